@@ -323,6 +323,39 @@ __device__ __forceinline__ int sroot(const volatile int *par, int x)
     return x;
 }
 
+// The same while other threads replace roots by border records (negative):
+// a node that holds one is a root.
+__device__ __forceinline__ int sroot_marked(const volatile int *par, int x)
+{
+    int p = par[x];
+    while (p >= 0 && p != x) {
+        x = p;
+        p = par[x];
+    }
+    return x;
+}
+
+// Index of the highest set bit of v, -1 when there is none (bfind).
+__device__ __forceinline__ int top_bit(uint32_t v)
+{
+    int r;
+    asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
+}
+
+// The two 16-bit halves selected from X (even positions) and Z (odd
+// positions) interleaved into one word: bits of half hf (0 or 1) of each.
+__device__ __forceinline__ uint32_t interleave16(uint32_t X, uint32_t Z, int hf)
+{
+    uint32_t v = __byte_perm(X, Z, hf ? 0x7362 : 0x5140);   // bytes x0 z0 x1 z1
+    uint32_t t = (v ^ (v >> 4)) & 0x00F000F0u;
+    v ^= t ^ (t << 4);
+    t = (v ^ (v >> 2)) & 0x0C0C0C0Cu;
+    v ^= t ^ (t << 2);
+    t = (v ^ (v >> 1)) & 0x22222222u;
+    return v ^ t ^ (t << 1);
+}
+
 // Packed per-root record written over a root's own forest entry once the
 // tile is labelled: INFO_BORDER | 0x8000 | slot for a piece that touches the
 // tile border (slot = its representative node), INFO_INTERIOR | spin << 14 |
@@ -440,6 +473,119 @@ __device__ void tile_label(volatile int *par, const uint32_t (*Hb)[TWW], const u
     __syncthreads();
 }
 
+// Connected components of the intra-tile bonds: B[y][2c] holds the right-link
+// bonds of word c of row y, B[y][2c + 1] its down-link bonds, both without the
+// links that leave the tile.  The tile is cut into 32 x 32 sub-tiles, one per
+// warp, lane = column:
+//   1. the warp goes down its 32 rows with every site's label in a register.
+//      A run (maximal chain of right bonds inside a sub-tile row) takes the
+//      label above its last bonded contact by one shuffle, or starts a new
+//      label, its own head, when it has none.  Labels are forest nodes: every
+//      site's entry is written once, pointing at the node its label was born
+//      at.  At T_c that settles 86% of the contacts with plain stores; the rest
+//      (a run whose contacts carry different labels: 86 of 499 a sub-tile,
+//      67 without repeats) are kept as a mask per row and united afterwards,
+//      lane = row;
+//   2. unions across the sub-tile boundaries inside the tile.
+// Links always hang the larger root under the smaller, so par[x] < x unless x
+// is a root and every root is the minimum local index of its piece; local
+// row-major order is the global order, so the root is the piece's minimum
+// site.  Forest indices are padded, y * PW + x, which keeps row-major order
+// and puts the rows of a column on distinct shared-memory banks.
+// The labelling is bound by instruction issue.  Uniting every contact by two
+// finds and a compare-and-swap, lane = row, cost 2.1K warp instructions a
+// sub-tile with 12.5 of 32 lanes active; this pass with the plain-store labels
+// and one code look-up a site took the 64-row tile kernel from 2.01 to 1.40 ms
+// at L=16384, T_c (111 -> 81M warp instructions a launch at L=4096).
+// Returns, to lane r, the heads of the runs of row r of the warp's sub-tile
+// that started a label (every root is one of them).
+template <int TH>
+__device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
+{
+    constexpr int NT = TileCfg<TH>::NT;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
+    const int rows = 32 * sx < tw ? min(32, th - y0) : 0;
+    uint32_t born = 0u, conf = 0u;
+    if (rows > 0) {
+        const uint32_t le = 0xFFFFFFFFu >> (31 - lane), gt = ~le;
+        int row = y0 * PW + 32 * sx;
+        uint2 hv = *reinterpret_cast<const uint2 *>(&B[y0][2 * sx]);
+        uint32_t heads = run_heads(hv.x);
+        int lab = row + top_bit(heads & le);
+        par[row + lane] = lab;
+        born = heads;
+#pragma unroll 4
+        for (int r = 1; r < rows; ++r) {
+            const uint32_t v = hv.y;   // down bonds from the row above
+            hv = *reinterpret_cast<const uint2 *>(&B[y0 + r][2 * sx]);
+            row += PW;
+            heads = ~(hv.x << 1);
+            const int hd = top_bit(heads & le);
+            const uint32_t n = heads & gt;                     // heads to the right: the run ends before them
+            const int c = top_bit(v & (n - 1u) & ~n);          // last contact at or left of the run's end
+            const bool has = c >= hd;
+            const int lc = __shfl_sync(0xFFFFFFFFu, lab, c);
+            const uint32_t cf = __ballot_sync(0xFFFFFFFFu, ((v >> lane) & 1u) && lab != lc);
+            const uint32_t nr = __ballot_sync(0xFFFFFFFFu, !has) & heads;
+            lab = has ? lc : row + hd;
+            par[row + lane] = lab;
+            if (lane == r) {
+                born = nr;
+                conf = cf;
+            }
+        }
+        __syncwarp();
+        const int base = (y0 + lane) * PW + 32 * sx;
+        int pa = -1, pb = -1;
+        for (; conf; conf &= conf - 1) {
+            const int i = base + __ffs(conf) - 1;
+            const int a = par[i - PW], b = par[i];
+            if (a != pa || b != pb) sunite(par, a, b);
+            pa = a;
+            pb = b;
+        }
+        if (lane >= rows) born = 0u;
+    }
+    __syncthreads();
+
+    // ---- 2. links across sub-tile boundaries: vertical boundaries between
+    //         sub-tile columns, horizontal ones between sub-tile rows.  A link
+    //         whose two sites point at the same nodes as those of the bonded
+    //         link before it along the boundary joins nothing new (a site's
+    //         entry is always in its own set, whatever unions are under way).
+    {
+        constexpr int NV = (TWW - 1) * TH;
+        constexpr int NH = (TH / 32 - 1) * TW;
+        for (int q = threadIdx.x; q < NV + NH; q += NT) {
+            int ia, ib, step;
+            bool before;
+            if (q < NV) {
+                const int bnd = q / TH + 1, y = q % TH;     // link (32 bnd - 1, y) - (32 bnd, y)
+                if (y >= th || !(B[y][2 * bnd - 2] >> 31)) continue;
+                before = y > 0 && (B[y - 1][2 * bnd - 2] >> 31);
+                ia = y * PW + 32 * bnd - 1;
+                ib = ia + 1;
+                step = PW;
+            } else {
+                const int r = q - NV;
+                const int bnd = r / TW + 1, x = r % TW;     // link (x, 32 bnd - 1) - (x, 32 bnd)
+                const int y = 32 * bnd - 1;
+                if (y + 1 >= th || !((B[y][2 * (x >> 5) + 1] >> (x & 31)) & 1u)) continue;
+                before = x > 0 && ((B[y][2 * ((x - 1) >> 5) + 1] >> ((x - 1) & 31)) & 1u);
+                ia = y * PW + x;
+                ib = ia + PW;
+                step = 1;
+            }
+            const int a = par[ia], b = par[ib];
+            if (before && par[ia - step] == a && par[ib - step] == b) continue;
+            sunite(par, a, b);
+        }
+    }
+    __syncthreads();
+    return born;
+}
+
 // ------------------------------------------------ global-memory union-find
 __device__ __forceinline__ int gload(const int32_t *p)
 {
@@ -519,18 +665,19 @@ __device__ __forceinline__ void cp_async_wait_all()
 // ------------------------------------------------------------ shared layout
 template <int TH>
 struct TileSmem {
-    int par[TH * PW];               // union-find forest over run heads (padded rows); in the
+    int par[TH * PW];               // union-find forest over the sites (padded rows); in the
                                     // finish half, the tile's site codes (TH * TW * 2 bytes)
-    uint32_t sp[TH + 1][TWW];       // spins as bits, row TH = halo row; in a tile narrower
-                                    // than TW, bit tw of a row = the halo column
-    uint32_t spx[TH / 32];          // halo column of a full-width tile: bit y = row y
-    uint32_t bh[TH][TWW];           // right-link bonds (bit x: link (x,y)-(x+1,y))
-    uint32_t bv[TH][TWW];           // down-link bonds
+    uint32_t sp[TH + 1][TWW];       // spins as bits, row TH = halo row
+    uint32_t spx[TH / 32];          // halo column (the site right of the tile's last): bit y = row y
+    // row y: first the raw draws (below), then the intra-tile bonds, [2c] the
+    // right links and [2c + 1] the down links of word c
+    __align__(16) uint32_t b[TH][2 * TWW];
     union {                         // never live at the same time:
-        uint32_t finfo[Slots<TH>::S];        // finish half: finals of the tile's own nodes
+        __align__(16) uint32_t finfo[Slots<TH>::S];   // finish half: finals of the tile's own nodes
         uint32_t spb[TH][TWW];               // start half: SPIN-stream bit of each site
-        long long red[TileCfg<TH>::NW][4];   // the reduction that ends each half
     } u;
+    int acc[4];                     // sums of the tile: bond_sum, mag (sweep k-1), nbonds, nclusters (sweep k)
+    unsigned long long acc_c2[2];   // RF_CSIZE: sum |C|^2 of sweep k-1 and of sweep k
     uint32_t pm[Slots<TH>::S][8];   // PCC: per border piece, columns and rows it occupies
 };
 
@@ -564,7 +711,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     constexpr int SPT = (S + NT - 1) / NT;   // node slots per thread
     constexpr int NQ = TH * TW / 8 / NT;     // 8-site groups per thread
     static_assert(NQ * 8 * NT == TH * TW, "tile sites must split into 8-site groups");
-    static_assert(TH * TWW == NT, "one 32-site word of the tile per thread");
+    static_assert(TH * TWW == NT && NW * 8 == TH, "one 32-site word of the tile per thread, eight rows per warp");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileSmem<TH> &sm = *reinterpret_cast<TileSmem<TH> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
@@ -585,29 +732,21 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     // column, the last tile row no down link in its last row
     const bool open_r = (F & FEAT_OPEN) && (R.flags & RF_OPEN) && t.tx == R.tiles_x - 1;
     const bool open_b = (F & FEAT_OPEN) && (R.flags & RF_OPEN) && t.ty == R.tiles_y - 1;
+    const bool csz = (F & FEAT_CSIZE) && (R.flags & RF_CSIZE) != 0;
+    const bool pcc = (F & FEAT_PCC) && (R.flags & RF_PCC) != 0;
     // site indices fit in 32 bits (N <= 2^30)
     const uint32_t uL = (uint32_t)L;
     const uint32_t gbase = (uint32_t)t.y0 * uL + (uint32_t)t.x0;   // global index of local site 0
     uint16_t *code = R.code + (size_t)t.lt * TH * TW;
-    // the intra-tile right bonds of word (y, c): the tile's last column links out
-    auto ih_of = [&](int y, int c) { return sm.bh[y][c] & valid_mask(c, t.tw - 1); };
-    // the spin word right of word (y, c), of which only bit 0 is used: the next
-    // word of the row, or the halo column of a full-width tile
-    auto right_of = [&](int y, int c) { return c + 1 < TWW ? sm.sp[y][c + 1] : sm.spx[y >> 5] >> (y & 31); };
-    // sets the halo-column spin of row y (the spin right of the tile's last column)
-    auto set_halo = [&](int y) {
-        if (t.tw == TW)
-            atomicOr(&sm.spx[y >> 5], 1u << (y & 31));
-        else
-            sm.sp[y][t.tw >> 5] |= 1u << (t.tw & 31);
-    };
+    // the thread's word of the tile: row wy, sites 32 wc .. 32 wc + 31
+    const int wy = tid >> 2, wc = tid & 3;
 
+    // ---- loads of the finish half, in flight during the draws
+    uint32_t fb = 0u, fr = 0u;
     if (fin) {
-        // ---- finish sweep k-1: resolve every site's cluster and flip it
-        const int jf = j - 1;
-        const bool last = j == R.nsweeps;
         // the tile's codes, 8 sites per 16-byte asynchronous copy straight
-        // into shared memory (the forest's space, unused until the labelling)
+        // into shared memory (the forest's space, unused until the labelling),
+        // and the finals of its own nodes
         const uint4 *code4 = reinterpret_cast<const uint4 *>(code);
         uint4 *scode4 = reinterpret_cast<uint4 *>(sm.par);
 #pragma unroll
@@ -615,13 +754,71 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             const int idx = tid + q * NT;
             if ((idx * 8) / TW < t.th) cp_async16(scode4 + idx, code4 + idx);
         }
-        for (int s = tid; s < S; s += NT) sm.u.finfo[s] = R.nfinal[(size_t)t.lt * S + s];
+        const uint32_t *nf = R.nfinal + (size_t)t.lt * S;
+        for (int s = tid; s < S / 4; s += NT) cp_async16(sm.u.finfo + 4 * s, nf + 4 * s);
         // the halos' finals (new spins of the top row of the tile below and of
-        // the left column of the tile to the right), issued with the codes
-        uint32_t fb = 0u, fr = 0u;
-        if (warp < TWW && 32 * warp + lane < t.tw) fb = R.nfinal[(size_t)t.g_down * S + SL::TOP + 32 * warp + lane];
+        // the left column of the tile to the right)
+        if (warp < TWW && tid < t.tw) fb = R.nfinal[(size_t)t.g_down * S + SL::TOP + tid];
         if (tid < t.th) fr = R.nfinal[(size_t)t.g_right * S + SL::LEFT + tid];
-        for (int w = tid; w < TH / 32; w += NT) sm.spx[w] = 0u;
+    }
+    if (tid < 4) sm.acc[tid] = 0;
+    if ((F & FEAT_CSIZE) && tid < 2) sm.acc_c2[tid] = 0ull;
+
+    // ---- Step 1 (Sec. I) of sweep k, its random part: link l = 2i + d draws
+    // word (l mod 4) of Philox(l/4, k, BOND), i.e. sites 2m and 2m+1 share
+    // block m.  Warp w draws rows 8w .. 8w+7, two at a time (four independent
+    // blocks in flight per lane): lane m the m-th and the (32+m)-th block of a
+    // row, counted from the one that holds the row's first site.  Four ballots
+    // per 32 blocks are the row's below-threshold bits with even and odd
+    // positions apart: x and z the right links, y and w the down links.  The
+    // thread that owns a word interleaves them (13 operations a word against
+    // a shuffle, a shift and two ballots a word for every lane of the warp).
+    const uint64_t k = R.sweep0 + (uint64_t)j;
+    const uint64_t thr = (F & FEAT_PCC) && (R.flags & RF_PCC) ? *R.thr_dev : R.thr;
+    const uint32_t klo = (uint32_t)k, khi = (uint32_t)(k >> 32);
+    const bool any_bond = start && thr != 0;      // t = 0: P = 0, nothing bonds
+    // an odd first site is the second one of its row's first block, so the
+    // row's 128 sites reach into a 65th block: lane r draws it for row r
+    uint32_t extra = 0u;
+    if (any_bond) {
+        const uint32_t tm1 = (uint32_t)(thr - 1);     // t in [1, 2^32] -> t - 1 fits 32 bits
+        const bool wide = t.tw > 64;                  // blocks 32 .. 63 of a row have sites in the tile
+        for (int i = 0; i < 8; i += 2) {
+            const int y = 8 * warp + i;
+            if (y >= t.th) break;
+            const uint32_t g0 = gbase + (uint32_t)y * uL;
+            const uint32_t b0 = (g0 >> 1) + lane, b2 = ((g0 + uL) >> 1) + lane;
+            const U4 r0 = philox4x32_10(b0, klo, khi, STREAM_BOND, R.key0, R.key1);
+            const U4 r2 = philox4x32_10(b2, klo, khi, STREAM_BOND, R.key0, R.key1);
+            U4 r1{}, r3{};
+            if (wide) {
+                r1 = philox4x32_10(b0 + 32, klo, khi, STREAM_BOND, R.key0, R.key1);
+                r3 = philox4x32_10(b2 + 32, klo, khi, STREAM_BOND, R.key0, R.key1);
+            }
+            auto ballots = [&](const U4 &r) {
+                return make_uint4(__ballot_sync(0xFFFFFFFFu, below(r.x, tm1)), __ballot_sync(0xFFFFFFFFu, below(r.y, tm1)),
+                                  __ballot_sync(0xFFFFFFFFu, below(r.z, tm1)), __ballot_sync(0xFFFFFFFFu, below(r.w, tm1)));
+            };
+            const uint4 q0 = ballots(r0), q1 = ballots(r1), q2 = ballots(r2), q3 = ballots(r3);
+            if (lane == 0) {
+                uint4 *raw = reinterpret_cast<uint4 *>(&sm.b[y][0]);
+                raw[0] = q0;
+                raw[1] = q1;
+                raw[2] = q2;
+                raw[3] = q3;
+            }
+        }
+        if ((uL | gbase) & 1u) {
+            const uint32_t g0 = gbase + (uint32_t)(8 * warp + (lane & 7)) * uL;
+            const U4 r = philox4x32_10((g0 >> 1) + 64u, klo, khi, STREAM_BOND, R.key0, R.key1);
+            extra = (below(r.x, tm1) ? 1u : 0u) | (below(r.y, tm1) ? 2u : 0u);
+        }
+    }
+
+    if (fin) {
+        // ---- finish sweep k-1: resolve every site's cluster and flip it
+        const bool last = j == R.nsweeps;
+        const uint4 *scode4 = reinterpret_cast<const uint4 *>(sm.par);
         cp_async_wait_all();
         __syncthreads();
 #pragma unroll
@@ -668,50 +865,17 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                 }
             }
         }
-        // bottom halo row: new spins of the top row of the tile below
+        // bottom halo row and right halo column
         if (warp < TWW) {
             const uint32_t word = __ballot_sync(0xFFFFFFFFu, (fb & FINAL_SPIN) != 0u);
             if (lane == 0) sm.sp[t.th][warp] = word;
         }
-        __syncthreads();
-        // right halo column: new spins of the left column of the tile to the right
-        if (fr & FINAL_SPIN) set_halo(tid);
-        __syncthreads();
-        long long bs = 0, mag = 0;
-        for (int w = tid; w < t.th * TWW; w += NT) {
-            const int y = w >> 2, c = w & 3;
-            const uint32_t vm = valid_mask(c, t.tw);
-            const uint32_t vr = open_r ? valid_mask(c, t.tw - 1) : vm;   // sites with a right link
-            const uint32_t vd = (open_b && y == t.th - 1) ? 0u : vm;      // sites with a down link
-            const uint32_t cur = sm.sp[y][c];
-            const uint32_t right = (cur >> 1) | (right_of(y, c) << 31);
-            const uint32_t down = sm.sp[y + 1][c];
-            bs += __popc(vr) - 2 * __popc((cur ^ right) & vr) + __popc(vd) - 2 * __popc((cur ^ down) & vd);
-            mag += 2 * __popc(cur & vm) - __popc(vm);
+        if (warp < TH / 32) {
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, (fr & FINAL_SPIN) != 0u);
+            if (lane == 0) sm.spx[warp] = word;
         }
-        // clusters that touch a tile border: their sizes were summed at their
-        // root nodes by the merge; each root node is in exactly one tile
-        long long c2 = 0;
-        if ((F & FEAT_CSIZE) && (R.flags & RF_CSIZE))
-            for (int s = tid; s < S; s += NT) {
-                const long long c = R.csize[(size_t)t.lt * S + s];
-                c2 += c * c;
-            }
-        long long v[4] = {bs, mag, c2, 0};
-        DevObs *o = R.obs + jf;
-        unsigned long long *const dst[4] = {&o->bond_sum, &o->mag, &o->csize2, nullptr};
-        block_sum_atomic<NT, 4>(v, dst, sm.u.red);
-        __syncthreads();
-    }
-
-    if (!start) return;
-
-    // ---- start sweep k
-    const uint64_t k = R.sweep0 + (uint64_t)j;
-    const uint64_t thr = (R.flags & RF_PCC) ? *R.thr_dev : R.thr;
-    if (!fin) {
+    } else {
         // first sweep of the call: spins (and halos) from global memory
-        for (int w = tid; w < TH / 32; w += NT) sm.spx[w] = 0u;
         for (int w = warp; w < (t.th + 1) * TWW; w += NW) {
             const int y = w >> 2, c = w & 3;
             const int x = 32 * c + lane;
@@ -721,328 +885,265 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             const uint32_t word = __ballot_sync(0xFFFFFFFFu, spin);
             if (lane == 0) sm.sp[y][c] = word;
         }
-        __syncthreads();
-        for (int y = tid; y < t.th; y += NT) {
-            const uint32_t gi = (uint32_t)(t.y0 + y) * uL + (uint32_t)((t.x0 + t.tw) % L);
-            if (R.spin[gi]) set_halo(y);
+        if (warp < TH / 32) {
+            int spin = 0;
+            if (tid < t.th) spin = R.spin[(uint32_t)(t.y0 + tid) * uL + (uint32_t)((t.x0 + t.tw) % L)];
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, spin);
+            if (lane == 0) sm.spx[warp] = word;
         }
-        __syncthreads();
     }
-    const bool pcc = (F & FEAT_PCC) && (R.flags & RF_PCC) != 0;
-    if (pcc)
-        for (int q = tid; q < S * 8; q += NT) (&sm.pm[0][0])[q] = 0u;
-    if (t.lt == 0 && tid == 0) {
-        R.obs[j].threshold = thr;
-        R.obs[j].spans_x = 0;
-        R.obs[j].spans_y = 0;
-    }
+    __syncthreads();
 
-    // Step 1 (Sec. I): bonds.  Link l = 2i + d draws word (l mod 4) of
-    // Philox(l/4, k, BOND), i.e. sites 2m and 2m+1 share block m.
-    const uint32_t klo = (uint32_t)k, khi = (uint32_t)(k >> 32);
-    const bool any_bond = thr != 0;               // t = 0: P = 0, nothing bonds
-    const uint32_t tm1 = (uint32_t)(thr - 1);     // t in [1, 2^32] -> t - 1 fits 32 bits
-    // the bonds of row y from its two horizontal-and-vertical draw words per
-    // 32-site word (rh, rv): keep the links whose spins agree, store them
-    // rows yA and yB at once: lane c < 4 takes word c of row yA, lane 4 + c
-    // word c of row yB (skipped when yB is past the tile)
-    auto store_rows = [&](int yA, const uint32_t (&rhA)[TWW], const uint32_t (&rvA)[TWW], int yB,
-                          const uint32_t (&rhB)[TWW], const uint32_t (&rvB)[TWW]) {
-        const bool second = lane >= TWW;
-        const int y = second ? yB : yA;
-        if (lane < 2 * TWW && y < t.th) {
-            const int c = lane & (TWW - 1);
-            const uint32_t rhc = second ? (c == 0 ? rhB[0] : c == 1 ? rhB[1] : c == 2 ? rhB[2] : rhB[3])
-                                        : (c == 0 ? rhA[0] : c == 1 ? rhA[1] : c == 2 ? rhA[2] : rhA[3]);
-            const uint32_t rvc = second ? (c == 0 ? rvB[0] : c == 1 ? rvB[1] : c == 2 ? rvB[2] : rvB[3])
-                                        : (c == 0 ? rvA[0] : c == 1 ? rvA[1] : c == 2 ? rvA[2] : rvA[3]);
-            const uint32_t vm = valid_mask(c, t.tw);
-            const uint32_t vr = open_r ? valid_mask(c, t.tw - 1) : vm;
-            const uint32_t vd = (open_b && y == t.th - 1) ? 0u : vm;
-            const uint32_t cur = sm.sp[y][c];
-            const uint32_t right = (cur >> 1) | (right_of(y, c) << 31);
-            const uint32_t down = sm.sp[y + 1][c];
-            const uint32_t h = rhc & ~(cur ^ right) & vr;
-            const uint32_t v = rvc & ~(cur ^ down) & vd;
-            sm.bh[y][c] = h;
-            sm.bv[y][c] = v;
+    // ---- the thread's word: spin agreement along its links, the sums of
+    //      sweep k-1 and the bonds of sweep k
+    const uint32_t vm = wy < t.th ? valid_mask(wc, t.tw) : 0u;
+    const int last_c = (t.tw - 1) >> 5, last_b = (t.tw - 1) & 31;   // the tile's last column
+    {
+        uint32_t eqr = 0u, eqd = 0u, cur = 0u;   // links that exist and join equal spins
+        uint32_t vr = vm, vd = vm;
+        if (wy < t.th) {
+            if (open_r) vr = valid_mask(wc, t.tw - 1);    // sites with a right link
+            if (open_b && wy == t.th - 1) vd = 0u;        // sites with a down link
+            cur = sm.sp[wy][wc];
+            uint32_t right = __funnelshift_r(cur, wc + 1 < TWW ? sm.sp[wy][wc + 1] : 0u, 1);
+            // (bits past the tile's last column are zero)
+            if (wc == last_c) right |= ((sm.spx[wy >> 5] >> (wy & 31)) & 1u) << last_b;
+            eqr = ~(cur ^ right) & vr;
+            eqd = ~(cur ^ sm.sp[wy + 1][wc]) & vd;
         }
-    };
-    auto store_row = [&](int y, const uint32_t (&rh)[TWW], const uint32_t (&rv)[TWW]) {
-        store_rows(y, rh, rv, t.th, rh, rv);
-    };
-    // aligned row: lane l drew the blocks of sites (2l, 2l+1) (r0) and
-    // (64+2l, 65+2l) (r1); lane x of each 32-site word fetches its two bits
-    // by shuffle
-    auto draws_aligned = [&](const U4 &r0, const U4 &r1, uint32_t (&rh)[TWW], uint32_t (&rv)[TWW]) {
-        const uint32_t nib0 = (below(r0.x, tm1) ? 1u : 0u) | (below(r0.y, tm1) ? 2u : 0u) |
-                              (below(r0.z, tm1) ? 4u : 0u) | (below(r0.w, tm1) ? 8u : 0u);
-        const uint32_t nib1 = (below(r1.x, tm1) ? 1u : 0u) | (below(r1.y, tm1) ? 2u : 0u) |
-                              (below(r1.z, tm1) ? 4u : 0u) | (below(r1.w, tm1) ? 8u : 0u);
-#pragma unroll
-        for (int q = 0; q < TWW; ++q) {
-            const uint32_t n = __shfl_sync(0xFFFFFFFFu, q < 2 ? nib0 : nib1, 16 * (q & 1) + (lane >> 1)) >>
-                               (2 * (lane & 1));
-            rh[q] = __ballot_sync(0xFFFFFFFFu, n & 1u);
-            rv[q] = __ballot_sync(0xFFFFFFFFu, n & 2u);
-        }
-    };
-    if (any_bond && (uL & 1u) == 0) {
-        // even L: every row starts on an even site; two rows per pass, four
-        // independent Philox blocks in flight per lane
-        for (int y = warp; y < t.th; y += 2 * NW) {
-            const int y2 = y + NW;
-            const uint32_t b0 = ((gbase + (uint32_t)y * uL) >> 1) + lane;
-            const uint32_t b2 = ((gbase + (uint32_t)y2 * uL) >> 1) + lane;
-            const U4 r0 = philox4x32_10(b0, klo, khi, STREAM_BOND, R.key0, R.key1);
-            const U4 r1 = philox4x32_10(b0 + 32, klo, khi, STREAM_BOND, R.key0, R.key1);
-            const U4 r2 = philox4x32_10(b2, klo, khi, STREAM_BOND, R.key0, R.key1);
-            const U4 r3 = philox4x32_10(b2 + 32, klo, khi, STREAM_BOND, R.key0, R.key1);
-            uint32_t rh[TWW], rv[TWW], rh2[TWW], rv2[TWW];
-            draws_aligned(r0, r1, rh, rv);
-            draws_aligned(r2, r3, rh2, rv2);
-            store_rows(y, rh, rv, y2, rh2, rv2);
-        }
-    } else {
-        for (int y = warp; y < t.th; y += NW) {
-            const uint32_t G0 = gbase + (uint32_t)y * uL;
-            uint32_t rh[TWW], rv[TWW];
-            if (!any_bond) {
-#pragma unroll
-                for (int q = 0; q < TWW; ++q) rh[q] = rv[q] = 0u;
-            } else if ((G0 & 1u) == 0) {
-                const uint32_t b0 = (G0 >> 1) + lane;
-                const U4 r0 = philox4x32_10(b0, klo, khi, STREAM_BOND, R.key0, R.key1);
-                const U4 r1 = philox4x32_10(b0 + 32, klo, khi, STREAM_BOND, R.key0, R.key1);
-                draws_aligned(r0, r1, rh, rv);
-            } else {
-                // odd row start (odd L): every site draws its own block
-#pragma unroll
-                for (int q = 0; q < TWW; ++q) {
-                    const uint32_t gi = G0 + 32 * q + lane;
-                    const U4 r = philox4x32_10(gi >> 1, klo, khi, STREAM_BOND, R.key0, R.key1);
-                    const bool odd = gi & 1u;
-                    rh[q] = __ballot_sync(0xFFFFFFFFu, below(odd ? r.z : r.x, tm1));
-                    rv[q] = __ballot_sync(0xFFFFFFFFu, below(odd ? r.w : r.y, tm1));
+        if (fin) {
+            // bond_sum: +1 a link between equal spins, -1 otherwise
+            const int bs = 2 * (__popc(eqr) + __popc(eqd)) - __popc(vr) - __popc(vd);
+            const int mag = 2 * __popc(cur) - __popc(vm);
+            const int ws = __reduce_add_sync(0xFFFFFFFFu, bs), wm = __reduce_add_sync(0xFFFFFFFFu, mag);
+            if (lane == 0) {
+                atomicAdd(&sm.acc[0], ws);
+                atomicAdd(&sm.acc[1], wm);
+            }
+            // clusters that touch a tile border: their sizes were summed at their
+            // root nodes by the merge; each root node is in exactly one tile
+            if (csz) {
+                unsigned long long c2 = 0ull;
+                for (int s = tid; s < S; s += NT) {
+                    const long long c = R.csize[(size_t)t.lt * S + s];
+                    c2 += (unsigned long long)(c * c);
                 }
-            }
-            store_row(y, rh, rv);
-        }
-    }
-    // The SPIN-stream bit of every site of the tile, for the clusters that end
-    // inside it (Sec. I step 3: one new random spin per cluster): bit (g mod
-    // 128) of Philox(g / 128, k, SPIN) for a site of global index g.  A row's
-    // 128 sites span the two blocks from the one holding its first site; one
-    // thread per row draws them and keeps the row's 128 bits.
-    for (int y = tid; y < t.th; y += NT) {
-        const uint32_t g0 = gbase + (uint32_t)y * uL;
-        const uint32_t pos = g0 & 127u;
-        const U4 r0 = philox4x32_10(g0 >> 7, klo, khi, STREAM_SPIN, R.key0, R.key1);
-        U4 r1 = r0;
-        if (pos) r1 = philox4x32_10((g0 >> 7) + 1, klo, khi, STREAM_SPIN, R.key0, R.key1);
-        // the 8 words from the first one the row needs: words pos/32 .. pos/32 + 4
-        uint32_t w[5];
-        switch (pos >> 5) {
-        case 0: w[0] = r0.x; w[1] = r0.y; w[2] = r0.z; w[3] = r0.w; w[4] = r1.x; break;
-        case 1: w[0] = r0.y; w[1] = r0.z; w[2] = r0.w; w[3] = r1.x; w[4] = r1.y; break;
-        case 2: w[0] = r0.z; w[1] = r0.w; w[2] = r1.x; w[3] = r1.y; w[4] = r1.z; break;
-        default: w[0] = r0.w; w[1] = r1.x; w[2] = r1.y; w[3] = r1.z; w[4] = r1.w; break;
-        }
-#pragma unroll
-        for (int c = 0; c < TWW; ++c) sm.u.spb[y][c] = __funnelshift_r(w[c], w[c + 1], pos & 31u);
-    }
-    __syncthreads();
-
-    long long nb = 0;
-    for (int w = tid; w < t.th * TWW; w += NT) {
-        const int y = w >> 2, c = w & 3;
-        nb += __popc(sm.bh[y][c]) + __popc(sm.bv[y][c]);
-    }
-    // crossing bonds: right edge (bit tw-1 of each row), bottom edge (row th-1)
-    for (int q = warp; q <= TH / 32; q += NW) {
-        if (q < TH / 32) {
-            const int y = 32 * q + lane;
-            const int bit = (y < t.th) ? (sm.bh[y][(t.tw - 1) >> 5] >> ((t.tw - 1) & 31)) & 1 : 0;
-            const uint32_t word = __ballot_sync(0xFFFFFFFFu, bit);
-            if (lane == 0) R.cross[(size_t)t.lt * CROSS_WORDS + q] = word;
-        } else if (lane < TWW) {
-            R.cross[(size_t)t.lt * CROSS_WORDS + TWW + lane] = sm.bv[t.th - 1][lane];
-        }
-    }
-    if (j == R.nsweeps - 1) {
-        // the last sweep of the call keeps its bonds for sw_get_bonds
-        uint32_t *bb = R.bondbits + (size_t)t.lt * TH * 2 * TWW;
-        for (int w = tid; w < t.th * TWW; w += NT) {
-            const int y = w >> 2, c = w & 3;
-            bb[y * 2 * TWW + c] = sm.bh[y][c];
-            bb[y * 2 * TWW + TWW + c] = sm.bv[y][c];
-        }
-    }
-
-    // Step 2 inside the tile (Hoshen-Kopelman's role in Sec. II.A slave step 1)
-    tile_label<TH>(sm.par, sm.bh, sm.bv, t.th, t.tw);
-
-    // One node per border site: key = global index of the piece's local root,
-    // parent = the piece's first border slot (the representative).
-    int rs[SPT];
-#pragma unroll
-    for (int q = 0; q < SPT; ++q) {
-        const int s = tid + q * NT;
-        int site;
-        rs[q] = -1;
-        if (s < S && slot_site<TH>(s, t.tw, t.th, site)) {
-            const int sy = site / TW, c = (site % TW) >> 5;
-            rs[q] = sroot(sm.par, head_of(run_heads(ih_of(sy, c)), sy * PW + 32 * c, site & 31));
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < SPT; ++q)
-        if (rs[q] >= 0) atomicMin((int *)&sm.par[rs[q]], (int)(INFO_BORDER | (uint32_t)(tid + q * NT)));
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < SPT; ++q) {
-        const int s = tid + q * NT;
-        if (s >= S) break;
-        const size_t node = (size_t)t.lt * S + s;
-        if (rs[q] >= 0) {
-            const int rep = sm.par[rs[q]] & 0x3FF;
-            R.npar[node] = (int32_t)((size_t)t.lt * S + rep);
-            R.nkey[node] = (int32_t)((gbase + (uint32_t)(rs[q] / PW) * uL + (uint32_t)(rs[q] % PW)) |
-                                     (rep == s ? KEY_REP : 0u));
-        } else {
-            R.npar[node] = (int32_t)node;
-            R.nkey[node] = (int32_t)KEY_NONE;
-        }
-        if ((F & FEAT_CSIZE) && (R.flags & RF_CSIZE)) R.csize[node] = 0;   // the merge adds piece sizes at root nodes
-    }
-    // Every run head learns its root; every interior root gets its record
-    // (the cluster's new spin, Sec. I step 3, drawn here) and is counted.
-    // A walk stops at a root, a border record or an interior record, and each
-    // thread writes only its own heads, so concurrent walks see ancestors.
-    long long ncl_interior = 0;
-    for (int w = tid; w < t.th * TWW; w += NT) {
-        const int y = w % t.th, c = w / t.th;   // a warp covers consecutive rows
-        const int base = y * PW + 32 * c;
-        for (uint32_t bits = run_heads(ih_of(y, c)); bits; bits &= bits - 1) {
-            const int hx = __ffs(bits) - 1;
-            const int hd = base + hx;
-            int x = hd, p = sm.par[x];
-            while (p != x && p >= 0 && (uint32_t)p < INFO_INTERIOR) {
-                x = p;
-                p = sm.par[x];
-            }
-            if (x != hd) {
-                // the root's record itself where it is already there (codes
-                // then need one load); the root otherwise.  Cluster sizes add
-                // at roots, so the feature variant keeps root indices.
-                sm.par[hd] = (!(F & FEAT_CSIZE) && (uint32_t)p >= INFO_INTERIOR && p != x) ? p : x;
-            } else if (p == hd && 32 * c + hx < t.tw) {
-                // an interior root inside the tile: its site's SPIN-stream bit
-                const uint32_t spin = (sm.u.spb[y][c] >> hx) & 1u;
-                sm.par[hd] = (int)(INFO_INTERIOR | (spin << 14) | (uint32_t)(y * TW + 32 * c + hx));
-                ++ncl_interior;
+                if (c2) atomicAdd(&sm.acc_c2[0], c2);
             }
         }
-    }
-    __syncthreads();
-    const bool csz = (F & FEAT_CSIZE) && (R.flags & RF_CSIZE) != 0;
-    if (csz) {
-        // cluster sizes: every run adds its length to bits 16-30 of its root's
-        // record (a piece holds at most TW*TH = 2^14 sites, an interior
-        // cluster at most (TW-2)(TH-2) < 2^14, so neither field overflows
-        // into the record's flag bits); the codes below read bits 0-15 only
-        for (int w = tid; w < t.th * TWW; w += NT) {
-            const int y = w % t.th, c = w / t.th;
-            const int base = y * PW + 32 * c;
-            const int vw = min(32, t.tw - 32 * c);   // real sites in this word
-            for (uint32_t bits = run_heads(ih_of(y, c)); bits;) {
-                const int hx = __ffs(bits) - 1;
-                bits &= bits - 1;
-                if (hx >= vw) break;
-                const int nx = bits ? __ffs(bits) - 1 : 32;
-                const int v = sm.par[base + hx];
-                const int root = (v < 0 || (uint32_t)v >= INFO_INTERIOR) ? base + hx : v;
-                atomicAdd((int *)&sm.par[root], (min(nx, vw) - hx) << 16);
-            }
-        }
-    }
-    // Every site's 2-byte code (the low half of its root's record): border
-    // pieces by node slot, interior clusters by local root and new spin.
-    // 8 sites per 16-byte store.
-    uint4 *code4 = reinterpret_cast<uint4 *>(code);
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int idx = tid + q * NT;
-        const int y = (idx * 8) / TW, xb = (idx * 8) % TW;
-        if (y >= t.th) continue;
-        uint32_t wv[4] = {0u, 0u, 0u, 0u};
-        const int c = xb >> 5;
-        const uint32_t heads = run_heads(ih_of(y, c));
-        const int base = y * PW + 32 * c;
-        int slot = -1;            // PCC: border piece of the sites gathered in cols
-        uint32_t cols = 0u;
-        int info = 0;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int x = xb + e;
-            if (x >= t.tw) break;
-            // a site inside a run shares the run head's code: look up only
-            // where a run starts (and for the group's first site)
-            if (e == 0 || ((heads >> (x & 31)) & 1u)) {
-                const int v = sm.par[e == 0 ? head_of(heads, base, x & 31) : base + (x & 31)];
-                info = ((uint32_t)v >= INFO_INTERIOR) ? v : sm.par[v];   // records: negative or >= INFO_INTERIOR
-            }
-            wv[e >> 1] |= ((uint32_t)info & 0xFFFFu) << (16 * (e & 1));
-            if (pcc && info < 0) {
-                // the columns and rows each border piece occupies (only a
-                // piece touching the border can belong to a spanning cluster)
-                const int sl = info & 0x3FF;
-                if (sl != slot) {
-                    if (slot >= 0) {
-                        atomicOr(&sm.pm[slot][c], cols);
-                        atomicOr(&sm.pm[slot][4 + (y >> 5)], 1u << (y & 31));
+        if (start) {
+            uint32_t rh = 0u, rv = 0u;   // links drawn below the threshold
+            if (any_bond) {
+                const uint4 raw = *reinterpret_cast<const uint4 *>(&sm.b[wy][4 * (wc >> 1)]);
+                rh = interleave16(raw.x, raw.z, wc & 1);
+                rv = interleave16(raw.y, raw.w, wc & 1);
+                if ((uL | gbase) & 1u) {
+                    // rows that start on an odd site are one site ahead of their blocks
+                    const uint32_t ex = __shfl_sync(0xFFFFFFFFu, extra, lane >> 2);
+                    uint32_t nh = __shfl_down_sync(0xFFFFFFFFu, rh, 1), nv = __shfl_down_sync(0xFFFFFFFFu, rv, 1);
+                    if (wc == TWW - 1) {
+                        nh = ex;
+                        nv = ex >> 1;
                     }
-                    slot = sl;
-                    cols = 0u;
-                }
-                cols |= 1u << (x & 31);
-            }
-        }
-        if (slot >= 0) {
-            atomicOr(&sm.pm[slot][c], cols);
-            atomicOr(&sm.pm[slot][4 + (y >> 5)], 1u << (y & 31));
-        }
-        code4[idx] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-    }
-    if (pcc) {
-        __syncthreads();
-        for (int q = tid; q < S * 8; q += NT) R.pmask[(size_t)t.lt * S * 8 + q] = (&sm.pm[0][0])[q];
-    }
-    long long c2 = 0;
-    if (csz) {
-        // every root: an interior cluster adds its |C|^2; a border piece
-        // hands its size to its representative node for the merge
-        __syncthreads();
-        for (int w = tid; w < t.th * TWW; w += NT) {
-            const int y = w % t.th, c = w / t.th;
-            const int base = y * PW + 32 * c;
-            const int vw = min(32, t.tw - 32 * c);
-            for (uint32_t bits = run_heads(ih_of(y, c)) & valid_mask(0, vw); bits; bits &= bits - 1) {
-                const int v = sm.par[base + __ffs(bits) - 1];
-                if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
-                    R.psize[(size_t)t.lt * S + (v & 0x3FF)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
-                } else if ((uint32_t)v >= INFO_INTERIOR) {   // bits 16-29 (bit 30 is the flag)
-                    const long long size = ((uint32_t)v >> 16) & 0x3FFFu;
-                    c2 += size * size;
+                    if ((gbase + (uint32_t)wy * uL) & 1u) {
+                        rh = __funnelshift_r(rh, nh, 1);
+                        rv = __funnelshift_r(rv, nv, 1);
+                    }
                 }
             }
+            const uint32_t h = rh & eqr, v = rv & eqd;
+            const int nb = __reduce_add_sync(0xFFFFFFFFu, __popc(h) + __popc(v));
+            if (lane == 0) atomicAdd(&sm.acc[2], nb);
+            // crossing bonds: right edge (the last column's bit of every row, a
+            // warp's eight rows a byte), bottom edge (the last row's down links)
+            {
+                uint32_t e = __ballot_sync(0xFFFFFFFFu, wc == last_c && ((h >> last_b) & 1u)) >> last_c;
+                e &= 0x11111111u;            // bit 4 r: row r
+                e = (e | (e >> 3)) & 0x03030303u;
+                e = (e | (e >> 6)) & 0x000F000Fu;
+                e = (e | (e >> 12)) & 0xFFu;
+                uint32_t *cross = R.cross + (size_t)t.lt * CROSS_WORDS;
+                if (lane == 0) reinterpret_cast<uint8_t *>(cross)[warp] = (uint8_t)e;
+                if (wy == t.th - 1) cross[TWW + wc] = v;
+            }
+            if (j == R.nsweeps - 1 && wy < t.th) {
+                // the last sweep of the call keeps its bonds for sw_get_bonds
+                uint32_t *bb = R.bondbits + (size_t)t.lt * TH * 2 * TWW + wy * 2 * TWW;
+                bb[wc] = h;
+                bb[TWW + wc] = v;
+            }
+            __syncwarp();   // the warp's rows: every draw is read before it is overwritten
+            *reinterpret_cast<uint2 *>(&sm.b[wy][2 * wc]) =
+                make_uint2(h & valid_mask(wc, t.tw - 1), wy < t.th - 1 ? v : 0u);
         }
     }
-    long long v4[4] = {nb, ncl_interior, c2, 0};
-    DevObs *o = R.obs + j;
-    unsigned long long *const dst[4] = {&o->nbonds, &o->nclusters, &o->csize2, nullptr};
-    block_sum_atomic<NT, 4>(v4, dst, sm.u.red);
+    if (start) {
+        // The SPIN-stream bit of every site of the tile, for the clusters that end
+        // inside it (Sec. I step 3: one new random spin per cluster): bit (g mod
+        // 128) of Philox(g / 128, k, SPIN) for a site of global index g.  A row's
+        // 128 sites span the two blocks from the one holding its first site; one
+        // thread per row draws them and keeps the row's 128 bits.
+        if (tid < t.th) {
+            const int y = tid;
+            const uint32_t g0 = gbase + (uint32_t)y * uL;
+            const uint32_t pos = g0 & 127u;
+            const U4 r0 = philox4x32_10(g0 >> 7, klo, khi, STREAM_SPIN, R.key0, R.key1);
+            U4 r1 = r0;
+            if (pos) r1 = philox4x32_10((g0 >> 7) + 1, klo, khi, STREAM_SPIN, R.key0, R.key1);
+            // the 8 words from the first one the row needs: words pos/32 .. pos/32 + 4
+            uint32_t w[5];
+            switch (pos >> 5) {
+            case 0: w[0] = r0.x; w[1] = r0.y; w[2] = r0.z; w[3] = r0.w; w[4] = r1.x; break;
+            case 1: w[0] = r0.y; w[1] = r0.z; w[2] = r0.w; w[3] = r1.x; w[4] = r1.y; break;
+            case 2: w[0] = r0.z; w[1] = r0.w; w[2] = r1.x; w[3] = r1.y; w[4] = r1.z; break;
+            default: w[0] = r0.w; w[1] = r1.x; w[2] = r1.y; w[3] = r1.z; w[4] = r1.w; break;
+            }
+#pragma unroll
+            for (int c = 0; c < TWW; ++c) sm.u.spb[y][c] = __funnelshift_r(w[c], w[c + 1], pos & 31u);
+        }
+        if (pcc)
+            for (int q = tid; q < S * 8; q += NT) (&sm.pm[0][0])[q] = 0u;
+        if (t.lt == 0 && tid == 0) {
+            R.obs[j].threshold = thr;
+            R.obs[j].spans_x = 0;
+            R.obs[j].spans_y = 0;
+        }
+    }
+    __syncthreads();
+
+    if (start) {
+        // Step 2 inside the tile (Hoshen-Kopelman's role in Sec. II.A slave step 1)
+        uint32_t born = tile_label_rows<TH>(sm.par, sm.b, t.th, t.tw);
+
+        // One node per border site: key = global index of the piece's local root,
+        // parent = the piece's first border slot (the representative).
+        int rs[SPT];
+#pragma unroll
+        for (int q = 0; q < SPT; ++q) {
+            const int s = tid + q * NT;
+            int site;
+            rs[q] = -1;
+            if (s < S && slot_site<TH>(s, t.tw, t.th, site)) {
+                rs[q] = sroot_marked(sm.par, site + site / TW);   // PW = TW + 1
+                atomicMin(&sm.par[rs[q]], (int)(INFO_BORDER | (uint32_t)s));
+            }
+        }
+        __syncthreads();
+        // Every interior root gets its record (the cluster's new spin, Sec. I
+        // step 3, drawn above) and is counted: lane r of a warp checks the nodes
+        // born in row r of its sub-tile.
+        {
+            const int sx = warp & (TWW - 1), y = 32 * (warp / TWW) + lane;
+            const int base = y * PW + 32 * sx;
+            born &= valid_mask(sx, t.tw);
+            int ncl = 0;
+            for (uint32_t bits = born; bits; bits &= bits - 1) {
+                const int hx = __ffs(bits) - 1;
+                if (sm.par[base + hx] == base + hx) {
+                    const uint32_t spin = (sm.u.spb[y][sx] >> hx) & 1u;
+                    sm.par[base + hx] = (int)(INFO_INTERIOR | (spin << 14) | (uint32_t)(y * TW + 32 * sx + hx));
+                    ++ncl;
+                }
+            }
+            ncl = __reduce_add_sync(0xFFFFFFFFu, ncl);
+            if (lane == 0 && ncl) atomicAdd(&sm.acc[3], ncl);
+        }
+#pragma unroll
+        for (int q = 0; q < SPT; ++q) {
+            const int s = tid + q * NT;
+            if (s >= S) break;
+            const size_t node = (size_t)t.lt * S + s;
+            if (rs[q] >= 0) {
+                const int rep = sm.par[rs[q]] & 0x3FF;
+                R.npar[node] = (int32_t)((size_t)t.lt * S + rep);
+                R.nkey[node] = (int32_t)((gbase + (uint32_t)(rs[q] / PW) * uL + (uint32_t)(rs[q] % PW)) |
+                                         (rep == s ? KEY_REP : 0u));
+            } else {
+                R.npar[node] = (int32_t)node;
+                R.nkey[node] = (int32_t)KEY_NONE;
+            }
+            if (csz) R.csize[node] = 0;   // the merge adds piece sizes at root nodes
+        }
+        __syncthreads();
+        // Every site's 2-byte code, the low half of its root's record: border
+        // pieces by node slot, interior clusters by local root and new spin.
+        // Lane = column: a site's entry, its label's and so on up to the root
+        // (2.0 steps at T_c for the slowest lane of a row).
+        {
+            const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
+            const int rows = min(32, t.th - y0);
+            const int x = 32 * sx + lane;
+            const bool site = x < t.tw;
+            uint16_t *cp = code + y0 * TW + x;
+            const int *pp = sm.par + y0 * PW + x;
+#pragma unroll 4
+            for (int r = 0; r < rows; ++r) {
+                int v = site ? pp[r * PW] : (int)INFO_BORDER;
+                int root = (y0 + r) * PW + x;
+                while ((uint32_t)v < INFO_INTERIOR) {   // records: negative or >= INFO_INTERIOR
+                    root = v;
+                    v = sm.par[v];
+                }
+                cp[r * TW] = site ? (uint16_t)v : (uint16_t)0;
+                if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) {
+                    // one lane per run (its head) for the whole run
+                    const uint32_t heads = run_heads(sm.b[y0 + r][2 * sx]);
+                    const uint32_t n = lane < 31 ? heads & (0xFFFFFFFFu << (lane + 1)) : 0u;
+                    const uint32_t run = (n - 1u) & ~n & (0xFFFFFFFFu << lane);
+                    if (site && ((heads >> lane) & 1u)) {
+                        // cluster sizes: every run adds its length to bits 16-30 of its root's
+                        // record (a piece holds at most TW*TH = 2^14 sites, an interior
+                        // cluster at most (TW-2)(TH-2) < 2^14, so neither field overflows
+                        // into the record's flag bits); the codes read bits 0-15 only
+                        if (csz) atomicAdd(&sm.par[root], __popc(run & valid_mask(sx, t.tw)) << 16);
+                        if (pcc && v < 0) {
+                            // the columns and rows each border piece occupies (only a
+                            // piece touching the border can belong to a spanning cluster)
+                            atomicOr(&sm.pm[v & 0x3FF][sx], run & valid_mask(sx, t.tw));
+                            atomicOr(&sm.pm[v & 0x3FF][4 + ((y0 + r) >> 5)], 1u << ((y0 + r) & 31));
+                        }
+                    }
+                }
+            }
+        }
+        if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) {
+            __syncthreads();
+            if (pcc)
+                for (int q = tid; q < S * 8; q += NT) R.pmask[(size_t)t.lt * S * 8 + q] = (&sm.pm[0][0])[q];
+            if (csz) {
+                // every root: an interior cluster adds its |C|^2; a border piece
+                // hands its size to its representative node for the merge
+                const int sx = warp & (TWW - 1), y = 32 * (warp / TWW) + lane;
+                unsigned long long c2 = 0ull;
+                for (uint32_t bits = born; bits; bits &= bits - 1) {
+                    const int v = sm.par[y * PW + 32 * sx + __ffs(bits) - 1];
+                    if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
+                        R.psize[(size_t)t.lt * S + (v & 0x3FF)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
+                    } else if ((uint32_t)v >= INFO_INTERIOR) {   // bits 16-29 (bit 30 is the flag)
+                        const unsigned long long size = ((uint32_t)v >> 16) & 0x3FFFu;
+                        c2 += size * size;
+                    }
+                }
+                if (c2) atomicAdd(&sm.acc_c2[1], c2);
+                __syncthreads();
+            }
+        }
+    }
+    // the tile's sums (every contribution but a sweep's own csize2 was added
+    // before a barrier above)
+    if (tid < 4) {
+        const int half = tid >> 1;            // 0: sweep k-1, 1: sweep k
+        if (half == 0 ? fin : start) {
+            DevObs *o = R.obs + (j - 1 + half);
+            const long long v = sm.acc[tid];
+            unsigned long long *dst = tid == 0 ? &o->bond_sum : tid == 1 ? &o->mag : tid == 2 ? &o->nbonds : &o->nclusters;
+            if (v) atomicAdd(dst, (unsigned long long)v);
+        }
+    } else if ((F & FEAT_CSIZE) && tid < 6) {
+        const int half = tid - 4;
+        if (csz && (half == 0 ? fin : start) && sm.acc_c2[half])
+            atomicAdd(&R.obs[j - 1 + half].csize2, sm.acc_c2[half]);
+    }
 }
 
 // ------------------------------------------------ union-find with offsets
