@@ -34,7 +34,7 @@ constexpr int CROSS_WORDS = 8;    // per tile: 4 words right-edge bits, 4 words 
 
 // 30-bit global roots: the GPU path supports N = L*L <= 2^30.
 constexpr uint32_t ROOT_MASK = 0x3FFFFFFFu;
-constexpr uint32_t FINAL_SPIN = 0x40000000u;
+constexpr uint32_t FINAL_SPIN = 0x80000000u;
 // A node key is a 30-bit site index (bits 0-29) plus KEY_REP; an edge slot
 // past the tile's sites holds KEY_NONE, outside that range, so it differs
 // from every real key up to site 2^30 - 1 (the corner of an L = 32768 lattice).
@@ -43,10 +43,14 @@ constexpr uint32_t KEY_REP = 0x40000000u;    // the node represents its piece
 constexpr uint32_t KEY_MASK = 0x3FFFFFFFu;
 
 // 2-byte tile-local cluster code of a site, written when a sweep starts and
-// read when it finishes.
-constexpr uint16_t CODE_BORDER = 0x8000u;   // bits 0-9: the piece's node slot
-constexpr uint16_t CODE_SPIN = 0x4000u;     // interior: the cluster's new spin
-constexpr uint16_t CODE_ROOT = 0x3FFFu;     // interior: tile-local root index
+// read when it finishes: the byte offset (4 x index) into the table of the
+// tile's finals, a piece's node slot, or one of the two entries after the
+// slots (an interior cluster's new spin, 0 or 1).  The last sweep of a call
+// writes CODE_LAST | spin << 14 | tile-local root index for the sites of
+// interior clusters instead: its finish also writes the labels.
+constexpr uint32_t CODE_LAST = 0x8000u;
+constexpr uint32_t CODE_SPIN = 0x4000u;
+constexpr uint32_t CODE_ROOT = 0x3FFFu;
 
 // Philox streams (counter word 3).
 constexpr uint32_t STREAM_INIT = 0u, STREAM_BOND = 1u, STREAM_SPIN = 2u;
@@ -281,6 +285,27 @@ __device__ __forceinline__ void sunite(volatile int *par, int a, int b)
     }
 }
 
+// As sunite, with STEPS tries that need no finds first: hang the larger of the
+// two nodes under the smaller if it is still a root, else go on from its
+// parent.  (A root a > b holds no node of smaller index, so b's set is another
+// one; b itself need not be a root.)  Most links join fresh nodes and end with
+// the first swap; the finds keep the trees shallow where many meet in one
+// set (hooks alone took 1.49 ms at L=16384, T=2.0, where three and then finds
+// take 1.19; finds alone 1.22).
+template <int STEPS>
+__device__ __forceinline__ void shook(volatile int *par, int a, int b)
+{
+    for (int i = 0; i < STEPS; ++i) {
+        if (a == b) return;
+        const int hi = max(a, b), lo = min(a, b);
+        const int old = atomicCAS((int *)&par[hi], hi, lo);
+        if (old == hi) return;
+        a = old;
+        b = lo;
+    }
+    sunite(par, a, b);
+}
+
 // As sunite, reporting whether this call linked two sets (false: a and b
 // were already in one set).
 __device__ __forceinline__ bool sunite_linked(volatile int *par, int a, int b)
@@ -357,12 +382,13 @@ __device__ __forceinline__ uint32_t interleave16(uint32_t X, uint32_t Z, int hf)
 }
 
 // Packed per-root record written over a root's own forest entry once the
-// tile is labelled: INFO_BORDER | 0x8000 | slot for a piece that touches the
-// tile border (slot = its representative node), INFO_INTERIOR | spin << 14 |
-// local index for a cluster that ends inside the tile.  The low 16 bits are
-// the site code.  Forest indices stay below INFO_INTERIOR.
-constexpr uint32_t INFO_BORDER = 0x80008000u;
+// tile is labelled: INFO_BORDER | 4 slot for a piece that touches the tile
+// border (slot = its representative node), INFO_INTERIOR | code for a cluster
+// that ends inside the tile.  The low 16 bits are the site code.  Forest
+// indices stay below INFO_INTERIOR.
+constexpr uint32_t INFO_BORDER = 0x80000000u;
 constexpr uint32_t INFO_INTERIOR = 0x40000000u;
+__device__ __forceinline__ int info_slot(int v) { return (v & 0xFFFF) >> 2; }
 
 // Run heads of a 32-site row word inside one sub-tile: bit x is set iff
 // x == 0 or the link (x-1, x) is not a bond (bit 31 of h, the link leaving
@@ -482,10 +508,9 @@ __device__ void tile_label(volatile int *par, const uint32_t (*Hb)[TWW], const u
 //      label above its last bonded contact by one shuffle, or starts a new
 //      label, its own head, when it has none.  Labels are forest nodes: every
 //      site's entry is written once, pointing at the node its label was born
-//      at.  At T_c that settles 86% of the contacts with plain stores; the rest
-//      (a run whose contacts carry different labels: 86 of 499 a sub-tile,
-//      67 without repeats) are kept as a mask per row and united afterwards,
-//      lane = row;
+//      at.  At T_c that settles 83% of the contacts with plain stores; the rest
+//      (a run whose contacts carry different labels: 86 of 499 a sub-tile) are
+//      kept as a mask per column and united afterwards;
 //   2. unions across the sub-tile boundaries inside the tile.
 // Links always hang the larger root under the smaller, so par[x] < x unless x
 // is a root and every root is the minimum local index of its piece; local
@@ -496,9 +521,11 @@ __device__ void tile_label(volatile int *par, const uint32_t (*Hb)[TWW], const u
 // finds and a compare-and-swap, lane = row, cost 2.1K warp instructions a
 // sub-tile with 12.5 of 32 lanes active; this pass with the plain-store labels
 // and one code look-up a site took the 64-row tile kernel from 2.01 to 1.40 ms
-// at L=16384, T_c (111 -> 81M warp instructions a launch at L=4096).
-// Returns, to lane r, the heads of the runs of row r of the warp's sub-tile
-// that started a label (every root is one of them).
+// at L=16384, T_c (111 -> 81M warp instructions a launch at L=4096), and masks
+// per column, the single-swap unions and the label nodes' copies of their root's
+// record (two loads a code) to 1.19 ms.
+// Returns, to lane x, the rows of column x of the warp's sub-tile whose site
+// started a label (every root is one of them).
 template <int TH>
 __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
 {
@@ -511,41 +538,33 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
         const uint32_t le = 0xFFFFFFFFu >> (31 - lane), gt = ~le;
         int row = y0 * PW + 32 * sx;
         uint2 hv = *reinterpret_cast<const uint2 *>(&B[y0][2 * sx]);
-        uint32_t heads = run_heads(hv.x);
-        int lab = row + top_bit(heads & le);
+        int hd = top_bit(run_heads(hv.x) & le);
+        int lab = row + hd;
         par[row + lane] = lab;
-        born = heads;
+        born = hd == lane;
 #pragma unroll 4
         for (int r = 1; r < rows; ++r) {
             const uint32_t v = hv.y;   // down bonds from the row above
             hv = *reinterpret_cast<const uint2 *>(&B[y0 + r][2 * sx]);
             row += PW;
-            heads = ~(hv.x << 1);
-            const int hd = top_bit(heads & le);
+            const uint32_t heads = ~(hv.x << 1);
+            hd = top_bit(heads & le);
             const uint32_t n = heads & gt;                     // heads to the right: the run ends before them
             const int c = top_bit(v & (n - 1u) & ~n);          // last contact at or left of the run's end
             const bool has = c >= hd;
             const int lc = __shfl_sync(0xFFFFFFFFu, lab, c);
-            const uint32_t cf = __ballot_sync(0xFFFFFFFFu, ((v >> lane) & 1u) && lab != lc);
-            const uint32_t nr = __ballot_sync(0xFFFFFFFFu, !has) & heads;
+            if (((v >> lane) & 1u) && lab != lc) conf |= 1u << r;
+            if (!has && hd == lane) born |= 1u << r;
             lab = has ? lc : row + hd;
             par[row + lane] = lab;
-            if (lane == r) {
-                born = nr;
-                conf = cf;
-            }
         }
         __syncwarp();
-        const int base = (y0 + lane) * PW + 32 * sx;
-        int pa = -1, pb = -1;
+        const int col = y0 * PW + 32 * sx + lane;
         for (; conf; conf &= conf - 1) {
-            const int i = base + __ffs(conf) - 1;
-            const int a = par[i - PW], b = par[i];
-            if (a != pa || b != pb) sunite(par, a, b);
-            pa = a;
-            pb = b;
+            const int i = col + (__ffs(conf) - 1) * PW;
+            shook<3>(par, par[i - PW], par[i]);
         }
-        if (lane >= rows) born = 0u;
+        if (32 * sx + lane >= tw) born = 0u;
     }
     __syncthreads();
 
@@ -579,7 +598,7 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
             }
             const int a = par[ia], b = par[ib];
             if (before && par[ia - step] == a && par[ib - step] == b) continue;
-            sunite(par, a, b);
+            shook<1>(par, a, b);
         }
     }
     __syncthreads();
@@ -673,7 +692,8 @@ struct TileSmem {
     // right links and [2c + 1] the down links of word c
     __align__(16) uint32_t b[TH][2 * TWW];
     union {                         // never live at the same time:
-        __align__(16) uint32_t finfo[Slots<TH>::S];   // finish half: finals of the tile's own nodes
+        __align__(16) uint32_t finfo[Slots<TH>::S + 4];   // finish half: finals of the tile's own nodes,
+                                                          // then spins 0 and 1 (entries S and S + 1)
         uint32_t spb[TH][TWW];               // start half: SPIN-stream bit of each site
     } u;
     int acc[4];                     // sums of the tile: bond_sum, mag (sweep k-1), nbonds, nclusters (sweep k)
@@ -756,6 +776,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         }
         const uint32_t *nf = R.nfinal + (size_t)t.lt * S;
         for (int s = tid; s < S / 4; s += NT) cp_async16(sm.u.finfo + 4 * s, nf + 4 * s);
+        if (tid < 2) sm.u.finfo[S + tid] = tid ? FINAL_SPIN : 0u;
         // the halos' finals (new spins of the top row of the tile below and of
         // the left column of the tile to the right)
         if (warp < TWW && tid < t.tw) fb = R.nfinal[(size_t)t.g_down * S + SL::TOP + tid];
@@ -828,25 +849,32 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (y >= t.th) continue;
             const uint4 cq = scode4[idx];
             const uint32_t wv[4] = {cq.x, cq.y, cq.z, cq.w};
+            // a site's spin: the top bit of its entry in the table of finals
+            auto entry = [&](uint32_t u) {
+                return *reinterpret_cast<const uint32_t *>(reinterpret_cast<const unsigned char *>(sm.u.finfo) + u);
+            };
             uint32_t bits = 0;
+            if (!last) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint32_t u = (wv[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
-                const uint32_t spin =
-                    (u & CODE_BORDER) ? (sm.u.finfo[u & 0x3FFu] >> 30) & 1u : (u >> 14) & 1u;
-                bits |= spin << e;
-            }
-            bits &= (1u << min(8, max(0, t.tw - xb))) - 1u;   // sites past tw are not spins
-            reinterpret_cast<uint8_t *>(&sm.sp[y][0])[xb >> 3] = (uint8_t)bits;
-            if (last) {
+                for (int e = 7; e >= 0; --e) {
+                    const uint32_t u = e & 1 ? wv[e >> 1] >> 16 : wv[e >> 1] & 0xFFFFu;
+                    bits = __funnelshift_l(entry(u), bits, 1);
+                }
+            } else {
                 const uint32_t gi0 = gbase + (uint32_t)y * uL + (uint32_t)xb;
                 uint32_t roots[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const uint32_t u = (wv[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
                     const uint32_t lr = u & CODE_ROOT;
-                    roots[e] = (u & CODE_BORDER) ? sm.u.finfo[u & 0x3FFu] & ROOT_MASK
-                                                 : gbase + (lr / TW) * uL + (lr % TW);
+                    if (u & CODE_LAST) {
+                        bits |= ((u >> 14) & 1u) << e;
+                        roots[e] = gbase + (lr / TW) * uL + (lr % TW);
+                    } else {
+                        const uint32_t w = entry(u);
+                        bits |= (w >> 31) << e;
+                        roots[e] = w & ROOT_MASK;
+                    }
                 }
                 const int nval = min(8, t.tw - xb);
                 if (nval == 8 && (gi0 & 7u) == 0) {
@@ -864,6 +892,8 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                     }
                 }
             }
+            // (sites past the tile's last column have the code of spin 0)
+            reinterpret_cast<uint8_t *>(&sm.sp[y][0])[xb >> 3] = (uint8_t)bits;
         }
         // bottom halo row and right halo column
         if (warp < TWW) {
@@ -1013,7 +1043,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
 
     if (start) {
         // Step 2 inside the tile (Hoshen-Kopelman's role in Sec. II.A slave step 1)
-        uint32_t born = tile_label_rows<TH>(sm.par, sm.b, t.th, t.tw);
+        const uint32_t born = tile_label_rows<TH>(sm.par, sm.b, t.th, t.tw);
 
         // One node per border site: key = global index of the piece's local root,
         // parent = the piece's first border slot (the representative).
@@ -1025,28 +1055,47 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             rs[q] = -1;
             if (s < S && slot_site<TH>(s, t.tw, t.th, site)) {
                 rs[q] = sroot_marked(sm.par, site + site / TW);   // PW = TW + 1
-                atomicMin(&sm.par[rs[q]], (int)(INFO_BORDER | (uint32_t)s));
+                atomicMin(&sm.par[rs[q]], (int)(INFO_BORDER | (uint32_t)(4 * s)));
             }
         }
         __syncthreads();
         // Every interior root gets its record (the cluster's new spin, Sec. I
-        // step 3, drawn above) and is counted: lane r of a warp checks the nodes
-        // born in row r of its sub-tile.
+        // step 3, drawn above) and is counted: lane x of a warp checks the nodes
+        // born in column x of its sub-tile.
+        const bool last_start = j == R.nsweeps - 1;
         {
-            const int sx = warp & (TWW - 1), y = 32 * (warp / TWW) + lane;
-            const int base = y * PW + 32 * sx;
-            born &= valid_mask(sx, t.tw);
+            const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
+            const int col = y0 * PW + 32 * sx + lane;
+            uint32_t linked = 0u;
             int ncl = 0;
             for (uint32_t bits = born; bits; bits &= bits - 1) {
-                const int hx = __ffs(bits) - 1;
-                if (sm.par[base + hx] == base + hx) {
-                    const uint32_t spin = (sm.u.spb[y][sx] >> hx) & 1u;
-                    sm.par[base + hx] = (int)(INFO_INTERIOR | (spin << 14) | (uint32_t)(y * TW + 32 * sx + hx));
+                const int r = __ffs(bits) - 1;
+                const int x = col + r * PW;
+                const int p = sm.par[x];
+                if (p == x) {
+                    const uint32_t spin = (sm.u.spb[y0 + r][sx] >> lane) & 1u;
+                    const uint32_t c = last_start ? CODE_LAST | (spin << 14) | (uint32_t)((y0 + r) * TW + 32 * sx + lane)
+                                                  : 4u * (S + spin);
+                    sm.par[x] = (int)(INFO_INTERIOR | c);
                     ++ncl;
+                } else if (p >= 0) {
+                    linked |= bits & -bits;
                 }
             }
             ncl = __reduce_add_sync(0xFFFFFFFFu, ncl);
             if (lane == 0 && ncl) atomicAdd(&sm.acc[3], ncl);
+            // the other labels' nodes take a copy of their root's record where it
+            // is there already, so that most sites find it two loads away (cluster
+            // sizes are added at the roots: their index instead)
+            for (; linked; linked &= linked - 1) {
+                const int x = col + (__ffs(linked) - 1) * PW;
+                int p = sm.par[x], q = sm.par[p];
+                while ((uint32_t)q < INFO_INTERIOR && q != p) {
+                    p = q;
+                    q = sm.par[p];
+                }
+                sm.par[x] = q == p || csz ? p : q;
+            }
         }
 #pragma unroll
         for (int q = 0; q < SPT; ++q) {
@@ -1054,7 +1103,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (s >= S) break;
             const size_t node = (size_t)t.lt * S + s;
             if (rs[q] >= 0) {
-                const int rep = sm.par[rs[q]] & 0x3FF;
+                const int rep = info_slot(sm.par[rs[q]]);
                 R.npar[node] = (int32_t)((size_t)t.lt * S + rep);
                 R.nkey[node] = (int32_t)((gbase + (uint32_t)(rs[q] / PW) * uL + (uint32_t)(rs[q] % PW)) |
                                          (rep == s ? KEY_REP : 0u));
@@ -1065,45 +1114,73 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (csz) R.csize[node] = 0;   // the merge adds piece sizes at root nodes
         }
         __syncthreads();
-        // Every site's 2-byte code, the low half of its root's record: border
-        // pieces by node slot, interior clusters by local root and new spin.
-        // Lane = column: a site's entry, its label's and so on up to the root
-        // (2.0 steps at T_c for the slowest lane of a row).
+        // Every site's 2-byte code, the low half of its root's record.  Lane =
+        // column: a site's entry, its label's node, seldom a third one.
         {
             const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
             const int rows = min(32, t.th - y0);
             const int x = 32 * sx + lane;
-            const bool site = x < t.tw;
             uint16_t *cp = code + y0 * TW + x;
             const int *pp = sm.par + y0 * PW + x;
-#pragma unroll 4
-            for (int r = 0; r < rows; ++r) {
-                int v = site ? pp[r * PW] : (int)INFO_BORDER;
-                int root = (y0 + r) * PW + x;
-                while ((uint32_t)v < INFO_INTERIOR) {   // records: negative or >= INFO_INTERIOR
-                    root = v;
-                    v = sm.par[v];
+            if (!((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) && rows == 32 && 32 * sx + 32 <= t.tw) {
+#pragma unroll 2
+                for (int r = 0; r < 32; r += 4) {
+                    int v[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = pp[(r + q) * PW];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = sm.par[v[q]];   // records: negative or >= INFO_INTERIOR
+                    while (min(min((uint32_t)v[0], (uint32_t)v[1]), min((uint32_t)v[2], (uint32_t)v[3])) < INFO_INTERIOR) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = sm.par[v[q]];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) cp[(r + q) * TW] = (uint16_t)v[q];
                 }
-                cp[r * TW] = site ? (uint16_t)v : (uint16_t)0;
-                if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) {
-                    // one lane per run (its head) for the whole run
-                    const uint32_t heads = run_heads(sm.b[y0 + r][2 * sx]);
-                    const uint32_t n = lane < 31 ? heads & (0xFFFFFFFFu << (lane + 1)) : 0u;
-                    const uint32_t run = (n - 1u) & ~n & (0xFFFFFFFFu << lane);
-                    if (site && ((heads >> lane) & 1u)) {
-                        // cluster sizes: every run adds its length to bits 16-30 of its root's
-                        // record (a piece holds at most TW*TH = 2^14 sites, an interior
-                        // cluster at most (TW-2)(TH-2) < 2^14, so neither field overflows
-                        // into the record's flag bits); the codes read bits 0-15 only
-                        if (csz) atomicAdd(&sm.par[root], __popc(run & valid_mask(sx, t.tw)) << 16);
-                        if (pcc && v < 0) {
-                            // the columns and rows each border piece occupies (only a
-                            // piece touching the border can belong to a spanning cluster)
-                            atomicOr(&sm.pm[v & 0x3FF][sx], run & valid_mask(sx, t.tw));
-                            atomicOr(&sm.pm[v & 0x3FF][4 + ((y0 + r) >> 5)], 1u << ((y0 + r) & 31));
+            } else {
+                const bool site = x < t.tw;
+                // Cluster sizes and piece masks, gathered down the lane's column and
+                // added when its cluster changes: a size goes to bits 16-30 of the
+                // root's record (a piece holds at most TW*TH = 2^14 sites, an interior
+                // cluster at most (TW-2)(TH-2) < 2^14, so neither field overflows into
+                // the record's flag bits; the codes read bits 0-15 only), the columns
+                // and rows of a border piece to its masks (only a piece touching the
+                // border can belong to a spanning cluster).
+                const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc);
+                int cur = -1, cur_v = 0;
+                uint32_t cur_rows = 0u;
+                auto flush = [&]() {
+                    if (!cur_rows) return;
+                    if (csz) atomicAdd(&sm.par[cur], __popc(cur_rows) << 16);
+                    if (pcc && cur_v < 0) {
+                        const int sl = info_slot(cur_v);
+                        atomicOr(&sm.pm[sl][sx], 1u << lane);
+                        atomicOr(&sm.pm[sl][4 + (y0 >> 5)], cur_rows);
+                    }
+                };
+#pragma unroll 2
+                for (int r = 0; r < rows; ++r) {
+                    int v = site ? pp[r * PW] : (int)(INFO_INTERIOR | 4u * S);
+                    int root = (y0 + r) * PW + x;
+                    while ((uint32_t)v < INFO_INTERIOR) {
+                        root = v;
+                        v = sm.par[v];
+                    }
+                    cp[r * TW] = (uint16_t)v;
+                    if (gather && site) {
+                        const int key = csz ? root : v;
+                        if (key != cur) {
+                            flush();
+                            cur = key;
+                            cur_v = v;
+                            cur_rows = 0u;
                         }
+                        cur_rows |= 1u << r;
                     }
                 }
+                if (gather) flush();
             }
         }
         if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) {
@@ -1113,12 +1190,12 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (csz) {
                 // every root: an interior cluster adds its |C|^2; a border piece
                 // hands its size to its representative node for the merge
-                const int sx = warp & (TWW - 1), y = 32 * (warp / TWW) + lane;
+                const int col = 32 * (warp / TWW) * PW + 32 * (warp & (TWW - 1)) + lane;
                 unsigned long long c2 = 0ull;
                 for (uint32_t bits = born; bits; bits &= bits - 1) {
-                    const int v = sm.par[y * PW + 32 * sx + __ffs(bits) - 1];
+                    const int v = sm.par[col + (__ffs(bits) - 1) * PW];
                     if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
-                        R.psize[(size_t)t.lt * S + (v & 0x3FF)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
+                        R.psize[(size_t)t.lt * S + info_slot(v)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
                     } else if ((uint32_t)v >= INFO_INTERIOR) {   // bits 16-29 (bit 30 is the flag)
                         const unsigned long long size = ((uint32_t)v >> 16) & 0x3FFFu;
                         c2 += size * size;

@@ -51,6 +51,10 @@ using namespace swg;
 namespace {
 
 constexpr uint32_t STREAM_QSPIN = 3;
+// A record of a piece that touches a tile face, and the code of its sites
+// (bits 0-14: its representative slot).
+constexpr uint32_t INFO_FACE = 0x80008000u;
+constexpr uint32_t CODE_FACE = 0x8000u;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr int PT = 256;   // threads of the per-site helper kernels
 
@@ -402,7 +406,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const uint32_t u = (wv[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
-                const uint32_t s = (u & CODE_BORDER) ? sm.f.s.fst[u & 0x7FFFu] : (u & 0xFFu);
+                const uint32_t s = (u & CODE_FACE) ? sm.f.s.fst[u & 0x7FFFu] : (u & 0xFFu);
                 if (e < 4) lo |= s << (8 * e);
                 else hi |= s << (8 * (e - 4));
             }
@@ -426,7 +430,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 // clusters' were written when the sweep started)
                 for (int e = 0; e < nval; ++e) {
                     const uint32_t u = (wv[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
-                    if (u & CODE_BORDER) p.label[gi0 + e] = (int32_t)(p.nfinal[nbase + (u & 0x7FFFu)] & ROOT_MASK);
+                    if (u & CODE_FACE) p.label[gi0 + e] = (int32_t)(p.nfinal[nbase + (u & 0x7FFFu)] & ROOT_MASK);
                 }
             }
         }
@@ -738,7 +742,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     __syncthreads();
 #pragma unroll
     for (int qq = 0; qq < G::SPT; ++qq)
-        if (rs[qq] >= 0) atomicMin((int *)&sm.f.par[rs[qq]], (int)(INFO_BORDER | (uint32_t)(tid + qq * NT)));
+        if (rs[qq] >= 0) atomicMin((int *)&sm.f.par[rs[qq]], (int)(INFO_FACE | (uint32_t)(tid + qq * NT)));
     __syncthreads();
 #pragma unroll
     for (int qq = 0; qq < G::SPT; ++qq) {
