@@ -51,10 +51,6 @@ using namespace swg;
 namespace {
 
 constexpr uint32_t STREAM_QSPIN = 3;
-// A record of a piece that touches a tile face, and the code of its sites
-// (bits 0-14: its representative slot).
-constexpr uint32_t INFO_FACE = 0x80008000u;
-constexpr uint32_t CODE_FACE = 0x8000u;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr int PT = 256;   // threads of the per-site helper kernels
 
@@ -179,85 +175,90 @@ __device__ __forceinline__ PTile ptile_of(const PottsDev &p, int lt)
 }
 
 // ------------------------------------------------- 3D tile union-find
-// Connected components of the bonds inside a 32 x 16 x 16 tile (X: +x bonds,
-// whose link leaving the tile's last column is ignored; Y, Z: +y / +z bonds,
-// ignored in the tile's last row / layer).  The forest lives on run heads (a
-// run = maximal chain of x bonds in a row; its head is its leftmost site):
-//   1. warp w holds the rows y = 4 (w mod 4) + (lane mod 4), z = 8 (w / 4) +
-//      lane / 4; lane = row unites its runs with those of the next row along
-//      y and along z inside the warp, skipping a bond when the bond of the
-//      same direction to its left joins the same two runs;
-//   2. the y and z bonds between the warps' row blocks, one thread per link,
-//      with the same skip rule.
+// Connected components of the bonds inside a 32 x 16 x 16 tile, B[r] = {+x,
+// +y, +z bonds} of row r = y + 16 z, all without the links that leave the
+// tile.  Warp w holds the rows y = 4 (w mod 4) .. + 3, z = 8 (w / 4) .. + 7,
+// lane = column, and goes through them with y innermost, the labels of the
+// row before along y and of the four rows before along z in registers:
+//   1. a run (maximal chain of x bonds in a row) takes the label of its last
+//      contact along y, else along z, by shuffle, or starts a new label, its own
+//      head; contacts with another label are kept as masks per column and united
+//      afterwards (sw_device.cuh's tile_label_rows with a second direction: at
+//      the 3D critical point 85% of the contacts inside a warp's rows need
+//      no union);
+//   2. the y and z bonds between the warps' row blocks, eight sites a thread.
+// With the thread-per-word comparisons and the table codes below this took the
+// tile kernel (bound by instruction issue) from 2.07 to 1.32 ms at L=512, q=2,
+// T_c, and the 2D one from 0.62 to 0.38 ms at L=8192, q=3.
 // Links hang the larger root under the smaller, so roots are piece minima in
-// local row-major order, which is global order.
-__device__ void tile_label3(volatile int *par, const uint32_t (*X)[1], const uint32_t (*Y)[1],
-                            const uint32_t (*Z)[1], int tw, int th, int td)
+// local row-major order, which is global order.  Returns, to lane x, the rows
+// (bit 4 zz + yy) of the warp whose site x started a label.
+__device__ __forceinline__ uint32_t tile_label3(volatile int *par, const uint32_t (*B)[3], int tw, int th, int td)
 {
     using G = PG<3>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int yy = lane & 3, zz = lane >> 2;
-    const int y = 4 * (warp & 3) + yy, z = 8 * (warp >> 2) + zz;
-    const int r = y + G::TY * z;
-    const bool ok = y < th && z < td;
-    const uint32_t vx = valid_mask(0, tw - 1);
-    const uint32_t heads = run_heads(ok ? X[r][0] & vx : 0u);
-    const uint32_t hy = __shfl_down_sync(FULL, heads, 1);   // row (y + 1, z) when yy < 3
-    const uint32_t hz = __shfl_down_sync(FULL, heads, 4);   // row (y, z + 1) when zz < 7
-    const int base = r * G::PW;
-    if (ok) {
+    const int yb = 4 * (warp & 3), zb = 8 * (warp >> 2);
+    const uint32_t le = 0xFFFFFFFFu >> (31 - lane), gt = ~le;
+    uint32_t born = 0u, cy = 0u, cz = 0u;
+    {
+        int labz[4] = {0, 0, 0, 0};
+        uint32_t zw[4] = {0u, 0u, 0u, 0u};
+        for (int zz = 0; zz < 8 && zb + zz < td; ++zz) {
+            int laby = 0;
+            uint32_t yw = 0u;
 #pragma unroll
-        for (int x = 0; x < 32; ++x) par[base + x] = base + x;
+            for (int yy = 0; yy < 4; ++yy) {
+                if (yb + yy >= th) break;
+                const int r = yb + yy + G::TY * (zb + zz), row = r * G::PW;
+                const uint32_t heads = run_heads(B[r][0]);
+                const int hd = top_bit(heads & le);
+                const uint32_t n = heads & gt, m = (n - 1u) & ~n;   // m: up to the run's end
+                const int py = top_bit(yw & m), pz = top_bit(zw[yy] & m);
+                const int ly = __shfl_sync(FULL, laby, py), lz = __shfl_sync(FULL, labz[yy], pz);
+                const bool hy = py >= hd, hz = pz >= hd;
+                const int lab = hy ? ly : hz ? lz : row + hd;
+                const uint32_t bit = 1u << (4 * zz + yy);
+                if (((yw >> lane) & 1u) && laby != lab) cy |= bit;
+                if (((zw[yy] >> lane) & 1u) && labz[yy] != lab) cz |= bit;
+                if (!hy && !hz && hd == lane) born |= bit;
+                par[row + lane] = lab;
+                laby = labz[yy] = lab;
+                yw = B[r][1];
+                zw[yy] = B[r][2];
+            }
+        }
     }
     __syncwarp();
-    const uint32_t vy = (ok && yy < 3 && y + 1 < th) ? Y[r][0] : 0u;
-    const uint32_t vz = (ok && zz < 7 && z + 1 < td) ? Z[r][0] : 0u;
-    const uint32_t uy = vy & (~(vy << 1) | heads | hy);
-    const uint32_t uz = vz & (~(vz << 1) | heads | hz);
-    int pa = -1, pb = -1, pr = 0;
-    for (uint32_t b = uy; b; b &= b - 1) {
-        const int x = __ffs(b) - 1;
-        const int ha = head_of(heads, base, x), hb = head_of(hy, base + G::PW, x);
-        pr = sunite_root(par, ha == pa ? pr : ha, hb == pb ? pr : hb);
-        pa = ha;
-        pb = hb;
+    const int col = (yb + G::TY * zb) * G::PW + lane;
+    auto node = [&](int i) { return col + ((i & 3) + G::TY * (i >> 2)) * G::PW; };
+    for (; cy; cy &= cy - 1) {
+        const int i = node(__ffs(cy) - 1);
+        shook<2>(par, par[i - G::PW], par[i]);
     }
-    pa = pb = -1;
-    for (uint32_t b = uz; b; b &= b - 1) {
-        const int x = __ffs(b) - 1;
-        const int ha = head_of(heads, base, x), hb = head_of(hz, base + G::TY * G::PW, x);
-        pr = sunite_root(par, ha == pa ? pr : ha, hb == pb ? pr : hb);
-        pa = ha;
-        pb = hb;
+    for (; cz; cz &= cz - 1) {
+        const int i = node(__ffs(cz) - 1);
+        shook<2>(par, par[i - G::TY * G::PW], par[i]);
     }
     __syncthreads();
-    // y bonds from rows y = 3, 7, 11 (every z), z bonds from layer z = 7 (every y)
-    constexpr int NYB = 3 * G::TZ * 32, NZB = G::TY * 32;
-    for (int q = threadIdx.x; q < NYB + NZB; q += G::NT) {
-        int A, B, x;
-        uint32_t bw;
-        if (q < NYB) {
-            const int bnd = q / (G::TZ * 32), rem = q % (G::TZ * 32);
-            const int zq = rem >> 5, yq = 4 * bnd + 3;
-            x = rem & 31;
-            if (yq + 1 >= th || zq >= td) continue;
-            A = yq + G::TY * zq;
-            B = A + 1;
-            bw = Y[A][0];
-        } else {
-            const int rem = q - NYB, yq = rem >> 5;
-            x = rem & 31;
-            if (8 >= td || yq >= th) continue;
-            A = yq + G::TY * 7;
-            B = A + G::TY;
-            bw = Z[A][0];
+    // y bonds from rows y = 3, 7, 11 (every z), z bonds from layer z = 7 (every
+    // y): 64 rows, a quarter of a row's word a thread
+    {
+        const int w = threadIdx.x >> 2, x0 = 8 * (threadIdx.x & 3);
+        const bool yd = w < 48;
+        const int y = yd ? 4 * (w % 3) + 3 : w - 48, z = yd ? w / 3 : 7;
+        const int A = y + G::TY * z, step = (yd ? 1 : G::TY) * G::PW;
+        uint32_t bits = y < th && z < td ? (B[A][yd ? 1 : 2] >> x0) & 0xFFu : 0u;
+        int pa = -1, pb = -1;
+        for (; bits; bits &= bits - 1) {
+            const int i = A * G::PW + x0 + __ffs(bits) - 1;
+            const int a = par[i], b = par[i + step];
+            if (a != pa || b != pb) shook<1>(par, a, b);
+            pa = a;
+            pb = b;
         }
-        if (!((bw >> x) & 1u)) continue;
-        const uint32_t hA = run_heads(X[A][0] & vx), hB = run_heads(X[B][0] & vx);
-        if (x > 0 && ((bw >> (x - 1)) & 1u) && !((hA >> x) & 1u) && !((hB >> x) & 1u)) continue;
-        sunite(par, head_of(hA, A * G::PW, x), head_of(hB, B * G::PW, x));
     }
     __syncthreads();
+    return tw > lane ? born : 0u;
 }
 
 // ------------------------------------------------------------ shared layout
@@ -267,19 +268,24 @@ __device__ void tile_label3(volatile int *par, const uint32_t (*X)[1], const uin
 template <int DIM>
 struct PSmem {
     using G = PG<DIM>;
+    static constexpr int BW = DIM == 2 ? 2 * G::TWW : 3;   // bond words of a row
     union {
-        int par[G::NR * G::PW];             // from the labelling on: union-find forest over run heads
+        int par[G::NR * G::PW];             // from the labelling on: union-find forest over the sites
         struct {
-            uint8_t fst[G::S];              // finish half: new states of the tile's pieces, by slot
-            uint8_t st[G::HZ][G::HY][G::RS];   // states; row TY, layer TZ and column tw: + halo
             alignas(16) uint16_t code[G::NS];  // finish half: the tile's site codes
+            alignas(16) uint32_t raw[G::NR][DIM == 2 ? 2 * G::TWW : 4];   // a row's random bond bits
+            // finish half: the table the codes index, the new states of the
+            // tile's pieces by slot, then every state itself
+            uint8_t fst[G::S + 256];
+            uint8_t st[G::HZ][G::HY][G::RS];   // states; row TY, layer TZ and column tw: + halo
         } s;
     } f;
     uint8_t qs[G::NR][G::TX];               // each site's state drawn from the QSPIN stream
-    uint32_t bx[G::NR][G::TWW];             // +x bonds (bit x of word c: site 32 c + x)
-    uint32_t by[G::NR][G::TWW];             // +y bonds
-    uint32_t bz[DIM == 3 ? G::NR : 1][G::TWW];   // +z bonds
-    long long red[G::NW][4];                // the reduction that ends each half
+    // a row's bonds inside the tile: in 2D [2c] the +x and [2c + 1] the +y
+    // bonds of word c, in 3D the +x, +y and +z bonds
+    alignas(16) uint32_t b[G::NR][BW];
+    int acc[4];                             // sums of the tile: bond_sum, mag (sweep j-1), nbonds, nclusters (sweep j)
+    unsigned long long acc_c2[2];           // RF_CSIZE: sum |C|^2 of sweep j-1 and of sweep j
     uint32_t pm[G::S][G::PMW];              // PCC: coordinates each border piece occupies
 };
 
@@ -292,10 +298,28 @@ constexpr size_t ptile_smem(bool pcc)
     return pcc ? sizeof(PSmem<DIM>) : offsetof(PSmem<DIM>, pm);
 }
 
-// bytes 0 .. n-1 of a word (n in [0, 4])
-__device__ __forceinline__ uint32_t byte_mask(int n)
+// Top bit of every byte of t that is zero (t = a ^ b: the bytes where a and b agree).
+__device__ __forceinline__ uint32_t zero_bytes(uint32_t t)
 {
-    return n >= 4 ? 0xFFFFFFFFu : (n <= 0 ? 0u : (1u << (8 * n)) - 1u);
+    return ~(((t & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | t) & 0x80808080u;
+}
+
+// The four flags of zero_bytes in bits 28-31.
+__device__ __forceinline__ uint32_t byte_flags(uint32_t z)
+{
+    return z * 0x00204081u;
+}
+
+// Bit m of byte q of v (q < 4, m < 8) to bit 4 m + q.
+__device__ __forceinline__ uint32_t interleave4x8(uint32_t v)
+{
+    auto spread = [](uint32_t x) {   // bit m to bit 4 m
+        x = (x | (x << 12)) & 0x000F000Fu;
+        x = (x | (x << 6)) & 0x03030303u;
+        return (x | (x << 3)) & 0x11111111u;
+    };
+    return spread(v & 0xFFu) | (spread((v >> 8) & 0xFFu) << 1) | (spread((v >> 16) & 0xFFu) << 2) |
+           (spread(v >> 24) << 3);
 }
 
 // ----------------------------------------------------------------- k_ptile
@@ -340,14 +364,17 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         z = r / G::TY;
         return y < th && z < td;
     };
-    // intra-tile x bonds of word (r, c): the link leaving the tile's last column is ignored
-    auto ih = [&](int r, int c) { return sm.bx[r][c] & valid_mask(c, tw - 1); };
+    // the thread's word of the tile: row wr = (wy, wz), sites 32 wc .. 32 wc + 31;
+    // warp w holds rows w NR / NW .. (w + 1) NR / NW - 1
+    constexpr int WROWS = G::NR / NW;
+    const int wr = tid / TWW, wc = tid % TWW, wy = wr % G::TY, wz = wr / G::TY;
+    const bool row_ok = wy < th && wz < td;
 
+    // ---- loads of the finish half, in flight during the draws
     if (fin) {
-        // ---- finish sweep j-1: every site's new state
-        const bool last = j == nsweeps;
         // the tile's codes, 8 sites per 16-byte asynchronous copy straight
-        // into shared memory (the forest's space, free until the labelling)
+        // into shared memory (the forest's space, free until the labelling),
+        // and the states of its own pieces
         const uint4 *code4 = reinterpret_cast<const uint4 *>(code);
         uint4 *scode4 = reinterpret_cast<uint4 *>(sm.f.s.code);
 #pragma unroll
@@ -356,45 +383,154 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             const int idx = tid + qq * NT;
             if (group(idx, x, y, z)) cp_async16(scode4 + idx, code4 + idx);
         }
-        {
-            const uint32_t *ns4 = reinterpret_cast<const uint32_t *>(p.nstate + nbase);
-            uint32_t *fs4 = reinterpret_cast<uint32_t *>(sm.f.s.fst);
-            for (int w = tid; w < S / 4; w += NT) fs4[w] = ns4[w];
+        for (int w = tid; w < S / 16; w += NT) cp_async16(sm.f.s.fst + 16 * w, p.nstate + nbase + 16 * w);
+        sm.f.s.fst[S + tid] = (uint8_t)tid;   // NT = 256
+    }
+    if (tid < 4) sm.acc[tid] = 0;
+    if ((F & FEAT_CSIZE) && tid < 2) sm.acc_c2[tid] = 0ull;
+
+    // ---- Step 1 (Sec. I) of sweep j, its random part: which links' Philox
+    // words are below the threshold, and every site's QSPIN state (the draws
+    // need no state, so they run while the loads above are in flight).  Each
+    // warp draws its own rows; ballots leave them in shared memory for the
+    // thread that owns the word.
+    const uint64_t k = sweep0 + (uint64_t)j;
+    const uint64_t thr = p.thr_dev ? *p.thr_dev : p.thr;
+    const uint32_t klo = (uint32_t)k, khi = (uint32_t)(k >> 32);
+    const bool any_bond = start && thr != 0;
+    const uint32_t tm1 = (uint32_t)(thr - 1);
+    // every row starts a QSPIN block (4 divides L): the bond draws also fill qs
+    const bool qsm = any_bond && (uL & 3u) == 0;
+    auto ballots = [&](const U4 &u, bool act) {
+        return make_uint4(__ballot_sync(FULL, act && below(u.x, tm1)), __ballot_sync(FULL, act && below(u.y, tm1)),
+                          __ballot_sync(FULL, act && below(u.z, tm1)), __ballot_sync(FULL, act && below(u.w, tm1)));
+    };
+    auto states4 = [&](const U4 &u) {
+        return (uint32_t)potts_state(u.x, q) | ((uint32_t)potts_state(u.y, q) << 8) |
+               ((uint32_t)potts_state(u.z, q) << 16) | ((uint32_t)potts_state(u.w, q) << 24);
+    };
+    uint32_t extra = 0u;   // 2D, rows from an odd site: lane r's first two words of its row's 65th block
+    if (any_bond) {
+        if constexpr (DIM == 2) {
+            // link l = 2i + d: sites 2m and 2m + 1 share Philox block m (the
+            // Ising path's draws, sw_device.cuh)
+            const bool wide = tw > 64;
+            for (int i = 0; i < WROWS; i += 2) {
+                const int y = WROWS * warp + i;
+                if (y >= th) break;
+                const uint32_t g0 = t.gbase + (uint32_t)y * uL, g2 = g0 + uL;
+                const uint32_t b0 = (g0 >> 1) + lane, b2 = (g2 >> 1) + lane;
+                const U4 r0 = philox4x32_10(b0, klo, khi, STREAM_BOND, k0, k1);
+                const U4 r2 = philox4x32_10(b2, klo, khi, STREAM_BOND, k0, k1);
+                U4 r1{}, r3{};
+                if (wide) {
+                    r1 = philox4x32_10(b0 + 32, klo, khi, STREAM_BOND, k0, k1);
+                    r3 = philox4x32_10(b2 + 32, klo, khi, STREAM_BOND, k0, k1);
+                }
+                const uint4 q0 = ballots(r0, true), q1 = ballots(r1, true), q2 = ballots(r2, true), q3 = ballots(r3, true);
+                if (lane == 0) {
+                    uint4 *raw = reinterpret_cast<uint4 *>(&sm.f.s.raw[y][0]);
+                    raw[0] = q0;
+                    raw[1] = q1;
+                    raw[2] = q2;
+                    raw[3] = q3;
+                }
+                if (qsm) {
+                    // lane l: the QSPIN block of sites 4l .. 4l + 3 of each row
+                    const U4 s0 = philox4x32_10((g0 >> 2) + lane, klo, khi, STREAM_QSPIN, k0, k1);
+                    const U4 s2 = philox4x32_10((g2 >> 2) + lane, klo, khi, STREAM_QSPIN, k0, k1);
+                    *reinterpret_cast<uint32_t *>(&sm.qs[y][4 * lane]) = states4(s0);
+                    *reinterpret_cast<uint32_t *>(&sm.qs[y + 1][4 * lane]) = states4(s2);
+                }
+            }
+            if ((uL | t.gbase) & 1u) {
+                const uint32_t g0 = t.gbase + (uint32_t)(WROWS * warp + (lane & (WROWS - 1))) * uL;
+                const U4 r = philox4x32_10((g0 >> 1) + 64u, klo, khi, STREAM_BOND, k0, k1);
+                extra = (below(r.x, tm1) ? 1u : 0u) | (below(r.y, tm1) ? 2u : 0u);
+            }
+        } else if (qsm) {
+            // link l = 3i + d.  Every row starts on a multiple of 4, so its 96
+            // links are exactly the 24 Philox blocks from 3 i0 / 4: three blocks
+            // for four sites.  Lane 8 c + m draws block 3 m + c (c < 3), so that
+            // byte c of the ballot of word w holds link 4 c + w of the m-th four
+            // sites at bit m; lanes 24-31 draw the row's eight QSPIN blocks.
+            const bool bl = lane < 24;
+            const uint32_t st_ = bl ? STREAM_BOND : STREAM_QSPIN;
+            const uint32_t off = bl ? 3u * (lane & 7) + (lane >> 3) : (uint32_t)(lane - 24);
+            for (int i = 0; i < WROWS; i += 2) {
+                // two rows y, y + 1 of a layer (WROWS and TY are even)
+                const int r = WROWS * warp + i, y = r % G::TY, z = r / G::TY;
+                if (y >= th || z >= td) continue;
+                const uint32_t i0 = gidx(0, y, z) >> 2, i2 = i0 + (uL >> 2);
+                const U4 u0 = philox4x32_10((bl ? 3u * i0 : i0) + off, klo, khi, st_, k0, k1);
+                const U4 u2 = philox4x32_10((bl ? 3u * i2 : i2) + off, klo, khi, st_, k0, k1);
+                const uint4 q0 = ballots(u0, true), q2 = ballots(u2, true);
+                if (lane == 0) {
+                    *reinterpret_cast<uint4 *>(&sm.f.s.raw[r][0]) = q0;
+                    *reinterpret_cast<uint4 *>(&sm.f.s.raw[r + 1][0]) = q2;
+                }
+                if (!bl) {
+                    *reinterpret_cast<uint32_t *>(&sm.qs[r][4 * (lane - 24)]) = states4(u0);
+                    *reinterpret_cast<uint32_t *>(&sm.qs[r + 1][4 * (lane - 24)]) = states4(u2);
+                }
+            }
+        } else {
+            // a row starts anywhere in a block: its 96 links lie in the 25 blocks
+            // from the one that holds its first; lane x takes its three bits
+            // from the ballots
+            for (int i = 0; i < WROWS; ++i) {
+                const int r = WROWS * warp + i, y = r % G::TY, z = r / G::TY;
+                if (y >= th || z >= td) continue;
+                const uint32_t l0 = 3u * gidx(0, y, z);
+                const U4 u = philox4x32_10((l0 >> 2) + lane, klo, khi, STREAM_BOND, k0, k1);
+                const uint4 B = ballots(u, true);
+                const int l = (int)(l0 & 3u) + 3 * lane;
+                auto bit_of = [&](int e) {
+                    const uint32_t w = e & 2 ? (e & 1 ? B.w : B.z) : (e & 1 ? B.y : B.x);
+                    return (w >> (e >> 2)) & 1u;
+                };
+                const uint32_t rx = __ballot_sync(FULL, bit_of(l)), ry = __ballot_sync(FULL, bit_of(l + 1)),
+                               rz = __ballot_sync(FULL, bit_of(l + 2));
+                if (lane == 0) *reinterpret_cast<uint4 *>(&sm.f.s.raw[r][0]) = make_uint4(rx, ry, rz, 0u);
+            }
         }
+    }
+
+    uint8_t *st = &sm.f.s.st[0][0][0];
+    if (fin) {
+        // ---- finish sweep j-1: every site's new state
+        const bool last = j == nsweeps;
         // the + halo: new states of the neighbours' "-" face sites (the merge
         // gives every "-" face slot its cluster's state)
         constexpr int HPT = (G::FT + NT - 1) / NT;
-        uint32_t hs[HPT];
-        int hnode[HPT], hpos[HPT];
 #pragma unroll
         for (int qq = 0; qq < HPT; ++qq) {
             const int h = tid + qq * NT;
-            hpos[qq] = -1;
-            hnode[qq] = 0;
+            int hnode = -1, hpos = 0;
             if (h < G::F0) {
                 const int y = h % G::TY, z = h / G::TY;
                 if (y < th && z < td) {
-                    hnode[qq] = t.nb[0] * S + face_off<DIM>(0, 0) + h;
-                    hpos[qq] = (z * G::HY + y) * G::RS + tw;
+                    hnode = t.nb[0] * S + face_off<DIM>(0, 0) + h;
+                    hpos = (z * G::HY + y) * G::RS + tw;
                 }
             } else if (h < G::F0 + G::F1) {
                 const int f = h - G::F0, x = f % G::TX, z = f / G::TX;
                 if (x < tw && z < td) {
-                    hnode[qq] = t.nb[1] * S + face_off<DIM>(1, 0) + f;
-                    hpos[qq] = (z * G::HY + th) * G::RS + x;
+                    hnode = t.nb[1] * S + face_off<DIM>(1, 0) + f;
+                    hpos = (z * G::HY + th) * G::RS + x;
                 }
             } else if (h < G::FT) {
                 const int f = h - G::F0 - G::F1, x = f % G::TX, y = f / G::TX;
                 if (x < tw && y < th) {
-                    hnode[qq] = t.nb[2] * S + face_off<DIM>(2, 0) + f;
-                    hpos[qq] = (td * G::HY + y) * G::RS + x;
+                    hnode = t.nb[2] * S + face_off<DIM>(2, 0) + f;
+                    hpos = (td * G::HY + y) * G::RS + x;
                 }
             }
-            hs[qq] = hpos[qq] >= 0 ? p.nstate[hnode[qq]] : 0u;
+            if (hnode >= 0) st[hpos] = p.nstate[hnode];
         }
         cp_async_wait_all();
         __syncthreads();
-        uint8_t *st = &sm.f.s.st[0][0][0];
+        const uint4 *scode4 = reinterpret_cast<const uint4 *>(sm.f.s.code);
 #pragma unroll
         for (int qq = 0; qq < G::NQ; ++qq) {
             int x, y, z;
@@ -405,8 +541,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             uint32_t lo = 0u, hi = 0u;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const uint32_t u = (wv[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
-                const uint32_t s = (u & CODE_FACE) ? sm.f.s.fst[u & 0x7FFFu] : (u & 0xFFu);
+                const uint32_t s = sm.f.s.fst[e & 1 ? wv[e >> 1] >> 16 : wv[e >> 1] & 0xFFFFu];
                 if (e < 4) lo |= s << (8 * e);
                 else hi |= s << (8 * (e - 4));
             }
@@ -430,69 +565,11 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 // clusters' were written when the sweep started)
                 for (int e = 0; e < nval; ++e) {
                     const uint32_t u = (wv[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
-                    if (u & CODE_FACE) p.label[gi0 + e] = (int32_t)(p.nfinal[nbase + (u & 0x7FFFu)] & ROOT_MASK);
+                    if (u < (uint32_t)S) p.label[gi0 + e] = (int32_t)(p.nfinal[nbase + u] & ROOT_MASK);
                 }
             }
         }
-#pragma unroll
-        for (int qq = 0; qq < HPT; ++qq) {
-            if (hpos[qq] >= 0) st[hpos[qq]] = (uint8_t)hs[qq];
-        }
-        __syncthreads();
-        // observables of sweep j-1: every link that exists, every site
-        long long bs = 0, mag = 0;
-        for (int w = tid; w < G::NR * TWW; w += NT) {
-            const int r = w / TWW, c = w % TWW;
-            const int y = r % G::TY, z = r / G::TY;
-            if (y >= th || z >= td) continue;
-            const uint8_t *row = st + (z * G::HY + y) * G::RS;
-            const uint8_t *rowy = row + G::RS;
-            const uint8_t *rowz = row + G::HY * G::RS;
-            const bool dy = !(open_y && y == th - 1), dz = DIM == 3 && !(open_z && z == td - 1);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const int x = 32 * c + 4 * m;
-                const int nv = min(4, tw - x);
-                if (nv <= 0) break;
-                const uint32_t cur = *reinterpret_cast<const uint32_t *>(row + x);
-                const uint32_t nxt = *reinterpret_cast<const uint32_t *>(row + x + 4);
-                const uint32_t right = __funnelshift_r(cur, nxt, 8);
-                const uint32_t vm = byte_mask(nv);
-                const int nr = min(4, tw - x - (open_x ? 1 : 0));
-                bs += 2 * (__popc(__vcmpeq4(cur, right) & byte_mask(nr)) >> 3) - max(nr, 0);
-                if (dy) {
-                    const uint32_t down = *reinterpret_cast<const uint32_t *>(rowy + x);
-                    bs += 2 * (__popc(__vcmpeq4(cur, down) & vm) >> 3) - nv;
-                }
-                if (dz) {
-                    const uint32_t back = *reinterpret_cast<const uint32_t *>(rowz + x);
-                    bs += 2 * (__popc(__vcmpeq4(cur, back) & vm) >> 3) - nv;
-                }
-                mag += (long long)q * (__popc(__vcmpeq4(cur, 0u) & vm) >> 3) - nv;
-            }
-        }
-        // clusters that touch a tile face: their sizes were summed at their
-        // root nodes by the merge; each root node is in exactly one tile
-        long long c2 = 0;
-        if (csz)
-            for (int s = tid; s < S; s += NT) {
-                const long long c = p.csize[nbase + s];
-                c2 += c * c;
-            }
-        long long v[4] = {bs, mag, c2, 0};
-        DevObs *o = obs + (j - 1);
-        unsigned long long *const dst[4] = {&o->bond_sum, &o->mag, &o->csize2, nullptr};
-        block_sum_atomic<NT, 4>(v, dst, sm.red);
-        __syncthreads();
-    }
-
-    if (!start) return;
-
-    // ---- start sweep j
-    const uint64_t k = sweep0 + (uint64_t)j;
-    const uint64_t thr = p.thr_dev ? *p.thr_dev : p.thr;
-    const uint32_t klo = (uint32_t)k, khi = (uint32_t)(k >> 32);
-    if (!fin) {
+    } else {
         // first sweep of the call: states and + halos from global memory
         const int hrows = (th + 1) * (DIM == 3 ? td + 1 : 1);
         for (int rw = warp; rw < hrows; rw += NW) {
@@ -505,399 +582,340 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 sm.f.s.st[hz][hy][x] = grow[gx];
             }
         }
-        __syncthreads();
-    }
-    if (pcc)
-        for (int w = tid; w < S * G::PMW; w += NT) (&sm.pm[0][0])[w] = 0u;
-    if (lt == 0 && tid == 0) {
-        obs[j].threshold = thr;
-        obs[j].spans_x = 0;
-        obs[j].spans_y = 0;
-    }
-
-    // Step 1 (Sec. I): bonds between equal states.
-    const bool any_bond = thr != 0;
-    const uint32_t tm1 = (uint32_t)(thr - 1);
-    // every row starts a QSPIN block (4 divides L): the bond draws also fill qs
-    const bool qsm = any_bond && (uL & 3u) == 0;
-    // row (y, z) from its random bond bits (rx, ry, rz: bit x of word c set
-    // iff the link's Philox word is below the threshold)
-    auto store_row = [&](int y, int z, const uint32_t (&rx)[TWW], const uint32_t (&ry)[TWW],
-                         const uint32_t (&rz)[TWW]) {
-        const int r = y + G::TY * z;
-        const bool dy = !(open_y && y == th - 1), dz = !(open_z && z == td - 1);
-#pragma unroll
-        for (int c = 0; c < TWW; ++c) {
-            const int x = 32 * c + lane;
-            const uint8_t s = sm.f.s.st[z][y][x];
-            const uint32_t ex = __ballot_sync(FULL, s == sm.f.s.st[z][y][x + 1]);
-            const uint32_t ey = __ballot_sync(FULL, s == sm.f.s.st[z][y + 1][x]);
-            uint32_t ez = 0u;
-            if (DIM == 3) ez = __ballot_sync(FULL, s == sm.f.s.st[DIM == 3 ? z + 1 : z][y][x]);
-            const uint32_t vm = valid_mask(c, tw);
-            const uint32_t vr = open_x ? valid_mask(c, tw - 1) : vm;
-            if (lane == c) {
-                sm.bx[r][c] = rx[c] & ex & vr;
-                sm.by[r][c] = dy ? ry[c] & ey & vm : 0u;
-                if (DIM == 3) sm.bz[DIM == 3 ? r : 0][c] = dz ? rz[c] & ez & vm : 0u;
-            }
-        }
-    };
-    if constexpr (DIM == 2) {
-        // link l = 2i + d: sites 2m and 2m + 1 share Philox block m
-        // aligned row: lane l drew the blocks of sites (2l, 2l+1) (r0) and
-        // (64+2l, 65+2l) (r1); lane x of each 32-site word takes its two bits
-        // by shuffle
-        auto draws_aligned = [&](const U4 &r0, const U4 &r1, uint32_t (&rh)[TWW], uint32_t (&rv)[TWW]) {
-            const uint32_t nib0 = (below(r0.x, tm1) ? 1u : 0u) | (below(r0.y, tm1) ? 2u : 0u) |
-                                  (below(r0.z, tm1) ? 4u : 0u) | (below(r0.w, tm1) ? 8u : 0u);
-            const uint32_t nib1 = (below(r1.x, tm1) ? 1u : 0u) | (below(r1.y, tm1) ? 2u : 0u) |
-                                  (below(r1.z, tm1) ? 4u : 0u) | (below(r1.w, tm1) ? 8u : 0u);
-#pragma unroll
-            for (int c = 0; c < TWW; ++c) {
-                const uint32_t n = __shfl_sync(FULL, c < 2 ? nib0 : nib1, 16 * (c & 1) + (lane >> 1)) >>
-                                   (2 * (lane & 1));
-                rh[c] = __ballot_sync(FULL, n & 1u);
-                rv[c] = __ballot_sync(FULL, n & 2u);
-            }
-        };
-        uint32_t rz[TWW] = {};
-        if (any_bond && (uL & 1u) == 0) {
-            for (int y = warp; y < th; y += 2 * NW) {
-                const int y2 = y + NW;
-                const uint32_t b0 = ((t.gbase + (uint32_t)y * uL) >> 1) + lane;
-                const uint32_t b2 = ((t.gbase + (uint32_t)y2 * uL) >> 1) + lane;
-                const U4 r0 = philox4x32_10(b0, klo, khi, STREAM_BOND, k0, k1);
-                const U4 r1 = philox4x32_10(b0 + 32, klo, khi, STREAM_BOND, k0, k1);
-                const U4 r2 = philox4x32_10(b2, klo, khi, STREAM_BOND, k0, k1);
-                const U4 r3 = philox4x32_10(b2 + 32, klo, khi, STREAM_BOND, k0, k1);
-                if (qsm) {
-                    // lane l: the QSPIN block of sites 4l .. 4l + 3 of each row
-                    const U4 s0 = philox4x32_10(((t.gbase + (uint32_t)y * uL) >> 2) + lane, klo, khi, STREAM_QSPIN, k0, k1);
-                    const U4 s2 = philox4x32_10(((t.gbase + (uint32_t)y2 * uL) >> 2) + lane, klo, khi, STREAM_QSPIN, k0, k1);
-                    *reinterpret_cast<uint32_t *>(&sm.qs[y][4 * lane]) =
-                        (uint32_t)potts_state(s0.x, q) | ((uint32_t)potts_state(s0.y, q) << 8) |
-                        ((uint32_t)potts_state(s0.z, q) << 16) | ((uint32_t)potts_state(s0.w, q) << 24);
-                    if (y2 < th)
-                        *reinterpret_cast<uint32_t *>(&sm.qs[y2][4 * lane]) =
-                            (uint32_t)potts_state(s2.x, q) | ((uint32_t)potts_state(s2.y, q) << 8) |
-                            ((uint32_t)potts_state(s2.z, q) << 16) | ((uint32_t)potts_state(s2.w, q) << 24);
-                }
-                uint32_t rh[TWW], rv[TWW], rh2[TWW], rv2[TWW];
-                draws_aligned(r0, r1, rh, rv);
-                draws_aligned(r2, r3, rh2, rv2);
-                store_row(y, 0, rh, rv, rz);
-                if (y2 < th) store_row(y2, 0, rh2, rv2, rz);
-            }
-        } else {
-            for (int y = warp; y < th; y += NW) {
-                const uint32_t G0 = t.gbase + (uint32_t)y * uL;
-                uint32_t rh[TWW], rv[TWW];
-#pragma unroll
-                for (int c = 0; c < TWW; ++c) {
-                    rh[c] = rv[c] = 0u;
-                    if (any_bond) {
-                        // odd L: a row may start on an odd site; every site draws its block
-                        const uint32_t gi = G0 + 32 * c + lane;
-                        const U4 r = philox4x32_10(gi >> 1, klo, khi, STREAM_BOND, k0, k1);
-                        const bool odd = gi & 1u;
-                        rh[c] = __ballot_sync(FULL, below(odd ? r.z : r.x, tm1));
-                        rv[c] = __ballot_sync(FULL, below(odd ? r.w : r.y, tm1));
-                    }
-                }
-                store_row(y, 0, rh, rv, rz);
-            }
-        }
-    } else {
-        // link l = 3i + d.  When 4 divides L every row starts on a multiple
-        // of 4, so its 96 links are exactly the 24 Philox blocks from 3 i0 / 4:
-        // lane b < 24 draws block b, and lane x takes bits 3x + d of the row's
-        // link string from four ballots (one per word of a block)
-        const int nrows = th * td;
-        auto bits_of = [&](const uint32_t (&B)[4], int l) { return (B[l & 3] >> (l >> 2)) & 1u; };
-        auto row_aligned = [&](const U4 &u, int r, uint32_t (&rx)[1], uint32_t (&ry)[1], uint32_t (&rz)[1]) {
-            const bool act = lane < 24;
-            if (!act && r >= 0)   // lanes 24..31 drew the row's QSPIN blocks: four sites' states each
-                *reinterpret_cast<uint32_t *>(&sm.qs[r][4 * (lane - 24)]) =
-                    (uint32_t)potts_state(u.x, q) | ((uint32_t)potts_state(u.y, q) << 8) |
-                    ((uint32_t)potts_state(u.z, q) << 16) | ((uint32_t)potts_state(u.w, q) << 24);
-            uint32_t B[4];
-            B[0] = __ballot_sync(FULL, act && below(u.x, tm1));
-            B[1] = __ballot_sync(FULL, act && below(u.y, tm1));
-            B[2] = __ballot_sync(FULL, act && below(u.z, tm1));
-            B[3] = __ballot_sync(FULL, act && below(u.w, tm1));
-            const int l = 3 * lane;
-            rx[0] = __ballot_sync(FULL, bits_of(B, l));
-            ry[0] = __ballot_sync(FULL, bits_of(B, l + 1));
-            rz[0] = __ballot_sync(FULL, bits_of(B, l + 2));
-        };
-        if (any_bond && (uL & 3u) == 0) {
-            for (int rw = warp; rw < nrows; rw += 2 * NW) {
-                const int rw2 = rw + NW;
-                const int y = rw % th, z = rw / th, y2 = rw2 % th, z2 = rw2 / th;
-                // lane b < 24: BOND block b of the row; lane 24 + b: QSPIN block b
-                const uint32_t i0 = gidx(0, y, z), i2 = gidx(0, y2, z2);
-                const bool bl = lane < 24;
-                const uint32_t st_ = bl ? STREAM_BOND : STREAM_QSPIN;
-                const uint32_t c0 = bl ? 3u * (i0 >> 2) + (uint32_t)lane : (i0 >> 2) + (uint32_t)(lane - 24);
-                const uint32_t c2 = bl ? 3u * (i2 >> 2) + (uint32_t)lane : (i2 >> 2) + (uint32_t)(lane - 24);
-                const U4 u0 = philox4x32_10(c0, klo, khi, st_, k0, k1);
-                const U4 u2 = philox4x32_10(c2, klo, khi, st_, k0, k1);
-                uint32_t rx[1], ry[1], rz[1], rx2[1], ry2[1], rz2[1];
-                row_aligned(u0, y + G::TY * z, rx, ry, rz);
-                row_aligned(u2, rw2 < nrows ? y2 + G::TY * z2 : -1, rx2, ry2, rz2);
-                store_row(y, z, rx, ry, rz);
-                if (rw2 < nrows) store_row(y2, z2, rx2, ry2, rz2);
-            }
-        } else {
-            for (int rw = warp; rw < nrows; rw += NW) {
-                const int y = rw % th, z = rw / th;
-                uint32_t rx[1] = {0u}, ry[1] = {0u}, rz[1] = {0u};
-                if (any_bond) {
-                    // each site's three links span one or two blocks
-                    const uint32_t l0 = 3u * gidx(lane, y, z);
-                    const uint32_t m0 = l0 >> 2, m1 = (l0 + 2u) >> 2;
-                    const U4 u0 = philox4x32_10(m0, klo, khi, STREAM_BOND, k0, k1);
-                    U4 u1 = u0;
-                    if (m1 != m0) u1 = philox4x32_10(m1, klo, khi, STREAM_BOND, k0, k1);
-                    bool bit[3];
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const uint32_t l = l0 + (uint32_t)d;
-                        bit[d] = below(u4_word((l >> 2) == m0 ? u0 : u1, (int)(l & 3u)), tm1);
-                    }
-                    rx[0] = __ballot_sync(FULL, bit[0]);
-                    ry[0] = __ballot_sync(FULL, bit[1]);
-                    rz[0] = __ballot_sync(FULL, bit[2]);
-                }
-                store_row(y, z, rx, ry, rz);
-            }
-        }
     }
     __syncthreads();
 
-    long long nb = 0;
-    for (int w = tid; w < G::NR * TWW; w += NT) {
-        const int r = w / TWW, c = w % TWW;
-        const int y = r % G::TY, z = r / G::TY;
-        if (y >= th || z >= td) continue;
-        nb += __popc(sm.bx[r][c]) + __popc(sm.by[r][c]) + (DIM == 3 ? __popc(sm.bz[DIM == 3 ? r : 0][c]) : 0);
-    }
-    // crossing bonds, bit f of face a at word (f / 32) of that face's block:
-    // x face f = r (the row), y face f = x + TX z, z face f = x + TX y
-    {
-        uint32_t *cross = p.cross + (size_t)lt * G::CW;
-        for (int qq = warp; qq < G::F0 / 32; qq += NW) {
-            const int r = 32 * qq + lane, y = r % G::TY, z = r / G::TY;
-            const int bit = (y < th && z < td) ? (sm.bx[r][(tw - 1) >> 5] >> ((tw - 1) & 31)) & 1 : 0;
-            const uint32_t word = __ballot_sync(FULL, bit);
-            if (lane == 0) cross[qq] = word;
-        }
-        for (int w = tid; w < G::F1 / 32; w += NT) {
-            const int c = w % TWW, z = w / TWW;
-            cross[G::F0 / 32 + w] = z < td ? sm.by[(th - 1) + G::TY * z][c] : 0u;
-        }
-        if (DIM == 3)
-            for (int w = tid; w < G::F2 / 32; w += NT) {
-                const int c = w % TWW, y = w / TWW;
-                cross[(G::F0 + G::F1) / 32 + w] = y < th ? sm.bz[DIM == 3 ? y + G::TY * (td - 1) : 0][c] : 0u;
-            }
-    }
+    // ---- the thread's word: state agreement along its links (four sites a
+    //      comparison), the sums of sweep j-1 and the bonds of sweep j
     const bool last_start = j == nsweeps - 1;
-    if (last_start) {
-        // the last sweep of the call keeps its bond bytes
-        for (int rw = warp; rw < th * td; rw += NW) {
-            const int y = rw % th, z = rw / th, r = y + G::TY * z;
-            const uint32_t g0 = gidx(0, y, z);
+    {
+        const uint32_t vm = row_ok ? valid_mask(wc, tw) : 0u;
+        const uint32_t vx = open_x && row_ok ? valid_mask(wc, tw - 1) : vm;
+        const uint32_t vy = open_y && wy == th - 1 ? 0u : vm;
+        const uint32_t vz = DIM == 2 || (open_z && wz == td - 1) ? 0u : vm;
+        uint32_t ex = 0u, ey = 0u, ez = 0u, zero = 0u;
+        if (row_ok) {
+            const uint32_t *row = reinterpret_cast<const uint32_t *>(st + (wz * G::HY + wy) * G::RS + 32 * wc);
+            const uint32_t *rowy = row + G::RS / 4;
+            const uint32_t *rowz = row + G::HY * (G::RS / 4);
+            uint32_t nxt = row[8];
 #pragma unroll
-            for (int c = 0; c < TWW; ++c) {
-                const int x = 32 * c + lane;
-                if (x >= tw) break;
-                uint32_t b = ((sm.bx[r][c] >> lane) & 1u) | (((sm.by[r][c] >> lane) & 1u) << 1);
-                if (DIM == 3) b |= ((sm.bz[DIM == 3 ? r : 0][c] >> lane) & 1u) << 2;
-                p.bond[g0 + (uint32_t)x] = (uint8_t)b;
+            for (int m = 7; m >= 0; --m) {
+                const uint32_t cur = row[m];
+                ex = __funnelshift_l(byte_flags(zero_bytes(cur ^ __funnelshift_r(cur, nxt, 8))), ex, 4);
+                ey = __funnelshift_l(byte_flags(zero_bytes(cur ^ rowy[m])), ey, 4);
+                if (DIM == 3) ez = __funnelshift_l(byte_flags(zero_bytes(cur ^ rowz[m])), ez, 4);
+                if (fin) zero = __funnelshift_l(byte_flags(zero_bytes(cur)), zero, 4);
+                nxt = cur;
             }
+            ex &= vx;
+            ey &= vy;
+            ez &= vz;
         }
-    }
-
-    // Step 2 inside the tile
-    if constexpr (DIM == 2)
-        tile_label<64>(sm.f.par, sm.bx, sm.by, th, tw);
-    else
-        tile_label3(sm.f.par, sm.bx, sm.by, sm.bz, tw, th, td);
-
-    // One node per face site: key = global index of the piece's local root,
-    // parent = the piece's first face slot (the representative).
-    int rs[G::SPT];
-#pragma unroll
-    for (int qq = 0; qq < G::SPT; ++qq) {
-        const int s = tid + qq * NT;
-        int x, y, z;
-        rs[qq] = -1;
-        if (s < S && slot_xyz<DIM>(s, t.e, x, y, z)) {
-            const int r = y + G::TY * z, c = x >> 5;
-            rs[qq] = sroot(sm.f.par, head_of(run_heads(ih(r, c)), r * G::PW + 32 * c, x & 31));
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int qq = 0; qq < G::SPT; ++qq)
-        if (rs[qq] >= 0) atomicMin((int *)&sm.f.par[rs[qq]], (int)(INFO_FACE | (uint32_t)(tid + qq * NT)));
-    __syncthreads();
-#pragma unroll
-    for (int qq = 0; qq < G::SPT; ++qq) {
-        const int s = tid + qq * NT;
-        if (s >= S) break;
-        const size_t node = nbase + s;
-        if (rs[qq] >= 0) {
-            const int rep = sm.f.par[rs[qq]] & 0x7FFF;
-            p.npar[node] = (int32_t)(nbase + rep);
-            p.nkey[node] = (int32_t)(gfor(rs[qq]) | (rep == s ? KEY_REP : 0u));
-        } else {
-            p.npar[node] = (int32_t)node;
-            p.nkey[node] = (int32_t)KEY_NONE;
-        }
-        if (csz) p.csize[node] = 0;   // the merge adds piece sizes at root nodes
-    }
-    // Every run head learns its root; every interior root gets its record:
-    // its cluster's new state (Sec. I step 3, drawn here), and is counted.
-    // A walk stops at a root, a border record or an interior record; each
-    // thread writes only its own heads, so concurrent walks see ancestors.
-    long long ncl_interior = 0;
-    const int nrows = th * td;
-    for (int w = tid; w < nrows * TWW; w += NT) {
-        const int rr = w % nrows, c = w / nrows;   // a warp covers consecutive rows
-        const int y = rr % th, z = rr / th, r = y + G::TY * z;
-        const int base = r * G::PW + 32 * c;
-        for (uint32_t bits = run_heads(ih(r, c)); bits; bits &= bits - 1) {
-            const int hx = __ffs(bits) - 1;
-            const int hd = base + hx;
-            int x = hd, pp = sm.f.par[x];
-            while (pp != x && pp >= 0 && (uint32_t)pp < INFO_INTERIOR) {
-                x = pp;
-                pp = sm.f.par[x];
+        if (fin) {
+            // bond_sum: +1 a link between equal states, -1 otherwise
+            const int bs = 2 * (__popc(ex) + __popc(ey) + __popc(ez)) - __popc(vx) - __popc(vy) - __popc(vz);
+            const int mag = q * __popc(zero & vm) - __popc(vm);
+            const int ws = __reduce_add_sync(FULL, bs), wm = __reduce_add_sync(FULL, mag);
+            if (lane == 0) {
+                atomicAdd(&sm.acc[0], ws);
+                atomicAdd(&sm.acc[1], wm);
             }
-            if (x != hd) {
-                sm.f.par[hd] = x;
-            } else if (pp == hd && 32 * c + hx < tw) {
-                const uint8_t s = qsm ? sm.qs[r][32 * c + hx] : cluster_state(gidx(32 * c + hx, y, z), klo, khi, k0, k1, q);
-                sm.f.par[hd] = (int)(INFO_INTERIOR | (uint32_t)s);
-                ++ncl_interior;
-            }
-        }
-    }
-    __syncthreads();
-    if (csz) {
-        // cluster sizes: every run adds its length to bits 16-30 of its root's
-        // record (a piece or cluster holds at most 8192 sites); the codes
-        // below read bits 0-15 only
-        for (int w = tid; w < nrows * TWW; w += NT) {
-            const int rr = w % nrows, c = w / nrows;
-            const int y = rr % th, z = rr / th, r = y + G::TY * z;
-            const int base = r * G::PW + 32 * c;
-            const int vw = min(32, tw - 32 * c);
-            for (uint32_t bits = run_heads(ih(r, c)); bits;) {
-                const int hx = __ffs(bits) - 1;
-                bits &= bits - 1;
-                if (hx >= vw) break;
-                const int nx = bits ? __ffs(bits) - 1 : 32;
-                const int v = sm.f.par[base + hx];
-                const int root = (v < 0 || (uint32_t)v >= INFO_INTERIOR) ? base + hx : v;
-                atomicAdd((int *)&sm.f.par[root], (min(nx, vw) - hx) << 16);
-            }
-        }
-        __syncthreads();
-    }
-    // Every site's 2-byte code (the low half of its root's record): border
-    // pieces by representative slot, interior clusters by new state.
-    uint4 *code4 = reinterpret_cast<uint4 *>(code);
-#pragma unroll
-    for (int qq = 0; qq < G::NQ; ++qq) {
-        int xb, y, z;
-        const int idx = tid + qq * NT;
-        if (!group(idx, xb, y, z)) continue;
-        const int r = y + G::TY * z, c = xb >> 5;
-        const uint32_t heads = run_heads(ih(r, c));
-        const int base = r * G::PW + 32 * c;
-        const uint32_t gi0 = gidx(xb, y, z);
-        uint32_t wv[4] = {0u, 0u, 0u, 0u};
-        int slot = -1;   // PCC: border piece of the sites gathered in cols
-        uint32_t cols = 0u;
-        int info = 0, root = 0;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int x = xb + e;
-            if (x >= tw) break;
-            if (e == 0 || ((heads >> (x & 31)) & 1u)) {
-                const int hd = e == 0 ? head_of(heads, base, x & 31) : base + (x & 31);
-                const int v = sm.f.par[hd];
-                if ((uint32_t)v >= INFO_INTERIOR) {   // records: negative or >= INFO_INTERIOR
-                    info = v;
-                    root = hd;
-                } else {
-                    info = sm.f.par[v];
-                    root = v;
+            // clusters that touch a tile face: their sizes were summed at their
+            // root nodes by the merge; each root node is in exactly one tile
+            if (csz) {
+                unsigned long long c2 = 0ull;
+                for (int s = tid; s < S; s += NT) {
+                    const long long c = p.csize[nbase + s];
+                    c2 += (unsigned long long)(c * c);
                 }
+                if (c2) atomicAdd(&sm.acc_c2[0], c2);
             }
-            wv[e >> 1] |= ((uint32_t)info & 0xFFFFu) << (16 * (e & 1));
-            if (last_start && info >= 0) p.label[gi0 + e] = (int32_t)gfor(root);
-            if (pcc && info < 0) {
-                const int sl = info & 0x7FFF;
-                if (sl != slot) {
-                    if (slot >= 0) {
-                        if (DIM == 2) {
-                            atomicOr(&sm.pm[slot][c], cols);
-                            atomicOr(&sm.pm[slot][4 + (y >> 5)], 1u << (y & 31));
-                        } else {
-                            atomicOr(&sm.pm[slot][0], cols);
-                            atomicOr(&sm.pm[slot][1], (1u << y) | (1u << (16 + z)));
+        }
+        if (start) {
+            uint32_t rx = 0u, ry = 0u, rz = 0u;
+            if (any_bond) {
+                const uint4 raw = *reinterpret_cast<const uint4 *>(&sm.f.s.raw[wr][DIM == 2 ? 4 * (wc >> 1) : 0]);
+                if (DIM == 2) {
+                    rx = interleave16(raw.x, raw.z, wc & 1);
+                    ry = interleave16(raw.y, raw.w, wc & 1);
+                    if ((uL | t.gbase) & 1u) {
+                        // rows that start on an odd site are one site ahead of their blocks
+                        const uint32_t e = __shfl_sync(FULL, extra, lane / TWW);
+                        uint32_t nx = __shfl_down_sync(FULL, rx, 1), ny = __shfl_down_sync(FULL, ry, 1);
+                        if (wc == TWW - 1) {
+                            nx = e;
+                            ny = e >> 1;
+                        }
+                        if ((t.gbase + (uint32_t)wy * uL) & 1u) {
+                            rx = __funnelshift_r(rx, nx, 1);
+                            ry = __funnelshift_r(ry, ny, 1);
                         }
                     }
-                    slot = sl;
-                    cols = 0u;
+                } else if (qsm) {
+                    // byte c of word w: link 4 c + w of the twelve links of four
+                    // sites; direction d of site i is link 3 i + d
+                    rx = interleave4x8(__byte_perm(__byte_perm(raw.x, raw.w, 0x0040), __byte_perm(raw.z, raw.y, 0x0061), 0x5410));
+                    ry = interleave4x8(__byte_perm(__byte_perm(raw.y, raw.x, 0x0050), __byte_perm(raw.w, raw.z, 0x0061), 0x5410));
+                    rz = interleave4x8(__byte_perm(__byte_perm(raw.z, raw.y, 0x0050), __byte_perm(raw.x, raw.w, 0x0062), 0x5410));
+                } else {
+                    rx = raw.x;
+                    ry = raw.y;
+                    rz = raw.z;
                 }
-                cols |= 1u << (x & 31);
             }
-        }
-        if (slot >= 0) {
-            if (DIM == 2) {
-                atomicOr(&sm.pm[slot][c], cols);
-                atomicOr(&sm.pm[slot][4 + (y >> 5)], 1u << (y & 31));
-            } else {
-                atomicOr(&sm.pm[slot][0], cols);
-                atomicOr(&sm.pm[slot][1], (1u << y) | (1u << (16 + z)));
+            const uint32_t bx = rx & ex, by = ry & ey, bz = rz & ez;
+            const int nb = __reduce_add_sync(FULL, __popc(bx) + __popc(by) + __popc(bz));
+            if (lane == 0) atomicAdd(&sm.acc[2], nb);
+            // crossing bonds, bit f of face a at word (f / 32) of that face's block:
+            // x face f = r (the row), y face f = x + TX z, z face f = x + TX y
+            {
+                uint32_t *cross = p.cross + (size_t)lt * G::CW;
+                const int last_c = (tw - 1) >> 5, last_b = (tw - 1) & 31;
+                const uint32_t e = __ballot_sync(FULL, wc == last_c && ((bx >> last_b) & 1u)) >> last_c;
+                if (DIM == 2) {
+                    // a warp's eight rows a byte: bit 4 r of e is row r
+                    uint32_t v = e & 0x11111111u;
+                    v = (v | (v >> 3)) & 0x03030303u;
+                    v = (v | (v >> 6)) & 0x000F000Fu;
+                    v = (v | (v >> 12)) & 0xFFu;
+                    if (lane == 0) reinterpret_cast<uint8_t *>(cross)[warp] = (uint8_t)v;
+                } else if (lane == 0) {
+                    cross[warp] = e;
+                }
+                // (layers past the tile: no bonds, by = bz = 0)
+                if (wy == th - 1) cross[G::F0 / 32 + wc + TWW * wz] = by;
+                if (DIM == 3 && wz == td - 1) cross[(G::F0 + G::F1) / 32 + wy] = bz;
             }
+            auto put = [&](uint32_t x, uint32_t y, uint32_t z) {
+                if constexpr (DIM == 2) {
+                    *reinterpret_cast<uint2 *>(&sm.b[wr][2 * wc]) = make_uint2(x, y);
+                } else {
+                    sm.b[wr][0] = x;
+                    sm.b[wr][1] = y;
+                    sm.b[wr][2] = z;
+                }
+            };
+            if (last_start) {
+                // the last sweep of the call keeps its bond bytes (the warp's own rows)
+                put(bx, by, bz);
+                __syncwarp();
+                for (int i = 0; i < WROWS; ++i) {
+                    const int r = WROWS * warp + i, y = r % G::TY, z = r / G::TY;
+                    if (y >= th || z >= td) continue;
+                    const uint32_t g0 = gidx(0, y, z);
+#pragma unroll
+                    for (int c = 0; c < TWW; ++c) {
+                        const int x = 32 * c + lane;
+                        if (x >= tw) break;
+                        uint32_t b = ((sm.b[r][DIM == 2 ? 2 * c : 0] >> lane) & 1u) |
+                                     (((sm.b[r][DIM == 2 ? 2 * c + 1 : 1] >> lane) & 1u) << 1);
+                        if (DIM == 3) b |= ((sm.b[r][2] >> lane) & 1u) << 2;
+                        p.bond[g0 + (uint32_t)x] = (uint8_t)b;
+                    }
+                }
+                __syncwarp();
+            }
+            put(bx & valid_mask(wc, tw - 1), wy < th - 1 ? by : 0u, wz < td - 1 ? bz : 0u);
         }
-        code4[idx] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+        if (start && pcc)
+            for (int w = tid; w < S * G::PMW; w += NT) (&sm.pm[0][0])[w] = 0u;
+        if (start && lt == 0 && tid == 0) {
+            obs[j].threshold = thr;
+            obs[j].spans_x = 0;
+            obs[j].spans_y = 0;
+        }
     }
-    if (pcc) {
+    __syncthreads();
+
+    if (start) {
+        // Step 2 inside the tile
+        uint32_t born;
+        if constexpr (DIM == 2)
+            born = tile_label_rows<64>(sm.f.par, sm.b, th, tw);
+        else
+            born = tile_label3(sm.f.par, sm.b, tw, th, td);
+        // the warp's rows of the labelling: bit i of its masks is row lrow(i) and
+        // its lanes are the sites lx
+        const int lx = DIM == 2 ? 32 * (warp % TWW) + lane : lane;
+        auto lrow = [&](int i) {
+            return DIM == 2 ? 32 * (warp / TWW) + i : 4 * (warp & 3) + (i & 3) + G::TY * (8 * (warp >> 2) + (i >> 2));
+        };
+
+        // One node per face site: key = global index of the piece's local root,
+        // parent = the piece's first face slot (the representative).
+        int rs[G::SPT];
+#pragma unroll
+        for (int qq = 0; qq < G::SPT; ++qq) {
+            const int s = tid + qq * NT;
+            int x, y, z;
+            rs[qq] = -1;
+            if (s < S && slot_xyz<DIM>(s, t.e, x, y, z)) {
+                rs[qq] = sroot_marked(sm.f.par, (y + G::TY * z) * G::PW + x);
+                atomicMin(&sm.f.par[rs[qq]], (int)(INFO_BORDER | (uint32_t)s));
+            }
+        }
         __syncthreads();
-        for (int w = tid; w < S * G::PMW; w += NT) p.pmask[nbase * G::PMW + w] = (&sm.pm[0][0])[w];
-    }
-    long long c2 = 0;
-    if (csz) {
-        // every root: an interior cluster adds its |C|^2; a border piece hands
-        // its size to its representative node for the merge
-        for (int w = tid; w < nrows * TWW; w += NT) {
-            const int rr = w % nrows, c = w / nrows;
-            const int y = rr % th, z = rr / th, r = y + G::TY * z;
-            const int base = r * G::PW + 32 * c;
-            const int vw = min(32, tw - 32 * c);
-            for (uint32_t bits = run_heads(ih(r, c)) & valid_mask(0, vw); bits; bits &= bits - 1) {
-                const int v = sm.f.par[base + __ffs(bits) - 1];
-                if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
-                    p.psize[nbase + (v & 0x7FFF)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
-                } else if ((uint32_t)v >= INFO_INTERIOR) {   // bits 16-29 (bit 30 is the flag)
-                    const long long size = ((uint32_t)v >> 16) & 0x3FFFu;
-                    c2 += size * size;
+        // Every interior root gets its record, its cluster's new state (Sec. I
+        // step 3), and is counted; the other labels' nodes take a copy of their
+        // root's record where it is there already (cluster sizes are added at
+        // the roots and labels are root indices: the root's index instead).
+        {
+            uint32_t linked = 0u;
+            int ncl = 0;
+            for (uint32_t bits = born; bits; bits &= bits - 1) {
+                const int r = lrow(__ffs(bits) - 1), x = r * G::PW + lx;
+                const int v = sm.f.par[x];
+                if (v == x) {
+                    const uint32_t s = qsm ? sm.qs[r][lx] : cluster_state(gidx(lx, r % G::TY, r / G::TY), klo, khi, k0, k1, q);
+                    sm.f.par[x] = (int)(INFO_INTERIOR | (S + s));
+                    ++ncl;
+                } else if (v >= 0) {
+                    linked |= bits & -bits;
                 }
+            }
+            ncl = __reduce_add_sync(FULL, ncl);
+            if (lane == 0 && ncl) atomicAdd(&sm.acc[3], ncl);
+            for (; linked; linked &= linked - 1) {
+                const int x = lrow(__ffs(linked) - 1) * G::PW + lx;
+                int v = sm.f.par[x], w = sm.f.par[v];
+                while ((uint32_t)w < INFO_INTERIOR && w != v) {
+                    v = w;
+                    w = sm.f.par[v];
+                }
+                sm.f.par[x] = w == v || csz || last_start ? v : w;
+            }
+        }
+#pragma unroll
+        for (int qq = 0; qq < G::SPT; ++qq) {
+            const int s = tid + qq * NT;
+            if (s >= S) break;
+            const size_t node = nbase + s;
+            if (rs[qq] >= 0) {
+                const int rep = sm.f.par[rs[qq]] & 0xFFFF;
+                p.npar[node] = (int32_t)(nbase + rep);
+                p.nkey[node] = (int32_t)(gfor(rs[qq]) | (rep == s ? KEY_REP : 0u));
+            } else {
+                p.npar[node] = (int32_t)node;
+                p.nkey[node] = (int32_t)KEY_NONE;
+            }
+            if (csz) p.csize[node] = 0;   // the merge adds piece sizes at root nodes
+        }
+        __syncthreads();
+        // Every site's 2-byte code (the low half of its root's record): border
+        // pieces by representative slot, interior clusters S + their new state.
+        // Lane = column: a site's entry, its label's node, seldom a third one.
+        const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc);
+        if (!gather && !last_start && tw == G::TX && th == G::TY && td == G::TZ) {
+#pragma unroll 2
+            for (int i = 0; i < 32; i += 4) {
+                int v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = sm.f.par[lrow(i + e) * G::PW + lx];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if ((uint32_t)v[e] < INFO_INTERIOR) v[e] = sm.f.par[v[e]];   // records: negative or >= INFO_INTERIOR
+                while (min(min((uint32_t)v[0], (uint32_t)v[1]), min((uint32_t)v[2], (uint32_t)v[3])) < INFO_INTERIOR) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if ((uint32_t)v[e] < INFO_INTERIOR) v[e] = sm.f.par[v[e]];
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) code[lrow(i + e) * G::TX + lx] = (uint16_t)v[e];
+            }
+        } else {
+            // Cluster sizes and piece masks, gathered down the lane's rows and added
+            // when its cluster changes: a size goes to bits 16-30 of the root's
+            // record (a piece or cluster holds at most 8192 sites; the codes read
+            // bits 0-15 only), the coordinates of a border piece to its masks.
+            int cur = -1, cur_v = 0;
+            uint32_t cur_rows = 0u;
+            auto flush = [&]() {
+                if (!cur_rows) return;
+                if (csz) atomicAdd(&sm.f.par[cur], __popc(cur_rows) << 16);
+                if (pcc && cur_v < 0) {
+                    uint32_t *pm = sm.pm[cur_v & 0xFFFF];
+                    if (DIM == 2) {
+                        atomicOr(pm + (warp % TWW), 1u << lane);
+                        atomicOr(pm + 4 + warp / TWW, cur_rows);
+                    } else {
+                        // bits y and 16 + z of the rows (bit 4 zz + yy of the mask)
+                        uint32_t ys = cur_rows | (cur_rows >> 16);
+                        ys |= ys >> 8;
+                        ys |= ys >> 4;
+                        uint32_t zs = cur_rows | (cur_rows >> 1);
+                        zs = (zs | (zs >> 2)) & 0x11111111u;   // bit 4 zz
+                        zs = (zs | (zs >> 3)) & 0x03030303u;
+                        zs = (zs | (zs >> 6)) & 0x000F000Fu;
+                        zs = (zs | (zs >> 12)) & 0xFFu;
+                        atomicOr(pm, 1u << lane);
+                        atomicOr(pm + 1, ((ys & 0xFu) << (4 * (warp & 3))) | (zs << (16 + 8 * (warp >> 2))));
+                    }
+                }
+            };
+#pragma unroll 2
+            for (int i = 0; i < 32; ++i) {
+                const int r = lrow(i), y = r % G::TY, z = r / G::TY;
+                if (y >= th || z >= td) continue;
+                int root = r * G::PW + lx;
+                int v = lx < tw ? sm.f.par[root] : (int)(INFO_INTERIOR | (uint32_t)S);
+                while ((uint32_t)v < INFO_INTERIOR) {
+                    root = v;
+                    v = sm.f.par[v];
+                }
+                code[r * G::TX + lx] = (uint16_t)v;
+                if (lx >= tw) continue;
+                if (last_start && v >= 0) p.label[gidx(lx, y, z)] = (int32_t)gfor(root);
+                if (gather) {
+                    const int key = csz ? root : v;
+                    if (key != cur) {
+                        flush();
+                        cur = key;
+                        cur_v = v;
+                        cur_rows = 0u;
+                    }
+                    cur_rows |= 1u << i;
+                }
+            }
+            if (gather) flush();
+        }
+        if (gather) {
+            __syncthreads();
+            if (pcc)
+                for (int w = tid; w < S * G::PMW; w += NT) p.pmask[nbase * G::PMW + w] = (&sm.pm[0][0])[w];
+            if (csz) {
+                // every root: an interior cluster adds its |C|^2; a border piece hands
+                // its size to its representative node for the merge
+                unsigned long long c2 = 0ull;
+                for (uint32_t bits = born; bits; bits &= bits - 1) {
+                    const int v = sm.f.par[lrow(__ffs(bits) - 1) * G::PW + lx];
+                    if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
+                        p.psize[nbase + (v & 0xFFFF)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
+                    } else if ((uint32_t)v >= INFO_INTERIOR) {   // bits 16-29 (bit 30 is the flag)
+                        const unsigned long long size = ((uint32_t)v >> 16) & 0x3FFFu;
+                        c2 += size * size;
+                    }
+                }
+                if (c2) atomicAdd(&sm.acc_c2[1], c2);
+                __syncthreads();
             }
         }
     }
-    long long v4[4] = {nb, ncl_interior, c2, 0};
-    DevObs *o = obs + j;
-    unsigned long long *const dst[4] = {&o->nbonds, &o->nclusters, &o->csize2, nullptr};
-    block_sum_atomic<NT, 4>(v4, dst, sm.red);
+    // the tile's sums (every contribution but a sweep's own csize2 was added
+    // before a barrier above)
+    if (tid < 4) {
+        const int half = tid >> 1;            // 0: sweep j-1, 1: sweep j
+        if (half == 0 ? fin : start) {
+            DevObs *o = obs + (j - 1 + half);
+            const long long v = sm.acc[tid];
+            unsigned long long *dst = tid == 0 ? &o->bond_sum : tid == 1 ? &o->mag : tid == 2 ? &o->nbonds : &o->nclusters;
+            if (v) atomicAdd(dst, (unsigned long long)v);
+        }
+    } else if ((F & FEAT_CSIZE) && tid < 6) {
+        const int half = tid - 4;
+        if (csz && (half == 0 ? fin : start) && sm.acc_c2[half])
+            atomicAdd(&obs[j - 1 + half].csize2, sm.acc_c2[half]);
+    }
 }
 
 // ------------------------------------------------ topological rule (RF_WIND)

@@ -32,3 +32,24 @@ def test_word_and_subtile_edges(sw, orc, L, tile_h):
                 np.testing.assert_array_equal(lat.spins(), ref.spin)
                 np.testing.assert_array_equal(lat.labels(), ref.label)
                 np.testing.assert_array_equal(lat.bonds(), ref.bond)
+
+
+# Potts tiles (128 x 64, 32 x 16 x 16): word edges and odd rows in 2D; in 3D
+# row blocks of 4 x 8, quarter words at their boundaries, and rows that start
+# at every place of a Philox block.  With and without csize (labels then keep
+# their roots' indices) and with the table's last states (q = 256).
+@pytest.mark.parametrize("csize", [False, True])
+@pytest.mark.parametrize("dim,L,q", [(2, 63, 3), (2, 66, 2), (2, 126, 256), (2, 191, 3), (2, 193, 2),
+                                     (3, 5, 2), (3, 12, 256), (3, 15, 3), (3, 18, 2), (3, 31, 2), (3, 47, 3),
+                                     (3, 52, 2)])
+def test_potts_word_and_block_edges(sw, orc, dim, L, q, csize):
+    tc = 1.0 / np.log(1 + np.sqrt(q)) if dim == 2 else (2.2557 if q == 2 else 1.8164)
+    for T in (0.8 * tc, tc, 1.5 * tc):
+        ref = orc.PottsChain(dim, L, q, 1.0, T, L, csize=csize)
+        with sw.PottsLattice(dim, L, q, T=T, seed=L, csize=csize) as lat:
+            for n in (1, 3):
+                lat.sweep(n)
+                assert_obs_equal(lat.observables(), ref.run(n))
+                np.testing.assert_array_equal(lat.spins(), ref.spin)
+                np.testing.assert_array_equal(lat.labels(), ref.label)
+                np.testing.assert_array_equal(lat.bonds(), ref.bond)
