@@ -35,12 +35,15 @@ constexpr int CROSS_WORDS = 8;    // per tile: 4 words right-edge bits, 4 words 
 // 30-bit global roots: the GPU path supports N = L*L <= 2^30.
 constexpr uint32_t ROOT_MASK = 0x3FFFFFFFu;
 constexpr uint32_t FINAL_SPIN = 0x80000000u;
-// A node key is a 30-bit site index (bits 0-29) plus KEY_REP; an edge slot
-// past the tile's sites holds KEY_NONE, outside that range, so it differs
-// from every real key up to site 2^30 - 1 (the corner of an L = 32768 lattice).
-constexpr uint32_t KEY_NONE = 0x80000000u;
+// A node of the border forest is {parent, key} in one 8-byte word, so that a
+// walk gets both with one load.  A key is a 30-bit site index (bits 0-29), the
+// minimum of the piece, with KEY_REP and, on the Ising path, the new spin that
+// the piece's cluster takes if that site is the cluster's minimum (FINAL_SPIN):
+// the merge needs no draw.  An edge slot past the tile's sites has parent
+// NODE_NONE and key 0.
 constexpr uint32_t KEY_REP = 0x40000000u;    // the node represents its piece
 constexpr uint32_t KEY_MASK = 0x3FFFFFFFu;
+constexpr int32_t NODE_NONE = -1;
 
 // 2-byte tile-local cluster code of a site, written when a sweep starts and
 // read when it finishes: the byte offset (4 x index) into the table of the
@@ -90,8 +93,7 @@ struct Replica {
     uint16_t *code;         // tiles * TH * TW site codes
     uint32_t *bondbits;     // tiles * TH * 8 words (last sweep of a call only)
     uint32_t *cross;        // tiles * CROSS_WORDS
-    int32_t *npar;          // tiles * S node parents
-    int32_t *nkey;          // tiles * S node keys (global root candidates)
+    int2 *node;             // tiles * S border nodes {parent, key}
     uint32_t *nfinal;       // tiles * S resolved (root | spin << 30)
     // PCC scratch (Sec. III): spanning candidates and their coverage (null otherwise)
     uint32_t *pmask;        // tiles * S * 8: a piece's column mask (4 words), row mask (4 words)
@@ -151,14 +153,6 @@ __device__ __forceinline__ U4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c
     return U4{c0, c1, c2, c3};
 }
 
-// The method's blocks: counter = (word, sweep lo, sweep hi, stream).
-__device__ __forceinline__ U4 stream_block(const Replica &R, uint64_t word, uint64_t sweep,
-                                           uint32_t stream)
-{
-    return philox4x32_10((uint32_t)word, (uint32_t)sweep, (uint32_t)(sweep >> 32), stream,
-                         R.key0, R.key1);
-}
-
 __device__ __forceinline__ uint32_t u4_word(const U4 &v, int i)
 {
     return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
@@ -181,7 +175,7 @@ __device__ __forceinline__ uint32_t valid_mask(int c, int tw)
 // Resolved final (root | spin << 30) of an edge slot: a representative holds
 // its cluster's, and so does every top or left slot (the ones a neighbour
 // reads for its halo).  Only nfinal is read: the tile kernel that reads a
-// neighbour's finals rewrites that neighbour's npar and nkey concurrently.
+// neighbour's finals rewrites that neighbour's nodes concurrently.
 
 // ------------------------------------------------------------ tile geometry
 struct Tile {
@@ -254,22 +248,6 @@ __device__ __forceinline__ int sfind(volatile int *par, int x)
     return x;
 }
 
-// As sunite, returning the root of the united set.
-__device__ __forceinline__ int sunite_root(volatile int *par, int a, int b)
-{
-    for (;;) {
-        a = sfind(par, a);
-        b = sfind(par, b);
-        if (a == b) return a;
-        if (a > b) {
-            const int t = a;
-            a = b;
-            b = t;
-        }
-        if (atomicCAS((int *)&par[b], b, a) == b) return a;
-    }
-}
-
 __device__ __forceinline__ void sunite(volatile int *par, int a, int b)
 {
     for (;;) {
@@ -337,19 +315,8 @@ struct TileCfg {
     static constexpr int MINB = TH == 32 ? 11 : TH == 64 ? 6 : TH == 96 ? 4 : 3;
 };
 
-// Root of x without writing (a forest no thread is changing any more).
-__device__ __forceinline__ int sroot(const volatile int *par, int x)
-{
-    int p = par[x];
-    while (p != x) {
-        x = p;
-        p = par[x];
-    }
-    return x;
-}
-
-// The same while other threads replace roots by border records (negative):
-// a node that holds one is a root.
+// Root of x without writing, while other threads replace roots by border
+// records (negative): a node that holds one is a root.
 __device__ __forceinline__ int sroot_marked(const volatile int *par, int x)
 {
     int p = par[x];
@@ -396,107 +363,6 @@ __device__ __forceinline__ int info_slot(int v) { return (v & 0xFFFF) >> 2; }
 __device__ __forceinline__ uint32_t run_heads(uint32_t h)
 {
     return ~((h & 0x7FFFFFFFu) << 1);
-}
-
-// Local index of the head of the run that holds bit x of a row word whose
-// first site has local index base.
-__device__ __forceinline__ int head_of(uint32_t heads, int base, int x)
-{
-    return base + 31 - __clz(heads & (0xFFFFFFFFu >> (31 - x)));
-}
-
-// Connected components of the intra-tile bonds (H: right links, whose link
-// leaving the tile's last column is ignored; V: down links, ignored in the
-// tile's last row).  The tile is cut into 32 x 32 sub-tiles, one per warp,
-// and the forest lives on run heads only (a run = maximal chain of right
-// bonds inside one sub-tile row; its head is its leftmost site):
-//   1. lane r of a warp owns row r of its sub-tile: it unites the runs of its
-//      row with the runs below at every down bond, skipping a bond when the
-//      bond to its left already joins the same two runs;
-//   2. unions across the sub-tile boundaries inside the tile.
-// Links always hang the larger root under the smaller, so par[x] < x unless x
-// is a root and every root is the minimum local index of its piece; local
-// row-major order is the global order, so the root is the piece's minimum
-// site.  Forest indices are padded, y * PW + x, which keeps row-major order
-// and puts the rows of a column on distinct shared-memory banks.
-template <int TH>
-__device__ void tile_label(volatile int *par, const uint32_t (*Hb)[TWW], const uint32_t (*Vb)[TWW],
-                           int th, int tw)
-{
-    constexpr int NT = TileCfg<TH>::NT;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int sx = warp & (TWW - 1), sy = warp / TWW;
-    // the intra-tile bonds: the tile's last column has no right link inside,
-    // its last row no down link inside
-    auto H = [&](int y, int c) { return Hb[y][c] & valid_mask(c, tw - 1); };
-    auto V = [&](int y, int c) { return y < th - 1 ? Vb[y][c] : 0u; };
-
-    // ---- 1. inside each sub-tile, lane = row
-    {
-        const int y = 32 * sy + lane;
-        const bool row_ok = y < th;
-        const uint32_t heads = run_heads(row_ok ? H(y, sx) : 0u);
-        const uint32_t heads_below = __shfl_down_sync(0xFFFFFFFFu, heads, 1);
-        const uint32_t v = (row_ok && lane < 31) ? V(y, sx) : 0u;
-        const uint32_t u = v & (~(v << 1) | heads | heads_below);
-        const int base = y * PW + 32 * sx;
-        if (row_ok) {   // every site of the row its own root (only run heads are used)
-#pragma unroll
-            for (int x = 0; x < 32; ++x) par[base + x] = base + x;
-        }
-        __syncwarp();
-        // consecutive contacts often share a run above or below: their
-        // finds start at the last union's root (an ancestor of that run's
-        // head), not at the head
-        int prev_a = -1, prev_b = -1, prev_r = 0;
-        for (uint32_t b = u; b; b &= b - 1) {
-            const int x = __ffs(b) - 1;
-            const int ha = head_of(heads, base, x), hb = head_of(heads_below, base + PW, x);
-            prev_r = sunite_root(par, ha == prev_a ? prev_r : ha, hb == prev_b ? prev_r : hb);
-            prev_a = ha;
-            prev_b = hb;
-        }
-    }
-    __syncthreads();
-
-    // ---- 2. links across sub-tile boundaries: vertical boundaries between
-    //         sub-tile columns, horizontal ones between sub-tile rows
-    {
-        constexpr int NV = (TWW - 1) * TH;
-        constexpr int NH = (TH / 32 - 1) * TW;
-        for (int q = threadIdx.x; q < NV + NH; q += NT) {
-            int a, b;
-            if (q < NV) {
-                const int bnd = q / TH + 1, y = q % TH;     // link (32 bnd - 1, y) - (32 bnd, y)
-                if (y >= th || !((H(y, bnd - 1) >> 31) & 1u)) continue;
-                // skip when the row above already joins the same two sites
-                // through down links inside the sub-tiles (united in phase 1;
-                // at a sub-tile row edge those down links are phase-2 links
-                // themselves and could justify each other in a cycle)
-                if ((y & 31) != 0 && ((H(y - 1, bnd - 1) >> 31) & 1u) &&
-                    ((V(y - 1, bnd - 1) >> 31) & 1u) && (V(y - 1, bnd) & 1u))
-                    continue;
-                a = head_of(run_heads(H(y, bnd - 1)), y * PW + 32 * (bnd - 1), 31);
-                b = y * PW + 32 * bnd;   // column 0 of a sub-tile row is always a head
-            } else {
-                const int r = q - NV;
-                const int bnd = r / TW + 1, x = r % TW;     // link (x, 32 bnd - 1) - (x, 32 bnd)
-                const int y = 32 * bnd - 1;
-                if (y + 1 >= th || !((V(y, x >> 5) >> (x & 31)) & 1u)) continue;
-                // skip when the column to the left already joins the same two
-                // sites through right links inside the sub-tiles
-                if ((x & 31) != 0 && ((V(y, (x - 1) >> 5) >> ((x - 1) & 31)) & 1u) &&
-                    ((H(y, (x - 1) >> 5) >> ((x - 1) & 31)) & 1u) &&
-                    ((H(y + 1, (x - 1) >> 5) >> ((x - 1) & 31)) & 1u))
-                    continue;
-                const int c = x >> 5;
-                a = head_of(run_heads(H(y, c)), y * PW + 32 * c, x & 31);
-                b = head_of(run_heads(H(y + 1, c)), (y + 1) * PW + 32 * c, x & 31);
-            }
-            sunite(par, a, b);
-        }
-    }
-    __syncthreads();
 }
 
 // Connected components of the intra-tile bonds: B[y][2c] holds the right-link
@@ -611,62 +477,22 @@ __device__ __forceinline__ int gload(const int32_t *p)
     return *(const volatile int32_t *)p;
 }
 
-__device__ __forceinline__ int gfind(int32_t *par, int x)
+// A node in one 8-byte load: {parent, key}.
+__device__ __forceinline__ int2 nload(const int2 *p)
 {
-    int p = gload(par + x);
-    while (p != x) {
-        const int gp = gload(par + p);
-        if (gp != p) *(volatile int32_t *)(par + x) = gp;
-        x = gp;
-        p = gload(par + x);
-    }
-    return x;
+    const unsigned long long v = *reinterpret_cast<const volatile unsigned long long *>(p);
+    return make_int2((int)(uint32_t)v, (int)(uint32_t)(v >> 32));
 }
 
-// Union of the node forest ordered by key: the root with the larger key is
-// hung under the root with the smaller one.  Keys are the global indices of
-// the pieces' local roots, distinct between pieces and equal only inside one
-// piece (whose non-representative nodes are never roots), so keys fall
-// strictly along every chain of root links (no cycle can form) and each
-// set's root carries the set's minimum key: the global cluster root.
-__device__ __forceinline__ void gunite_by_key(int32_t *par, const int32_t *key, int a, int b)
+__device__ __forceinline__ int pload(const int2 *p)
 {
-    for (;;) {
-        a = gfind(par, a);
-        b = gfind(par, b);
-        if (a == b) return;
-        if (key[a] > key[b]) {
-            const int t = a;
-            a = b;
-            b = t;
-        }
-        if (atomicCAS(par + b, b, a) == b) return;
-    }
+    return gload(&p->x);
 }
 
-// --------------------------------------------------------- block reductions
-template <int NT, int K>
-__device__ __forceinline__ void block_sum_atomic(long long (&v)[K], unsigned long long *const dst[K],
-                                                 long long (*red)[K])
+// Points node n at p (an ancestor).
+__device__ __forceinline__ void pstore(int2 *n, int p)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-        long long x = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o);
-        if (lane == 0) red[warp][q] = x;
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < K; ++q) {
-            long long x = lane < NT / 32 ? red[lane][q] : 0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o);
-            if (lane == 0 && dst[q] && x != 0) atomicAdd(dst[q], (unsigned long long)x);
-        }
-    }
+    *(volatile int32_t *)&n->x = p;
 }
 
 // 16 bytes from global to shared memory without passing through registers
@@ -1104,12 +930,13 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             const size_t node = (size_t)t.lt * S + s;
             if (rs[q] >= 0) {
                 const int rep = info_slot(sm.par[rs[q]]);
-                R.npar[node] = (int32_t)((size_t)t.lt * S + rep);
-                R.nkey[node] = (int32_t)((gbase + (uint32_t)(rs[q] / PW) * uL + (uint32_t)(rs[q] % PW)) |
-                                         (rep == s ? KEY_REP : 0u));
+                const int ry = rs[q] / PW, rx = rs[q] - ry * PW;
+                const uint32_t spin = (sm.u.spb[ry][rx >> 5] >> (rx & 31)) << 31;   // FINAL_SPIN
+                R.node[node] = make_int2((int)((size_t)t.lt * S + rep),
+                                         (int)((gbase + (uint32_t)ry * uL + (uint32_t)rx) |
+                                               (rep == s ? KEY_REP : 0u) | spin));
             } else {
-                R.npar[node] = (int32_t)node;
-                R.nkey[node] = (int32_t)KEY_NONE;
+                R.node[node] = make_int2(NODE_NONE, 0);
             }
             if (csz) R.csize[node] = 0;   // the merge adds piece sizes at root nodes
         }
@@ -1288,11 +1115,11 @@ __device__ __forceinline__ int wfind(unsigned long long *lk, int x, uint32_t &of
     return x;
 }
 
-// Union by key (as gunite_by_key) of the nodes a and b joined by a bond that
-// moves by d from a to b.  If they already share a root, the bond closes a
+// Union by key of the nodes a and b joined by a bond that moves by d from a to
+// b: the root with the larger key hangs under the other.  If they already share a root, the bond closes a
 // cycle: a non-zero displacement around it is a winding, recorded in the
 // sweep's spans_x / spans_y.
-__device__ __forceinline__ void wunite(unsigned long long *lk, const int32_t *key, int a, int b, uint32_t d,
+__device__ __forceinline__ void wunite(unsigned long long *lk, const int2 *node, int a, int b, uint32_t d,
                                        DevObs *o)
 {
     for (;;) {
@@ -1307,7 +1134,7 @@ __device__ __forceinline__ void wunite(unsigned long long *lk, const int32_t *ke
         }
         int lo = ra, hi = rb;
         uint32_t off = rel;
-        if ((uint32_t)key[ra] > (uint32_t)key[rb]) {
+        if (((uint32_t)node[ra].y & KEY_MASK) > ((uint32_t)node[rb].y & KEY_MASK)) {
             lo = rb;
             hi = ra;
             off = wind_neg(rel);
@@ -1390,8 +1217,8 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
 #pragma unroll
         for (int q = 0; q < MC::EPT; ++q) {
             if (!prev[q]) continue;
-            const uint32_t ka = (uint32_t)R.nkey[na[q]] ^ (uint32_t)R.nkey[na[q] - 1];
-            const uint32_t kb = (uint32_t)R.nkey[nb[q]] ^ (uint32_t)R.nkey[nb[q] - 1];
+            const uint32_t ka = (uint32_t)R.node[na[q]].y ^ (uint32_t)R.node[na[q] - 1].y;
+            const uint32_t kb = (uint32_t)R.node[nb[q]].y ^ (uint32_t)R.node[nb[q] - 1].y;
             if (((ka | kb) & KEY_MASK) == 0) na[q] = -1;
         }
 #pragma unroll
@@ -1399,7 +1226,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
             if (na[q] < 0) continue;
             // a right link moves by (+1, 0), a down link by (0, +1)
             const bool right = threadIdx.x + q * MC::MT < TH;
-            wunite(R.nlink, R.nkey, na[q], nb[q], right ? wind_off(1, 0) : wind_off(0, 1), R.obs + j);
+            wunite(R.nlink, R.node, na[q], nb[q], right ? wind_off(1, 0) : wind_off(0, 1), R.obs + j);
         }
         return;
     }
@@ -1418,10 +1245,11 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
 #pragma unroll
     for (int q = 0; q < MC::EPT; ++q) {
         if (na[q] < 0) continue;
-        pa[q] = gload(R.npar + na[q]);
-        pb[q] = gload(R.npar + nb[q]);
-        ka[q] = R.nkey[na[q]];
-        kb[q] = R.nkey[nb[q]];
+        const int2 va = nload(R.node + na[q]), vb = nload(R.node + nb[q]);
+        pa[q] = va.x;
+        ka[q] = va.y;
+        pb[q] = vb.x;
+        kb[q] = vb.y;
     }
     __syncthreads();
     bool live[MC::EPT];
@@ -1448,10 +1276,9 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
         const bool u_hi = ((uint32_t)ka[q] & KEY_MASK) > ((uint32_t)kb[q] & KEY_MASK);
         const int hi = u_hi ? u : v, lo = u_hi ? v : u;
         const bool inner = u_hi ? (ra && pa[q] != na[q]) : (rb && pb[q] != nb[q]);
-        if (!inner && atomicCAS(R.npar + hi, hi, lo) == hi) live[q] = false;
+        if (!inner && atomicCAS(&R.node[hi].x, hi, lo) == hi) live[q] = false;
     }
-    // The thread's remaining unions (gunite_by_key's steps) advance in lock
-    // step, both finds of every link at once, so their L2 round trips
+    // The thread's remaining unions advance in lock step, both finds of every link at once, so their L2 round trips
     // overlap: each pass climbs every find that is not at a root (path
     // splitting: the node it came from is pointed at the parent just read, an
     // ancestor), links two distinct roots by compare-and-swap, the larger key
@@ -1475,12 +1302,12 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
                 // path splitting rewrites representatives only: a slot that
                 // is not one keeps its own representative as its parent
                 if (!ra) {
-                    if (sa[q] >= 0) *(volatile int32_t *)(R.npar + sa[q]) = pa[q];
+                    if (sa[q] >= 0) pstore(R.node + sa[q], pa[q]);
                     sa[q] = ((uint32_t)ka[q] & KEY_REP) ? xa[q] : -1;
                     xa[q] = pa[q];
                 }
                 if (!rb) {
-                    if (sb[q] >= 0) *(volatile int32_t *)(R.npar + sb[q]) = pb[q];
+                    if (sb[q] >= 0) pstore(R.node + sb[q], pb[q]);
                     sb[q] = ((uint32_t)kb[q] & KEY_REP) ? xb[q] : -1;
                     xb[q] = pb[q];
                 }
@@ -1488,9 +1315,9 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
             } else if (xa[q] == xb[q]) {
                 live[q] = false;
             } else {
-                const bool a_lo = ka[q] < kb[q];
+                const bool a_lo = ((uint32_t)ka[q] & KEY_MASK) < ((uint32_t)kb[q] & KEY_MASK);
                 const int lo = a_lo ? xa[q] : xb[q], hi = a_lo ? xb[q] : xa[q];
-                if (atomicCAS(R.npar + hi, hi, lo) == hi) live[q] = false;
+                if (atomicCAS(&R.node[hi].x, hi, lo) == hi) live[q] = false;
                 else more = true;
             }
         }
@@ -1498,10 +1325,11 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
 #pragma unroll
         for (int q = 0; q < MC::EPT; ++q) {
             if (!live[q]) continue;
-            pa[q] = gload(R.npar + xa[q]);
-            pb[q] = gload(R.npar + xb[q]);
-            ka[q] = R.nkey[xa[q]];
-            kb[q] = R.nkey[xb[q]];
+            const int2 va = nload(R.node + xa[q]), vb = nload(R.node + xb[q]);
+            pa[q] = va.x;
+            ka[q] = va.y;
+            pb[q] = vb.x;
+            kb[q] = vb.y;
         }
     }
 }
@@ -1522,7 +1350,8 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_init(const SweepArgs 
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
         const int s = threadIdx.x + q * MC::MT, n = base + s;
-        const int p = R.npar[n];
+        int p = R.node[n].x;
+        if (p == NODE_NONE) p = n;
         uint32_t off = 0u;
         int site, rsite;
         if (p != n && slot_site<TH>(s, t.tw, t.th, site) && slot_site<TH>(p - base, t.tw, t.th, rsite))
@@ -1556,7 +1385,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_jump(const SweepArgs
             unsigned long long v[MC::NPT], w[MC::NPT];
 #pragma unroll
             for (int q = 0; q < MC::NPT; ++q)
-                v[q] = ((uint32_t)R.nkey[base + threadIdx.x + q * MC::MT] & KEY_REP)
+                v[q] = ((uint32_t)R.node[base + threadIdx.x + q * MC::MT].y & KEY_REP)
                            ? wload(R.nlink + base + threadIdx.x + q * MC::MT) : ~0ull;
 #pragma unroll
             for (int q = 0; q < MC::NPT; ++q) w[q] = v[q] != ~0ull ? wload(R.nlink + (uint32_t)v[q]) : ~0ull;
@@ -1568,21 +1397,18 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_jump(const SweepArgs
         }
         return;
     }
-    uint32_t key[MC::NPT];
     int p[MC::NPT], gp[MC::NPT];
 #pragma unroll
-    for (int q = 0; q < MC::NPT; ++q) key[q] = (uint32_t)R.nkey[base + threadIdx.x + q * MC::MT];
-#pragma unroll
-    for (int q = 0; q < MC::NPT; ++q) {   // loaded with the key, not after it: one round trip less
-        const int pq = gload(R.npar + base + threadIdx.x + q * MC::MT);
-        p[q] = (key[q] & KEY_REP) ? pq : -1;
+    for (int q = 0; q < MC::NPT; ++q) {
+        const int2 v = nload(R.node + base + threadIdx.x + q * MC::MT);
+        p[q] = ((uint32_t)v.y & KEY_REP) ? v.x : -1;
     }
     for (int r = 0; r < MERGE_JUMP_ROUNDS; ++r) {
 #pragma unroll
-        for (int q = 0; q < MC::NPT; ++q) gp[q] = p[q] >= 0 ? gload(R.npar + p[q]) : -1;
+        for (int q = 0; q < MC::NPT; ++q) gp[q] = p[q] >= 0 ? pload(R.node + p[q]) : -1;
 #pragma unroll
         for (int q = 0; q < MC::NPT; ++q) {
-            if (gp[q] != p[q]) *(volatile int32_t *)(R.npar + base + threadIdx.x + q * MC::MT) = gp[q];
+            if (gp[q] != p[q]) pstore(R.node + base + threadIdx.x + q * MC::MT, gp[q]);
             p[q] = gp[q];
         }
     }
@@ -1591,8 +1417,8 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_jump(const SweepArgs
 // Resolve every node once the unions are done: each representative walks to
 // its root r (key: the cluster's minimum site index), for PCC lattices writes
 // r over every node of the walk (full path compression: no union happens any
-// more, so every node on it has root r) and stores the cluster's root and new spin,
-// bit (root mod 128) of Philox(root/128, k, SPIN) (Sec. I step 3); a top or
+// more, so every node on it has root r) and stores the cluster's root and new
+// spin, both in r's key (Sec. I step 3); a top or
 // left slot that is not a representative then copies its representative's.
 // Counts the clusters that touch a tile border (one root node each).
 template <int TH, bool W>
@@ -1605,17 +1431,22 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;
     const bool wind = W && (R.flags & RF_WIND);   // the forest lives in nlink
-    auto parent = [&](int x) { return wind ? (int)(uint32_t)wload(R.nlink + x) : gload(R.npar + x); };
-    uint32_t key[MC::NPT];
+    // node x with its forest's parent
+    auto node_of = [&](int x) {
+        int2 v = nload(R.node + x);
+        if (wind) v.x = (int)(uint32_t)wload(R.nlink + x);
+        return v;
+    };
+    uint32_t key[MC::NPT], rkey[MC::NPT];   // of the slot, and of the node its walk is at
     int r[MC::NPT], p[MC::NPT];
-#pragma unroll
-    for (int q = 0; q < MC::NPT; ++q) key[q] = (uint32_t)R.nkey[base + threadIdx.x + q * MC::MT];
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
         r[q] = base + threadIdx.x + q * MC::MT;
         // a representative walks its forest; any other slot keeps its parent
         // from the tile kernel (its representative) for the copy below
-        p[q] = (wind && (key[q] & KEY_REP)) ? parent(r[q]) : gload(R.npar + r[q]);
+        const int2 v = nload(R.node + r[q]);
+        key[q] = rkey[q] = (uint32_t)v.y;
+        p[q] = (wind && (key[q] & KEY_REP)) ? node_of(r[q]).x : v.x;
     }
     // the walks of the thread's representatives advance in lock step
     for (;;) {
@@ -1630,13 +1461,13 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
         if (!more) break;
 #pragma unroll
         for (int q = 0; q < MC::NPT; ++q)
-            if (key[q] & KEY_REP) p[q] = parent(r[q]);
+            if ((key[q] & KEY_REP) && p[q] == r[q]) {   // the node just reached
+                const int2 v = node_of(r[q]);
+                p[q] = v.x;
+                rkey[q] = (uint32_t)v.y;
+            }
     }
     __shared__ uint32_t rfin[MC::S];   // the finals of the representatives
-    uint32_t rkey[MC::NPT];
-#pragma unroll
-    for (int q = 0; q < MC::NPT; ++q) rkey[q] = (key[q] & KEY_REP) ? (uint32_t)R.nkey[r[q]] & KEY_MASK : 0u;
-    const uint64_t k = R.sweep0 + (uint64_t)j;
     int nroots = 0;
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
@@ -1662,18 +1493,16 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
                 // straight from its parent; no other kernel reads the forest
                 // again before the next tile launch rewrites it
                 for (int x = n; x != r[q];) {
-                    const int nx = gload(R.npar + x);
-                    *(volatile int32_t *)(R.npar + x) = r[q];
+                    const int nx = pload(R.node + x);
+                    pstore(R.node + x, r[q]);
                     x = nx;
                 }
             }
             nroots += r[q] == n;
             if (R.flags & RF_CSIZE) atomicAdd(R.csize + r[q], R.psize[n]);
-            const U4 u = stream_block(R, rkey[q] >> 7, k, STREAM_SPIN);
-            const int bit = rkey[q] & 127;
-            const uint32_t spin = (u4_word(u, bit >> 5) >> (bit & 31)) & 1u;
-            R.nfinal[n] = rkey[q] | (spin ? FINAL_SPIN : 0u);
-            rfin[threadIdx.x + q * MC::MT] = R.nfinal[n];
+            const uint32_t f = rkey[q] & ~KEY_REP;
+            R.nfinal[n] = f;
+            rfin[threadIdx.x + q * MC::MT] = f;
         }
     }
     __syncthreads();
@@ -1686,7 +1515,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
     for (int q = 0; q < MC::NPT; ++q) {
         const int s = threadIdx.x + q * MC::MT;
         if (!(key[q] & KEY_REP) && (s < Slots<TH>::BOTTOM || (s >= Slots<TH>::LEFT && s < Slots<TH>::RIGHT)))
-            R.nfinal[base + s] = key[q] == KEY_NONE ? 0u : rfin[p[q] - base];
+            R.nfinal[base + s] = p[q] == NODE_NONE ? 0u : rfin[p[q] - base];
     }
     // every thread of the block gets here; the last warp may be partial
     const int wb = threadIdx.x & ~31;
@@ -1733,8 +1562,9 @@ __global__ void k_pcc_candidates(const SweepArgs a)
         axis = 1;
         node = t.lt * S + SL::TOP + x;
     }
-    int r = gload(R.npar + node);
-    if (!((uint32_t)R.nkey[node] & KEY_REP)) r = gload(R.npar + r);   // via the representative
+    const int2 v = nload(R.node + node);
+    int r = v.x;
+    if (!((uint32_t)v.y & KEY_REP)) r = pload(R.node + r);   // via the representative
     int32_t *c = R.cid + (size_t)r * 2 + axis;
     if (atomicCAS(c, 0, 1) == 0) {
         const int id = atomicAdd(R.ncand + axis, 1);   // < L: at most one per edge site
@@ -1761,7 +1591,7 @@ __global__ void k_pcc_cover(const SweepArgs a)
     const uint4 *pm4 = reinterpret_cast<const uint4 *>(R.pmask + (size_t)nl * 8);
     const uint4 c4 = pm4[0], r4 = pm4[1];
     if (!(c4.x | c4.y | c4.z | c4.w | r4.x | r4.y | r4.z | r4.w)) return;
-    const int r = gload(R.npar + nl);
+    const int r = pload(R.node + nl);
     const Tile t = tile_of(R, g, TH);
     const int cx = R.cid[(size_t)r * 2 + 0], cy = R.cid[(size_t)r * 2 + 1];
     if (cx >= 2) {

@@ -242,7 +242,7 @@ struct sw_ctx {
     uint16_t *code = nullptr;
     uint32_t *bondbits = nullptr;
     uint32_t *cross = nullptr;
-    int32_t *npar = nullptr, *nkey = nullptr;
+    int2 *node = nullptr;
     uint32_t *nfinal = nullptr;
     uint64_t *thr_dev = nullptr;
     Replica *rep_dev = nullptr;
@@ -292,7 +292,7 @@ void ctx_free(sw_ctx *c)
     c->graphs.clear();
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
     c->ev_pool.clear();
-    void *ptrs[] = {c->spin, c->label, c->code, c->bondbits, c->cross, c->npar, c->nkey,
+    void *ptrs[] = {c->spin, c->label, c->code, c->bondbits, c->cross, c->node,
                     c->nfinal, c->thr_dev, c->rep_dev, c->tile_rep, c->jbase, c->bond_bytes, c->obs,
                     c->pmask, c->cid, c->cand, c->ncand, c->cov, c->psize, c->csize, c->nlink, c->nstate, c->wlink};
     for (void *p : ptrs)
@@ -354,8 +354,7 @@ int ctx_create(sw_ctx **out, int32_t L, uint64_t thr, uint64_t seed, bool pcc, u
     if ((e = dalloc(&c->code, nt * c->TH * TW)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->bondbits, nt * c->TH * 2 * TWW)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->cross, nt * CROSS_WORDS)) != cudaSuccess) return fail(e);
-    if ((e = dalloc(&c->npar, nt * c->S)) != cudaSuccess) return fail(e);
-    if ((e = dalloc(&c->nkey, nt * c->S)) != cudaSuccess) return fail(e);
+    if ((e = dalloc(&c->node, nt * c->S)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->nfinal, nt * c->S)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->thr_dev, 1)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->rep_dev, 1)) != cudaSuccess) return fail(e);
@@ -403,8 +402,7 @@ int ctx_create(sw_ctx **out, int32_t L, uint64_t thr, uint64_t seed, bool pcc, u
     R.code = c->code;
     R.bondbits = c->bondbits;
     R.cross = c->cross;
-    R.npar = c->npar;
-    R.nkey = c->nkey;
+    R.node = c->node;
     R.nfinal = c->nfinal;
     R.pmask = c->pmask;
     R.cid = c->cid;
@@ -549,7 +547,7 @@ int run_sweeps(sw_ctx *c, int32_t n)
                 SW_CUDA(cudaEventRecord(e0, c->stream));
                 SW_CUDA(potts_enqueue_tile(c->pd, j, n, c->sweep, obs, c->stream));
                 SW_CUDA(cudaEventRecord(e1, c->stream));
-                if (j < n) SW_CUDA(potts_enqueue_merge(c->pd, j, c->sweep, obs, c->stream));
+                if (j < n) SW_CUDA(potts_enqueue_merge(c->pd, j, n, c->sweep, obs, c->stream));
                 SW_CUDA(cudaEventRecord(e2, c->stream));
                 c->ev_marks.push_back(e0);
                 c->ev_marks.push_back(e1);
@@ -732,10 +730,9 @@ int potts_create(sw_ctx **out, int32_t dim, int32_t L, int32_t q, uint64_t thr, 
     if ((e = dalloc(&c->jbase, 1)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->code, nt * (size_t)g.sites_per_tile)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->cross, nt * (size_t)g.cross_words)) != cudaSuccess) return fail(e);
-    if ((e = dalloc(&c->npar, nt * S)) != cudaSuccess) return fail(e);
-    if ((e = dalloc(&c->nkey, nt * S)) != cudaSuccess) return fail(e);
+    if ((e = dalloc(&c->node, nt * S)) != cudaSuccess) return fail(e);
     if ((e = dalloc(&c->nfinal, nt * S)) != cudaSuccess) return fail(e);
-    if ((e = dalloc(&c->nstate, nt * S)) != cudaSuccess) return fail(e);
+    if ((e = dalloc(&c->nstate, 2 * nt * S)) != cudaSuccess) return fail(e);   // nstate, then kstate
     if (flags & SW_FLAG_CSIZE) {
         if ((e = dalloc(&c->psize, nt * S)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->csize, nt * S)) != cudaSuccess) return fail(e);
@@ -759,10 +756,10 @@ int potts_create(sw_ctx **out, int32_t dim, int32_t L, int32_t q, uint64_t thr, 
     p.label = c->label;
     p.code = c->code;
     p.cross = c->cross;
-    p.npar = c->npar;
-    p.nkey = c->nkey;
+    p.node = c->node;
     p.nfinal = c->nfinal;
     p.nstate = c->nstate;
+    p.kstate = c->nstate + nt * S;
     p.psize = c->psize;
     p.csize = c->csize;
     p.wlink = c->wlink;

@@ -47,9 +47,10 @@ struct PottsDev {
     int32_t *label;                    // N labels of the last sweep
     uint16_t *code;                    // ntiles * sites-per-tile
     uint32_t *cross;                   // ntiles * cross words
-    int32_t *npar, *nkey;              // ntiles * slots
-    uint32_t *nfinal;                  // ntiles * slots: a representative's cluster root
+    int2 *node;                        // ntiles * slots: {parent, key}
+    uint32_t *nfinal;                  // ntiles * slots: a representative's cluster root (last sweep of a call)
     uint8_t *nstate;                   // ntiles * slots: a representative's new state
+    uint8_t *kstate;                   // ntiles * slots: the state a representative's piece takes as a cluster's root
     int32_t *psize, *csize;            // ntiles * slots (RF_CSIZE only)
     int4 *wlink;                       // RF_WIND: ntiles * slots node links {parent, dx, dy, dz}
     // PCC (null otherwise): the threshold lives on the device and follows the
@@ -74,8 +75,8 @@ __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_hot_start(const 
 // Launch j (0 .. nsweeps) of a call: the tile kernel, then (j < nsweeps) the merge of sweep j.
 __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_tile(const PottsDev &p, int j, int nsweeps,
                                                                      uint64_t sweep0, DevObs *obs, cudaStream_t st);
-__attribute__((visibility("hidden"))) cudaError_t potts_enqueue_merge(const PottsDev &p, int j, uint64_t sweep0,
-                                                                      DevObs *obs, cudaStream_t st);
+__attribute__((visibility("hidden"))) cudaError_t potts_enqueue_merge(const PottsDev &p, int j, int nsweeps,
+                                                                      uint64_t sweep0, DevObs *obs, cudaStream_t st);
 // One call of nsweeps sweeps (observables into obs[0 .. nsweeps-1]).
 __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_sweeps(const PottsDev &p, int nsweeps,
                                                                        uint64_t sweep0, DevObs *obs,

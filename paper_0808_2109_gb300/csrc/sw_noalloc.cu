@@ -51,9 +51,8 @@ constexpr size_t OFF_JBASE = OFF_TILE_REP + al(MAX_TILES_STATIC * sizeof(int32_t
 constexpr size_t OFF_CODE = OFF_JBASE + al(sizeof(int32_t));
 constexpr size_t OFF_BONDBITS = OFF_CODE + al((size_t)MAX_TILES_STATIC * TH_STATIC * TW * sizeof(uint16_t));
 constexpr size_t OFF_CROSS = OFF_BONDBITS + al((size_t)MAX_TILES_STATIC * TH_STATIC * 2 * TWW * sizeof(uint32_t));
-constexpr size_t OFF_NPAR = OFF_CROSS + al((size_t)MAX_TILES_STATIC * CROSS_WORDS * sizeof(uint32_t));
-constexpr size_t OFF_NKEY = OFF_NPAR + al((size_t)MAX_TILES_STATIC * S_STATIC * sizeof(int32_t));
-constexpr size_t OFF_NFINAL = OFF_NKEY + al((size_t)MAX_TILES_STATIC * S_STATIC * sizeof(int32_t));
+constexpr size_t OFF_NODE = OFF_CROSS + al((size_t)MAX_TILES_STATIC * CROSS_WORDS * sizeof(uint32_t));
+constexpr size_t OFF_NFINAL = OFF_NODE + al((size_t)MAX_TILES_STATIC * S_STATIC * sizeof(int2));
 constexpr size_t SCRATCH_BYTES = OFF_NFINAL + al((size_t)MAX_TILES_STATIC * S_STATIC * sizeof(uint32_t));
 static_assert(SCRATCH_BYTES == 2755328, "the size quoted in the comments and the header");
 
@@ -141,8 +140,7 @@ extern "C" int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_
     R.code = reinterpret_cast<uint16_t *>(scratch + OFF_CODE);
     R.bondbits = reinterpret_cast<uint32_t *>(scratch + OFF_BONDBITS);
     R.cross = reinterpret_cast<uint32_t *>(scratch + OFF_CROSS);
-    R.npar = reinterpret_cast<int32_t *>(scratch + OFF_NPAR);
-    R.nkey = reinterpret_cast<int32_t *>(scratch + OFF_NKEY);
+    R.node = reinterpret_cast<int2 *>(scratch + OFF_NODE);
     R.nfinal = reinterpret_cast<uint32_t *>(scratch + OFF_NFINAL);
 
     if (spin_in != spin_out &&

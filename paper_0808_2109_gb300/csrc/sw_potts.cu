@@ -793,11 +793,16 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             const size_t node = nbase + s;
             if (rs[qq] >= 0) {
                 const int rep = sm.f.par[rs[qq]] & 0xFFFF;
-                p.npar[node] = (int32_t)(nbase + rep);
-                p.nkey[node] = (int32_t)(gfor(rs[qq]) | (rep == s ? KEY_REP : 0u));
+                const uint32_t key = gfor(rs[qq]);
+                p.node[node] = make_int2((int)(nbase + rep), (int)(key | (rep == s ? KEY_REP : 0u)));
+                // a representative's new state if its piece's minimum is its
+                // cluster's
+                if (rep == s) {
+                    const int r = rs[qq] / G::PW;
+                    p.kstate[node] = qsm ? sm.qs[r][rs[qq] - r * G::PW] : cluster_state(key, klo, khi, k0, k1, q);
+                }
             } else {
-                p.npar[node] = (int32_t)node;
-                p.nkey[node] = (int32_t)KEY_NONE;
+                p.node[node] = make_int2(NODE_NONE, 0);
             }
             if (csz) p.csize[node] = 0;   // the merge adds piece sizes at root nodes
         }
@@ -967,7 +972,7 @@ __device__ __forceinline__ int wfind3(WLink *wl, int x, int &ox, int &oy, int &o
 // set: the cycle it closes has net displacement pos(a) + e_ax - pos(b) through
 // the tree, non-zero exactly when it winds (recorded per axis).  Else the root
 // of larger key hangs under the other with its displacement from it.
-__device__ __forceinline__ void wunite3(WLink *wl, const int32_t *key, int a, int b, int ax, DevObs *o)
+__device__ __forceinline__ void wunite3(WLink *wl, const int2 *node, int a, int b, int ax, DevObs *o)
 {
     for (;;) {
         int oax, oay, oaz, obx, oby, obz;
@@ -980,7 +985,7 @@ __device__ __forceinline__ void wunite3(WLink *wl, const int32_t *key, int a, in
             if (cy || cz) atomicOr(&o->spans_y, 1);   // y, or in 3D y or z
             return;
         }
-        const bool a_lo = (uint32_t)key[ra] < (uint32_t)key[rb];
+        const bool a_lo = (uint32_t)node[ra].y < (uint32_t)node[rb].y;
         const int lo = a_lo ? ra : rb, hi = a_lo ? rb : ra;
         const WLink root{hi, 0, 0, 0};
         const WLink nl = a_lo ? WLink{lo, cx, cy, cz} : WLink{lo, -cx, -cy, -cz};
@@ -1034,17 +1039,18 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
         WLink *wl = reinterpret_cast<WLink *>(p.wlink);
 #pragma unroll
         for (int qq = 0; qq < MC::EPT; ++qq)
-            if (na[qq] >= 0) wunite3(wl, p.nkey, na[qq], nb[qq], ax[qq], obs + j);
+            if (na[qq] >= 0) wunite3(wl, p.node, na[qq], nb[qq], ax[qq], obs + j);
         return;
     }
     int pa[MC::EPT], pb[MC::EPT], ka[MC::EPT], kb[MC::EPT];
 #pragma unroll
     for (int qq = 0; qq < MC::EPT; ++qq) {
         if (na[qq] < 0) continue;
-        pa[qq] = gload(p.npar + na[qq]);
-        pb[qq] = gload(p.npar + nb[qq]);
-        ka[qq] = p.nkey[na[qq]];
-        kb[qq] = p.nkey[nb[qq]];
+        const int2 va = nload(p.node + na[qq]), vb = nload(p.node + nb[qq]);
+        pa[qq] = va.x;
+        ka[qq] = va.y;
+        pb[qq] = vb.x;
+        kb[qq] = vb.y;
     }
     bool live[MC::EPT];
 #pragma unroll
@@ -1067,7 +1073,7 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
         const int hi = u_hi ? u : v, lo = u_hi ? v : u;
         // a representative whose parent was read as another node is no root
         const bool inner = u_hi ? (ra && pa[qq] != na[qq]) : (rb && pb[qq] != nb[qq]);
-        if (!inner && atomicCAS(p.npar + hi, hi, lo) == hi) live[qq] = false;
+        if (!inner && atomicCAS(&p.node[hi].x, hi, lo) == hi) live[qq] = false;
     }
     // the remaining unions in lock step (path splitting on the way up; the
     // larger key's root is hung under the smaller by compare-and-swap)
@@ -1088,12 +1094,12 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
                 // path splitting rewrites representatives only: a slot that
                 // is not one keeps its own representative as its parent
                 if (!ra) {
-                    if (sa[qq] >= 0) *(volatile int32_t *)(p.npar + sa[qq]) = pa[qq];
+                    if (sa[qq] >= 0) pstore(p.node + sa[qq], pa[qq]);
                     sa[qq] = ((uint32_t)ka[qq] & KEY_REP) ? xa[qq] : -1;
                     xa[qq] = pa[qq];
                 }
                 if (!rb) {
-                    if (sb[qq] >= 0) *(volatile int32_t *)(p.npar + sb[qq]) = pb[qq];
+                    if (sb[qq] >= 0) pstore(p.node + sb[qq], pb[qq]);
                     sb[qq] = ((uint32_t)kb[qq] & KEY_REP) ? xb[qq] : -1;
                     xb[qq] = pb[qq];
                 }
@@ -1103,7 +1109,7 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
             } else {
                 const bool a_lo = ka[qq] < kb[qq];
                 const int lo = a_lo ? xa[qq] : xb[qq], hi = a_lo ? xb[qq] : xa[qq];
-                if (atomicCAS(p.npar + hi, hi, lo) == hi) live[qq] = false;
+                if (atomicCAS(&p.node[hi].x, hi, lo) == hi) live[qq] = false;
                 else more = true;
             }
         }
@@ -1111,10 +1117,11 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
 #pragma unroll
         for (int qq = 0; qq < MC::EPT; ++qq) {
             if (!live[qq]) continue;
-            pa[qq] = gload(p.npar + xa[qq]);
-            pb[qq] = gload(p.npar + xb[qq]);
-            ka[qq] = p.nkey[xa[qq]];
-            kb[qq] = p.nkey[xb[qq]];
+            const int2 va = nload(p.node + xa[qq]), vb = nload(p.node + xb[qq]);
+            pa[qq] = va.x;
+            ka[qq] = va.y;
+            pb[qq] = vb.x;
+            kb[qq] = vb.y;
         }
     }
 }
@@ -1133,10 +1140,10 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_init(const PottsDev p)
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
         const int s = threadIdx.x + qq * MC::MT, n = base + s;
-        const int rep = p.npar[n];
+        const int rep = p.node[n].x;
         WLink w{n, 0, 0, 0};
         int x, y, z, xr, yr, zr;
-        if ((uint32_t)p.nkey[n] != KEY_NONE && rep != n && slot_xyz<DIM>(s, t.e, x, y, z) &&
+        if (rep != NODE_NONE && rep != n && slot_xyz<DIM>(s, t.e, x, y, z) &&
             slot_xyz<DIM>(rep - base, t.e, xr, yr, zr))
             w = WLink{rep, x - xr, y - yr, z - zr};
         wl[n] = w;
@@ -1155,8 +1162,7 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_jump(const PottsDev p)
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
         const int n = base + threadIdx.x + qq * MC::MT;
-        const uint32_t key = (uint32_t)p.nkey[n];
-        if (key == KEY_NONE || !(key & KEY_REP)) continue;
+        if (!((uint32_t)p.node[n].y & KEY_REP)) continue;
         const WLink w = wl_read(wl + n);
         if (w.parent == n) continue;
         const WLink g = wl_read(wl + w.parent);
@@ -1164,72 +1170,71 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_jump(const PottsDev p)
     }
 }
 
-// Every representative walks to its root r (key: the cluster's minimum site)
-// and stores the cluster's root and new state (Sec. I step 3); under PCC it
-// also points every node of its walk at r.  A "-" face slot that is not a
-// representative then takes its representative's state (its parent, in the
-// same tile: the unions rewrite representatives only) for the neighbour's
-// halo.  Counts the clusters that touch a tile face (one root node each).
+// Every representative that is not its cluster's root walks to the root r and
+// takes r's state, which the tile kernel left in kstate (Sec. I step 3; nstate
+// itself the tile kernel must not write: its neighbours read it for their
+// halos meanwhile).  On the last sweep of a call every representative also stores
+// its root's key (the label); under PCC it points every node of its walk at r.
+// A "-" face slot that is not a representative then takes its
+// representative's state (its parent, in the same tile: the unions rewrite
+// representatives only) for the neighbour's halo.  Counts the clusters that
+// touch a tile face (one root node each).
 template <int DIM, bool W>
-__global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, uint64_t sweep0,
-                                                                 DevObs *obs)
+__global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, bool last, DevObs *obs)
 {
     using MC = PMC<DIM>;
     const int base = blockIdx.x * PG<DIM>::S;
     // under the topological rule the forest lives in the node links (their
-    // first word is the parent); npar keeps each node's representative
+    // first word is the parent); node.x keeps each node's representative
     const bool wind = W && (p.flags & RF_WIND);
     const int32_t *wpar = reinterpret_cast<const int32_t *>(p.wlink);
-    auto parent = [&](int x) { return wind ? gload(wpar + 4 * (size_t)x) : gload(p.npar + x); };
-    uint32_t key[MC::NPT];
+    auto parent = [&](int x) { return wind ? gload(wpar + 4 * (size_t)x) : pload(p.node + x); };
+    bool is_rep[MC::NPT];
     int r[MC::NPT], pr[MC::NPT], rep[MC::NPT];
-#pragma unroll
-    for (int qq = 0; qq < MC::NPT; ++qq) key[qq] = (uint32_t)p.nkey[base + threadIdx.x + qq * MC::MT];
+    uint32_t st[MC::NPT];
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
         r[qq] = base + threadIdx.x + qq * MC::MT;
-        rep[qq] = gload(p.npar + r[qq]);
-        pr[qq] = wind ? parent(r[qq]) : rep[qq];
+        const int2 v = nload(p.node + r[qq]);
+        st[qq] = p.kstate[r[qq]];
+        is_rep[qq] = ((uint32_t)v.y & KEY_REP) != 0u;
+        rep[qq] = v.x;
+        pr[qq] = wind && is_rep[qq] ? parent(r[qq]) : v.x;
     }
-    auto is_rep = [](uint32_t kk) { return kk != KEY_NONE && (kk & KEY_REP); };
     __shared__ uint8_t rst[PG<DIM>::S];   // the new state of each representative slot
     for (;;) {
         bool more = false;
 #pragma unroll
         for (int qq = 0; qq < MC::NPT; ++qq)
-            if (is_rep(key[qq]) && pr[qq] != r[qq]) {
+            if (is_rep[qq] && pr[qq] != r[qq]) {
                 r[qq] = pr[qq];
                 more = true;
             }
         if (!more) break;
 #pragma unroll
         for (int qq = 0; qq < MC::NPT; ++qq)
-            if (is_rep(key[qq])) pr[qq] = parent(r[qq]);
+            if (is_rep[qq]) pr[qq] = parent(r[qq]);
     }
-    const uint64_t k = sweep0 + (uint64_t)j;
-    const uint32_t klo = (uint32_t)k, khi = (uint32_t)(k >> 32);
-    const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
-    const bool pcc = (p.flags & RF_PCC) != 0 && !wind;   // the extension rule's candidates read npar
+    const bool pcc = (p.flags & RF_PCC) != 0 && !wind;   // the extension rule's candidates read the parents
     int nroots = 0;
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
         const int s = threadIdx.x + qq * MC::MT, n = base + s;
-        if (is_rep(key[qq])) {
+        if (is_rep[qq]) {
+            if (r[qq] != n) st[qq] = p.kstate[r[qq]];
+            p.nstate[n] = (uint8_t)st[qq];
             if (pcc) {
                 // the PCC kernels read a representative's root from its parent
                 for (int x = n; x != r[qq];) {
-                    const int nx = gload(p.npar + x);
-                    *(volatile int32_t *)(p.npar + x) = r[qq];
+                    const int nx = pload(p.node + x);
+                    pstore(p.node + x, r[qq]);
                     x = nx;
                 }
             }
             nroots += r[qq] == n;
             if (p.flags & RF_CSIZE) atomicAdd(p.csize + r[qq], p.psize[n]);
-            const uint32_t rkey = (uint32_t)p.nkey[r[qq]] & KEY_MASK;
-            const uint8_t st = cluster_state(rkey, klo, khi, k0, k1, p.q);
-            p.nstate[n] = st;
-            rst[s] = st;
-            p.nfinal[n] = rkey;
+            rst[s] = (uint8_t)st[qq];
+            if (last) p.nfinal[n] = (uint32_t)p.node[r[qq]].y & KEY_MASK;
         }
     }
     __syncthreads();
@@ -1239,7 +1244,7 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
         const int s = threadIdx.x + qq * MC::MT;
-        if (!is_rep(key[qq]) && key[qq] != KEY_NONE && minus_slot<DIM>(s)) p.nstate[base + s] = rst[rep[qq] - base];
+        if (!is_rep[qq] && rep[qq] != NODE_NONE && minus_slot<DIM>(s)) p.nstate[base + s] = rst[rep[qq] - base];
     }
     const int wb = threadIdx.x & ~31;
     const unsigned wm = MC::MT - wb >= 32 ? 0xFFFFFFFFu : (1u << (MC::MT - wb)) - 1u;
@@ -1268,10 +1273,10 @@ __global__ void k_ppcc_candidates(const PottsDev p, int64_t F)
     const PTile t = ptile_of<DIM>(p, lt);
     if (t.c[a] != 0) return;
     const int node = lt * S + face_off<DIM>(a, 0) + f;
-    const uint32_t key = (uint32_t)p.nkey[node];
-    if (key == KEY_NONE) return;
-    int r = gload(p.npar + node);
-    if (!(key & KEY_REP)) r = gload(p.npar + r);   // via a representative
+    const int2 v = nload(p.node + node);
+    if (v.x == NODE_NONE) return;
+    int r = v.x;
+    if (!((uint32_t)v.y & KEY_REP)) r = pload(p.node + r);   // via a representative
     int32_t *c = p.cid + (size_t)r * DIM + a;
     if (atomicCAS(c, 0, 1) == 0) {
         const int id = atomicAdd(p.ncand + a, 1);   // < F: at most one per face site
@@ -1286,14 +1291,14 @@ __global__ void k_ppcc_cover(const PottsDev p)
     using G = PG<DIM>;
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= (int64_t)p.ntiles * G::S) return;
-    const uint32_t key = (uint32_t)p.nkey[n];
-    if (key == KEY_NONE || !(key & KEY_REP)) return;
+    const int2 v = nload(p.node + n);
+    if (!((uint32_t)v.y & KEY_REP)) return;
     uint32_t m[G::PMW];
     uint32_t any = 0u;
 #pragma unroll
     for (int w = 0; w < G::PMW; ++w) any |= (m[w] = p.pmask[(size_t)n * G::PMW + w]);
     if (!any) return;
-    const int r = gload(p.npar + n);
+    const int r = v.x;
     const PTile t = ptile_of<DIM>(p, (int)(n / G::S));
     const uint32_t W = ((uint32_t)p.L + 31u) / 32u;
     const int64_t F = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
@@ -1424,7 +1429,7 @@ void launch_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs 
 }
 
 template <int DIM>
-void launch_merge(const PottsDev &p, int j, uint64_t sweep0, DevObs *obs, cudaStream_t st)
+void launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
 {
     using G = PG<DIM>;
     const bool pcc = (p.flags & RF_PCC) != 0;
@@ -1434,13 +1439,13 @@ void launch_merge(const PottsDev &p, int j, uint64_t sweep0, DevObs *obs, cudaSt
         k_pwind_init<DIM><<<tiles, PMC<DIM>::MT, 0, st>>>(p);
         k_pmerge_union<DIM, true><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, obs);
         k_pwind_jump<DIM><<<tiles, PMC<DIM>::MT, 0, st>>>(p);
-        k_pmerge_resolve<DIM, true><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, sweep0, obs);
+        k_pmerge_resolve<DIM, true><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, j == nsweeps - 1, obs);
     } else {
         // no pointer-jumping round: after the unions' single-swap links the
         // walks are short, and the round cost more than it saved (3D 2.99 ->
         // 2.94 ms a sweep without it)
         k_pmerge_union<DIM, false><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, obs);
-        k_pmerge_resolve<DIM, false><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, sweep0, obs);
+        k_pmerge_resolve<DIM, false><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, j == nsweeps - 1, obs);
     }
     if (pcc && wind) {
         // the flags are the windings the unions recorded: the feedback only
@@ -1493,10 +1498,10 @@ cudaError_t potts_enqueue_tile(const PottsDev &p, int j, int nsweeps, uint64_t s
 }
 
 // ... and, for j < nsweeps, the merge of sweep j.
-cudaError_t potts_enqueue_merge(const PottsDev &p, int j, uint64_t sweep0, DevObs *obs, cudaStream_t st)
+cudaError_t potts_enqueue_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
 {
-    if (p.dim == 2) launch_merge<2>(p, j, sweep0, obs, st);
-    else launch_merge<3>(p, j, sweep0, obs, st);
+    if (p.dim == 2) launch_merge<2>(p, j, nsweeps, sweep0, obs, st);
+    else launch_merge<3>(p, j, nsweeps, sweep0, obs, st);
     return cudaGetLastError();
 }
 
@@ -1506,7 +1511,7 @@ cudaError_t potts_enqueue_sweeps(const PottsDev &p, int nsweeps, uint64_t sweep0
 {
     for (int j = 0; j <= nsweeps; ++j) {
         cudaError_t e = potts_enqueue_tile(p, j, nsweeps, sweep0, obs, st);
-        if (e == cudaSuccess && j < nsweeps) e = potts_enqueue_merge(p, j, sweep0, obs, st);
+        if (e == cudaSuccess && j < nsweeps) e = potts_enqueue_merge(p, j, nsweeps, sweep0, obs, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -64,7 +64,8 @@ struct Job {
     int32_t *label = nullptr;
     uint16_t *code = nullptr;
     uint32_t *bondbits = nullptr, *cross = nullptr, *nfinal = nullptr, *pmask = nullptr, *cov = nullptr;
-    int32_t *npar = nullptr, *nkey = nullptr, *cid = nullptr, *cand = nullptr, *ncand = nullptr;
+    int2 *node = nullptr;
+    int32_t *cid = nullptr, *cand = nullptr, *ncand = nullptr;
     uint64_t *thr_dev = nullptr;
     DevObs *obs = nullptr;
     int32_t *psize = nullptr, *csize = nullptr;   // SW_FLAG_CSIZE
@@ -77,7 +78,7 @@ struct Job {
 // Byte offsets of a job's buffers inside its one device block, each on a
 // 256-byte boundary; PCC scratch last, in one range that starts zeroed.
 struct JobLayout {
-    size_t spin, label, code, bondbits, cross, npar, nkey, nfinal, thr, obs, psize, csize, nlink;
+    size_t spin, label, code, bondbits, cross, node, nfinal, thr, obs, psize, csize, nlink;
     size_t pmask, cid, cand, ncand, cov, pcc_end, total;
 };
 
@@ -98,8 +99,7 @@ JobLayout job_layout(int L, int TH, int nsweeps, bool pcc, bool csize, bool wind
     o.code = take(nt * TH * TW * 2);
     o.bondbits = take(nt * TH * 2 * TWW * 4);
     o.cross = take(nt * CROSS_WORDS * 4);
-    o.npar = take(nt * S * 4);
-    o.nkey = take(nt * S * 4);
+    o.node = take(nt * S * 8);
     o.nfinal = take(nt * S * 4);
     o.thr = take(8);
     o.obs = take((size_t)nsweeps * sizeof(DevObs));
@@ -197,8 +197,7 @@ cudaError_t job_alloc(Job *j, cudaStream_t st)
     j->code = reinterpret_cast<uint16_t *>(b + o.code);
     j->bondbits = reinterpret_cast<uint32_t *>(b + o.bondbits);
     j->cross = reinterpret_cast<uint32_t *>(b + o.cross);
-    j->npar = reinterpret_cast<int32_t *>(b + o.npar);
-    j->nkey = reinterpret_cast<int32_t *>(b + o.nkey);
+    j->node = reinterpret_cast<int2 *>(b + o.node);
     j->nfinal = reinterpret_cast<uint32_t *>(b + o.nfinal);
     j->thr_dev = reinterpret_cast<uint64_t *>(b + o.thr);
     j->obs = reinterpret_cast<DevObs *>(b + o.obs);
@@ -242,8 +241,7 @@ Replica replica_of(const Job *j)
     R.code = j->code;
     R.bondbits = j->bondbits;
     R.cross = j->cross;
-    R.npar = j->npar;
-    R.nkey = j->nkey;
+    R.node = j->node;
     R.nfinal = j->nfinal;
     R.pmask = j->pmask;
     R.cid = j->cid;
