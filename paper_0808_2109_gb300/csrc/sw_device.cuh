@@ -11,7 +11,7 @@
 //            shared-memory union-find over the bonds inside the tile, the new
 //            spin of every cluster that does not touch the tile border, and
 //            one "node" per border site (the master's "new lattice").
-//   k_merge_union / k_merge_jump / k_merge_resolve
+//   k_merge_union / k_merge_resolve
 //            the master's step 2 (Sec. II.A): union-find over the border
 //            nodes joined by the bonds that cross tile edges, including the
 //            periodic wrap; the root of a global cluster is the minimum site
@@ -124,6 +124,30 @@ struct SweepArgs {
 __device__ __forceinline__ int lattice_launch(const SweepArgs &a, const Replica &R)
 {
     return a.j + *a.jbase - R.jstart;
+}
+
+// Programmatic dependent launch: the kernels of a call form one chain in which
+// each may start while the one before it drains.  Every kernel lets its
+// successor start at once, and every block waits (griddepcontrol.wait: all of
+// the predecessor's work done and visible) before it touches anything that a
+// kernel of the chain writes.  What the host wrote before the chain (Replica,
+// tile table, launch offset, the threshold of a plain lattice) may be read
+// first, and so may draws be made.  No block returns without the wait, so a
+// kernel that has finished implies that all before it have.
+// A kernel lets its successor start first thing, so that short kernels are all
+// in place when their turn comes (L=64: 23.0 us a sweep against 24.9 when they
+// start after the wait and 27.0 without the chain; L=4096, T=3.0: 93.7, 97.9 and
+// 104 us), except the merge kernels of the topological rule and of PCC, which
+// do so after their wait: their chains are longer, and blocks of several kernels
+// ahead crowd the tile kernel's onto the same SMs (every option at L=1001: 92 us
+// against 111; without the chain 94; PCC L=2048: 95 against 96 and 97).
+__device__ __forceinline__ void chain_next()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ------------------------------------------------------------------ Philox
@@ -300,6 +324,10 @@ __device__ __forceinline__ bool sunite_linked(volatile int *par, int a, int b)
         if (atomicCAS((int *)&par[b], b, a) == b) return true;
     }
 }
+
+// SMs of the GPU this is written for: the blocks of a grid that start at once
+// are about this many times a kernel's blocks per SM.
+constexpr int FIRST_WAVE_SMS = 152;
 
 // Threads of a tile CTA: one warp per 32 x 32 sub-tile.
 template <int TH>
@@ -562,16 +590,17 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     TileSmem<TH> &sm = *reinterpret_cast<TileSmem<TH> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
 
+    chain_next();
     const int g = blockIdx.x;
-    if (g >= a.n_tiles) return;
-    const int ri = a.tile_rep[g];
-    if (ri < 0) return;
-    const Replica &R = a.reps[ri];
-    const int j = lattice_launch(a, R);   // finishes sweep j-1, starts sweep j
-    if (j < 0) return;
-    const bool fin = j >= 1 && j <= R.nsweeps;
+    const int ri = g < a.n_tiles ? a.tile_rep[g] : -1;
+    const Replica &R = a.reps[max(ri, 0)];
+    const int j = ri < 0 ? -1 : lattice_launch(a, R);   // finishes sweep j-1, starts sweep j
+    if (j < 0 || j > R.nsweeps) {
+        chain_wait();
+        return;
+    }
+    const bool fin = j >= 1;
     const bool start = j < R.nsweeps;
-    if (!fin && !start) return;
     const Tile t = tile_of(R, g, TH);
     const int L = R.L;
     // open boundaries: the last tile column has no right link in its last
@@ -589,7 +618,9 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
 
     // ---- loads of the finish half, in flight during the draws
     uint32_t fb = 0u, fr = 0u;
-    if (fin) {
+    auto finish_loads = [&]() {
+        chain_wait();
+        if (!fin) return;
         // the tile's codes, 8 sites per 16-byte asynchronous copy straight
         // into shared memory (the forest's space, unused until the labelling),
         // and the finals of its own nodes
@@ -607,7 +638,12 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         // the left column of the tile to the right)
         if (warp < TWW && tid < t.tw) fb = R.nfinal[(size_t)t.g_down * S + SL::TOP + tid];
         if (tid < t.th) fr = R.nfinal[(size_t)t.g_right * S + SL::LEFT + tid];
-    }
+    };
+    // A block of the first wave may start before the merge is done: it draws
+    // first and then waits and loads.  Later ones find the merge done.  (A PCC
+    // lattice's threshold comes from the merge: no draws before it.)
+    const bool early = g < FIRST_WAVE_SMS * TileCfg<TH>::MINB && !pcc;
+    if (!early) finish_loads();
     if (tid < 4) sm.acc[tid] = 0;
     if ((F & FEAT_CSIZE) && tid < 2) sm.acc_c2[tid] = 0ull;
 
@@ -662,6 +698,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         }
     }
 
+    if (early) finish_loads();
     if (fin) {
         // ---- finish sweep k-1: resolve every site's cluster and flip it
         const bool last = j == R.nsweeps;
@@ -1161,13 +1198,26 @@ struct MergeCfg {
 
 // The lattice of tile g and its launch index, or null when the tile is idle
 // or the lattice has no sweep in this launch (uniform across the block).
-__device__ __forceinline__ const Replica *merge_lattice(const SweepArgs &a, int g, int &j)
+__device__ __forceinline__ const Replica *launch_lattice(const SweepArgs &a, int g, int &j)
 {
     const int ri = a.tile_rep[g];
     if (ri < 0) return nullptr;
     const Replica *R = a.reps + ri;
     j = lattice_launch(a, *R);
     return (j < 0 || j >= R->nsweeps) ? nullptr : R;
+}
+
+// The same at the start of a merge kernel (W: with the topological rule): the
+// successor may start, the predecessor's work is done.
+template <bool W>
+__device__ __forceinline__ const Replica *merge_lattice(const SweepArgs &a, int g, int &j)
+{
+    const Replica *R = launch_lattice(a, g, j);
+    const bool late = W || (R && (R->flags & RF_PCC));
+    if (!late) chain_next();
+    chain_wait();
+    if (late) chain_next();
+    return R;
 }
 
 // Master step 2 of Sec. II.A: only links between neighbouring domains are
@@ -1183,7 +1233,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
     using MC = MergeCfg<TH>;
     constexpr int S = SL::S;
     int j;
-    const Replica *Rp = merge_lattice(a, blockIdx.x, j);
+    const Replica *Rp = merge_lattice<W>(a, blockIdx.x, j);
     if (!Rp) return;
     const Replica &R = *Rp;
     const Tile t = tile_of(R, blockIdx.x, TH);
@@ -1342,7 +1392,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_init(const SweepArgs 
 {
     using MC = MergeCfg<TH>;
     int j;
-    const Replica *Rp = merge_lattice(a, blockIdx.x, j);
+    const Replica *Rp = merge_lattice<true>(a, blockIdx.x, j);
     if (!Rp || !(Rp->flags & RF_WIND)) return;
     const Replica &R = *Rp;
     const Tile t = tile_of(R, blockIdx.x, TH);
@@ -1360,58 +1410,31 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_init(const SweepArgs 
     }
 }
 
-// Pointer jumping over the representatives (every parent replaced by its
-// grandparent, MERGE_JUMP_ROUNDS times) between the unions and the
-// resolve: it cuts the depth of the chains that unions across many tiles
-// leave behind.  The rounds run in one launch, so a round may read a parent
-// that its own thread has already moved up; every value read is still an
-// ancestor, and the resolve kernel walks to the root whatever depth is left.
-// One round is best since the unions split their paths (L=16384, 64-row
-// tiles, merge per sweep with 0 / 1 / 2 / 3 rounds: 0.31 / 0.28 / 0.29 / 0.34
-// ms at T_c, 0.45 / 0.50 / 0.59 ms for 1 / 2 / 3 rounds at T = 2.0).
-// Other slots keep their piece's representative as parent.
-constexpr int MERGE_JUMP_ROUNDS = 1;
-template <int TH, bool W>
-__global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_jump(const SweepArgs a)
+// Topological rule: one round of pointer jumping over the representatives'
+// links (the wind unions hang roots under roots, so walks grow longer than on
+// the plain path, which has no such round: without it the merge takes 0.21 ms
+// instead of 0.23 at L=16384, T_c, 64-row tiles, 17 us instead of 20 at L=64).
+template <int TH>
+__global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_jump(const SweepArgs a)
 {
     using MC = MergeCfg<TH>;
     int j;
-    const Replica *Rp = merge_lattice(a, blockIdx.x, j);
-    if (!Rp) return;
+    const Replica *Rp = merge_lattice<true>(a, blockIdx.x, j);
+    if (!Rp || !(Rp->flags & RF_WIND)) return;
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;   // the lattice's own nodes
-    if (W && (R.flags & RF_WIND)) {
-        for (int r = 0; r < MERGE_JUMP_ROUNDS; ++r) {
-            unsigned long long v[MC::NPT], w[MC::NPT];
+    unsigned long long v[MC::NPT], w[MC::NPT];
 #pragma unroll
-            for (int q = 0; q < MC::NPT; ++q)
-                v[q] = ((uint32_t)R.node[base + threadIdx.x + q * MC::MT].y & KEY_REP)
-                           ? wload(R.nlink + base + threadIdx.x + q * MC::MT) : ~0ull;
+    for (int q = 0; q < MC::NPT; ++q)
+        v[q] = ((uint32_t)R.node[base + threadIdx.x + q * MC::MT].y & KEY_REP)
+                   ? wload(R.nlink + base + threadIdx.x + q * MC::MT) : ~0ull;
 #pragma unroll
-            for (int q = 0; q < MC::NPT; ++q) w[q] = v[q] != ~0ull ? wload(R.nlink + (uint32_t)v[q]) : ~0ull;
+    for (int q = 0; q < MC::NPT; ++q) w[q] = v[q] != ~0ull ? wload(R.nlink + (uint32_t)v[q]) : ~0ull;
 #pragma unroll
-            for (int q = 0; q < MC::NPT; ++q)
-                if (v[q] != ~0ull && (uint32_t)w[q] != (uint32_t)v[q])
-                    *(volatile unsigned long long *)(R.nlink + base + threadIdx.x + q * MC::MT) =
-                        wind_link((int)(uint32_t)w[q], wind_add((uint32_t)(v[q] >> 32), (uint32_t)(w[q] >> 32)));
-        }
-        return;
-    }
-    int p[MC::NPT], gp[MC::NPT];
-#pragma unroll
-    for (int q = 0; q < MC::NPT; ++q) {
-        const int2 v = nload(R.node + base + threadIdx.x + q * MC::MT);
-        p[q] = ((uint32_t)v.y & KEY_REP) ? v.x : -1;
-    }
-    for (int r = 0; r < MERGE_JUMP_ROUNDS; ++r) {
-#pragma unroll
-        for (int q = 0; q < MC::NPT; ++q) gp[q] = p[q] >= 0 ? pload(R.node + p[q]) : -1;
-#pragma unroll
-        for (int q = 0; q < MC::NPT; ++q) {
-            if (gp[q] != p[q]) pstore(R.node + base + threadIdx.x + q * MC::MT, gp[q]);
-            p[q] = gp[q];
-        }
-    }
+    for (int q = 0; q < MC::NPT; ++q)
+        if (v[q] != ~0ull && (uint32_t)w[q] != (uint32_t)v[q])
+            *(volatile unsigned long long *)(R.nlink + base + threadIdx.x + q * MC::MT) =
+                wind_link((int)(uint32_t)w[q], wind_add((uint32_t)(v[q] >> 32), (uint32_t)(w[q] >> 32)));
 }
 
 // Resolve every node once the unions are done: each representative walks to
@@ -1426,7 +1449,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
 {
     using MC = MergeCfg<TH>;
     int j;
-    const Replica *Rp = merge_lattice(a, blockIdx.x, j);
+    const Replica *Rp = merge_lattice<W>(a, blockIdx.x, j);
     if (!Rp) return;
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;
@@ -1539,6 +1562,8 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
 template <int TH>
 __global__ void k_pcc_candidates(const SweepArgs a)
 {
+    chain_wait();
+    chain_next();
     using SL = Slots<TH>;
     constexpr int S = SL::S;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1578,6 +1603,8 @@ __global__ void k_pcc_candidates(const SweepArgs a)
 template <int TH>
 __global__ void k_pcc_cover(const SweepArgs a)
 {
+    chain_wait();
+    chain_next();
     constexpr int S = Slots<TH>::S;
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= (int64_t)a.n_tiles * S) return;
@@ -1625,6 +1652,8 @@ constexpr int PCC_DECIDE_BLOCKS = 8;
 template <int TH>
 __global__ void k_pcc_decide(const SweepArgs a, int n_reps)
 {
+    chain_wait();
+    chain_next();
     const int rr = blockIdx.y;
     if (rr >= n_reps) return;
     const Replica &R = a.reps[rr];

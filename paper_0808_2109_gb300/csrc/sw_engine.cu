@@ -48,76 +48,65 @@ cudaError_t tile_prepare()
 }
 
 template <int TH>
-void launch_tile(const SweepArgs &a, bool pcc, int feat, cudaStream_t st)
+cudaError_t launch_tile(const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
-    const size_t smem = tile_smem<TH>(pcc);
-    if (pcc || (feat & FEAT_TILE))
-        k_tile<TH, FEAT_TILE><<<a.n_tiles, TileCfg<TH>::NT, smem, st>>>(a);
-    else
-        k_tile<TH, 0><<<a.n_tiles, TileCfg<TH>::NT, smem, st>>>(a);
+    return launch_kernel(pcc || (feat & FEAT_TILE) ? k_tile<TH, FEAT_TILE> : k_tile<TH, 0>, dim3(a.n_tiles),
+                         TileCfg<TH>::NT, tile_smem<TH>(pcc), st, chained, a);
 }
 
-// The merge of launch group j: unions across tile edges, one round of
-// pointer jumping, every node's resolved root and new spin; then for PCC
-// lattices the span test and the feedback.
-template <int TH, bool W>
-void launch_merge_w(const SweepArgs &a, bool pcc, int n_reps, cudaStream_t st)
+// The merge of launch group j: unions across tile edges, every node's resolved
+// root and new spin; then for PCC lattices the span test and the feedback.
+template <int TH>
+cudaError_t launch_merge(const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st, bool chained)
 {
     constexpr int S = Slots<TH>::S;
     constexpr int MT = MergeCfg<TH>::MT;
-    const int64_t nu = (int64_t)a.n_tiles * (TH + TW);
-    const int64_t nn = (int64_t)a.n_tiles * S;
-    const unsigned bu = (unsigned)((nu + MERGE_THREADS - 1) / MERGE_THREADS);
-    const unsigned bn = (unsigned)((nn + MERGE_THREADS - 1) / MERGE_THREADS);
-    const unsigned tiles = (unsigned)a.n_tiles;
-    if (W) k_wind_init<TH><<<tiles, MT, 0, st>>>(a);
-    k_merge_union<TH, W><<<tiles, MT, 0, st>>>(a);
-    k_merge_jump<TH, W><<<tiles, MT, 0, st>>>(a);
-    k_merge_resolve<TH, W><<<tiles, MT, 0, st>>>(a);
+    const bool wind = (feat & FEAT_WIND) != 0;
+    const dim3 tiles(a.n_tiles);
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto *k, dim3 grid, unsigned threads, auto... args) {
+        if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, args...);
+    };
+    if (wind) go(k_wind_init<TH>, tiles, MT, a);
+    go(wind ? k_merge_union<TH, true> : k_merge_union<TH, false>, tiles, MT, a);
+    if (wind) go(k_wind_jump<TH>, tiles, MT, a);
+    go(wind ? k_merge_resolve<TH, true> : k_merge_resolve<TH, false>, tiles, MT, a);
     if (pcc) {   // reads the compressed forest; the spins do not depend on it
-        k_pcc_candidates<TH><<<bu, MERGE_THREADS, 0, st>>>(a);
-        k_pcc_cover<TH><<<bn, MERGE_THREADS, 0, st>>>(a);
-        k_pcc_decide<TH><<<dim3(PCC_DECIDE_BLOCKS, n_reps), 256, 0, st>>>(a, n_reps);
+        const int64_t nu = (int64_t)a.n_tiles * (TH + TW), nn = (int64_t)a.n_tiles * S;
+        go(k_pcc_candidates<TH>, dim3((unsigned)((nu + MERGE_THREADS - 1) / MERGE_THREADS)), MERGE_THREADS, a);
+        go(k_pcc_cover<TH>, dim3((unsigned)((nn + MERGE_THREADS - 1) / MERGE_THREADS)), MERGE_THREADS, a);
+        go(k_pcc_decide<TH>, dim3(PCC_DECIDE_BLOCKS, n_reps), 256, a, n_reps);
     }
+    return e;
 }
 
-template <int TH>
-void launch_merge(const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st)
-{
-    if (feat & FEAT_WIND)
-        launch_merge_w<TH, true>(a, pcc, n_reps, st);
-    else
-        launch_merge_w<TH, false>(a, pcc, n_reps, st);
-}
-
-cudaError_t enqueue_tile(int TH, const SweepArgs &a, bool pcc, int feat, cudaStream_t st)
+cudaError_t enqueue_tile(int TH, const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
     switch (TH) {
-    case 32: launch_tile<32>(a, pcc, feat, st); break;
-    case 64: launch_tile<64>(a, pcc, feat, st); break;
-    case 96: launch_tile<96>(a, pcc, feat, st); break;
-    default: launch_tile<128>(a, pcc, feat, st); break;
+    case 32: return launch_tile<32>(a, pcc, feat, st, chained);
+    case 64: return launch_tile<64>(a, pcc, feat, st, chained);
+    case 96: return launch_tile<96>(a, pcc, feat, st, chained);
+    default: return launch_tile<128>(a, pcc, feat, st, chained);
     }
-    return cudaGetLastError();
 }
 
-cudaError_t enqueue_merge(int TH, const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st)
+cudaError_t enqueue_merge(int TH, const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st, bool chained)
 {
     switch (TH) {
-    case 32: launch_merge<32>(a, pcc, feat, n_reps, st); break;
-    case 64: launch_merge<64>(a, pcc, feat, n_reps, st); break;
-    case 96: launch_merge<96>(a, pcc, feat, n_reps, st); break;
-    default: launch_merge<128>(a, pcc, feat, n_reps, st); break;
+    case 32: return launch_merge<32>(a, pcc, feat, n_reps, st, chained);
+    case 64: return launch_merge<64>(a, pcc, feat, n_reps, st, chained);
+    case 96: return launch_merge<96>(a, pcc, feat, n_reps, st, chained);
+    default: return launch_merge<128>(a, pcc, feat, n_reps, st, chained);
     }
-    return cudaGetLastError();
 }
 
 // One launch group: the tile kernel of launch j, then the merge of sweep j.
-cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st)
+cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st,
+                              bool chained)
 {
-    cudaError_t e = enqueue_tile(TH, a, pcc, feat, st);
+    cudaError_t e = enqueue_tile(TH, a, pcc, feat, st, chained);
     if (e != cudaSuccess) return e;
-    return enqueue_merge(TH, a, pcc, feat, n_reps, st);
+    return enqueue_merge(TH, a, pcc, feat, n_reps, st, true);
 }
 
 cudaError_t prepare_th(int TH)
@@ -472,7 +461,7 @@ int graph_for(sw_ctx *c, int m, cudaGraphExec_t *out)
     cudaError_t e = cudaSuccess;
     for (int j = 0; j < m && e == cudaSuccess; ++j) {
         a.j = j;
-        e = enqueue_launch_th(c->TH, a, c->pcc, ctx_features(c), 1, c->cap_stream);
+        e = enqueue_launch_th(c->TH, a, c->pcc, ctx_features(c), 1, c->cap_stream, j > 0);
     }
     cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -514,9 +503,9 @@ int enqueue_profiled(sw_ctx *c, int32_t n)
         SW_CUDA(next_event(c, &e2));
         a.j = j;
         SW_CUDA(cudaEventRecord(e0, c->stream));
-        SW_CUDA(enqueue_tile(c->TH, a, c->pcc, ctx_features(c), c->stream));
+        SW_CUDA(enqueue_tile(c->TH, a, c->pcc, ctx_features(c), c->stream, false));
         SW_CUDA(cudaEventRecord(e1, c->stream));
-        if (j < n) SW_CUDA(enqueue_merge(c->TH, a, c->pcc, ctx_features(c), 1, c->stream));
+        if (j < n) SW_CUDA(enqueue_merge(c->TH, a, c->pcc, ctx_features(c), 1, c->stream, false));
         SW_CUDA(cudaEventRecord(e2, c->stream));
         c->ev_marks.push_back(e0);
         c->ev_marks.push_back(e1);
@@ -545,9 +534,9 @@ int run_sweeps(sw_ctx *c, int32_t n)
                 SW_CUDA(next_event(c, &e1));
                 SW_CUDA(next_event(c, &e2));
                 SW_CUDA(cudaEventRecord(e0, c->stream));
-                SW_CUDA(potts_enqueue_tile(c->pd, j, n, c->sweep, obs, c->stream));
+                SW_CUDA(potts_enqueue_tile(c->pd, j, n, c->sweep, obs, c->stream, false));
                 SW_CUDA(cudaEventRecord(e1, c->stream));
-                if (j < n) SW_CUDA(potts_enqueue_merge(c->pd, j, n, c->sweep, obs, c->stream));
+                if (j < n) SW_CUDA(potts_enqueue_merge(c->pd, j, n, c->sweep, obs, c->stream, false));
                 SW_CUDA(cudaEventRecord(e2, c->stream));
                 c->ev_marks.push_back(e0);
                 c->ev_marks.push_back(e1);
@@ -594,7 +583,7 @@ int run_sweeps(sw_ctx *c, int32_t n)
             SweepArgs a = args_of(c);
             for (int j = 0; j < m; ++j) {
                 a.j = j;
-                SW_CUDA(enqueue_launch_th(c->TH, a, c->pcc, ctx_features(c), 1, c->stream));
+                SW_CUDA(enqueue_launch_th(c->TH, a, c->pcc, ctx_features(c), 1, c->stream, j > 0));
             }
         }
         done += m;

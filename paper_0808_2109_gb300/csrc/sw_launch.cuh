@@ -17,18 +17,40 @@ constexpr int MERGE_THREADS = 256;
 // runs).
 __attribute__((visibility("hidden"))) cudaError_t prepare_th(int TH);
 // feat: FEAT_* bits of the tile-kernel variant to launch (the union of what
-// the launch's lattices need)
+// the launch's lattices need).  chained: the call's first kernel depends on the
+// kernel before it in the stream as the others do on theirs (false: after
+// memory operations, events or other kernels).
 __attribute__((visibility("hidden"))) cudaError_t enqueue_tile(int TH, const SweepArgs &a, bool pcc, int feat,
-                                                               cudaStream_t st);
+                                                               cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_merge(int TH, const SweepArgs &a, bool pcc, int feat,
-                                                                int n_reps, cudaStream_t st);
+                                                                int n_reps, cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat,
-                                                                    int n_reps, cudaStream_t st);
+                                                                    int n_reps, cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_hot_start(uint8_t *spin, int64_t N, uint64_t seed,
                                                                     cudaStream_t st);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_job_init(uint8_t *spin, int64_t N, uint64_t seed, void *obs,
                                                                    int64_t obs_bytes, uint64_t *thr_dev, uint64_t thr,
                                                                    cudaStream_t st);
+
+// Launches kernel k; chained: as a dependent of the kernel before it in the
+// stream, which it may overlap (chain_next / chain_wait in sw_device.cuh).  The
+// first kernel after anything else in the stream is not chained.
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, bool chained,
+                          A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
 
 inline int slots_of(int TH) { return 2 * TW + 2 * TH; }
 
@@ -74,9 +96,11 @@ __attribute__((visibility("hidden"))) void potts_geometry(int dim, int L, PottsG
 __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_hot_start(const PottsDev &p, cudaStream_t st);
 // Launch j (0 .. nsweeps) of a call: the tile kernel, then (j < nsweeps) the merge of sweep j.
 __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_tile(const PottsDev &p, int j, int nsweeps,
-                                                                     uint64_t sweep0, DevObs *obs, cudaStream_t st);
+                                                                     uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                                                                     bool chained);
 __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_merge(const PottsDev &p, int j, int nsweeps,
-                                                                      uint64_t sweep0, DevObs *obs, cudaStream_t st);
+                                                                      uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                                                                      bool chained);
 // One call of nsweeps sweeps (observables into obs[0 .. nsweeps-1]).
 __attribute__((visibility("hidden"))) cudaError_t potts_enqueue_sweeps(const PottsDev &p, int nsweeps,
                                                                        uint64_t sweep0, DevObs *obs,

@@ -334,8 +334,8 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PSmem<DIM> &sm = *reinterpret_cast<PSmem<DIM> *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int lt = blockIdx.x;
-    if (lt >= p.ntiles) return;
+    chain_next();
+    const int lt = blockIdx.x;   // the grid is the lattice's tiles
     const bool fin = j >= 1, start = j < nsweeps;
     const PTile t = ptile_of<DIM>(p, lt);
     const int tw = t.e[0], th = t.e[1], td = t.e[2];
@@ -371,7 +371,9 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     const bool row_ok = wy < th && wz < td;
 
     // ---- loads of the finish half, in flight during the draws
-    if (fin) {
+    auto finish_loads = [&]() {
+        chain_wait();
+        if (!fin) return;
         // the tile's codes, 8 sites per 16-byte asynchronous copy straight
         // into shared memory (the forest's space, free until the labelling),
         // and the states of its own pieces
@@ -385,7 +387,10 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         }
         for (int w = tid; w < S / 16; w += NT) cp_async16(sm.f.s.fst + 16 * w, p.nstate + nbase + 16 * w);
         sm.f.s.fst[S + tid] = (uint8_t)tid;   // NT = 256
-    }
+    };
+    // a block of the first wave draws first (sw_device.cuh's k_tile)
+    const bool early = lt < FIRST_WAVE_SMS * 5 && !p.thr_dev;
+    if (!early) finish_loads();
     if (tid < 4) sm.acc[tid] = 0;
     if ((F & FEAT_CSIZE) && tid < 2) sm.acc_c2[tid] = 0ull;
 
@@ -497,6 +502,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     }
 
     uint8_t *st = &sm.f.s.st[0][0][0];
+    if (early) finish_loads();
     if (fin) {
         // ---- finish sweep j-1: every site's new state
         const bool last = j == nsweeps;
@@ -1013,6 +1019,10 @@ struct PMC {
 template <int DIM, bool W>
 __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p, int j, DevObs *obs)
 {
+    const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
+    if (!late) chain_next();
+    chain_wait();
+    if (late) chain_next();
     using G = PG<DIM>;
     using MC = PMC<DIM>;
     constexpr int S = G::S;
@@ -1132,6 +1142,8 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
 template <int DIM>
 __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_init(const PottsDev p)
 {
+    chain_wait();
+    chain_next();
     using G = PG<DIM>;
     using MC = PMC<DIM>;
     const int lt = blockIdx.x, base = lt * G::S;
@@ -1156,6 +1168,8 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_init(const PottsDev p)
 template <int DIM>
 __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_jump(const PottsDev p)
 {
+    chain_wait();
+    chain_next();
     using MC = PMC<DIM>;
     const int base = blockIdx.x * PG<DIM>::S;
     WLink *wl = reinterpret_cast<WLink *>(p.wlink);
@@ -1182,6 +1196,10 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_jump(const PottsDev p)
 template <int DIM, bool W>
 __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, bool last, DevObs *obs)
 {
+    const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
+    if (!late) chain_next();
+    chain_wait();
+    if (late) chain_next();
     using MC = PMC<DIM>;
     const int base = blockIdx.x * PG<DIM>::S;
     // under the topological rule the forest lives in the node links (their
@@ -1263,6 +1281,8 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
 template <int DIM>
 __global__ void k_ppcc_candidates(const PottsDev p, int64_t F)
 {
+    chain_wait();
+    chain_next();
     using G = PG<DIM>;
     constexpr int S = G::S;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1288,6 +1308,8 @@ __global__ void k_ppcc_candidates(const PottsDev p, int64_t F)
 template <int DIM>
 __global__ void k_ppcc_cover(const PottsDev p)
 {
+    chain_wait();
+    chain_next();
     using G = PG<DIM>;
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= (int64_t)p.ntiles * G::S) return;
@@ -1335,6 +1357,8 @@ __global__ void k_ppcc_cover(const PottsDev p)
 constexpr int PPCC_DECIDE = 16;
 __global__ void k_ppcc_decide(const PottsDev p, int64_t F, int j, uint64_t sweep0, DevObs *obs)
 {
+    chain_wait();
+    chain_next();
     const uint32_t L = (uint32_t)p.L, W = (L + 31) / 32;
     DevObs *o = obs + j;
     int sx = 0, sy = 0;
@@ -1415,49 +1439,49 @@ cudaError_t potts_prepare()
 }
 
 template <int DIM>
-void launch_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
+cudaError_t launch_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                        bool chained)
 {
-    using G = PG<DIM>;
-    const bool pcc = (p.flags & RF_PCC) != 0;
     const bool feat = (p.flags & (RF_PCC | RF_OPEN | RF_CSIZE)) != 0;
-    const unsigned tiles = (unsigned)p.ntiles;
-    const size_t smem = ptile_smem<DIM>(pcc);
-    if (feat)
-        k_ptile<DIM, FEAT_TILE><<<tiles, G::NT, smem, st>>>(p, j, nsweeps, sweep0, obs);
-    else
-        k_ptile<DIM, 0><<<tiles, G::NT, smem, st>>>(p, j, nsweeps, sweep0, obs);
+    return launch_kernel(feat ? k_ptile<DIM, FEAT_TILE> : k_ptile<DIM, 0>, dim3((unsigned)p.ntiles), PG<DIM>::NT,
+                         ptile_smem<DIM>((p.flags & RF_PCC) != 0), st, chained, p, j, nsweeps, sweep0, obs);
 }
 
 template <int DIM>
-void launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
+cudaError_t launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                         bool chained)
 {
     using G = PG<DIM>;
-    const bool pcc = (p.flags & RF_PCC) != 0;
-    const unsigned tiles = (unsigned)p.ntiles;
-    const bool wind = (p.flags & RF_WIND) != 0;
+    constexpr int MT = PMC<DIM>::MT;
+    const bool pcc = (p.flags & RF_PCC) != 0, wind = (p.flags & RF_WIND) != 0;
+    const dim3 tiles((unsigned)p.ntiles);
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto *k, dim3 grid, unsigned threads, auto... args) {
+        if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, args...);
+    };
+    const bool last = j == nsweeps - 1;
     if (wind) {
-        k_pwind_init<DIM><<<tiles, PMC<DIM>::MT, 0, st>>>(p);
-        k_pmerge_union<DIM, true><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, obs);
-        k_pwind_jump<DIM><<<tiles, PMC<DIM>::MT, 0, st>>>(p);
-        k_pmerge_resolve<DIM, true><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, j == nsweeps - 1, obs);
+        go(k_pwind_init<DIM>, tiles, MT, p);
+        go(k_pmerge_union<DIM, true>, tiles, MT, p, j, obs);
+        go(k_pwind_jump<DIM>, tiles, MT, p);
+        go(k_pmerge_resolve<DIM, true>, tiles, MT, p, j, last, obs);
     } else {
         // no pointer-jumping round: after the unions' single-swap links the
         // walks are short, and the round cost more than it saved (3D 2.99 ->
         // 2.94 ms a sweep without it)
-        k_pmerge_union<DIM, false><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, obs);
-        k_pmerge_resolve<DIM, false><<<tiles, PMC<DIM>::MT, 0, st>>>(p, j, j == nsweeps - 1, obs);
+        go(k_pmerge_union<DIM, false>, tiles, MT, p, j, obs);
+        go(k_pmerge_resolve<DIM, false>, tiles, MT, p, j, last, obs);
     }
-    if (pcc && wind) {
-        // the flags are the windings the unions recorded: the feedback only
+    if (pcc) {
         const int64_t F = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
-        k_ppcc_decide<<<PPCC_DECIDE, PT, 0, st>>>(p, F, j, sweep0, obs);
-    } else if (pcc) {
-        const int64_t F = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
-        const int64_t nc = (int64_t)p.ntiles * G::FT, nn = (int64_t)p.ntiles * G::S;
-        k_ppcc_candidates<DIM><<<(unsigned)((nc + PT - 1) / PT), PT, 0, st>>>(p, F);
-        k_ppcc_cover<DIM><<<(unsigned)((nn + PT - 1) / PT), PT, 0, st>>>(p);
-        k_ppcc_decide<<<PPCC_DECIDE, PT, 0, st>>>(p, F, j, sweep0, obs);
+        if (!wind) {   // under the topological rule the unions recorded the flags
+            const int64_t nc = (int64_t)p.ntiles * G::FT, nn = (int64_t)p.ntiles * G::S;
+            go(k_ppcc_candidates<DIM>, dim3((unsigned)((nc + PT - 1) / PT)), PT, p, F);
+            go(k_ppcc_cover<DIM>, dim3((unsigned)((nn + PT - 1) / PT)), PT, p);
+        }
+        go(k_ppcc_decide, dim3(PPCC_DECIDE), PT, p, F, j, sweep0, obs);
     }
+    return e;
 }
 
 }  // namespace
@@ -1488,21 +1512,21 @@ cudaError_t potts_enqueue_hot_start(const PottsDev &p, cudaStream_t st)
 
 // Launch j of a call of nsweeps sweeps: the tile kernel (finishing sweep
 // j-1, starting sweep j) ...
-cudaError_t potts_enqueue_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
+cudaError_t potts_enqueue_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                               bool chained)
 {
     cudaError_t e = potts_prepare();
     if (e != cudaSuccess) return e;
-    if (p.dim == 2) launch_tile<2>(p, j, nsweeps, sweep0, obs, st);
-    else launch_tile<3>(p, j, nsweeps, sweep0, obs, st);
-    return cudaGetLastError();
+    return p.dim == 2 ? launch_tile<2>(p, j, nsweeps, sweep0, obs, st, chained)
+                      : launch_tile<3>(p, j, nsweeps, sweep0, obs, st, chained);
 }
 
 // ... and, for j < nsweeps, the merge of sweep j.
-cudaError_t potts_enqueue_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
+cudaError_t potts_enqueue_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                                bool chained)
 {
-    if (p.dim == 2) launch_merge<2>(p, j, nsweeps, sweep0, obs, st);
-    else launch_merge<3>(p, j, nsweeps, sweep0, obs, st);
-    return cudaGetLastError();
+    return p.dim == 2 ? launch_merge<2>(p, j, nsweeps, sweep0, obs, st, chained)
+                      : launch_merge<3>(p, j, nsweeps, sweep0, obs, st, chained);
 }
 
 // The launches of one call of nsweeps sweeps: tile kernel j = 0 .. nsweeps,
@@ -1510,8 +1534,8 @@ cudaError_t potts_enqueue_merge(const PottsDev &p, int j, int nsweeps, uint64_t 
 cudaError_t potts_enqueue_sweeps(const PottsDev &p, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st)
 {
     for (int j = 0; j <= nsweeps; ++j) {
-        cudaError_t e = potts_enqueue_tile(p, j, nsweeps, sweep0, obs, st);
-        if (e == cudaSuccess && j < nsweeps) e = potts_enqueue_merge(p, j, nsweeps, sweep0, obs, st);
+        cudaError_t e = potts_enqueue_tile(p, j, nsweeps, sweep0, obs, st, j > 0);
+        if (e == cudaSuccess && j < nsweeps) e = potts_enqueue_merge(p, j, nsweeps, sweep0, obs, st, true);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

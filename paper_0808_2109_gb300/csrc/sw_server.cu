@@ -354,7 +354,7 @@ cudaError_t lane_capture(Lane &ln, cudaStream_t cap_stream, bool pcc, int feat)
     SweepArgs a = lane_args(ln);
     for (int j = 0; j < GROUPS_PER_STEP && e == cudaSuccess; ++j) {
         a.j = j;
-        e = enqueue_launch_th(ln.TH, a, pcc, feat, ln.cap_reps, cap_stream);
+        e = enqueue_launch_th(ln.TH, a, pcc, feat, ln.cap_reps, cap_stream, j > 0);
     }
     cudaError_t e2 = cudaStreamEndCapture(cap_stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
