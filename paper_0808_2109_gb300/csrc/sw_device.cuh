@@ -1183,18 +1183,50 @@ __device__ __forceinline__ void wunite(unsigned long long *lk, const int2 *node,
 
 // ------------------------------------------------------------- merge phase
 // Launch shape of the merge kernels: one block per tile (blockIdx.x = the
-// tile's index in the tile table) of S/4 threads; thread i takes the slots
-// i + q*S/4 (q < 4) and the crossing links i + q*S/4 (q < 2).  The tile's
-// lattice, launch and range checks are read once per thread instead of once
-// per node, and the loads of a thread's nodes are issued together.
+// tile's index in the tile table), so that the tile's lattice, launch and
+// range checks are read once per thread instead of once per node.  The kernels
+// are bound by latency and by instructions issued for lanes without work, so a
+// block first lists what there is to do in shared memory: the crossing links
+// that are bonded (half of them at T_c; 0.24 in 3D) and the representatives that
+// are not their cluster's root.
 template <int TH>
 struct MergeCfg {
     static constexpr int S = Slots<TH>::S;
-    static constexpr int MT = S / 4;                    // threads per block
+    static constexpr int MT = S / 4;                    // threads per block: four slots each
     static constexpr int NPT = 4;                       // slots per thread
-    static constexpr int EPT = (TH + TW + MT - 1) / MT; // crossing links per thread
-    static_assert(S % 4 == 0 && EPT == 2, "merge launch shape");
+    static constexpr int LW = TH / 32 + TWW;            // words of crossing bits
+    static constexpr int UT = TH <= 64 ? 96 : 128;      // threads of the union kernel, two links each
+    static_assert(S % 4 == 0 && 32 * LW <= 2 * UT, "merge launch shape");
 };
+
+// The set bits of NWORDS words (word(w), w < NWORDS <= 64) as a list of their
+// positions 32 w + bit in shared memory, by a block of NT threads (whole warps).
+// Returns their number; the caller's next barrier makes the list visible.
+template <int NWORDS, int NT, typename W>
+__device__ __forceinline__ int list_bits(W word, uint16_t *list)
+{
+    static_assert(NWORDS <= 64 && NT % 32 == 0, "two words a lane");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t w0 = lane < NWORDS ? word(lane) : 0u;
+    const uint32_t w1 = NWORDS > 32 && 32 + lane < NWORDS ? word(32 + lane) : 0u;
+    // both halves' running counts in one scan (16 bits each)
+    const uint32_t own = (uint32_t)__popc(w0) | ((uint32_t)__popc(w1) << 16);
+    uint32_t sum = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, sum, o);
+        if (lane >= o) sum += v;
+    }
+    const uint32_t all = __shfl_sync(0xFFFFFFFFu, sum, 31);
+    const uint32_t before = sum - own;   // per half
+    for (int w = warp; w < NWORDS; w += NT / 32) {
+        const uint32_t v = __shfl_sync(0xFFFFFFFFu, w < 32 ? w0 : w1, w & 31);
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, before, w & 31);
+        const int at = w < 32 ? (int)(b & 0xFFFFu) : (int)((all & 0xFFFFu) + (b >> 16));
+        if ((v >> lane) & 1u) list[at + __popc(v & ((1u << lane) - 1u))] = (uint16_t)(32 * w + lane);
+    }
+    return (int)((all & 0xFFFFu) + (all >> 16));
+}
 
 // The lattice of tile g and its launch index, or null when the tile is idle
 // or the lattice has no sweep in this launch (uniform across the block).
@@ -1227,59 +1259,21 @@ __device__ __forceinline__ const Replica *merge_lattice(const SweepArgs &a, int 
 // W: compiled with the topological rule (lattices with RF_WIND unite their
 // nodes with displacements in nlink); every kernel of the merge has it.
 template <int TH, bool W>
-__global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31) / 32)) k_merge_union(const SweepArgs a)
+__global__ void __launch_bounds__(MergeCfg<TH>::UT, 64 / (MergeCfg<TH>::UT / 32)) k_merge_union(const SweepArgs a)
 {
     using SL = Slots<TH>;
     using MC = MergeCfg<TH>;
-    constexpr int S = SL::S;
+    constexpr int S = SL::S, EPT = 2;
+    __shared__ uint16_t links[32 * MC::LW];
     int j;
     const Replica *Rp = merge_lattice<W>(a, blockIdx.x, j);
     if (!Rp) return;
     const Replica &R = *Rp;
     const Tile t = tile_of(R, blockIdx.x, TH);
     const uint32_t *cross = R.cross + (size_t)t.lt * CROSS_WORDS;
-    int na[MC::EPT], nb[MC::EPT];
-    bool prev[MC::EPT];   // the link before it along the edge is bonded too
-#pragma unroll
-    for (int q = 0; q < MC::EPT; ++q) {
-        const int e = threadIdx.x + q * MC::MT;
-        na[q] = -1;
-        prev[q] = false;
-        if (e < TH) {
-            if (e < t.th && ((cross[e >> 5] >> (e & 31)) & 1u)) {
-                na[q] = t.lt * S + SL::RIGHT + e;
-                nb[q] = t.g_right * S + SL::LEFT + e;
-                prev[q] = e > 0 && ((cross[(e - 1) >> 5] >> ((e - 1) & 31)) & 1u);
-            }
-        } else if (e < TH + TW) {
-            const int x = e - TH;
-            if (x < t.tw && ((cross[TWW + (x >> 5)] >> (x & 31)) & 1u)) {
-                na[q] = t.lt * S + SL::BOTTOM + x;
-                nb[q] = t.g_down * S + SL::TOP + x;
-                prev[q] = x > 0 && ((cross[TWW + ((x - 1) >> 5)] >> ((x - 1) & 31)) & 1u);
-            }
-        }
-    }
-    if (W && (R.flags & RF_WIND)) {
-        // A link whose two ends lie in the same two pieces as the bonded link
-        // just before it along the edge joins nothing new (pieces are known
-        // by their keys, which no union changes): skip it.
-#pragma unroll
-        for (int q = 0; q < MC::EPT; ++q) {
-            if (!prev[q]) continue;
-            const uint32_t ka = (uint32_t)R.node[na[q]].y ^ (uint32_t)R.node[na[q] - 1].y;
-            const uint32_t kb = (uint32_t)R.node[nb[q]].y ^ (uint32_t)R.node[nb[q] - 1].y;
-            if (((ka | kb) & KEY_MASK) == 0) na[q] = -1;
-        }
-#pragma unroll
-        for (int q = 0; q < MC::EPT; ++q) {
-            if (na[q] < 0) continue;
-            // a right link moves by (+1, 0), a down link by (0, +1)
-            const bool right = threadIdx.x + q * MC::MT < TH;
-            wunite(R.nlink, R.node, na[q], nb[q], right ? wind_off(1, 0) : wind_off(0, 1), R.obs + j);
-        }
-        return;
-    }
+    // (bits past the tile's last row or column are zero)
+    const int total = list_bits<MC::LW, MC::UT>(
+        [&](int w) { return cross[w < TH / 32 ? w : TWW + w - TH / 32]; }, links);
     // The block's links first meet in a small forest in shared memory over
     // the pieces they touch: the tile's own pieces (ids [0, S): a piece's
     // representative slot), the right neighbour's ([S, 2S)) and the lower
@@ -1290,10 +1284,49 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
     // its parent, which is its representative: no find ever passes through a
     // slot that is not a representative, and each such slot ends one link only.
     __shared__ int lp[3 * S];
-    for (int i = threadIdx.x; i < 3 * S; i += MC::MT) lp[i] = i;
-    int pa[MC::EPT], pb[MC::EPT], ka[MC::EPT], kb[MC::EPT];
+    const bool wind = W && (R.flags & RF_WIND);
+    if (!wind)
+        for (int i = threadIdx.x; i < 3 * S; i += MC::UT) lp[i] = i;
+    __syncthreads();
+    int na[EPT], nb[EPT];
+    bool right[EPT];
 #pragma unroll
-    for (int q = 0; q < MC::EPT; ++q) {
+    for (int q = 0; q < EPT; ++q) {
+        const int i = threadIdx.x + q * MC::UT;
+        na[q] = nb[q] = -1;
+        right[q] = false;
+        if (i < total) {
+            const int e = links[i];
+            right[q] = e < TH;
+            na[q] = t.lt * S + (right[q] ? SL::RIGHT + e : SL::BOTTOM + e - TH);
+            nb[q] = right[q] ? t.g_right * S + SL::LEFT + e : t.g_down * S + SL::TOP + e - TH;
+        }
+    }
+    if (wind) {
+        // A link whose two ends lie in the same two pieces as the bonded link
+        // just before it along the edge joins nothing new (pieces are known
+        // by their keys, which no union changes): skip it.
+#pragma unroll
+        for (int q = 0; q < EPT; ++q) {
+            const int i = threadIdx.x + q * MC::UT;
+            if (i == 0 || i >= total) continue;
+            const int e = links[i];
+            if (links[i - 1] != e - 1 || e == TH) continue;   // the one before along the same edge
+            const uint32_t ka = (uint32_t)R.node[na[q]].y ^ (uint32_t)R.node[na[q] - 1].y;
+            const uint32_t kb = (uint32_t)R.node[nb[q]].y ^ (uint32_t)R.node[nb[q] - 1].y;
+            if (((ka | kb) & KEY_MASK) == 0) na[q] = -1;
+        }
+#pragma unroll
+        for (int q = 0; q < EPT; ++q) {
+            if (na[q] < 0) continue;
+            // a right link moves by (+1, 0), a down link by (0, +1)
+            wunite(R.nlink, R.node, na[q], nb[q], right[q] ? wind_off(1, 0) : wind_off(0, 1), R.obs + j);
+        }
+        return;
+    }
+    int pa[EPT], pb[EPT], ka[EPT], kb[EPT];
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
         if (na[q] < 0) continue;
         const int2 va = nload(R.node + na[q]), vb = nload(R.node + nb[q]);
         pa[q] = va.x;
@@ -1301,16 +1334,14 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
         pb[q] = vb.x;
         kb[q] = vb.y;
     }
-    __syncthreads();
-    bool live[MC::EPT];
+    bool live[EPT];
 #pragma unroll
-    for (int q = 0; q < MC::EPT; ++q) {
+    for (int q = 0; q < EPT; ++q) {
         live[q] = false;
         if (na[q] < 0) continue;
-        const bool right = threadIdx.x + q * MC::MT < TH;
-        const int own = t.lt * S, nbr = (right ? t.g_right : t.g_down) * S;
+        const int own = t.lt * S, nbr = (right[q] ? t.g_right : t.g_down) * S;
         const int la = ((uint32_t)ka[q] & KEY_REP) ? na[q] - own : pa[q] - own;
-        const int lb = (right ? S : 2 * S) + (((uint32_t)kb[q] & KEY_REP) ? nb[q] - nbr : pb[q] - nbr);
+        const int lb = (right[q] ? S : 2 * S) + (((uint32_t)kb[q] & KEY_REP) ? nb[q] - nbr : pb[q] - nbr);
         live[q] = sunite_linked(lp, la, lb);
     }
     // First try, one compare-and-swap: hang the larger-key one of the two
@@ -1319,7 +1350,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
     // if that representative is still a root, the two sets differ and the
     // link joins them (its new parent need not be a root).
 #pragma unroll
-    for (int q = 0; q < MC::EPT; ++q) {
+    for (int q = 0; q < EPT; ++q) {
         if (!live[q]) continue;
         const bool ra = ((uint32_t)ka[q] & KEY_REP) != 0u, rb = ((uint32_t)kb[q] & KEY_REP) != 0u;
         const int u = ra ? na[q] : pa[q], v = rb ? nb[q] : pb[q];
@@ -1335,9 +1366,9 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
     // under the smaller (a failed swap climbs on from the root that was
     // linked meanwhile), and loads the parent and key of every current node
     // for the next pass (the first pass uses the loads above).
-    int xa[MC::EPT], xb[MC::EPT], sa[MC::EPT], sb[MC::EPT];
+    int xa[EPT], xb[EPT], sa[EPT], sb[EPT];
 #pragma unroll
-    for (int q = 0; q < MC::EPT; ++q) {
+    for (int q = 0; q < EPT; ++q) {
         xa[q] = na[q];
         xb[q] = nb[q];
         sa[q] = sb[q] = -1;
@@ -1345,7 +1376,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
     for (;;) {
         bool more = false;
 #pragma unroll
-        for (int q = 0; q < MC::EPT; ++q) {
+        for (int q = 0; q < EPT; ++q) {
             if (!live[q]) continue;
             const bool ra = pa[q] == xa[q], rb = pb[q] == xb[q];
             if (!ra || !rb) {
@@ -1373,7 +1404,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT, 64 / ((MergeCfg<TH>::MT + 31
         }
         if (!more) break;
 #pragma unroll
-        for (int q = 0; q < MC::EPT; ++q) {
+        for (int q = 0; q < EPT; ++q) {
             if (!live[q]) continue;
             const int2 va = nload(R.node + xa[q]), vb = nload(R.node + xb[q]);
             pa[q] = va.x;
@@ -1441,112 +1472,107 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_jump(const SweepArgs 
 // its root r (key: the cluster's minimum site index), for PCC lattices writes
 // r over every node of the walk (full path compression: no union happens any
 // more, so every node on it has root r) and stores the cluster's root and new
-// spin, both in r's key (Sec. I step 3); a top or
-// left slot that is not a representative then copies its representative's.
+// spin, both in r's key (Sec. I step 3); a slot that is not a representative
+// then copies its representative's.
 // Counts the clusters that touch a tile border (one root node each).
 template <int TH, bool W>
 __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepArgs a)
 {
     using MC = MergeCfg<TH>;
+    __shared__ uint32_t rfin[MC::S];   // the finals of the representatives
+    __shared__ int2 walks[MC::S];      // representatives that are no roots: slot, parent
+    __shared__ int nwalks;
+    if (threadIdx.x == 0) nwalks = 0;
     int j;
     const Replica *Rp = merge_lattice<W>(a, blockIdx.x, j);
     if (!Rp) return;
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;
     const bool wind = W && (R.flags & RF_WIND);   // the forest lives in nlink
-    // node x with its forest's parent
-    auto node_of = [&](int x) {
-        int2 v = nload(R.node + x);
-        if (wind) v.x = (int)(uint32_t)wload(R.nlink + x);
-        return v;
-    };
-    uint32_t key[MC::NPT], rkey[MC::NPT];   // of the slot, and of the node its walk is at
-    int r[MC::NPT], p[MC::NPT];
+    // every thread of the block gets here; the last warp may be partial
+    const int lane = threadIdx.x & 31, wb = threadIdx.x & ~31;
+    const unsigned wm = MC::MT - wb >= 32 ? 0xFFFFFFFFu : (1u << (MC::MT - wb)) - 1u;
+    uint32_t key[MC::NPT];
+    int p[MC::NPT];   // parent from the tile kernel (the representative of its piece)
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
-        r[q] = base + threadIdx.x + q * MC::MT;
-        // a representative walks its forest; any other slot keeps its parent
-        // from the tile kernel (its representative) for the copy below
-        const int2 v = nload(R.node + r[q]);
-        key[q] = rkey[q] = (uint32_t)v.y;
-        p[q] = (wind && (key[q] & KEY_REP)) ? node_of(r[q]).x : v.x;
+        const int2 v = nload(R.node + base + threadIdx.x + q * MC::MT);
+        p[q] = v.x;
+        key[q] = (uint32_t)v.y;
     }
-    // the walks of the thread's representatives advance in lock step
-    for (;;) {
-        bool more = false;
-#pragma unroll
-        for (int q = 0; q < MC::NPT; ++q) {
-            if ((key[q] & KEY_REP) && p[q] != r[q]) {
-                r[q] = p[q];
-                more = true;
-            }
-        }
-        if (!more) break;
-#pragma unroll
-        for (int q = 0; q < MC::NPT; ++q)
-            if ((key[q] & KEY_REP) && p[q] == r[q]) {   // the node just reached
-                const int2 v = node_of(r[q]);
-                p[q] = v.x;
-                rkey[q] = (uint32_t)v.y;
-            }
-    }
-    __shared__ uint32_t rfin[MC::S];   // the finals of the representatives
+    __syncthreads();
     int nroots = 0;
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
-        const int n = base + threadIdx.x + q * MC::MT;
-        if (key[q] & KEY_REP) {
-            if (wind) {
-                // displacement from the root along the walk, then every link
-                // of the walk rewritten to the root with its own displacement
-                uint32_t tot = 0u;
-                for (int x = n; x != r[q];) {
-                    const unsigned long long v = wload(R.nlink + x);
-                    tot = wind_add(tot, (uint32_t)(v >> 32));
-                    x = (int)(uint32_t)v;
-                }
-                for (int x = n; x != r[q];) {
-                    const unsigned long long v = wload(R.nlink + x);
-                    *(volatile unsigned long long *)(R.nlink + x) = wind_link(r[q], tot);
-                    tot = wind_add(tot, wind_neg((uint32_t)(v >> 32)));
-                    x = (int)(uint32_t)v;
-                }
-            } else if (R.flags & RF_PCC) {
-                // the PCC kernels that follow read a representative's root
-                // straight from its parent; no other kernel reads the forest
-                // again before the next tile launch rewrites it
-                for (int x = n; x != r[q];) {
-                    const int nx = pload(R.node + x);
-                    pstore(R.node + x, r[q]);
-                    x = nx;
-                }
-            }
-            nroots += r[q] == n;
-            if (R.flags & RF_CSIZE) atomicAdd(R.csize + r[q], R.psize[n]);
-            const uint32_t f = rkey[q] & ~KEY_REP;
-            R.nfinal[n] = f;
-            rfin[threadIdx.x + q * MC::MT] = f;
+        const int s = threadIdx.x + q * MC::MT, n = base + s;
+        const bool rep = (key[q] & KEY_REP) != 0u;
+        const int up = wind && rep ? (int)(uint32_t)wload(R.nlink + n) : p[q];
+        const bool walk = rep && up != n;
+        if (rep && !walk) {   // a cluster's root: its own final
+            ++nroots;
+            rfin[s] = key[q] & ~KEY_REP;
+            if (R.flags & RF_CSIZE) atomicAdd(R.csize + n, R.psize[n]);
         }
+        const unsigned m = __ballot_sync(wm, walk);
+        int at = 0;
+        if (lane == 0 && m) at = atomicAdd(&nwalks, __popc(m));
+        at = __shfl_sync(wm, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (walk) walks[at] = make_int2(s, up);
     }
     __syncthreads();
-    // a top or left slot that is not a representative, whose final a
-    // neighbour's tile kernel reads for its halo: its representative's (its
-    // parent since the tile kernel, in this tile: the unions rewrite
-    // representatives only); past the tile's sites, 0.  No kernel reads the
-    // final of any other slot that is not a representative.
+    for (int i = threadIdx.x; i < nwalks; i += MC::MT) {
+        const int2 w = walks[i];
+        const int n = base + w.x;
+        int r = w.y;
+        uint32_t rkey;
+        for (;;) {
+            const int2 v = nload(R.node + r);
+            const int up = wind ? (int)(uint32_t)wload(R.nlink + r) : v.x;
+            rkey = (uint32_t)v.y;
+            if (up == r) break;
+            r = up;
+        }
+        if (wind) {
+            // displacement from the root along the walk, then every link
+            // of the walk rewritten to the root with its own displacement
+            uint32_t tot = 0u;
+            for (int x = n; x != r;) {
+                const unsigned long long v = wload(R.nlink + x);
+                tot = wind_add(tot, (uint32_t)(v >> 32));
+                x = (int)(uint32_t)v;
+            }
+            for (int x = n; x != r;) {
+                const unsigned long long v = wload(R.nlink + x);
+                *(volatile unsigned long long *)(R.nlink + x) = wind_link(r, tot);
+                tot = wind_add(tot, wind_neg((uint32_t)(v >> 32)));
+                x = (int)(uint32_t)v;
+            }
+        } else if (R.flags & RF_PCC) {
+            // the PCC kernels that follow read a representative's root
+            // straight from its parent; no other kernel reads the forest
+            // again before the next tile launch rewrites it
+            for (int x = n; x != r;) {
+                const int nx = pload(R.node + x);
+                pstore(R.node + x, r);
+                x = nx;
+            }
+        }
+        if (R.flags & RF_CSIZE) atomicAdd(R.csize + r, R.psize[n]);
+        rfin[w.x] = rkey & ~KEY_REP;
+    }
+    __syncthreads();
+    // every slot's final: a slot that is not a representative has its
+    // representative's (its parent since the tile kernel, in this tile: the
+    // unions rewrite representatives only), which a neighbour's tile kernel
+    // reads for its halo; past the tile's sites, 0
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
         const int s = threadIdx.x + q * MC::MT;
-        if (!(key[q] & KEY_REP) && (s < Slots<TH>::BOTTOM || (s >= Slots<TH>::LEFT && s < Slots<TH>::RIGHT)))
-            R.nfinal[base + s] = p[q] == NODE_NONE ? 0u : rfin[p[q] - base];
+        R.nfinal[base + s] = p[q] == NODE_NONE ? 0u : rfin[(key[q] & KEY_REP) ? s : p[q] - base];
     }
-    // every thread of the block gets here; the last warp may be partial
-    const int wb = threadIdx.x & ~31;
-    const unsigned wm = MC::MT - wb >= 32 ? 0xFFFFFFFFu : (1u << (MC::MT - wb)) - 1u;
     nroots = __reduce_add_sync(wm, nroots);
-    if ((threadIdx.x & 31) == 0 && nroots) atomicAdd(&R.obs[j].nclusters, (unsigned long long)nroots);
+    if (lane == 0 && nroots) atomicAdd(&R.obs[j].nclusters, (unsigned long long)nroots);
 }
-
 // ------------------------------------------------------------------- PCC
 // Extension rule under periodic boundaries (Sec. III): a cluster spans x
 // iff its projection on the x axis, the range P_x(C), is all of [0, L-1],

@@ -68,7 +68,7 @@ cudaError_t launch_merge(const SweepArgs &a, bool pcc, int feat, int n_reps, cud
         if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, args...);
     };
     if (wind) go(k_wind_init<TH>, tiles, MT, a);
-    go(wind ? k_merge_union<TH, true> : k_merge_union<TH, false>, tiles, MT, a);
+    go(wind ? k_merge_union<TH, true> : k_merge_union<TH, false>, tiles, MergeCfg<TH>::UT, a);
     if (wind) go(k_wind_jump<TH>, tiles, MT, a);
     go(wind ? k_merge_resolve<TH, true> : k_merge_resolve<TH, false>, tiles, MT, a);
     if (pcc) {   // reads the compressed forest; the spins do not depend on it

@@ -13,8 +13,8 @@
 //             union-find over the bonds inside the tile, the new state of
 //             every cluster that ends inside the tile, one node per site of
 //             each tile face, and the site codes.
-//   k_pmerge_union / k_pmerge_resolve (with k_pwind_init / k_pwind_jump under
-//             the topological rule)
+//   k_pmerge_union / k_pmerge_resolve (with k_pwind_init under the
+//             topological rule)
 //             the master's step 2: a union-find over the face nodes joined by
 //             the bonds that leave a tile (the wrapping links included),
 //             smaller key (cluster minimum) wins; then every representative
@@ -129,15 +129,6 @@ __device__ __forceinline__ bool slot_xyz(int s, const int (&e)[3], int &x, int &
         y = f / G::TX;
     }
     return x < e[0] && y < e[1] && z < e[2];
-}
-
-// A slot on a "-" face: the halo of the neighbour on that side reads its final.
-template <int DIM>
-__device__ __forceinline__ bool minus_slot(int s)
-{
-    using G = PG<DIM>;
-    return s < G::F0 || (s >= 2 * G::F0 && s < 2 * G::F0 + G::F1) ||
-           (DIM == 3 && s >= 2 * G::F0 + 2 * G::F1 && s < 2 * G::F0 + 2 * G::F1 + G::F2);
 }
 
 struct PTile {
@@ -1003,21 +994,26 @@ __device__ __forceinline__ void wunite3(WLink *wl, const int2 *node, int a, int 
 // ------------------------------------------------------------------ merge
 template <int DIM>
 struct PMC {
-    static constexpr int MT = DIM == 2 ? 96 : 512;                  // threads per block (measured best)
-    static constexpr int EPT = (PG<DIM>::FT + MT - 1) / MT;        // crossing links per thread
-    static constexpr int NPT = PG<DIM>::S / MT;                    // slots per thread
-    static_assert(PG<DIM>::S % MT == 0, "merge launch shape");
+    // threads of the union kernel (two links each a pass) and of the others;
+    // measured over 2D 64-128 and 96-192, 3D 128-512 and 160-640: 3D L=512,
+    // q=2 within 1% from 320 / 256 to 384 / 320, which is the best of the small
+    // lattices (L=50 PCC with the topological rule 97 us a sweep against 102)
+    static constexpr int UT = DIM == 2 ? 96 : 384;
+    static constexpr int UB = DIM == 2 ? 21 : 5;          // its blocks per SM
+    static constexpr int MT = DIM == 2 ? 64 : 320;
+    static constexpr int NPT = PG<DIM>::S / MT;           // slots per thread
+    static_assert(PG<DIM>::S % MT == 0 && PG<DIM>::S % 16 == 0, "merge launch shape");
 };
 
 // Master step 2 of Sec. II.A on the face nodes: link e of a tile joins slot
 // f of its + face along axis a to slot f of the - face of the next tile
 // along a (e = f, F0 + f, F0 + F1 + f for a = 0, 1, 2); union by key, the
-// finds of all of a thread's links advancing in lock step.  (A per-block
+// finds of a thread's two links advancing in lock step.  (A per-block
 // shared-memory forest that filters links joining pieces already joined, as
 // the Ising merge has, made the 3D merge slower: its pieces are small and
 // seldom meet twice.)
 template <int DIM, bool W>
-__global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p, int j, DevObs *obs)
+__global__ void __launch_bounds__(PMC<DIM>::UT, PMC<DIM>::UB) k_pmerge_union(const PottsDev p, int j, DevObs *obs)
 {
     const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
     if (!late) chain_next();
@@ -1025,113 +1021,117 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_union(const PottsDev p,
     if (late) chain_next();
     using G = PG<DIM>;
     using MC = PMC<DIM>;
-    constexpr int S = G::S;
+    constexpr int S = G::S, EPT = 2;
+    __shared__ uint16_t links[G::FT];   // the bonded crossing links
     const int lt = blockIdx.x;
     const PTile t = ptile_of<DIM>(p, lt);
     const uint32_t *cross = p.cross + (size_t)lt * G::CW;
-    int na[MC::EPT], nb[MC::EPT], ax[MC::EPT], nt[MC::EPT];
+    const int total = list_bits<G::CW, MC::UT>([&](int w) { return cross[w]; }, links);
+    __syncthreads();
+    for (int i0 = threadIdx.x; i0 < total; i0 += EPT * MC::UT) {
+        int na[EPT], nb[EPT], ax[EPT];
 #pragma unroll
-    for (int qq = 0; qq < MC::EPT; ++qq) {
-        const int e = threadIdx.x + qq * MC::MT;
-        na[qq] = -1;
-        ax[qq] = 0;
-        nt[qq] = 0;
-        if (e < G::FT && ((cross[e >> 5] >> (e & 31)) & 1u)) {
-            const int a = e < G::F0 ? 0 : e < G::F0 + G::F1 ? 1 : 2;
-            const int f = e - (a == 0 ? 0 : a == 1 ? G::F0 : G::F0 + G::F1);
-            nt[qq] = a == 0 ? t.nb[0] : a == 1 ? t.nb[1] : t.nb[2];
-            na[qq] = lt * S + face_off<DIM>(a, 1) + f;
-            nb[qq] = nt[qq] * S + face_off<DIM>(a, 0) + f;
-            ax[qq] = a;
-        }
-    }
-    if (W && (p.flags & RF_WIND)) {
-        WLink *wl = reinterpret_cast<WLink *>(p.wlink);
-#pragma unroll
-        for (int qq = 0; qq < MC::EPT; ++qq)
-            if (na[qq] >= 0) wunite3(wl, p.node, na[qq], nb[qq], ax[qq], obs + j);
-        return;
-    }
-    int pa[MC::EPT], pb[MC::EPT], ka[MC::EPT], kb[MC::EPT];
-#pragma unroll
-    for (int qq = 0; qq < MC::EPT; ++qq) {
-        if (na[qq] < 0) continue;
-        const int2 va = nload(p.node + na[qq]), vb = nload(p.node + nb[qq]);
-        pa[qq] = va.x;
-        ka[qq] = va.y;
-        pb[qq] = vb.x;
-        kb[qq] = vb.y;
-    }
-    bool live[MC::EPT];
-#pragma unroll
-    for (int qq = 0; qq < MC::EPT; ++qq) live[qq] = na[qq] >= 0;
-    // First try, one compare-and-swap: hang the larger-key one of the two
-    // pieces' representatives under the other.  Every parent carries a smaller
-    // key than its children, so a root of key k holds no node of smaller key:
-    // if that representative is still a root, the two sets differ and the
-    // link joins them (its new parent need not be a root).
-#pragma unroll
-    for (int qq = 0; qq < MC::EPT; ++qq) {
-        if (!live[qq]) continue;
-        const bool ra = ((uint32_t)ka[qq] & KEY_REP) != 0u, rb = ((uint32_t)kb[qq] & KEY_REP) != 0u;
-        const int u = ra ? na[qq] : pa[qq], v = rb ? nb[qq] : pb[qq];
-        if (u == v) {
-            live[qq] = false;
-            continue;
-        }
-        const bool u_hi = ((uint32_t)ka[qq] & KEY_MASK) > ((uint32_t)kb[qq] & KEY_MASK);
-        const int hi = u_hi ? u : v, lo = u_hi ? v : u;
-        // a representative whose parent was read as another node is no root
-        const bool inner = u_hi ? (ra && pa[qq] != na[qq]) : (rb && pb[qq] != nb[qq]);
-        if (!inner && atomicCAS(&p.node[hi].x, hi, lo) == hi) live[qq] = false;
-    }
-    // the remaining unions in lock step (path splitting on the way up; the
-    // larger key's root is hung under the smaller by compare-and-swap)
-    int xa[MC::EPT], xb[MC::EPT], sa[MC::EPT], sb[MC::EPT];
-#pragma unroll
-    for (int qq = 0; qq < MC::EPT; ++qq) {
-        xa[qq] = na[qq];
-        xb[qq] = nb[qq];
-        sa[qq] = sb[qq] = -1;
-    }
-    for (;;) {
-        bool more = false;
-#pragma unroll
-        for (int qq = 0; qq < MC::EPT; ++qq) {
-            if (!live[qq]) continue;
-            const bool ra = pa[qq] == xa[qq], rb = pb[qq] == xb[qq];
-            if (!ra || !rb) {
-                // path splitting rewrites representatives only: a slot that
-                // is not one keeps its own representative as its parent
-                if (!ra) {
-                    if (sa[qq] >= 0) pstore(p.node + sa[qq], pa[qq]);
-                    sa[qq] = ((uint32_t)ka[qq] & KEY_REP) ? xa[qq] : -1;
-                    xa[qq] = pa[qq];
-                }
-                if (!rb) {
-                    if (sb[qq] >= 0) pstore(p.node + sb[qq], pb[qq]);
-                    sb[qq] = ((uint32_t)kb[qq] & KEY_REP) ? xb[qq] : -1;
-                    xb[qq] = pb[qq];
-                }
-                more = true;
-            } else if (xa[qq] == xb[qq]) {
-                live[qq] = false;
-            } else {
-                const bool a_lo = ka[qq] < kb[qq];
-                const int lo = a_lo ? xa[qq] : xb[qq], hi = a_lo ? xb[qq] : xa[qq];
-                if (atomicCAS(&p.node[hi].x, hi, lo) == hi) live[qq] = false;
-                else more = true;
+        for (int qq = 0; qq < EPT; ++qq) {
+            const int i = i0 + qq * MC::UT;
+            na[qq] = -1;
+            ax[qq] = 0;
+            if (i < total) {
+                const int e = links[i];
+                const int a = e < G::F0 ? 0 : e < G::F0 + G::F1 ? 1 : 2;
+                const int f = e - (a == 0 ? 0 : a == 1 ? G::F0 : G::F0 + G::F1);
+                na[qq] = lt * S + face_off<DIM>(a, 1) + f;
+                nb[qq] = (a == 0 ? t.nb[0] : a == 1 ? t.nb[1] : t.nb[2]) * S + face_off<DIM>(a, 0) + f;
+                ax[qq] = a;
             }
         }
-        if (!more) break;
+        if (W && (p.flags & RF_WIND)) {
+            WLink *wl = reinterpret_cast<WLink *>(p.wlink);
 #pragma unroll
-        for (int qq = 0; qq < MC::EPT; ++qq) {
-            if (!live[qq]) continue;
-            const int2 va = nload(p.node + xa[qq]), vb = nload(p.node + xb[qq]);
+            for (int qq = 0; qq < EPT; ++qq)
+                if (na[qq] >= 0) wunite3(wl, p.node, na[qq], nb[qq], ax[qq], obs + j);
+            continue;
+        }
+        int pa[EPT], pb[EPT], ka[EPT], kb[EPT];
+#pragma unroll
+        for (int qq = 0; qq < EPT; ++qq) {
+            if (na[qq] < 0) continue;
+            const int2 va = nload(p.node + na[qq]), vb = nload(p.node + nb[qq]);
             pa[qq] = va.x;
             ka[qq] = va.y;
             pb[qq] = vb.x;
             kb[qq] = vb.y;
+        }
+        bool live[EPT];
+#pragma unroll
+        for (int qq = 0; qq < EPT; ++qq) live[qq] = na[qq] >= 0;
+        // First try, one compare-and-swap: hang the larger-key one of the two
+        // pieces' representatives under the other.  Every parent carries a smaller
+        // key than its children, so a root of key k holds no node of smaller key:
+        // if that representative is still a root, the two sets differ and the
+        // link joins them (its new parent need not be a root).
+#pragma unroll
+        for (int qq = 0; qq < EPT; ++qq) {
+            if (!live[qq]) continue;
+            const bool ra = ((uint32_t)ka[qq] & KEY_REP) != 0u, rb = ((uint32_t)kb[qq] & KEY_REP) != 0u;
+            const int u = ra ? na[qq] : pa[qq], v = rb ? nb[qq] : pb[qq];
+            if (u == v) {
+                live[qq] = false;
+                continue;
+            }
+            const bool u_hi = ((uint32_t)ka[qq] & KEY_MASK) > ((uint32_t)kb[qq] & KEY_MASK);
+            const int hi = u_hi ? u : v, lo = u_hi ? v : u;
+            // a representative whose parent was read as another node is no root
+            const bool inner = u_hi ? (ra && pa[qq] != na[qq]) : (rb && pb[qq] != nb[qq]);
+            if (!inner && atomicCAS(&p.node[hi].x, hi, lo) == hi) live[qq] = false;
+        }
+        // the remaining unions in lock step (path splitting on the way up; the
+        // larger key's root is hung under the smaller by compare-and-swap)
+        int xa[EPT], xb[EPT], sa[EPT], sb[EPT];
+#pragma unroll
+        for (int qq = 0; qq < EPT; ++qq) {
+            xa[qq] = na[qq];
+            xb[qq] = nb[qq];
+            sa[qq] = sb[qq] = -1;
+        }
+        for (;;) {
+            bool more = false;
+#pragma unroll
+            for (int qq = 0; qq < EPT; ++qq) {
+                if (!live[qq]) continue;
+                const bool ra = pa[qq] == xa[qq], rb = pb[qq] == xb[qq];
+                if (!ra || !rb) {
+                    // path splitting rewrites representatives only: a slot that
+                    // is not one keeps its own representative as its parent
+                    if (!ra) {
+                        if (sa[qq] >= 0) pstore(p.node + sa[qq], pa[qq]);
+                        sa[qq] = ((uint32_t)ka[qq] & KEY_REP) ? xa[qq] : -1;
+                        xa[qq] = pa[qq];
+                    }
+                    if (!rb) {
+                        if (sb[qq] >= 0) pstore(p.node + sb[qq], pb[qq]);
+                        sb[qq] = ((uint32_t)kb[qq] & KEY_REP) ? xb[qq] : -1;
+                        xb[qq] = pb[qq];
+                    }
+                    more = true;
+                } else if (xa[qq] == xb[qq]) {
+                    live[qq] = false;
+                } else {
+                    const bool a_lo = ka[qq] < kb[qq];
+                    const int lo = a_lo ? xa[qq] : xb[qq], hi = a_lo ? xb[qq] : xa[qq];
+                    if (atomicCAS(&p.node[hi].x, hi, lo) == hi) live[qq] = false;
+                    else more = true;
+                }
+            }
+            if (!more) break;
+#pragma unroll
+            for (int qq = 0; qq < EPT; ++qq) {
+                if (!live[qq]) continue;
+                const int2 va = nload(p.node + xa[qq]), vb = nload(p.node + xb[qq]);
+                pa[qq] = va.x;
+                ka[qq] = va.y;
+                pb[qq] = vb.x;
+                kb[qq] = vb.y;
+            }
         }
     }
 }
@@ -1162,36 +1162,14 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_init(const PottsDev p)
     }
 }
 
-// Topological rule: one round of pointer jumping on the representatives'
-// links (the wind unions hang roots under roots, so the walks grow longer
-// than on the plain path, which has no such round).
-template <int DIM>
-__global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_jump(const PottsDev p)
-{
-    chain_wait();
-    chain_next();
-    using MC = PMC<DIM>;
-    const int base = blockIdx.x * PG<DIM>::S;
-    WLink *wl = reinterpret_cast<WLink *>(p.wlink);
-#pragma unroll
-    for (int qq = 0; qq < MC::NPT; ++qq) {
-        const int n = base + threadIdx.x + qq * MC::MT;
-        if (!((uint32_t)p.node[n].y & KEY_REP)) continue;
-        const WLink w = wl_read(wl + n);
-        if (w.parent == n) continue;
-        const WLink g = wl_read(wl + w.parent);
-        if (g.parent != w.parent) atomicCAS(wl + n, w, WLink{g.parent, w.dx + g.dx, w.dy + g.dy, w.dz + g.dz});
-    }
-}
-
 // Every representative that is not its cluster's root walks to the root r and
 // takes r's state, which the tile kernel left in kstate (Sec. I step 3; nstate
 // itself the tile kernel must not write: its neighbours read it for their
 // halos meanwhile).  On the last sweep of a call every representative also stores
 // its root's key (the label); under PCC it points every node of its walk at r.
-// A "-" face slot that is not a representative then takes its
-// representative's state (its parent, in the same tile: the unions rewrite
-// representatives only) for the neighbour's halo.  Counts the clusters that
+// A slot that is not a representative then takes its representative's state
+// (its parent, in the same tile: the unions rewrite representatives only) for
+// the neighbour's halo.  Counts the clusters that
 // touch a tile face (one root node each).
 template <int DIM, bool W>
 __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, bool last, DevObs *obs)
@@ -1207,67 +1185,72 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
     const bool wind = W && (p.flags & RF_WIND);
     const int32_t *wpar = reinterpret_cast<const int32_t *>(p.wlink);
     auto parent = [&](int x) { return wind ? gload(wpar + 4 * (size_t)x) : pload(p.node + x); };
+    __shared__ alignas(16) uint8_t rst[PG<DIM>::S];   // the new state of every slot
+    __shared__ int2 walks[PG<DIM>::S];   // representatives that are no roots: slot, parent
+    __shared__ int nwalks;
+    if (threadIdx.x == 0) nwalks = 0;
+    // (every slot's state, kept for the representatives below)
+    for (int i = threadIdx.x; i < PG<DIM>::S / 16; i += MC::MT)
+        reinterpret_cast<uint4 *>(rst)[i] = reinterpret_cast<const uint4 *>(p.kstate + base)[i];
     bool is_rep[MC::NPT];
-    int r[MC::NPT], pr[MC::NPT], rep[MC::NPT];
-    uint32_t st[MC::NPT];
+    int rep[MC::NPT];
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
-        r[qq] = base + threadIdx.x + qq * MC::MT;
-        const int2 v = nload(p.node + r[qq]);
-        st[qq] = p.kstate[r[qq]];
+        const int2 v = nload(p.node + base + threadIdx.x + qq * MC::MT);
         is_rep[qq] = ((uint32_t)v.y & KEY_REP) != 0u;
         rep[qq] = v.x;
-        pr[qq] = wind && is_rep[qq] ? parent(r[qq]) : v.x;
     }
-    __shared__ uint8_t rst[PG<DIM>::S];   // the new state of each representative slot
-    for (;;) {
-        bool more = false;
-#pragma unroll
-        for (int qq = 0; qq < MC::NPT; ++qq)
-            if (is_rep[qq] && pr[qq] != r[qq]) {
-                r[qq] = pr[qq];
-                more = true;
-            }
-        if (!more) break;
-#pragma unroll
-        for (int qq = 0; qq < MC::NPT; ++qq)
-            if (is_rep[qq]) pr[qq] = parent(r[qq]);
-    }
-    const bool pcc = (p.flags & RF_PCC) != 0 && !wind;   // the extension rule's candidates read the parents
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
     int nroots = 0;
 #pragma unroll
     for (int qq = 0; qq < MC::NPT; ++qq) {
         const int s = threadIdx.x + qq * MC::MT, n = base + s;
-        if (is_rep[qq]) {
-            if (r[qq] != n) st[qq] = p.kstate[r[qq]];
-            p.nstate[n] = (uint8_t)st[qq];
-            if (pcc) {
-                // the PCC kernels read a representative's root from its parent
-                for (int x = n; x != r[qq];) {
-                    const int nx = pload(p.node + x);
-                    pstore(p.node + x, r[qq]);
-                    x = nx;
-                }
-            }
-            nroots += r[qq] == n;
-            if (p.flags & RF_CSIZE) atomicAdd(p.csize + r[qq], p.psize[n]);
-            rst[s] = (uint8_t)st[qq];
-            if (last) p.nfinal[n] = (uint32_t)p.node[r[qq]].y & KEY_MASK;
+        const int up = wind && is_rep[qq] ? parent(n) : rep[qq];
+        const bool walk = is_rep[qq] && up != n;
+        if (is_rep[qq] && !walk) {   // a cluster's root: its own state
+            ++nroots;
+            if (p.flags & RF_CSIZE) atomicAdd(p.csize + n, p.psize[n]);
+            if (last) p.nfinal[n] = (uint32_t)p.node[n].y & KEY_MASK;
         }
+        const unsigned m = __ballot_sync(FULL, walk);
+        int at = 0;
+        if (lane == 0 && m) at = atomicAdd(&nwalks, __popc(m));
+        at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (walk) walks[at] = make_int2(s, up);
     }
     __syncthreads();
-    // a "-" face slot that is not a representative (whose parent is still its
-    // own representative in this tile) takes its cluster's new state too: the
-    // neighbour's halo reads it with one load
-#pragma unroll
-    for (int qq = 0; qq < MC::NPT; ++qq) {
-        const int s = threadIdx.x + qq * MC::MT;
-        if (!is_rep[qq] && rep[qq] != NODE_NONE && minus_slot<DIM>(s)) p.nstate[base + s] = rst[rep[qq] - base];
+    const bool pcc = (p.flags & RF_PCC) != 0 && !wind;   // the extension rule's candidates read the parents
+    for (int i = threadIdx.x; i < nwalks; i += MC::MT) {
+        const int2 w = walks[i];
+        const int n = base + w.x;
+        int r = w.y;
+        for (int up = parent(r); up != r; up = parent(r)) r = up;
+        if (pcc) {
+            // the PCC kernels read a representative's root from its parent
+            for (int x = n; x != r;) {
+                const int nx = pload(p.node + x);
+                pstore(p.node + x, r);
+                x = nx;
+            }
+        }
+        if (p.flags & RF_CSIZE) atomicAdd(p.csize + r, p.psize[n]);
+        if (last) p.nfinal[n] = (uint32_t)p.node[r].y & KEY_MASK;
+        rst[w.x] = p.kstate[r];
     }
-    const int wb = threadIdx.x & ~31;
-    const unsigned wm = MC::MT - wb >= 32 ? 0xFFFFFFFFu : (1u << (MC::MT - wb)) - 1u;
-    nroots = __reduce_add_sync(wm, nroots);
-    if ((threadIdx.x & 31) == 0 && nroots) atomicAdd(&obs[j].nclusters, (unsigned long long)nroots);
+    __syncthreads();
+    // a slot that is not a representative (whose parent is still its own
+    // representative in this tile) takes its cluster's new state too: the
+    // neighbour's halo reads it with one load.  (Slots past the tile's sites
+    // keep whatever they have: nobody reads them.)
+#pragma unroll
+    for (int qq = 0; qq < MC::NPT; ++qq)
+        if (!is_rep[qq] && rep[qq] != NODE_NONE) rst[threadIdx.x + qq * MC::MT] = rst[rep[qq] - base];
+    __syncthreads();
+    for (int i = threadIdx.x; i < PG<DIM>::S / 16; i += MC::MT)
+        reinterpret_cast<uint4 *>(p.nstate + base)[i] = reinterpret_cast<const uint4 *>(rst)[i];
+    nroots = __reduce_add_sync(FULL, nroots);
+    if (lane == 0 && nroots) atomicAdd(&obs[j].nclusters, (unsigned long long)nroots);
 }
 
 // ------------------------------------------------------------------- PCC
@@ -1462,14 +1445,14 @@ cudaError_t launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0,
     const bool last = j == nsweeps - 1;
     if (wind) {
         go(k_pwind_init<DIM>, tiles, MT, p);
-        go(k_pmerge_union<DIM, true>, tiles, MT, p, j, obs);
-        go(k_pwind_jump<DIM>, tiles, MT, p);
+        go(k_pmerge_union<DIM, true>, tiles, PMC<DIM>::UT, p, j, obs);
         go(k_pmerge_resolve<DIM, true>, tiles, MT, p, j, last, obs);
     } else {
-        // no pointer-jumping round: after the unions' single-swap links the
-        // walks are short, and the round cost more than it saved (3D 2.99 ->
-        // 2.94 ms a sweep without it)
-        go(k_pmerge_union<DIM, false>, tiles, MT, p, j, obs);
+        // no pointer-jumping round, here or above: after the unions'
+        // single-swap links the walks are short, and the round cost more than it
+        // saved (3D 2.99 -> 2.94 ms a sweep without it; the topological rule at
+        // L=128 146 -> 135 us)
+        go(k_pmerge_union<DIM, false>, tiles, PMC<DIM>::UT, p, j, obs);
         go(k_pmerge_resolve<DIM, false>, tiles, MT, p, j, last, obs);
     }
     if (pcc) {
