@@ -1760,6 +1760,21 @@ static __global__ void k_hot_start(uint8_t *spin, int64_t N, uint32_t key0, uint
     spin[i] = (uint8_t)((u4_word(r, bit >> 5) >> (bit & 31)) & 1u);
 }
 
+// The start of a call in one launch: the lattice's descriptor (none when rep is
+// null), the launch offset of the chunk that follows and zeroed observables
+// (n_obs 8-byte words), where two copies and a memset would each be an
+// operation of their own in the stream.
+static __global__ void k_call_begin(const Replica R, Replica *rep, int32_t *jbase, int32_t jb,
+                                    unsigned long long *obs, int64_t n_obs)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n_obs) obs[i] = 0ull;
+    if (i == 0) {
+        *jbase = jb;
+        if (rep) *rep = R;
+    }
+}
+
 // A served lattice's initial device state in one launch: the hot start, zero
 // observables (n_obs 8-byte words) and the threshold word.
 static __global__ void k_job_init(uint8_t *spin, int64_t N, uint32_t key0, uint32_t key1,

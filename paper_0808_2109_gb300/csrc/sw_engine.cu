@@ -109,6 +109,16 @@ cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat, in
     return enqueue_merge(TH, a, pcc, feat, n_reps, st, true);
 }
 
+cudaError_t enqueue_groups(int TH, SweepArgs a, bool pcc, int feat, int m, bool last, cudaStream_t st)
+{
+    for (a.j = 0; a.j < m; ++a.j) {
+        const cudaError_t e = last && a.j == m - 1 ? enqueue_tile(TH, a, pcc, feat, st, a.j > 0)
+                                                   : enqueue_launch_th(TH, a, pcc, feat, 1, st, a.j > 0);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t prepare_th(int TH)
 {
     switch (TH) {
@@ -446,10 +456,12 @@ int ensure_obs(sw_ctx *c, int64_t n)
     return SW_OK;
 }
 
-// Graph of `m` launch groups j = 0..m-1 (offset by *jbase at run time).
-int graph_for(sw_ctx *c, int m, cudaGraphExec_t *out)
+// Graph of `m` launch groups j = 0..m-1 (offset by *jbase at run time); last:
+// the final one ends the call and has no merge.
+int graph_for(sw_ctx *c, int m, bool last, cudaGraphExec_t *out)
 {
-    auto it = c->graphs.find(m);
+    const int key = 2 * m + (last ? 1 : 0);
+    auto it = c->graphs.find(key);
     if (it != c->graphs.end()) {
         *out = it->second;
         return SW_OK;
@@ -457,12 +469,7 @@ int graph_for(sw_ctx *c, int m, cudaGraphExec_t *out)
     cudaGraph_t g = nullptr;
     std::lock_guard<std::mutex> lk(sw_capture_mutex());
     SW_CUDA(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    SweepArgs a = args_of(c);
-    cudaError_t e = cudaSuccess;
-    for (int j = 0; j < m && e == cudaSuccess; ++j) {
-        a.j = j;
-        e = enqueue_launch_th(c->TH, a, c->pcc, ctx_features(c), 1, c->cap_stream, j > 0);
-    }
+    cudaError_t e = enqueue_groups(c->TH, args_of(c), c->pcc, ctx_features(c), m, last, c->cap_stream);
     cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -472,7 +479,7 @@ int graph_for(sw_ctx *c, int m, cudaGraphExec_t *out)
     e = cudaGraphInstantiate(&ex, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return sw_cuda_fail(e);
-    c->graphs[m] = ex;
+    c->graphs[key] = ex;
     *out = ex;
     return SW_OK;
 }
@@ -493,8 +500,6 @@ cudaError_t next_event(sw_ctx *c, cudaEvent_t *ev)
 // kernel and the three merge kernels of every group bracketed by events.
 int enqueue_profiled(sw_ctx *c, int32_t n)
 {
-    int32_t zero = 0;
-    SW_CUDA(cudaMemcpyAsync(c->jbase, &zero, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     SweepArgs a = args_of(c);
     for (int j = 0; j <= n; ++j) {
         cudaEvent_t e0, e1, e2;
@@ -555,8 +560,11 @@ int run_sweeps(sw_ctx *c, int32_t n)
     R.nsweeps = n;
     R.thr = c->thr;
     R.obs = c->obs + c->obs_tail;
-    SW_CUDA(cudaMemcpyAsync(c->rep_dev, &R, sizeof(Replica), cudaMemcpyHostToDevice, c->stream));
-    SW_CUDA(cudaMemsetAsync(R.obs, 0, (size_t)n * sizeof(DevObs), c->stream));
+    // the descriptor, launch offset 0 and zeroed observables
+    const int64_t words = (int64_t)n * (int64_t)(sizeof(DevObs) / 8);
+    k_call_begin<<<(unsigned)((words + 255) / 256), 256, 0, c->stream>>>(
+        R, c->rep_dev, c->jbase, 0, reinterpret_cast<unsigned long long *>(R.obs), words);
+    SW_CUDA(cudaGetLastError());
     if (c->profiling) {
         rc = enqueue_profiled(c, n);
         if (rc != SW_OK) return rc;
@@ -570,21 +578,20 @@ int run_sweeps(sw_ctx *c, int32_t n)
     const int64_t total = (int64_t)n + 1;
     while (done < total) {
         const int m = (int)std::min<int64_t>(MAX_CHUNK, total - done);
-        int32_t jb = (int32_t)done;
-        SW_CUDA(cudaMemcpyAsync(c->jbase, &jb, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
+        const bool last = done + m == total;
+        if (done > 0) {
+            k_call_begin<<<1, 32, 0, c->stream>>>(R, nullptr, c->jbase, (int32_t)done, nullptr, 0);
+            SW_CUDA(cudaGetLastError());
+        }
         cudaGraphExec_t ex = nullptr;
-        rc = graph_for(c, m, &ex);
+        rc = graph_for(c, m, last, &ex);
         if (rc == SW_OK) {
             SW_CUDA(cudaGraphLaunch(ex, c->stream));
         } else {
             // capture refused (e.g. invalidated by another thread): the same
             // launch groups, enqueued directly
             cudaGetLastError();
-            SweepArgs a = args_of(c);
-            for (int j = 0; j < m; ++j) {
-                a.j = j;
-                SW_CUDA(enqueue_launch_th(c->TH, a, c->pcc, ctx_features(c), 1, c->stream, j > 0));
-            }
+            SW_CUDA(enqueue_groups(c->TH, args_of(c), c->pcc, ctx_features(c), m, last, c->stream));
         }
         done += m;
     }

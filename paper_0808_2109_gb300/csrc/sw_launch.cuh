@@ -26,6 +26,10 @@ __attribute__((visibility("hidden"))) cudaError_t enqueue_merge(int TH, const Sw
                                                                 int n_reps, cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat,
                                                                     int n_reps, cudaStream_t st, bool chained);
+// Launch groups j = 0 .. m-1 of one lattice; last: the final one is a call's
+// last and has no merge.
+__attribute__((visibility("hidden"))) cudaError_t enqueue_groups(int TH, SweepArgs a, bool pcc, int feat, int m,
+                                                                 bool last, cudaStream_t st);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_hot_start(uint8_t *spin, int64_t N, uint64_t seed,
                                                                     cudaStream_t st);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_job_init(uint8_t *spin, int64_t N, uint64_t seed, void *obs,
