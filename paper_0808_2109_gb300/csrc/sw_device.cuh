@@ -211,14 +211,14 @@ __device__ __forceinline__ Tile tile_of(const Replica &R, int g, int TH)
     Tile t;
     t.g = g;
     t.lt = g - R.tile_base;
-    t.tx = t.lt % R.tiles_x;
-    t.ty = t.lt / R.tiles_x;
+    t.ty = (int)((uint32_t)t.lt / (uint32_t)R.tiles_x);   // the only division
+    t.tx = t.lt - t.ty * R.tiles_x;
     t.x0 = t.tx * TW;
     t.y0 = t.ty * TH;
     t.tw = min(TW, R.L - t.x0);
     t.th = min(TH, R.L - t.y0);
-    t.g_right = t.ty * R.tiles_x + (t.tx + 1) % R.tiles_x;        // local tile indices
-    t.g_down = ((t.ty + 1) % R.tiles_y) * R.tiles_x + t.tx;
+    t.g_right = t.lt + (t.tx + 1 < R.tiles_x ? 1 : 1 - R.tiles_x);        // local tile indices
+    t.g_down = t.ty + 1 < R.tiles_y ? t.lt + R.tiles_x : t.tx;
     return t;
 }
 
@@ -293,7 +293,8 @@ __device__ __forceinline__ void sunite(volatile int *par, int a, int b)
 // one; b itself need not be a root.)  Most links join fresh nodes and end with
 // the first swap; the finds keep the trees shallow where many meet in one
 // set (hooks alone took 1.49 ms at L=16384, T=2.0, where three and then finds
-// take 1.19; finds alone 1.22).
+// took 1.19; finds alone 1.22; four inside a sub-tile and two at its edges are
+// 0.5% faster than three and one, two and one 1% slower).
 template <int STEPS>
 __device__ __forceinline__ void shook(volatile int *par, int a, int b)
 {
@@ -456,43 +457,36 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
         const int col = y0 * PW + 32 * sx + lane;
         for (; conf; conf &= conf - 1) {
             const int i = col + (__ffs(conf) - 1) * PW;
-            shook<3>(par, par[i - PW], par[i]);
+            shook<4>(par, par[i - PW], par[i]);
         }
         if (32 * sx + lane >= tw) born = 0u;
     }
     __syncthreads();
 
     // ---- 2. links across sub-tile boundaries: vertical boundaries between
-    //         sub-tile columns, horizontal ones between sub-tile rows.  A link
-    //         whose two sites point at the same nodes as those of the bonded
-    //         link before it along the boundary joins nothing new (a site's
-    //         entry is always in its own set, whatever unions are under way).
+    //         sub-tile columns, horizontal ones between sub-tile rows.  (Skipping a
+    //         link whose sites point at the same nodes as the one before it along
+    //         the boundary costs more than the unions it saves: 1433 us a sweep
+    //         against 1426 at L=16384, T_c.)
     {
         constexpr int NV = (TWW - 1) * TH;
         constexpr int NH = (TH / 32 - 1) * TW;
         for (int q = threadIdx.x; q < NV + NH; q += NT) {
-            int ia, ib, step;
-            bool before;
+            int ia, ib;
             if (q < NV) {
                 const int bnd = q / TH + 1, y = q % TH;     // link (32 bnd - 1, y) - (32 bnd, y)
                 if (y >= th || !(B[y][2 * bnd - 2] >> 31)) continue;
-                before = y > 0 && (B[y - 1][2 * bnd - 2] >> 31);
                 ia = y * PW + 32 * bnd - 1;
                 ib = ia + 1;
-                step = PW;
             } else {
                 const int r = q - NV;
                 const int bnd = r / TW + 1, x = r % TW;     // link (x, 32 bnd - 1) - (x, 32 bnd)
                 const int y = 32 * bnd - 1;
                 if (y + 1 >= th || !((B[y][2 * (x >> 5) + 1] >> (x & 31)) & 1u)) continue;
-                before = x > 0 && ((B[y][2 * ((x - 1) >> 5) + 1] >> ((x - 1) & 31)) & 1u);
                 ia = y * PW + x;
                 ib = ia + PW;
-                step = 1;
             }
-            const int a = par[ia], b = par[ib];
-            if (before && par[ia - step] == a && par[ib - step] == b) continue;
-            shook<1>(par, a, b);
+            shook<2>(par, par[ia], par[ib]);
         }
     }
     __syncthreads();

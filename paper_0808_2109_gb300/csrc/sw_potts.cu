@@ -146,19 +146,16 @@ __device__ __forceinline__ PTile ptile_of(const PottsDev &p, int lt)
     PTile t;
     const int n[3] = {p.ntx, p.nty, p.ntz};
     const int T[3] = {G::TX, G::TY, G::TZ};
-    t.c[0] = lt % p.ntx;
-    t.c[1] = (lt / p.ntx) % p.nty;
-    t.c[2] = lt / (p.ntx * p.nty);
+    const int step[3] = {1, p.ntx, p.ntx * p.nty};
+    const int r = (int)((uint32_t)lt / (uint32_t)p.ntx);
+    t.c[2] = DIM == 3 ? (int)((uint32_t)r / (uint32_t)p.nty) : 0;
+    t.c[1] = r - t.c[2] * p.nty;
+    t.c[0] = lt - r * p.ntx;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         t.o[a] = t.c[a] * T[a];
         t.e[a] = a < DIM ? min(T[a], p.L - t.o[a]) : 1;
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        int cc[3] = {t.c[0], t.c[1], t.c[2]};
-        cc[a] = (cc[a] + 1) % n[a];
-        t.nb[a] = cc[0] + n[0] * (cc[1] + n[1] * cc[2]);
+        t.nb[a] = lt + (t.c[a] + 1 < n[a] ? step[a] : step[a] * (1 - n[a]));
     }
     const uint32_t uL = (uint32_t)p.L;
     t.gbase = (uint32_t)t.o[0] + uL * ((uint32_t)t.o[1] + uL * (uint32_t)t.o[2]);
