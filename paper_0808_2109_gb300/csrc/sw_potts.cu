@@ -131,6 +131,34 @@ __device__ __forceinline__ bool slot_xyz(int s, const int (&e)[3], int &x, int &
     return x < e[0] && y < e[1] && z < e[2];
 }
 
+// The same for slot tid + NT q, the q-th of a tile kernel's thread (q is known
+// when the code is compiled, and with it the face).
+template <int DIM>
+__device__ __forceinline__ bool slot_of(int q, int tid, const int (&e)[3], int &x, int &y, int &z)
+{
+    using G = PG<DIM>;
+    if constexpr (DIM == 2) {
+        static_assert(DIM != 2 || (G::NT == 256 && G::F0 == 64 && G::F1 == 128), "slots of a thread");
+        const bool side = tid < 128;   // q = 0: x-, x+, y-; q = 1: y+
+        z = 0;
+        x = q == 0 ? (side ? (tid < 64 ? 0 : e[0] - 1) : tid - 128) : tid;
+        y = q == 0 ? (side ? tid & 63 : 0) : e[1] - 1;
+    } else {
+        static_assert(DIM != 3 || (G::NT == 256 && G::F0 == 256 && G::F1 == 512 && G::F2 == 512), "slots of a thread");
+        if (q < 2) {
+            x = q ? e[0] - 1 : 0;
+            y = tid & 15;
+            z = tid >> 4;
+        } else {
+            const int f = tid + 256 * (q & 1);
+            x = f & 31;
+            y = q < 6 ? (q < 4 ? 0 : e[1] - 1) : f >> 5;
+            z = q < 6 ? f >> 5 : (q < 8 ? 0 : e[2] - 1);
+        }
+    }
+    return x < e[0] && y < e[1] && z < e[2];
+}
+
 struct PTile {
     int c[3];      // tile coordinates
     int o[3];      // origin (sites)
@@ -221,11 +249,11 @@ __device__ __forceinline__ uint32_t tile_label3(volatile int *par, const uint32_
     auto node = [&](int i) { return col + ((i & 3) + G::TY * (i >> 2)) * G::PW; };
     for (; cy; cy &= cy - 1) {
         const int i = node(__ffs(cy) - 1);
-        shook<2>(par, par[i - G::PW], par[i]);
+        shook<4>(par, par[i - G::PW], par[i]);
     }
     for (; cz; cz &= cz - 1) {
         const int i = node(__ffs(cz) - 1);
-        shook<2>(par, par[i - G::TY * G::PW], par[i]);
+        shook<4>(par, par[i - G::TY * G::PW], par[i]);
     }
     __syncthreads();
     // y bonds from rows y = 3, 7, 11 (every z), z bonds from layer z = 7 (every
@@ -240,7 +268,7 @@ __device__ __forceinline__ uint32_t tile_label3(volatile int *par, const uint32_
         for (; bits; bits &= bits - 1) {
             const int i = A * G::PW + x0 + __ffs(bits) - 1;
             const int a = par[i], b = par[i + step];
-            if (a != pa || b != pb) shook<1>(par, a, b);
+            if (a != pa || b != pb) shook<2>(par, a, b);
             pa = a;
             pb = b;
         }
@@ -736,49 +764,68 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             return DIM == 2 ? 32 * (warp / TWW) + i : 4 * (warp & 3) + (i & 3) + G::TY * (8 * (warp >> 2) + (i >> 2));
         };
 
+        // The labels' nodes that are no roots point at theirs, so that a site's
+        // root is two loads away below (a walk a slot took a quarter of the 3D
+        // kernel: 10 slots a thread).
+        uint32_t linked = 0u;
+        for (uint32_t bits = born; bits; bits &= bits - 1) {
+            const int x = lrow(__ffs(bits) - 1) * G::PW + lx;
+            int v = sm.f.par[x];
+            if (v == x) continue;
+            linked |= bits & -bits;
+            int w = sm.f.par[v];
+            if (w == v) continue;
+            while (w != v) {
+                v = w;
+                w = sm.f.par[v];
+            }
+            sm.f.par[x] = v;
+        }
+        const uint32_t roots = born & ~linked;
+        __syncthreads();
+
         // One node per face site: key = global index of the piece's local root,
         // parent = the piece's first face slot (the representative).
+        // (A slot whose left neighbour has the same root leaves the mark to it: at
+        // T_c a few big pieces hold most slots, and 32 lanes at one address wait
+        // for each other.)
         int rs[G::SPT];
 #pragma unroll
         for (int qq = 0; qq < G::SPT; ++qq) {
             const int s = tid + qq * NT;
             int x, y, z;
             rs[qq] = -1;
-            if (s < S && slot_xyz<DIM>(s, t.e, x, y, z)) {
+            if (s < S && slot_of<DIM>(qq, tid, t.e, x, y, z))
                 rs[qq] = sroot_marked(sm.f.par, (y + G::TY * z) * G::PW + x);
-                atomicMin(&sm.f.par[rs[qq]], (int)(INFO_BORDER | (uint32_t)s));
+            const int left = __shfl_up_sync(FULL, rs[qq], 1);
+            if (rs[qq] >= 0 && (lane == 0 || left != rs[qq])) {
+                const int mark = (int)(INFO_BORDER | (uint32_t)s);
+                if (*(volatile int *)&sm.f.par[rs[qq]] > mark) atomicMin(&sm.f.par[rs[qq]], mark);
             }
         }
         __syncthreads();
         // Every interior root gets its record, its cluster's new state (Sec. I
         // step 3), and is counted; the other labels' nodes take a copy of their
         // root's record where it is there already (cluster sizes are added at
-        // the roots and labels are root indices: the root's index instead).
+        // the roots and labels are root indices: they keep the root's index).
         {
-            uint32_t linked = 0u;
             int ncl = 0;
-            for (uint32_t bits = born; bits; bits &= bits - 1) {
+            for (uint32_t bits = roots; bits; bits &= bits - 1) {
                 const int r = lrow(__ffs(bits) - 1), x = r * G::PW + lx;
                 const int v = sm.f.par[x];
                 if (v == x) {
                     const uint32_t s = qsm ? sm.qs[r][lx] : cluster_state(gidx(lx, r % G::TY, r / G::TY), klo, khi, k0, k1, q);
                     sm.f.par[x] = (int)(INFO_INTERIOR | (S + s));
                     ++ncl;
-                } else if (v >= 0) {
-                    linked |= bits & -bits;
                 }
             }
             ncl = __reduce_add_sync(FULL, ncl);
             if (lane == 0 && ncl) atomicAdd(&sm.acc[3], ncl);
-            for (; linked; linked &= linked - 1) {
-                const int x = lrow(__ffs(linked) - 1) * G::PW + lx;
-                int v = sm.f.par[x], w = sm.f.par[v];
-                while ((uint32_t)w < INFO_INTERIOR && w != v) {
-                    v = w;
-                    w = sm.f.par[v];
+            if (!csz && !last_start)
+                for (; linked; linked &= linked - 1) {
+                    const int x = lrow(__ffs(linked) - 1) * G::PW + lx;
+                    sm.f.par[x] = sm.f.par[sm.f.par[x]];   // (a root that has no record yet is its own entry)
                 }
-                sm.f.par[x] = w == v || csz || last_start ? v : w;
-            }
         }
 #pragma unroll
         for (int qq = 0; qq < G::SPT; ++qq) {
@@ -886,7 +933,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 // every root: an interior cluster adds its |C|^2; a border piece hands
                 // its size to its representative node for the merge
                 unsigned long long c2 = 0ull;
-                for (uint32_t bits = born; bits; bits &= bits - 1) {
+                for (uint32_t bits = roots; bits; bits &= bits - 1) {
                     const int v = sm.f.par[lrow(__ffs(bits) - 1) * G::PW + lx];
                     if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
                         p.psize[nbase + (v & 0xFFFF)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
