@@ -94,20 +94,19 @@ struct Replica {
     uint32_t *bondbits;     // tiles * TH * 8 words (last sweep of a call only)
     uint32_t *cross;        // tiles * CROSS_WORDS
     int2 *node;             // tiles * S border nodes {parent, key}
-    uint32_t *nfinal;       // tiles * S resolved (root | spin << 30)
+    uint32_t *nfinal;       // tiles * S resolved (root | spin << 31)
     // PCC scratch (Sec. III): spanning candidates and their coverage (null otherwise)
     uint32_t *pmask;        // tiles * S * 8: a piece's column mask (4 words), row mask (4 words)
     int32_t *cid;           // tiles * S * 2: candidate id + 2 of a root node (x, y), 0 = none
-    int32_t *cand;          // [2][L] candidate roots (x, then y)
-    int32_t *ncand;         // [3]: candidate counts (x, y), decide blocks finished
-    uint32_t *cov;
+    int32_t *ncand;         // [3]: candidate counts (x, y), cover blocks finished
+    uint32_t *cov;          // [L][tiles_x][4] column coverage, then [L][tiles_y][4] row coverage
     // cluster sizes (RF_CSIZE): sites of each border piece at its
     // representative node, and of each cluster at its root node
     int32_t *psize, *csize;
     // topological rule (RF_WIND): per node, parent (low 32 bits) and the
     // node's unwrapped displacement from its parent (high 32 bits, see
     // wind_off) -- one 64-bit word, so both change together
-    unsigned long long *nlink;          // [L][tiles_x][4] column coverage, then [L][tiles_y][4] row coverage
+    unsigned long long *nlink;
 };
 
 // A launch: every tile of every lattice in the tile table (entries of -1
@@ -137,10 +136,15 @@ __device__ __forceinline__ int lattice_launch(const SweepArgs &a, const Replica 
 // A kernel lets its successor start first thing, so that short kernels are all
 // in place when their turn comes (L=64: 23.0 us a sweep against 24.9 when they
 // start after the wait and 27.0 without the chain; L=4096, T=3.0: 93.7, 97.9 and
-// 104 us), except the merge kernels of the topological rule and of PCC, which
-// do so after their wait: their chains are longer, and blocks of several kernels
-// ahead crowd the tile kernel's onto the same SMs (every option at L=1001: 92 us
-// against 111; without the chain 94; PCC L=2048: 95 against 96 and 97).
+// 104 us).  Where a grid does not fill the GPU that has a price: blocks started
+// ahead go to the few SMs with room and run crowded there.  So
+//   - the merge kernels of the topological rule and of PCC let theirs start after
+//     their own wait (every option at L=1001: 92 us against 111);
+//   - the cover kernel of PCC lets the tile kernel start only when it ends (the
+//     tiles of such a lattice have nothing to do before: 2D Potts L=1024 58 us
+//     against 76);
+//   - the Potts tile kernel under the topological rule, whose unions are long,
+//     lets them start before its codes (3D L=128: 85 us against 109).
 __device__ __forceinline__ void chain_next()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -529,6 +533,41 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
+// ------------------------------------------------ union-find with offsets
+// Topological rule (Sec. III): a cluster winds around the box when one of
+// its cycles has a non-zero net displacement.  Nodes carry their unwrapped
+// displacement from their parent; each component is held as a residue mod
+// WIND_M, a prime above any lattice side.  A cycle's net displacement is
+// (n_x L, n_y L) with |n| <= L, which is zero mod WIND_M only for n = 0.
+constexpr uint32_t WIND_M = 65521u;
+
+__device__ __forceinline__ uint32_t wind_off(int dx, int dy)
+{
+    int x = dx % (int)WIND_M, y = dy % (int)WIND_M;
+    x += x < 0 ? (int)WIND_M : 0;
+    y += y < 0 ? (int)WIND_M : 0;
+    return (uint32_t)x | ((uint32_t)y << 16);
+}
+
+__device__ __forceinline__ uint32_t wind_add(uint32_t a, uint32_t b)
+{
+    uint32_t x = (a & 0xFFFFu) + (b & 0xFFFFu), y = (a >> 16) + (b >> 16);
+    x -= x >= WIND_M ? WIND_M : 0u;
+    y -= y >= WIND_M ? WIND_M : 0u;
+    return x | (y << 16);
+}
+
+__device__ __forceinline__ uint32_t wind_neg(uint32_t a)
+{
+    const uint32_t x = a & 0xFFFFu, y = a >> 16;
+    return (x ? WIND_M - x : 0u) | ((y ? WIND_M - y : 0u) << 16);
+}
+
+__device__ __forceinline__ unsigned long long wind_link(int parent, uint32_t off)
+{
+    return (unsigned long long)(uint32_t)parent | ((unsigned long long)off << 32);
+}
+
 // ------------------------------------------------------------ shared layout
 template <int TH>
 struct TileSmem {
@@ -565,9 +604,9 @@ constexpr size_t tile_smem(bool pcc)
 // and without FEAT_WIND.
 constexpr int FEAT_CSIZE = 1;   // cluster sizes (RF_CSIZE)
 constexpr int FEAT_OPEN = 2;    // open boundaries (RF_OPEN)
-constexpr int FEAT_WIND = 4;    // topological rule (RF_WIND; merge kernels only)
+constexpr int FEAT_WIND = 4;    // topological rule (RF_WIND)
 constexpr int FEAT_PCC = 8;     // PCC piece masks (RF_PCC)
-constexpr int FEAT_TILE = FEAT_CSIZE | FEAT_OPEN | FEAT_PCC;
+constexpr int FEAT_TILE = FEAT_CSIZE | FEAT_OPEN | FEAT_WIND | FEAT_PCC;
 
 template <int TH, int F>
 __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(const SweepArgs a)
@@ -584,10 +623,11 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     TileSmem<TH> &sm = *reinterpret_cast<TileSmem<TH> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
 
-    chain_next();
     const int g = blockIdx.x;
     const int ri = g < a.n_tiles ? a.tile_rep[g] : -1;
     const Replica &R = a.reps[max(ri, 0)];
+    const bool wind = (F & FEAT_WIND) && (R.flags & RF_WIND);
+    chain_next();
     const int j = ri < 0 ? -1 : lattice_launch(a, R);   // finishes sweep j-1, starts sweep j
     if (j < 0 || j > R.nsweeps) {
         chain_wait();
@@ -603,6 +643,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     const bool open_b = (F & FEAT_OPEN) && (R.flags & RF_OPEN) && t.ty == R.tiles_y - 1;
     const bool csz = (F & FEAT_CSIZE) && (R.flags & RF_CSIZE) != 0;
     const bool pcc = (F & FEAT_PCC) && (R.flags & RF_PCC) != 0;
+    const bool ext = pcc && !(R.flags & RF_WIND);   // PCC by the extension rule
     // site indices fit in 32 bits (N <= 2^30)
     const uint32_t uL = (uint32_t)L;
     const uint32_t gbase = (uint32_t)t.y0 * uL + (uint32_t)t.x0;   // global index of local site 0
@@ -888,8 +929,19 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
 #pragma unroll
             for (int c = 0; c < TWW; ++c) sm.u.spb[y][c] = __funnelshift_r(w[c], w[c + 1], pos & 31u);
         }
-        if (pcc)
+        if (ext) {
             for (int q = tid; q < S * 8; q += NT) (&sm.pm[0][0])[q] = 0u;
+            // the tiles together clear what the last sweep's candidates left (the
+            // union kernel then resets their counts)
+            const int nt = R.tiles_x * R.tiles_y, i0 = t.lt * NT + tid, di = nt * NT;
+            uint4 *cov4 = reinterpret_cast<uint4 *>(R.cov);
+#pragma unroll
+            for (int ax = 0; ax < 2; ++ax) {
+                const int words = R.ncand[ax] * (ax == 0 ? R.tiles_x : R.tiles_y);
+                for (int i = i0; i < words; i += di) cov4[i] = make_uint4(0u, 0u, 0u, 0u);
+                cov4 += (size_t)L * R.tiles_x;
+            }
+        }
         if (t.lt == 0 && tid == 0) {
             R.obs[j].threshold = thr;
             R.obs[j].spans_x = 0;
@@ -970,6 +1022,19 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                 R.node[node] = make_int2(NODE_NONE, 0);
             }
             if (csz) R.csize[node] = 0;   // the merge adds piece sizes at root nodes
+            if (ext) *reinterpret_cast<int2 *>(R.cid + 2 * node) = make_int2(0, 0);
+            if (wind) {
+                // topological rule: the node's link before the unions -- its
+                // representative and its displacement from it, both in this tile
+                int site, rsite, p = s;
+                uint32_t off = 0u;
+                if (rs[q] >= 0) {
+                    p = info_slot(sm.par[rs[q]]);
+                    if (slot_site<TH>(s, t.tw, t.th, site) && slot_site<TH>(p, t.tw, t.th, rsite))
+                        off = wind_off(site % TW - rsite % TW, site / TW - rsite / TW);
+                }
+                R.nlink[node] = wind_link((int)((size_t)t.lt * S + p), off);
+            }
         }
         __syncthreads();
         // Every site's 2-byte code, the low half of its root's record.  Lane =
@@ -980,7 +1045,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             const int x = 32 * sx + lane;
             uint16_t *cp = code + y0 * TW + x;
             const int *pp = sm.par + y0 * PW + x;
-            if (!((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) && rows == 32 && 32 * sx + 32 <= t.tw) {
+            if (!((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext)) && rows == 32 && 32 * sx + 32 <= t.tw) {
 #pragma unroll 2
                 for (int r = 0; r < 32; r += 4) {
                     int v[4];
@@ -1006,13 +1071,13 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                 // the record's flag bits; the codes read bits 0-15 only), the columns
                 // and rows of a border piece to its masks (only a piece touching the
                 // border can belong to a spanning cluster).
-                const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc);
+                const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext);
                 int cur = -1, cur_v = 0;
                 uint32_t cur_rows = 0u;
                 auto flush = [&]() {
                     if (!cur_rows) return;
                     if (csz) atomicAdd(&sm.par[cur], __popc(cur_rows) << 16);
-                    if (pcc && cur_v < 0) {
+                    if (ext && cur_v < 0) {
                         const int sl = info_slot(cur_v);
                         atomicOr(&sm.pm[sl][sx], 1u << lane);
                         atomicOr(&sm.pm[sl][4 + (y0 >> 5)], cur_rows);
@@ -1041,9 +1106,9 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                 if (gather) flush();
             }
         }
-        if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc)) {
+        if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext)) {
             __syncthreads();
-            if (pcc)
+            if (ext)
                 for (int q = tid; q < S * 8; q += NT) R.pmask[(size_t)t.lt * S * 8 + q] = (&sm.pm[0][0])[q];
             if (csz) {
                 // every root: an interior cluster adds its |C|^2; a border piece
@@ -1079,41 +1144,6 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         if (csz && (half == 0 ? fin : start) && sm.acc_c2[half])
             atomicAdd(&R.obs[j - 1 + half].csize2, sm.acc_c2[half]);
     }
-}
-
-// ------------------------------------------------ union-find with offsets
-// Topological rule (Sec. III): a cluster winds around the box when one of
-// its cycles has a non-zero net displacement.  Nodes carry their unwrapped
-// displacement from their parent; each component is held as a residue mod
-// WIND_M, a prime above any lattice side.  A cycle's net displacement is
-// (n_x L, n_y L) with |n| <= L, which is zero mod WIND_M only for n = 0.
-constexpr uint32_t WIND_M = 65521u;
-
-__device__ __forceinline__ uint32_t wind_off(int dx, int dy)
-{
-    int x = dx % (int)WIND_M, y = dy % (int)WIND_M;
-    x += x < 0 ? (int)WIND_M : 0;
-    y += y < 0 ? (int)WIND_M : 0;
-    return (uint32_t)x | ((uint32_t)y << 16);
-}
-
-__device__ __forceinline__ uint32_t wind_add(uint32_t a, uint32_t b)
-{
-    uint32_t x = (a & 0xFFFFu) + (b & 0xFFFFu), y = (a >> 16) + (b >> 16);
-    x -= x >= WIND_M ? WIND_M : 0u;
-    y -= y >= WIND_M ? WIND_M : 0u;
-    return x | (y << 16);
-}
-
-__device__ __forceinline__ uint32_t wind_neg(uint32_t a)
-{
-    const uint32_t x = a & 0xFFFFu, y = a >> 16;
-    return (x ? WIND_M - x : 0u) | ((y ? WIND_M - y : 0u) << 16);
-}
-
-__device__ __forceinline__ unsigned long long wind_link(int parent, uint32_t off)
-{
-    return (unsigned long long)(uint32_t)parent | ((unsigned long long)off << 32);
 }
 
 __device__ __forceinline__ unsigned long long wload(const unsigned long long *p)
@@ -1173,6 +1203,18 @@ __device__ __forceinline__ void wunite(unsigned long long *lk, const int2 *node,
         const unsigned long long root = (unsigned long long)(uint32_t)hi;   // self link, offset 0
         if (atomicCAS(lk + hi, root, wind_link(lo, off)) == root) return;
     }
+}
+
+// PCC feedback on the threshold for the next sweep (Sec. III): down by delta_k
+// if the clusters percolate, up otherwise, delta_k = 2^(32 - min(8 +
+// floor(k/1000), 20)), clamped to [0, 2^32].
+__device__ __forceinline__ void pcc_feedback(uint64_t *thr, int percolates, uint64_t k)
+{
+    const uint64_t e = 8 + k / 1000;
+    const uint64_t delta = (uint64_t)1 << (32 - (e < 20 ? e : 20));
+    const uint64_t top = (uint64_t)1 << 32;
+    const uint64_t t = *thr;
+    *thr = percolates ? (t > delta ? t - delta : 0) : (t + delta < top ? t + delta : top);
 }
 
 // ------------------------------------------------------------- merge phase
@@ -1264,6 +1306,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::UT, 64 / (MergeCfg<TH>::UT / 32)
     if (!Rp) return;
     const Replica &R = *Rp;
     const Tile t = tile_of(R, blockIdx.x, TH);
+    if ((R.flags & RF_PCC) && t.lt == 0 && threadIdx.x < 2) R.ncand[threadIdx.x] = 0;
     const uint32_t *cross = R.cross + (size_t)t.lt * CROSS_WORDS;
     // (bits past the tile's last row or column are zero)
     const int total = list_bits<MC::LW, MC::UT>(
@@ -1409,32 +1452,6 @@ __global__ void __launch_bounds__(MergeCfg<TH>::UT, 64 / (MergeCfg<TH>::UT / 32)
     }
 }
 
-// Topological rule: every node's link before the unions -- its parent from
-// the tile kernel (a piece's representative, or itself) and its displacement
-// from it, both inside one tile.
-template <int TH>
-__global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_init(const SweepArgs a)
-{
-    using MC = MergeCfg<TH>;
-    int j;
-    const Replica *Rp = merge_lattice<true>(a, blockIdx.x, j);
-    if (!Rp || !(Rp->flags & RF_WIND)) return;
-    const Replica &R = *Rp;
-    const Tile t = tile_of(R, blockIdx.x, TH);
-    const int base = (blockIdx.x - R.tile_base) * MC::S;
-#pragma unroll
-    for (int q = 0; q < MC::NPT; ++q) {
-        const int s = threadIdx.x + q * MC::MT, n = base + s;
-        int p = R.node[n].x;
-        if (p == NODE_NONE) p = n;
-        uint32_t off = 0u;
-        int site, rsite;
-        if (p != n && slot_site<TH>(s, t.tw, t.th, site) && slot_site<TH>(p - base, t.tw, t.th, rsite))
-            off = wind_off(site % TW - rsite % TW, site / TW - rsite / TW);
-        R.nlink[n] = wind_link(p, off);
-    }
-}
-
 // Topological rule: one round of pointer jumping over the representatives'
 // links (the wind unions hang roots under roots, so walks grow longer than on
 // the plain path, which has no such round: without it the merge takes 0.21 ms
@@ -1475,6 +1492,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
     using MC = MergeCfg<TH>;
     __shared__ uint32_t rfin[MC::S];   // the finals of the representatives
     __shared__ int2 walks[MC::S];      // representatives that are no roots: slot, parent
+    __shared__ int rroot[MC::S];       // the root nodes of the representatives (PCC)
     __shared__ int nwalks;
     if (threadIdx.x == 0) nwalks = 0;
     int j;
@@ -1483,6 +1501,10 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;
     const bool wind = W && (R.flags & RF_WIND);   // the forest lives in nlink
+    const bool ext = (R.flags & RF_PCC) && !wind;   // PCC by the extension rule
+    // under the topological rule the unions have recorded the flags: feed back
+    if (wind && (R.flags & RF_PCC) && base == 0 && threadIdx.x == 0)
+        pcc_feedback(R.thr_dev, R.obs[j].spans_x | R.obs[j].spans_y, R.sweep0 + (uint64_t)j);
     // every thread of the block gets here; the last warp may be partial
     const int lane = threadIdx.x & 31, wb = threadIdx.x & ~31;
     const unsigned wm = MC::MT - wb >= 32 ? 0xFFFFFFFFu : (1u << (MC::MT - wb)) - 1u;
@@ -1505,6 +1527,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
         if (rep && !walk) {   // a cluster's root: its own final
             ++nroots;
             rfin[s] = key[q] & ~KEY_REP;
+            if (ext) rroot[s] = n;
             if (R.flags & RF_CSIZE) atomicAdd(R.csize + n, R.psize[n]);
         }
         const unsigned m = __ballot_sync(wm, walk);
@@ -1541,10 +1564,11 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
                 tot = wind_add(tot, wind_neg((uint32_t)(v >> 32)));
                 x = (int)(uint32_t)v;
             }
-        } else if (R.flags & RF_PCC) {
-            // the PCC kernels that follow read a representative's root
-            // straight from its parent; no other kernel reads the forest
-            // again before the next tile launch rewrites it
+        } else if (ext) {
+            // the cover kernel reads a representative's root straight from its
+            // parent; no other kernel reads the forest again before the next
+            // tile launch rewrites it
+            rroot[w.x] = r;
             for (int x = n; x != r;) {
                 const int nx = pload(R.node + x);
                 pstore(R.node + x, r);
@@ -1562,7 +1586,21 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
 #pragma unroll
     for (int q = 0; q < MC::NPT; ++q) {
         const int s = threadIdx.x + q * MC::MT;
-        R.nfinal[base + s] = p[q] == NODE_NONE ? 0u : rfin[(key[q] & KEY_REP) ? s : p[q] - base];
+        const int rs = (key[q] & KEY_REP) ? s : p[q] - base;   // the representative's slot
+        R.nfinal[base + s] = p[q] == NODE_NONE ? 0u : rfin[rs];
+        // PCC, extension rule: the roots of the left-edge nodes of tile column 0
+        // and of the top-edge nodes of tile row 0 are the candidates
+        if (ext && p[q] != NODE_NONE) {
+            using SL = Slots<TH>;
+            const int lt = blockIdx.x - R.tile_base;
+            const int ax = s < SL::BOTTOM ? (lt < R.tiles_x ? 1 : -1)
+                                          : s >= SL::LEFT && s < SL::RIGHT && lt % R.tiles_x == 0 ? 0 : -1;
+            if (ax >= 0) {
+                int32_t *c = R.cid + (size_t)rroot[rs] * 2 + ax;
+                if (gload(c) == 0 && atomicCAS(c, 0, 1) == 0)
+                    *(volatile int32_t *)c = atomicAdd(R.ncand + ax, 1) + 2;   // < L + 2: at most one per edge site
+            }
+        }
     }
     nroots = __reduce_add_sync(wm, nroots);
     if (lane == 0 && nroots) atomicAdd(&R.obs[j].nclusters, (unsigned long long)nroots);
@@ -1575,172 +1613,78 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
 // pieces of one global cluster are united (the paper's update of P_x on a
 // merge) as bit sets per tile column (tile row).
 //
-// Step 1: candidates.  A cluster occupying every column holds a site of
-// column 0, on the left edge of a tile of tile column 0; one occupying every
-// row holds a site of row 0, on the top edge of a tile of tile row 0.  Those
-// edge nodes' roots get compact candidate ids (cid = id + 2).
+// A cluster occupying every column holds a site of column 0, on the left edge
+// of a tile of tile column 0; one occupying every row holds a site of row 0, on
+// the top edge of a tile of tile row 0.  The resolve kernel gave those edge
+// nodes' roots compact candidate ids (cid = id + 2).  Here every border piece
+// ORs the columns (rows) it occupies into its candidate cluster's coverage of
+// the piece's tile column (tile row).  The lattice's last block to finish (a
+// counter taken after a fence: no block waits for another) checks the
+// candidates -- a candidate spans x iff its coverage of every tile column is that
+// column's full mask, y alike; most fail at their first word -- and applies the
+// feedback.  (Separate kernels for the candidates and for checking and clearing
+// took 16 us a sweep at L=2048; counting the fresh bits of every OR instead of
+// checking made this kernel 15 us, four returning atomics in a row.  The tile
+// kernel clears.)
 template <int TH>
-__global__ void k_pcc_candidates(const SweepArgs a)
+__global__ void __launch_bounds__(Slots<TH>::S) k_pcc_cover(const SweepArgs a)
 {
-    chain_wait();
-    chain_next();
-    using SL = Slots<TH>;
-    constexpr int S = SL::S;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)a.n_tiles * (TH + TW)) return;
-    const int g = (int)(idx / (TH + TW));
-    const int e = (int)(idx % (TH + TW));
-    const int ri = a.tile_rep[g];
-    if (ri < 0) return;
-    const Replica &R = a.reps[ri];
-    const int j = lattice_launch(a, R);
-    if (!(R.flags & RF_PCC) || (R.flags & RF_WIND) || j < 0 || j >= R.nsweeps) return;
-    const Tile t = tile_of(R, g, TH);
-    int axis, node;
-    if (e < TH) {
-        if (t.tx != 0 || e >= t.th) return;
-        axis = 0;
-        node = t.lt * S + SL::LEFT + e;
-    } else {
-        const int x = e - TH;
-        if (t.ty != 0 || x >= t.tw) return;
-        axis = 1;
-        node = t.lt * S + SL::TOP + x;
-    }
-    const int2 v = nload(R.node + node);
-    int r = v.x;
-    if (!((uint32_t)v.y & KEY_REP)) r = pload(R.node + r);   // via the representative
-    int32_t *c = R.cid + (size_t)r * 2 + axis;
-    if (atomicCAS(c, 0, 1) == 0) {
-        const int id = atomicAdd(R.ncand + axis, 1);   // < L: at most one per edge site
-        R.cand[axis * R.L + id] = r;
-        *(volatile int32_t *)c = id + 2;
-    }
-}
-
-// Step 2: every border piece ORs the columns (rows) it occupies into its
-// candidate cluster's coverage of the piece's tile column (tile row).
-template <int TH>
-__global__ void k_pcc_cover(const SweepArgs a)
-{
-    chain_wait();
-    chain_next();
     constexpr int S = Slots<TH>::S;
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (int64_t)a.n_tiles * S) return;
-    const int g = (int)(n / S);
-    const int ri = a.tile_rep[g];
-    if (ri < 0) return;
-    const Replica &R = a.reps[ri];
-    const int j = lattice_launch(a, R);
-    if (!(R.flags & RF_PCC) || (R.flags & RF_WIND) || j < 0 || j >= R.nsweeps) return;
-    const int64_t nl = n - (int64_t)R.tile_base * S;   // the lattice's own node
-    const uint4 *pm4 = reinterpret_cast<const uint4 *>(R.pmask + (size_t)nl * 8);
-    const uint4 c4 = pm4[0], r4 = pm4[1];
-    if (!(c4.x | c4.y | c4.z | c4.w | r4.x | r4.y | r4.z | r4.w)) return;
-    const int r = pload(R.node + nl);
-    const Tile t = tile_of(R, g, TH);
-    const int cx = R.cid[(size_t)r * 2 + 0], cy = R.cid[(size_t)r * 2 + 1];
-    if (cx >= 2) {
-        uint32_t *cov = R.cov + ((size_t)(cx - 2) * R.tiles_x + t.tx) * 4;
-        const uint32_t w[4] = {c4.x, c4.y, c4.z, c4.w};
+    chain_wait();   // (the tile kernel starts when this one ends: see the chain)
+    int j;
+    const Replica *Rp = launch_lattice(a, blockIdx.x, j);
+    if (!Rp || !(Rp->flags & RF_PCC) || (Rp->flags & RF_WIND)) return;
+    const Replica &R = *Rp;
+    const Tile t = tile_of(R, blockIdx.x, TH);
+    uint32_t *covx = R.cov, *covy = R.cov + (size_t)R.L * R.tiles_x * 4;
+    {
+        const size_t n = (size_t)t.lt * S + threadIdx.x;
+        const uint4 *pm4 = reinterpret_cast<const uint4 *>(R.pmask + n * 8);
+        const uint4 m4[2] = {pm4[0], pm4[1]};   // columns, rows (pieces' representatives only)
+        const int2 id = *reinterpret_cast<const int2 *>(R.cid + 2 * (size_t)max(pload(R.node + n), 0));
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (w[q]) atomicOr(cov + q, w[q]);
-    }
-    if (cy >= 2) {
-        uint32_t *cov = R.cov + (size_t)R.L * R.tiles_x * 4 + ((size_t)(cy - 2) * R.tiles_y + t.ty) * 4;
-        const uint32_t w[4] = {r4.x, r4.y, r4.z, r4.w};
+        for (int ax = 0; ax < 2; ++ax) {
+            const int c = ax == 0 ? id.x : id.y;
+            if (c < 2) continue;
+            uint32_t *cov = ax == 0 ? covx + ((size_t)(c - 2) * R.tiles_x + t.tx) * 4
+                                    : covy + ((size_t)(c - 2) * R.tiles_y + t.ty) * 4;
+            const uint32_t w[4] = {m4[ax].x, m4[ax].y, m4[ax].z, m4[ax].w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (w[q]) atomicOr(cov + q, w[q]);
-    }
-}
-
-// Step 3 (PCC_DECIDE_BLOCKS blocks per lattice, blockIdx.y = the lattice): a
-// candidate spans x iff its coverage of every tile column is that column's
-// full mask (P_x(C) = [0, L-1]); y alike.  Each block checks its share of the
-// candidates, clears their scratch and ORs what it found into the sweep's
-// spans_x / spans_y; the lattice's last block to finish (a counter, ncand[2],
-// taken after a fence: no block waits for another) applies the PCC feedback
-// to the threshold for the next sweep -- down by delta_k if the clusters
-// percolate, up otherwise, delta_k = 2^(32 - min(8 + floor(k/1000), 20)),
-// clamped to [0, 2^32] -- and resets the counts.  Under the topological rule
-// (RF_WIND) there are no candidates: the flags are the windings the unions
-// recorded.
-constexpr int PCC_DECIDE_BLOCKS = 8;
-template <int TH>
-__global__ void k_pcc_decide(const SweepArgs a, int n_reps)
-{
-    chain_wait();
-    chain_next();
-    const int rr = blockIdx.y;
-    if (rr >= n_reps) return;
-    const Replica &R = a.reps[rr];
-    if (R.L <= 0) return;                  // unused slot of a batch
-    const int j = lattice_launch(a, R);
-    if (!(R.flags & RF_PCC) || j < 0 || j >= R.nsweeps) return;
-    const int nx = R.ncand[0], ny = R.ncand[1];
-    uint32_t *covx = R.cov;
-    uint32_t *covy = R.cov + (size_t)R.L * R.tiles_x * 4;
-    // block b takes a contiguous range of each axis's candidates: checks stop
-    // at the first tile column (row) a candidate does not cover, and the
-    // range's coverage is cleared with coalesced stores afterwards
-    const int cx = (nx + gridDim.x - 1) / gridDim.x, cy = (ny + gridDim.x - 1) / gridDim.x;
-    const int x0 = blockIdx.x * cx, x1 = min(nx, x0 + cx);
-    const int y0 = blockIdx.x * cy, y1 = min(ny, y0 + cy);
-    int sx = 0, sy = 0;
-    for (int id = x0 + threadIdx.x; id < x1; id += blockDim.x) {
-        bool full = true;
-        for (int tx = 0; tx < R.tiles_x && full; ++tx) {
-            const int tw = min(TW, R.L - TW * tx);
-            const uint32_t *cv = covx + ((size_t)id * R.tiles_x + tx) * 4;
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t m = valid_mask(q, tw);
-                full &= (cv[q] & m) == m;
-            }
+            for (int q = 0; q < 4; ++q)
+                if (w[q]) atomicOr(cov + q, w[q]);
         }
-        sx |= full;
-        R.cid[(size_t)R.cand[id] * 2 + 0] = 0;
     }
-    for (int id = y0 + threadIdx.x; id < y1; id += blockDim.x) {
-        bool full = true;
-        for (int ty = 0; ty < R.tiles_y && full; ++ty) {
-            const int th = min(TH, R.L - TH * ty);
-            const uint32_t *cv = covy + ((size_t)id * R.tiles_y + ty) * 4;
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t m = valid_mask(q, th);
-                full &= (cv[q] & m) == m;
+    __shared__ int is_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = atomicAdd(R.ncand + 2, 1) == R.tiles_x * R.tiles_y - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!is_last) return;   // else: every other block's coverage is visible
+    int span[2] = {0, 0};
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax) {
+        const int nc = R.ncand[ax], nt = ax == 0 ? R.tiles_x : R.tiles_y, side = ax == 0 ? TW : TH;
+        const uint4 *cov4 = reinterpret_cast<const uint4 *>(ax == 0 ? covx : covy);
+        for (int id = threadIdx.x; id < nc; id += S) {
+            bool full = true;
+            for (int q = 0; q < nt && full; ++q) {
+                const uint4 v = cov4[(size_t)id * nt + q];
+                const int n = min(side, R.L - side * q);
+                full = ((~v.x & valid_mask(0, n)) | (~v.y & valid_mask(1, n)) | (~v.z & valid_mask(2, n)) |
+                        (~v.w & valid_mask(3, n))) == 0u;
             }
+            span[ax] |= full;
         }
-        sy |= full;
-        R.cid[(size_t)R.cand[R.L + id] * 2 + 1] = 0;
+        span[ax] = __syncthreads_or(span[ax]);
     }
-    __syncthreads();   // every check of this block's range has read its coverage
-    for (int64_t q = (int64_t)x0 * R.tiles_x * 4 + threadIdx.x; q < (int64_t)x1 * R.tiles_x * 4; q += blockDim.x)
-        covx[q] = 0u;
-    for (int64_t q = (int64_t)y0 * R.tiles_y * 4 + threadIdx.x; q < (int64_t)y1 * R.tiles_y * 4; q += blockDim.x)
-        covy[q] = 0u;
-    sx = __syncthreads_or(sx);
-    sy = __syncthreads_or(sy);
     if (threadIdx.x != 0) return;
-    DevObs &o = R.obs[j];
-    if (sx) atomicOr(&o.spans_x, 1);
-    if (sy) atomicOr(&o.spans_y, 1);
-    __threadfence();
-    if (atomicAdd(R.ncand + 2, 1) != (int)gridDim.x - 1) return;
-    // the last block: every other block's flags are visible
-    __threadfence();
-    const int fx = *(volatile int32_t *)&o.spans_x, fy = *(volatile int32_t *)&o.spans_y;
-    const uint64_t k = R.sweep0 + (uint64_t)j;
-    const uint64_t e = 8 + k / 1000;
-    const uint64_t delta = (uint64_t)1 << (32 - (e < 20 ? e : 20));
-    const uint64_t top = (uint64_t)1 << 32;
-    const uint64_t t = *R.thr_dev;
-    *R.thr_dev = (fx || fy) ? (t > delta ? t - delta : 0) : (t + delta < top ? t + delta : top);
-    R.ncand[0] = 0;
-    R.ncand[1] = 0;
     R.ncand[2] = 0;
+    R.obs[j].spans_x = span[0];
+    R.obs[j].spans_y = span[1];
+    pcc_feedback(R.thr_dev, span[0] | span[1], R.sweep0 + (uint64_t)j);
 }
 
 // ------------------------------------------------------------ small kernels

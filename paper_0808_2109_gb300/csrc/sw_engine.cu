@@ -57,9 +57,8 @@ cudaError_t launch_tile(const SweepArgs &a, bool pcc, int feat, cudaStream_t st,
 // The merge of launch group j: unions across tile edges, every node's resolved
 // root and new spin; then for PCC lattices the span test and the feedback.
 template <int TH>
-cudaError_t launch_merge(const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st, bool chained)
+cudaError_t launch_merge(const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
-    constexpr int S = Slots<TH>::S;
     constexpr int MT = MergeCfg<TH>::MT;
     const bool wind = (feat & FEAT_WIND) != 0;
     const dim3 tiles(a.n_tiles);
@@ -67,16 +66,10 @@ cudaError_t launch_merge(const SweepArgs &a, bool pcc, int feat, int n_reps, cud
     auto go = [&](auto *k, dim3 grid, unsigned threads, auto... args) {
         if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, args...);
     };
-    if (wind) go(k_wind_init<TH>, tiles, MT, a);
     go(wind ? k_merge_union<TH, true> : k_merge_union<TH, false>, tiles, MergeCfg<TH>::UT, a);
     if (wind) go(k_wind_jump<TH>, tiles, MT, a);
     go(wind ? k_merge_resolve<TH, true> : k_merge_resolve<TH, false>, tiles, MT, a);
-    if (pcc) {   // reads the compressed forest; the spins do not depend on it
-        const int64_t nu = (int64_t)a.n_tiles * (TH + TW), nn = (int64_t)a.n_tiles * S;
-        go(k_pcc_candidates<TH>, dim3((unsigned)((nu + MERGE_THREADS - 1) / MERGE_THREADS)), MERGE_THREADS, a);
-        go(k_pcc_cover<TH>, dim3((unsigned)((nn + MERGE_THREADS - 1) / MERGE_THREADS)), MERGE_THREADS, a);
-        go(k_pcc_decide<TH>, dim3(PCC_DECIDE_BLOCKS, n_reps), 256, a, n_reps);
-    }
+    if (pcc) go(k_pcc_cover<TH>, tiles, Slots<TH>::S, a);   // reads the compressed forest; the spins do not depend on it
     return e;
 }
 
@@ -90,30 +83,30 @@ cudaError_t enqueue_tile(int TH, const SweepArgs &a, bool pcc, int feat, cudaStr
     }
 }
 
-cudaError_t enqueue_merge(int TH, const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st, bool chained)
+cudaError_t enqueue_merge(int TH, const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
     switch (TH) {
-    case 32: return launch_merge<32>(a, pcc, feat, n_reps, st, chained);
-    case 64: return launch_merge<64>(a, pcc, feat, n_reps, st, chained);
-    case 96: return launch_merge<96>(a, pcc, feat, n_reps, st, chained);
-    default: return launch_merge<128>(a, pcc, feat, n_reps, st, chained);
+    case 32: return launch_merge<32>(a, pcc, feat, st, chained);
+    case 64: return launch_merge<64>(a, pcc, feat, st, chained);
+    case 96: return launch_merge<96>(a, pcc, feat, st, chained);
+    default: return launch_merge<128>(a, pcc, feat, st, chained);
     }
 }
 
 // One launch group: the tile kernel of launch j, then the merge of sweep j.
-cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat, int n_reps, cudaStream_t st,
+cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat, cudaStream_t st,
                               bool chained)
 {
     cudaError_t e = enqueue_tile(TH, a, pcc, feat, st, chained);
     if (e != cudaSuccess) return e;
-    return enqueue_merge(TH, a, pcc, feat, n_reps, st, true);
+    return enqueue_merge(TH, a, pcc, feat, st, true);
 }
 
 cudaError_t enqueue_groups(int TH, SweepArgs a, bool pcc, int feat, int m, bool last, cudaStream_t st)
 {
     for (a.j = 0; a.j < m; ++a.j) {
         const cudaError_t e = last && a.j == m - 1 ? enqueue_tile(TH, a, pcc, feat, st, a.j > 0)
-                                                   : enqueue_launch_th(TH, a, pcc, feat, 1, st, a.j > 0);
+                                                   : enqueue_launch_th(TH, a, pcc, feat, st, a.j > 0);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -250,7 +243,7 @@ struct sw_ctx {
     uint8_t *bond_bytes = nullptr;
     // PCC scratch
     uint32_t *pmask = nullptr;
-    int32_t *cid = nullptr, *cand = nullptr, *ncand = nullptr;
+    int32_t *cid = nullptr, *ccount = nullptr, *ncand = nullptr;
     uint32_t *cov = nullptr;
     // cluster sizes (SW_FLAG_CSIZE)
     int32_t *psize = nullptr, *csize = nullptr;
@@ -293,7 +286,7 @@ void ctx_free(sw_ctx *c)
     c->ev_pool.clear();
     void *ptrs[] = {c->spin, c->label, c->code, c->bondbits, c->cross, c->node,
                     c->nfinal, c->thr_dev, c->rep_dev, c->tile_rep, c->jbase, c->bond_bytes, c->obs,
-                    c->pmask, c->cid, c->cand, c->ncand, c->cov, c->psize, c->csize, c->nlink, c->nstate, c->wlink};
+                    c->pmask, c->cid, c->ccount, c->ncand, c->cov, c->psize, c->csize, c->nlink, c->nstate, c->wlink};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
@@ -364,7 +357,6 @@ int ctx_create(sw_ctx **out, int32_t L, uint64_t thr, uint64_t seed, bool pcc, u
         const size_t ncov = (size_t)L * (c->tiles_x + c->tiles_y) * 4;
         if ((e = dalloc(&c->pmask, nt * c->S * 8)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->cid, nt * c->S * 2)) != cudaSuccess) return fail(e);
-        if ((e = dalloc(&c->cand, (size_t)2 * L)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->ncand, 3)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->cov, ncov)) != cudaSuccess) return fail(e);
         if ((e = cudaMemsetAsync(c->cid, 0, nt * c->S * 2 * sizeof(int32_t), c->stream)) != cudaSuccess) return fail(e);
@@ -405,7 +397,6 @@ int ctx_create(sw_ctx **out, int32_t L, uint64_t thr, uint64_t seed, bool pcc, u
     R.nfinal = c->nfinal;
     R.pmask = c->pmask;
     R.cid = c->cid;
-    R.cand = c->cand;
     R.ncand = c->ncand;
     R.cov = c->cov;
     R.psize = c->psize;
@@ -510,7 +501,7 @@ int enqueue_profiled(sw_ctx *c, int32_t n)
         SW_CUDA(cudaEventRecord(e0, c->stream));
         SW_CUDA(enqueue_tile(c->TH, a, c->pcc, ctx_features(c), c->stream, false));
         SW_CUDA(cudaEventRecord(e1, c->stream));
-        if (j < n) SW_CUDA(enqueue_merge(c->TH, a, c->pcc, ctx_features(c), 1, c->stream, false));
+        if (j < n) SW_CUDA(enqueue_merge(c->TH, a, c->pcc, ctx_features(c), c->stream, false));
         SW_CUDA(cudaEventRecord(e2, c->stream));
         c->ev_marks.push_back(e0);
         c->ev_marks.push_back(e1);
@@ -767,11 +758,12 @@ int potts_create(sw_ctx **out, int32_t dim, int32_t L, int32_t q, uint64_t thr, 
         if ((e = dalloc(&c->thr_dev, 1)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->cid, nt * S * (size_t)dim)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->pmask, nt * S * (size_t)g.pmask_words)) != cudaSuccess) return fail(e);
-        if ((e = dalloc(&c->cand, (size_t)dim * F)) != cudaSuccess) return fail(e);
+        if ((e = dalloc(&c->ccount, (size_t)dim * F)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->ncand, 4)) != cudaSuccess) return fail(e);
         if ((e = dalloc(&c->cov, (size_t)dim * F * W)) != cudaSuccess) return fail(e);
         if ((e = cudaMemsetAsync(c->cid, 0, nt * S * (size_t)dim * sizeof(int32_t), c->stream)) != cudaSuccess)
             return fail(e);
+        if ((e = cudaMemsetAsync(c->ccount, 0, (size_t)dim * F * sizeof(int32_t), c->stream)) != cudaSuccess) return fail(e);
         if ((e = cudaMemsetAsync(c->ncand, 0, 4 * sizeof(int32_t), c->stream)) != cudaSuccess) return fail(e);
         if ((e = cudaMemsetAsync(c->cov, 0, (size_t)dim * F * W * sizeof(uint32_t), c->stream)) != cudaSuccess)
             return fail(e);
@@ -781,7 +773,7 @@ int potts_create(sw_ctx **out, int32_t dim, int32_t L, int32_t q, uint64_t thr, 
         p.thr_dev = c->thr_dev;
         p.pmask = c->pmask;
         p.cid = c->cid;
-        p.cand = c->cand;
+        p.ccount = c->ccount;
         p.ncand = c->ncand;
         p.cov = c->cov;
     }

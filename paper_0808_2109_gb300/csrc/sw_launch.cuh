@@ -9,8 +9,6 @@
 
 namespace swg {
 
-constexpr int MERGE_THREADS = 256;
-
 // Defined once, in sw_engine.cu: every kernel template is instantiated in
 // that translation unit only, so each kernel has a single module copy (and
 // the shared-memory attribute set by prepare_th applies to the copy that
@@ -23,9 +21,9 @@ __attribute__((visibility("hidden"))) cudaError_t prepare_th(int TH);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_tile(int TH, const SweepArgs &a, bool pcc, int feat,
                                                                cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_merge(int TH, const SweepArgs &a, bool pcc, int feat,
-                                                                int n_reps, cudaStream_t st, bool chained);
+                                                                cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat,
-                                                                    int n_reps, cudaStream_t st, bool chained);
+                                                                    cudaStream_t st, bool chained);
 // Launch groups j = 0 .. m-1 of one lattice; last: the final one is a call's
 // last and has no merge.
 __attribute__((visibility("hidden"))) cudaError_t enqueue_groups(int TH, SweepArgs a, bool pcc, int feat, int m,
@@ -81,13 +79,13 @@ struct PottsDev {
     int4 *wlink;                       // RF_WIND: ntiles * slots node links {parent, dx, dy, dz}
     // PCC (null otherwise): the threshold lives on the device and follows the
     // feedback; per node and axis a < dim, a root's candidate id (cid, id + 2),
-    // per border piece its occupied coordinates (pmask), per axis the
-    // candidates (cand + a F, F = L^(dim-1) face sites), their counts
-    // (ncand[a]; ncand[3] counts finished decision blocks) and coverage
-    // (cov + a F W, W = ceil(L / 32) words per candidate)
+    // per border piece its occupied coordinates (pmask), per axis the number of
+    // candidates (ncand[a]; ncand[3] counts finished cover blocks), their
+    // coverage (cov + a F W, F = L^(dim-1) face sites, W = ceil(L / 32) words per
+    // candidate) and how many coordinates each covers (ccount + a F)
     uint64_t *thr_dev;
     uint32_t *pmask;
-    int32_t *cid, *cand, *ncand;
+    int32_t *cid, *ccount, *ncand;
     uint32_t *cov;
 };
 

@@ -13,13 +13,12 @@
 //             union-find over the bonds inside the tile, the new state of
 //             every cluster that ends inside the tile, one node per site of
 //             each tile face, and the site codes.
-//   k_pmerge_union / k_pmerge_resolve (with k_pwind_init under the
-//             topological rule)
+//   k_pmerge_union / k_pmerge_resolve
 //             the master's step 2: a union-find over the face nodes joined by
 //             the bonds that leave a tile (the wrapping links included),
 //             smaller key (cluster minimum) wins; then every representative
 //             node gets its cluster's root and new state.
-//   k_ppcc_candidates / k_ppcc_cover / k_ppcc_decide
+//   k_ppcc_cover
 //             PCC (Sec. III): the extension rule per axis on the merged
 //             clusters, and the feedback on the threshold.
 //
@@ -190,6 +189,12 @@ __device__ __forceinline__ PTile ptile_of(const PottsDev &p, int lt)
     return t;
 }
 
+// A node's link under the topological rule (below): its parent and its
+// displacement from it.
+struct alignas(16) WLink {
+    int32_t parent, dx, dy, dz;
+};
+
 // ------------------------------------------------- 3D tile union-find
 // Connected components of the bonds inside a 32 x 16 x 16 tile, B[r] = {+x,
 // +y, +z bonds} of row r = y + 16 z, all without the links that leave the
@@ -350,7 +355,8 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PSmem<DIM> &sm = *reinterpret_cast<PSmem<DIM> *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    chain_next();
+    const bool wind = (F & FEAT_WIND) && (p.flags & RF_WIND);
+    if (!wind) chain_next();   // (topological rule: below)
     const int lt = blockIdx.x;   // the grid is the lattice's tiles
     const bool fin = j >= 1, start = j < nsweeps;
     const PTile t = ptile_of<DIM>(p, lt);
@@ -362,7 +368,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     const bool open_y = open && t.c[1] == p.nty - 1;
     const bool open_z = DIM == 3 && open && t.c[2] == p.ntz - 1;
     const bool csz = (F & FEAT_CSIZE) && (p.flags & RF_CSIZE);
-    const bool pcc = (F & FEAT_PCC) && (p.flags & RF_PCC);
+    const bool ext = (F & FEAT_PCC) && (p.flags & RF_PCC) && !(p.flags & RF_WIND);   // PCC by the extension rule
     uint16_t *code = p.code + (size_t)lt * G::NS;
     const size_t nbase = (size_t)lt * S;
     const uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
@@ -740,8 +746,18 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             }
             put(bx & valid_mask(wc, tw - 1), wy < th - 1 ? by : 0u, wz < td - 1 ? bz : 0u);
         }
-        if (start && pcc)
+        if (start && ext) {
             for (int w = tid; w < S * G::PMW; w += NT) (&sm.pm[0][0])[w] = 0u;
+            // the tiles together clear what the last sweep's candidates left
+            // (the union kernel then resets their counts)
+            const int64_t W = (p.L + 31) / 32, FS = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
+            const int64_t i0 = (int64_t)lt * NT + tid, di = (int64_t)p.ntiles * NT;
+            for (int a = 0; a < DIM; ++a) {
+                const int64_t nc = p.ncand[a];
+                for (int64_t i = i0; i < nc * W; i += di) p.cov[a * FS * W + i] = 0u;
+                for (int64_t i = i0; i < nc; i += di) p.ccount[a * FS + i] = 0;
+            }
+        }
         if (start && lt == 0 && tid == 0) {
             obs[j].threshold = thr;
             obs[j].spans_x = 0;
@@ -846,12 +862,27 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 p.node[node] = make_int2(NODE_NONE, 0);
             }
             if (csz) p.csize[node] = 0;   // the merge adds piece sizes at root nodes
+            if (ext)
+                for (int a = 0; a < DIM; ++a) p.cid[node * DIM + a] = 0;
+            if (wind) {
+                // topological rule: the node's link before the unions -- its
+                // representative and its displacement from it, both in this tile
+                WLink w{(int)node, 0, 0, 0};
+                int x, y, z, xr, yr, zr;
+                if (rs[qq] >= 0) {
+                    const int rep = sm.f.par[rs[qq]] & 0xFFFF;
+                    if (slot_xyz<DIM>(s, t.e, x, y, z) && slot_xyz<DIM>(rep, t.e, xr, yr, zr))
+                        w = WLink{(int)(nbase + rep), x - xr, y - yr, z - zr};
+                }
+                reinterpret_cast<WLink *>(p.wlink)[node] = w;
+            }
         }
         __syncthreads();
+        if (wind) chain_next();
         // Every site's 2-byte code (the low half of its root's record): border
         // pieces by representative slot, interior clusters S + their new state.
         // Lane = column: a site's entry, its label's node, seldom a third one.
-        const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || pcc);
+        const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext);
         if (!gather && !last_start && tw == G::TX && th == G::TY && td == G::TZ) {
 #pragma unroll 2
             for (int i = 0; i < 32; i += 4) {
@@ -879,7 +910,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             auto flush = [&]() {
                 if (!cur_rows) return;
                 if (csz) atomicAdd(&sm.f.par[cur], __popc(cur_rows) << 16);
-                if (pcc && cur_v < 0) {
+                if (ext && cur_v < 0) {
                     uint32_t *pm = sm.pm[cur_v & 0xFFFF];
                     if (DIM == 2) {
                         atomicOr(pm + (warp % TWW), 1u << lane);
@@ -927,7 +958,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         }
         if (gather) {
             __syncthreads();
-            if (pcc)
+            if (ext)
                 for (int w = tid; w < S * G::PMW; w += NT) p.pmask[nbase * G::PMW + w] = (&sm.pm[0][0])[w];
             if (csz) {
                 // every root: an interior cluster adds its |C|^2; a border piece hands
@@ -971,10 +1002,6 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
 // changed by 16-byte compare-and-swap so that the four move together; a root
 // links to itself with displacement 0.  The displacements are exact: a set's
 // nodes lift to a connected set of at most N sites, so they stay below 2^30.
-struct alignas(16) WLink {
-    int32_t parent, dx, dy, dz;
-};
-
 __device__ __forceinline__ WLink wl_read(WLink *w)
 {
     const WLink z{0, 0, 0, 0};
@@ -1046,6 +1073,7 @@ struct PMC {
     static constexpr int UB = DIM == 2 ? 21 : 5;          // its blocks per SM
     static constexpr int MT = DIM == 2 ? 64 : 320;
     static constexpr int NPT = PG<DIM>::S / MT;           // slots per thread
+    static constexpr int CT = DIM == 2 ? 384 : 512;       // threads of the cover kernel
     static_assert(PG<DIM>::S % MT == 0 && PG<DIM>::S % 16 == 0, "merge launch shape");
 };
 
@@ -1068,6 +1096,7 @@ __global__ void __launch_bounds__(PMC<DIM>::UT, PMC<DIM>::UB) k_pmerge_union(con
     constexpr int S = G::S, EPT = 2;
     __shared__ uint16_t links[G::FT];   // the bonded crossing links
     const int lt = blockIdx.x;
+    if ((p.flags & RF_PCC) && lt == 0 && threadIdx.x < DIM) p.ncand[threadIdx.x] = 0;
     const PTile t = ptile_of<DIM>(p, lt);
     const uint32_t *cross = p.cross + (size_t)lt * G::CW;
     const int total = list_bits<G::CW, MC::UT>([&](int w) { return cross[w]; }, links);
@@ -1180,32 +1209,6 @@ __global__ void __launch_bounds__(PMC<DIM>::UT, PMC<DIM>::UB) k_pmerge_union(con
     }
 }
 
-// Topological rule: every node's link before the unions -- its parent from
-// the tile kernel (its piece's representative, or itself) and its
-// displacement from it, both sites of one tile.
-template <int DIM>
-__global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_init(const PottsDev p)
-{
-    chain_wait();
-    chain_next();
-    using G = PG<DIM>;
-    using MC = PMC<DIM>;
-    const int lt = blockIdx.x, base = lt * G::S;
-    const PTile t = ptile_of<DIM>(p, lt);
-    WLink *wl = reinterpret_cast<WLink *>(p.wlink);
-#pragma unroll
-    for (int qq = 0; qq < MC::NPT; ++qq) {
-        const int s = threadIdx.x + qq * MC::MT, n = base + s;
-        const int rep = p.node[n].x;
-        WLink w{n, 0, 0, 0};
-        int x, y, z, xr, yr, zr;
-        if (rep != NODE_NONE && rep != n && slot_xyz<DIM>(s, t.e, x, y, z) &&
-            slot_xyz<DIM>(rep - base, t.e, xr, yr, zr))
-            w = WLink{rep, x - xr, y - yr, z - zr};
-        wl[n] = w;
-    }
-}
-
 // Every representative that is not its cluster's root walks to the root r and
 // takes r's state, which the tile kernel left in kstate (Sec. I step 3; nstate
 // itself the tile kernel must not write: its neighbours read it for their
@@ -1216,7 +1219,7 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pwind_init(const PottsDev p)
 // the neighbour's halo.  Counts the clusters that
 // touch a tile face (one root node each).
 template <int DIM, bool W>
-__global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, bool last, DevObs *obs)
+__global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, bool last, uint64_t sweep0, DevObs *obs)
 {
     const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
     if (!late) chain_next();
@@ -1232,6 +1235,9 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
     __shared__ alignas(16) uint8_t rst[PG<DIM>::S];   // the new state of every slot
     __shared__ int2 walks[PG<DIM>::S];   // representatives that are no roots: slot, parent
     __shared__ int nwalks;
+    // under the topological rule the unions have recorded the flags: feed back
+    if (wind && (p.flags & RF_PCC) && base == 0 && threadIdx.x == 0)
+        pcc_feedback(p.thr_dev, obs[j].spans_x | obs[j].spans_y, sweep0 + (uint64_t)j);
     if (threadIdx.x == 0) nwalks = 0;
     // (every slot's state, kept for the representatives below)
     for (int i = threadIdx.x; i < PG<DIM>::S / 16; i += MC::MT)
@@ -1264,14 +1270,14 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
         if (walk) walks[at] = make_int2(s, up);
     }
     __syncthreads();
-    const bool pcc = (p.flags & RF_PCC) != 0 && !wind;   // the extension rule's candidates read the parents
+    const bool ext = (p.flags & RF_PCC) != 0 && !wind;   // PCC by the extension rule
     for (int i = threadIdx.x; i < nwalks; i += MC::MT) {
         const int2 w = walks[i];
         const int n = base + w.x;
         int r = w.y;
         for (int up = parent(r); up != r; up = parent(r)) r = up;
-        if (pcc) {
-            // the PCC kernels read a representative's root from its parent
+        if (ext) {
+            // the cover kernel reads a representative's root from its parent
             for (int x = n; x != r;) {
                 const int nx = pload(p.node + x);
                 pstore(p.node + x, r);
@@ -1283,6 +1289,25 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
         rst[w.x] = p.kstate[r];
     }
     __syncthreads();
+    if (ext) {
+        // the roots of the "-" face nodes of the tiles of coordinate 0 along an
+        // axis are that axis's candidates (cid = id + 2)
+        const PTile t = ptile_of<DIM>(p, blockIdx.x);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            if (t.c[a] != 0) continue;
+            const int n0 = base + face_off<DIM>(a, 0), nf = a == 0 ? PG<DIM>::F0 : a == 1 ? PG<DIM>::F1 : PG<DIM>::F2;
+            for (int f = threadIdx.x; f < nf; f += MC::MT) {
+                const int2 v = nload(p.node + n0 + f);
+                if (v.x == NODE_NONE) continue;
+                // a representative's parent is its root by now, another slot's its representative
+                const int r = ((uint32_t)v.y & KEY_REP) ? v.x : pload(p.node + v.x);
+                int32_t *c = p.cid + (size_t)r * DIM + a;
+                if (gload(c) == 0 && atomicCAS(c, 0, 1) == 0)
+                    *(volatile int32_t *)c = atomicAdd(p.ncand + a, 1) + 2;   // < F + 2: at most one per face site
+            }
+        }
+    }
     // a slot that is not a representative (whose parent is still its own
     // representative in this tile) takes its cluster's new state too: the
     // neighbour's halo reads it with one load.  (Slots past the tile's sites
@@ -1301,128 +1326,86 @@ __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev 
 // The extension rule in d dimensions (Sec. III): a cluster spans axis a iff
 // it occupies all L hyperplanes perpendicular to a.  Such a cluster holds a
 // site of the hyperplane a = 0, on the - face of a tile of tile coordinate 0
-// along a: those nodes' roots are the candidates (cid of the root node, per
-// axis: id + 2).  Every border piece then ORs the coordinates it occupies
-// along a into its candidate root's coverage (L bits), and a candidate spans
-// iff its coverage is full.  Interior clusters touch no face and span nothing.
+// along a: the resolve kernel made those nodes' roots the candidates (cid of
+// the root node, per axis: id + 2).  Here every border piece ORs the coordinates
+// it occupies along a into its candidate root's coverage (L bits): in 3D, where a
+// piece has one word an axis and the candidates of a face are many, the bits
+// that were not there yet are added to the candidate's count, and a count of
+// L spans; in 2D the last block checks the candidates' words (most fail at the
+// first).  spans_x reports axis x, spans_y y, in 3D y or z.  Interior clusters
+// touch no face and span nothing.  The last block to finish (a counter after a
+// fence: no block waits) applies the feedback.
 template <int DIM>
-__global__ void k_ppcc_candidates(const PottsDev p, int64_t F)
+__global__ void __launch_bounds__(PMC<DIM>::CT) k_ppcc_cover(const PottsDev p, int j, uint64_t sweep0, DevObs *obs)
 {
-    chain_wait();
-    chain_next();
     using G = PG<DIM>;
-    constexpr int S = G::S;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)p.ntiles * G::FT) return;
-    const int lt = (int)(idx / G::FT), e = (int)(idx % G::FT);
-    const int a = e < G::F0 ? 0 : e < G::F0 + G::F1 ? 1 : 2;
-    const int f = e - (a == 0 ? 0 : a == 1 ? G::F0 : G::F0 + G::F1);
+    constexpr int CT = PMC<DIM>::CT;
+    chain_wait();   // (the tile kernel starts when this one ends: sw_device.cuh)
+    const int lt = blockIdx.x;
     const PTile t = ptile_of<DIM>(p, lt);
-    if (t.c[a] != 0) return;
-    const int node = lt * S + face_off<DIM>(a, 0) + f;
-    const int2 v = nload(p.node + node);
-    if (v.x == NODE_NONE) return;
-    int r = v.x;
-    if (!((uint32_t)v.y & KEY_REP)) r = pload(p.node + r);   // via a representative
-    int32_t *c = p.cid + (size_t)r * DIM + a;
-    if (atomicCAS(c, 0, 1) == 0) {
-        const int id = atomicAdd(p.ncand + a, 1);   // < F: at most one per face site
-        p.cand[(size_t)a * F + id] = r;
-        *(volatile int32_t *)c = id + 2;
-    }
-}
-
-template <int DIM>
-__global__ void k_ppcc_cover(const PottsDev p)
-{
-    chain_wait();
-    chain_next();
-    using G = PG<DIM>;
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (int64_t)p.ntiles * G::S) return;
-    const int2 v = nload(p.node + n);
-    if (!((uint32_t)v.y & KEY_REP)) return;
-    uint32_t m[G::PMW];
-    uint32_t any = 0u;
-#pragma unroll
-    for (int w = 0; w < G::PMW; ++w) any |= (m[w] = p.pmask[(size_t)n * G::PMW + w]);
-    if (!any) return;
-    const int r = v.x;
-    const PTile t = ptile_of<DIM>(p, (int)(n / G::S));
     const uint32_t W = ((uint32_t)p.L + 31u) / 32u;
     const int64_t F = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
+    DevObs *o = obs + j;
+    for (int s = threadIdx.x; s < G::S; s += CT) {
+        const size_t n = (size_t)lt * G::S + s;
+        const int2 v = nload(p.node + n);
+        uint32_t m[G::PMW];
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        const int c = p.cid[(size_t)r * DIM + a];
-        if (c < 2) continue;
-        uint32_t *cov = p.cov + ((size_t)a * F + (size_t)(c - 2)) * W + (size_t)(t.o[a] >> 5);
-        if (DIM == 2) {
-            if (a == 0) {
+        for (int w = 0; w < G::PMW; ++w) m[w] = p.pmask[n * G::PMW + w];
+        if (!((uint32_t)v.y & KEY_REP)) continue;
 #pragma unroll
-                for (int w = 0; w < 4; ++w)
-                    if (m[w]) atomicOr(cov + w, m[w]);
+        for (int a = 0; a < DIM; ++a) {
+            const int c = p.cid[(size_t)v.x * DIM + a];
+            if (c < 2) continue;
+            uint32_t *cov = p.cov + ((size_t)a * F + (size_t)(c - 2)) * W + (size_t)(t.o[a] >> 5);
+            if constexpr (DIM == 2) {
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    const uint32_t bits = a == 0 ? m[w] : w < 2 ? m[G::PMW - 2 + w] : 0u;
+                    if (bits) atomicOr(cov + w, bits);
+                }
             } else {
-#pragma unroll
-                for (int w = 0; w < 2; ++w)
-                    if (m[4 + w]) atomicOr(cov + w, m[4 + w]);
+                // 32-site x words; 16-site y and z halves at an origin that is a
+                // multiple of 16
+                const uint32_t half = a == 0 ? m[0] : a == 1 ? (m[1] & 0xFFFFu) : (m[1] >> 16);
+                const uint32_t bits = a == 0 ? half : half << (t.o[a] & 31);
+                if (!bits) continue;
+                const int fresh = __popc(bits & ~atomicOr(cov, bits));
+                if (fresh && atomicAdd(p.ccount + a * F + (c - 2), fresh) + fresh == p.L)
+                    atomicOr(a == 0 ? &o->spans_x : &o->spans_y, 1);
             }
-        } else {
-            // 32-site x words; 16-site y and z halves at an origin that is a
-            // multiple of 16
-            const uint32_t bits = a == 0 ? m[0] : a == 1 ? (m[1] & 0xFFFFu) : (m[1] >> 16);
-            if (bits) atomicOr(cov, a == 0 ? bits : bits << (t.o[a] & 31));
         }
     }
-}
-
-// PPCC_DECIDE blocks: each checks a contiguous range of every axis's
-// candidates, clears their scratch and ORs its flags into the sweep's
-// spans_x (axis x) / spans_y (axis y, and z in 3D); the last block to finish
-// (a counter after a fence: no block waits) applies the feedback -- down by
-// delta_k if some cluster spans, up otherwise, delta_k = 2^(32 - min(8 +
-// floor(k / 1000), 20)), clamped to [0, 2^32] -- and resets the counts.
-constexpr int PPCC_DECIDE = 16;
-__global__ void k_ppcc_decide(const PottsDev p, int64_t F, int j, uint64_t sweep0, DevObs *obs)
-{
-    chain_wait();
-    chain_next();
-    const uint32_t L = (uint32_t)p.L, W = (L + 31) / 32;
-    DevObs *o = obs + j;
-    int sx = 0, sy = 0;
-    for (int a = 0; a < p.dim; ++a) {
-        const int n = p.ncand[a];
-        const int chunk = (n + gridDim.x - 1) / gridDim.x;
-        const int c0 = blockIdx.x * chunk, c1 = min(n, c0 + chunk);
-        uint32_t *cov = p.cov + (size_t)a * F * W;
-        int s = 0;
-        for (int id = c0 + threadIdx.x; id < c1; id += blockDim.x) {
-            bool full = true;
-            for (uint32_t w = 0; w < W && full; ++w) {
-                const uint32_t m = w + 1 < W || (L & 31u) == 0 ? 0xFFFFFFFFu : (1u << (L & 31u)) - 1u;
-                full = (cov[(size_t)id * W + w] & m) == m;
+    __shared__ int is_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = atomicAdd(p.ncand + 3, 1) == (int)gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!is_last) return;   // else: every other block's coverage and flags are visible
+    if constexpr (DIM == 2) {
+        for (int a = 0; a < 2; ++a) {
+            const uint32_t *cov = p.cov + (size_t)a * F * W;
+            const int nc = p.ncand[a];
+            int span = 0;
+            for (int id = threadIdx.x; id < nc; id += CT) {
+                bool full = true;
+                for (uint32_t w = 0; w < W && full; ++w) {
+                    const uint32_t m = valid_mask((int)w, p.L);
+                    full = (cov[(size_t)id * W + w] & m) == m;
+                }
+                span |= full;
             }
-            s |= full;
-            p.cid[(size_t)p.cand[(size_t)a * F + id] * p.dim + a] = 0;
+            span = __syncthreads_or(span);
+            if (threadIdx.x == 0) (a == 0 ? o->spans_x : o->spans_y) = span;
         }
-        s = __syncthreads_or(s);   // also: every check of this range has read its coverage
-        for (int64_t qq = (int64_t)c0 * W + threadIdx.x; qq < (int64_t)c1 * W; qq += blockDim.x) cov[qq] = 0u;
-        if (a == 0) sx |= s;
-        else sy |= s;
     }
     if (threadIdx.x != 0) return;
-    if (sx) atomicOr(&o->spans_x, 1);
-    if (sy) atomicOr(&o->spans_y, 1);
-    __threadfence();
-    if (atomicAdd(p.ncand + 3, 1) != (int)gridDim.x - 1) return;
-    __threadfence();   // the last block: every other block's flags are visible
-    const int fx = *(volatile int32_t *)&o->spans_x, fy = *(volatile int32_t *)&o->spans_y;
-    const uint64_t k = sweep0 + (uint64_t)j;
-    const uint64_t e = 8 + k / 1000;
-    const uint64_t delta = (uint64_t)1 << (32 - (e < 20 ? e : 20));
-    const uint64_t top = (uint64_t)1 << 32;
-    const uint64_t tt = *p.thr_dev;
-    *p.thr_dev = (fx || fy) ? (tt > delta ? tt - delta : 0) : (tt + delta < top ? tt + delta : top);
-    for (int a = 0; a < 4; ++a) p.ncand[a] = 0;
+    p.ncand[3] = 0;
+    const int flags = *(volatile int32_t *)&o->spans_x | *(volatile int32_t *)&o->spans_y;
+    pcc_feedback(p.thr_dev, flags, sweep0 + (uint64_t)j);
 }
 
 // ------------------------------------------------------------ small kernels
@@ -1469,16 +1452,15 @@ template <int DIM>
 cudaError_t launch_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
                         bool chained)
 {
-    const bool feat = (p.flags & (RF_PCC | RF_OPEN | RF_CSIZE)) != 0;
+    const bool feat = (p.flags & (RF_PCC | RF_OPEN | RF_CSIZE | RF_WIND)) != 0;
     return launch_kernel(feat ? k_ptile<DIM, FEAT_TILE> : k_ptile<DIM, 0>, dim3((unsigned)p.ntiles), PG<DIM>::NT,
-                         ptile_smem<DIM>((p.flags & RF_PCC) != 0), st, chained, p, j, nsweeps, sweep0, obs);
+                         ptile_smem<DIM>((p.flags & RF_PCC) && !(p.flags & RF_WIND)), st, chained, p, j, nsweeps, sweep0, obs);
 }
 
 template <int DIM>
 cudaError_t launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
                          bool chained)
 {
-    using G = PG<DIM>;
     constexpr int MT = PMC<DIM>::MT;
     const bool pcc = (p.flags & RF_PCC) != 0, wind = (p.flags & RF_WIND) != 0;
     const dim3 tiles((unsigned)p.ntiles);
@@ -1488,26 +1470,17 @@ cudaError_t launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0,
     };
     const bool last = j == nsweeps - 1;
     if (wind) {
-        go(k_pwind_init<DIM>, tiles, MT, p);
         go(k_pmerge_union<DIM, true>, tiles, PMC<DIM>::UT, p, j, obs);
-        go(k_pmerge_resolve<DIM, true>, tiles, MT, p, j, last, obs);
+        go(k_pmerge_resolve<DIM, true>, tiles, MT, p, j, last, sweep0, obs);
     } else {
         // no pointer-jumping round, here or above: after the unions'
         // single-swap links the walks are short, and the round cost more than it
         // saved (3D 2.99 -> 2.94 ms a sweep without it; the topological rule at
         // L=128 146 -> 135 us)
         go(k_pmerge_union<DIM, false>, tiles, PMC<DIM>::UT, p, j, obs);
-        go(k_pmerge_resolve<DIM, false>, tiles, MT, p, j, last, obs);
+        go(k_pmerge_resolve<DIM, false>, tiles, MT, p, j, last, sweep0, obs);
     }
-    if (pcc) {
-        const int64_t F = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
-        if (!wind) {   // under the topological rule the unions recorded the flags
-            const int64_t nc = (int64_t)p.ntiles * G::FT, nn = (int64_t)p.ntiles * G::S;
-            go(k_ppcc_candidates<DIM>, dim3((unsigned)((nc + PT - 1) / PT)), PT, p, F);
-            go(k_ppcc_cover<DIM>, dim3((unsigned)((nn + PT - 1) / PT)), PT, p);
-        }
-        go(k_ppcc_decide, dim3(PPCC_DECIDE), PT, p, F, j, sweep0, obs);
-    }
+    if (pcc && !wind) go(k_ppcc_cover<DIM>, tiles, PMC<DIM>::CT, p, j, sweep0, obs);
     return e;
 }
 

@@ -65,7 +65,7 @@ struct Job {
     uint16_t *code = nullptr;
     uint32_t *bondbits = nullptr, *cross = nullptr, *nfinal = nullptr, *pmask = nullptr, *cov = nullptr;
     int2 *node = nullptr;
-    int32_t *cid = nullptr, *cand = nullptr, *ncand = nullptr;
+    int32_t *cid = nullptr, *ncand = nullptr;
     uint64_t *thr_dev = nullptr;
     DevObs *obs = nullptr;
     int32_t *psize = nullptr, *csize = nullptr;   // SW_FLAG_CSIZE
@@ -79,7 +79,7 @@ struct Job {
 // 256-byte boundary; PCC scratch last, in one range that starts zeroed.
 struct JobLayout {
     size_t spin, label, code, bondbits, cross, node, nfinal, thr, obs, psize, csize, nlink;
-    size_t pmask, cid, cand, ncand, cov, pcc_end, total;
+    size_t pmask, cid, ncand, cov, pcc_end, total;
 };
 
 JobLayout job_layout(int L, int TH, int nsweeps, bool pcc, bool csize, bool wind)
@@ -109,11 +109,10 @@ JobLayout job_layout(int L, int TH, int nsweeps, bool pcc, bool csize, bool wind
         o.csize = take(nt * S * 4);
     }
     o.nlink = wind ? take(nt * S * 8) : at;
-    o.pmask = o.cid = o.cand = o.ncand = o.cov = o.pcc_end = at;
+    o.pmask = o.cid = o.ncand = o.cov = o.pcc_end = at;
     if (pcc) {
         o.pmask = take(nt * S * 8 * 4);
         o.cid = take(nt * S * 2 * 4);
-        o.cand = take(2 * (size_t)L * 4);
         o.ncand = take(3 * 4);
         o.cov = take((size_t)L * (tx + ty) * 4 * 4);
         o.pcc_end = at;
@@ -209,7 +208,6 @@ cudaError_t job_alloc(Job *j, cudaStream_t st)
     if (j->pcc) {
         j->pmask = reinterpret_cast<uint32_t *>(b + o.pmask);
         j->cid = reinterpret_cast<int32_t *>(b + o.cid);
-        j->cand = reinterpret_cast<int32_t *>(b + o.cand);
         j->ncand = reinterpret_cast<int32_t *>(b + o.ncand);
         j->cov = reinterpret_cast<uint32_t *>(b + o.cov);
         if ((e = cudaMemsetAsync(b + o.pmask, 0, o.pcc_end - o.pmask, st)) != cudaSuccess) return e;
@@ -245,7 +243,6 @@ Replica replica_of(const Job *j)
     R.nfinal = j->nfinal;
     R.pmask = j->pmask;
     R.cid = j->cid;
-    R.cand = j->cand;
     R.ncand = j->ncand;
     R.cov = j->cov;
     R.psize = j->psize;
@@ -354,7 +351,7 @@ cudaError_t lane_capture(Lane &ln, cudaStream_t cap_stream, bool pcc, int feat)
     SweepArgs a = lane_args(ln);
     for (int j = 0; j < GROUPS_PER_STEP && e == cudaSuccess; ++j) {
         a.j = j;
-        e = enqueue_launch_th(ln.TH, a, pcc, feat, ln.cap_reps, cap_stream, j > 0);
+        e = enqueue_launch_th(ln.TH, a, pcc, feat, cap_stream, j > 0);
     }
     cudaError_t e2 = cudaStreamEndCapture(cap_stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
