@@ -1002,10 +1002,18 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
 // changed by 16-byte compare-and-swap so that the four move together; a root
 // links to itself with displacement 0.  The displacements are exact: a set's
 // nodes lift to a connected set of at most N sites, so they stay below 2^30.
-__device__ __forceinline__ WLink wl_read(WLink *w)
+__device__ __forceinline__ WLink wl_read(const WLink *w)
 {
-    const WLink z{0, 0, 0, 0};
-    return atomicCAS(w, z, z);   // an atomic 16-byte read (rewrites an equal word)
+    // one 16-byte load, single-copy atomic as the swaps are (a swap by equal
+    // words as the read serialised the walks of a big cluster at its root: 3D
+    // L=256, T=2.0: 1956 us a sweep against 338)
+    unsigned long long lo, hi;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(w)
+                 : "memory");
+    return WLink{(int32_t)(uint32_t)lo, (int32_t)(uint32_t)(lo >> 32), (int32_t)(uint32_t)hi,
+                 (int32_t)(uint32_t)(hi >> 32)};
 }
 
 // Root of x with pos(x) - pos(root); the walk halves the path (x's link is
