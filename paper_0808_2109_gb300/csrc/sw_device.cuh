@@ -568,6 +568,16 @@ __device__ __forceinline__ unsigned long long wind_link(int parent, uint32_t off
     return (unsigned long long)(uint32_t)parent | ((unsigned long long)off << 32);
 }
 
+// Adds the warp's values to *dst in shared memory.  (A 64-bit add there is a
+// loop of compare-and-swaps: one a warp, where one a thread took 20 us of a tile
+// kernel of 384 threads.)
+__device__ __forceinline__ void warp_add64(unsigned long long *dst, unsigned long long v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
+}
+
 // ------------------------------------------------------------ shared layout
 template <int TH>
 struct TileSmem {
@@ -856,7 +866,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                     const long long c = R.csize[(size_t)t.lt * S + s];
                     c2 += (unsigned long long)(c * c);
                 }
-                if (c2) atomicAdd(&sm.acc_c2[0], c2);
+                warp_add64(&sm.acc_c2[0], c2);
             }
         }
         if (start) {
@@ -1083,24 +1093,35 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                         atomicOr(&sm.pm[sl][4 + (y0 >> 5)], cur_rows);
                     }
                 };
-#pragma unroll 2
-                for (int r = 0; r < rows; ++r) {
-                    int v = site ? pp[r * PW] : (int)(INFO_INTERIOR | 4u * S);
-                    int root = (y0 + r) * PW + x;
-                    while ((uint32_t)v < INFO_INTERIOR) {
-                        root = v;
-                        v = sm.par[v];
+                for (int r = 0; r < rows; r += 4) {   // four rows' look-ups in flight
+                    int v[4], root[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        root[q] = (y0 + r + q) * PW + x;
+                        v[q] = site && r + q < rows ? pp[(r + q) * PW] : (int)(INFO_INTERIOR | 4u * S);
                     }
-                    cp[r * TW] = (uint16_t)v;
-                    if (gather && site) {
-                        const int key = csz ? root : v;
-                        if (key != cur) {
-                            flush();
-                            cur = key;
-                            cur_v = v;
-                            cur_rows = 0u;
+                    while (min(min((uint32_t)v[0], (uint32_t)v[1]), min((uint32_t)v[2], (uint32_t)v[3])) < INFO_INTERIOR) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if ((uint32_t)v[q] < INFO_INTERIOR) {
+                                root[q] = v[q];
+                                v[q] = sm.par[v[q]];
+                            }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (r + q >= rows) break;
+                        cp[(r + q) * TW] = (uint16_t)v[q];
+                        if (gather && site) {
+                            const int key = csz ? root[q] : v[q];
+                            if (key != cur) {
+                                flush();
+                                cur = key;
+                                cur_v = v[q];
+                                cur_rows = 0u;
+                            }
+                            cur_rows |= 1u << (r + q);
                         }
-                        cur_rows |= 1u << r;
                     }
                 }
                 if (gather) flush();
@@ -1124,7 +1145,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                         c2 += size * size;
                     }
                 }
-                if (c2) atomicAdd(&sm.acc_c2[1], c2);
+                warp_add64(&sm.acc_c2[1], c2);
                 __syncthreads();
             }
         }
@@ -1295,7 +1316,7 @@ __device__ __forceinline__ const Replica *merge_lattice(const SweepArgs &a, int 
 // W: compiled with the topological rule (lattices with RF_WIND unite their
 // nodes with displacements in nlink); every kernel of the merge has it.
 template <int TH, bool W>
-__global__ void __launch_bounds__(MergeCfg<TH>::UT, 64 / (MergeCfg<TH>::UT / 32)) k_merge_union(const SweepArgs a)
+__global__ void __launch_bounds__(MergeCfg<TH>::UT, (W ? 40 : 64) / (MergeCfg<TH>::UT / 32)) k_merge_union(const SweepArgs a)
 {
     using SL = Slots<TH>;
     using MC = MergeCfg<TH>;

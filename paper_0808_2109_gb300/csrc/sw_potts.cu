@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                     const long long c = p.csize[nbase + s];
                     c2 += (unsigned long long)(c * c);
                 }
-                if (c2) atomicAdd(&sm.acc_c2[0], c2);
+                warp_add64(&sm.acc_c2[0], c2);
             }
         }
         if (start) {
@@ -930,28 +930,41 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                     }
                 }
             };
-#pragma unroll 2
-            for (int i = 0; i < 32; ++i) {
-                const int r = lrow(i), y = r % G::TY, z = r / G::TY;
-                if (y >= th || z >= td) continue;
-                int root = r * G::PW + lx;
-                int v = lx < tw ? sm.f.par[root] : (int)(INFO_INTERIOR | (uint32_t)S);
-                while ((uint32_t)v < INFO_INTERIOR) {
-                    root = v;
-                    v = sm.f.par[v];
+            for (int i = 0; i < 32; i += 4) {   // four rows' look-ups in flight
+                int v[4], root[4];
+                bool row[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int r = lrow(i + e);
+                    row[e] = r % G::TY < th && r / G::TY < td;
+                    root[e] = r * G::PW + lx;
+                    v[e] = row[e] && lx < tw ? sm.f.par[root[e]] : (int)(INFO_INTERIOR | (uint32_t)S);
                 }
-                code[r * G::TX + lx] = (uint16_t)v;
-                if (lx >= tw) continue;
-                if (last_start && v >= 0) p.label[gidx(lx, y, z)] = (int32_t)gfor(root);
-                if (gather) {
-                    const int key = csz ? root : v;
-                    if (key != cur) {
-                        flush();
-                        cur = key;
-                        cur_v = v;
-                        cur_rows = 0u;
+                while (min(min((uint32_t)v[0], (uint32_t)v[1]), min((uint32_t)v[2], (uint32_t)v[3])) < INFO_INTERIOR) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if ((uint32_t)v[e] < INFO_INTERIOR) {
+                            root[e] = v[e];
+                            v[e] = sm.f.par[v[e]];
+                        }
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (!row[e]) continue;
+                    const int r = lrow(i + e);
+                    code[r * G::TX + lx] = (uint16_t)v[e];
+                    if (lx >= tw) continue;
+                    if (last_start && v[e] >= 0) p.label[gidx(lx, r % G::TY, r / G::TY)] = (int32_t)gfor(root[e]);
+                    if (gather) {
+                        const int key = csz ? root[e] : v[e];
+                        if (key != cur) {
+                            flush();
+                            cur = key;
+                            cur_v = v[e];
+                            cur_rows = 0u;
+                        }
+                        cur_rows |= 1u << (i + e);
                     }
-                    cur_rows |= 1u << i;
                 }
             }
             if (gather) flush();
@@ -973,7 +986,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                         c2 += size * size;
                     }
                 }
-                if (c2) atomicAdd(&sm.acc_c2[1], c2);
+                warp_add64(&sm.acc_c2[1], c2);
                 __syncthreads();
             }
         }
@@ -1078,7 +1091,8 @@ struct PMC {
     // q=2 within 1% from 320 / 256 to 384 / 320, which is the best of the small
     // lattices (L=50 PCC with the topological rule 97 us a sweep against 102)
     static constexpr int UT = DIM == 2 ? 96 : 384;
-    static constexpr int UB = DIM == 2 ? 21 : 5;          // its blocks per SM
+    static constexpr int UB = DIM == 2 ? 21 : 5;          // its blocks per SM (WB: with the topological rule)
+    static constexpr int WB = DIM == 2 ? 12 : 3;
     static constexpr int MT = DIM == 2 ? 64 : 320;
     static constexpr int NPT = PG<DIM>::S / MT;           // slots per thread
     static constexpr int CT = DIM == 2 ? 384 : 512;       // threads of the cover kernel
@@ -1093,7 +1107,7 @@ struct PMC {
 // the Ising merge has, made the 3D merge slower: its pieces are small and
 // seldom meet twice.)
 template <int DIM, bool W>
-__global__ void __launch_bounds__(PMC<DIM>::UT, PMC<DIM>::UB) k_pmerge_union(const PottsDev p, int j, DevObs *obs)
+__global__ void __launch_bounds__(PMC<DIM>::UT, W ? PMC<DIM>::WB : PMC<DIM>::UB) k_pmerge_union(const PottsDev p, int j, DevObs *obs)
 {
     const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
     if (!late) chain_next();
