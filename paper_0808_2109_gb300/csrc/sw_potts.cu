@@ -426,8 +426,13 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     const uint32_t klo = (uint32_t)k, khi = (uint32_t)(k >> 32);
     const bool any_bond = start && thr != 0;
     const uint32_t tm1 = (uint32_t)(thr - 1);
-    // every row starts a QSPIN block (4 divides L): the bond draws also fill qs
-    const bool qsm = any_bond && (uL & 3u) == 0;
+    // every row starts a QSPIN block (4 divides L): the bond draws also fill qs.
+    // Otherwise qs is drawn apart, or every interior root and representative
+    // draws its own: in 3D, where they are many (L=255, q=3, T_c: 279 us a sweep
+    // against 298; q=2, T=2.0 the same), and in 2D grids of one wave, where the
+    // roots' draws are a chain (L=1001: 35.5 us against 38.2; L=8190: 492 against 485)
+    const bool aligned = (uL & 3u) == 0;
+    const bool qsm = any_bond && (aligned || DIM == 3 || p.ntiles <= FIRST_WAVE_SMS * 5);
     auto ballots = [&](const U4 &u, bool act) {
         return make_uint4(__ballot_sync(FULL, act && below(u.x, tm1)), __ballot_sync(FULL, act && below(u.y, tm1)),
                           __ballot_sync(FULL, act && below(u.z, tm1)), __ballot_sync(FULL, act && below(u.w, tm1)));
@@ -462,7 +467,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                     raw[2] = q2;
                     raw[3] = q3;
                 }
-                if (qsm) {
+                if (aligned) {
                     // lane l: the QSPIN block of sites 4l .. 4l + 3 of each row
                     const U4 s0 = philox4x32_10((g0 >> 2) + lane, klo, khi, STREAM_QSPIN, k0, k1);
                     const U4 s2 = philox4x32_10((g2 >> 2) + lane, klo, khi, STREAM_QSPIN, k0, k1);
@@ -475,7 +480,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 const U4 r = philox4x32_10((g0 >> 1) + 64u, klo, khi, STREAM_BOND, k0, k1);
                 extra = (below(r.x, tm1) ? 1u : 0u) | (below(r.y, tm1) ? 2u : 0u);
             }
-        } else if (qsm) {
+        } else if (aligned) {
             // link l = 3i + d.  Every row starts on a multiple of 4, so its 96
             // links are exactly the 24 Philox blocks from 3 i0 / 4: three blocks
             // for four sites.  Lane 8 c + m draws block 3 m + c (c < 3), so that
@@ -519,6 +524,21 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 const uint32_t rx = __ballot_sync(FULL, bit_of(l)), ry = __ballot_sync(FULL, bit_of(l + 1)),
                                rz = __ballot_sync(FULL, bit_of(l + 2));
                 if (lane == 0) *reinterpret_cast<uint4 *>(&sm.f.s.raw[r][0]) = make_uint4(rx, ry, rz, 0u);
+            }
+        }
+        if (qsm && !aligned) {
+            // rows that start inside a QSPIN block: the blocks of all the warp's rows
+            // dealt to its lanes
+            const int nb = (tw + 3) / 4 + 1;   // blocks of a row
+            for (int i = lane; i < WROWS * nb; i += 32) {
+                const int r = WROWS * warp + i / nb, b = i % nb, y = r % G::TY, z = r / G::TY;
+                if (y >= th || z >= td) continue;
+                const uint32_t i0 = gidx(0, y, z);
+                const uint32_t v = states4(philox4x32_10((i0 >> 2) + (uint32_t)b, klo, khi, STREAM_QSPIN, k0, k1));
+                const int x = 4 * b - (int)(i0 & 3u);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if ((uint32_t)(x + e) < (uint32_t)G::TX) sm.qs[r][x + e] = (uint8_t)(v >> (8 * e));
             }
         }
     }
@@ -680,7 +700,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                             ry = __funnelshift_r(ry, ny, 1);
                         }
                     }
-                } else if (qsm) {
+                } else if (aligned) {
                     // byte c of word w: link 4 c + w of the twelve links of four
                     // sites; direction d of site i is link 3 i + d
                     rx = interleave4x8(__byte_perm(__byte_perm(raw.x, raw.w, 0x0040), __byte_perm(raw.z, raw.y, 0x0061), 0x5410));
