@@ -486,28 +486,35 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
     uint32_t born = 0u, conf = 0u;
     if (rows > 0) {
         const uint32_t le = 0xFFFFFFFFu >> (31 - lane), gt = ~le;
-        int row = y0 * PW + 32 * sx;
-        uint2 hv = *reinterpret_cast<const uint2 *>(&B[y0][2 * sx]);
-        int hd = top_bit(run_heads(hv.x) & le);
-        int lab = row + hd;
-        par[row + lane] = lab;
-        born = hd == lane;
-#pragma unroll 4
-        for (int r = 1; r < rows; ++r) {
-            const uint32_t v = hv.y;   // down bonds from the row above
-            hv = *reinterpret_cast<const uint2 *>(&B[y0 + r][2 * sx]);
-            row += PW;
-            const uint32_t heads = ~(hv.x << 1);
-            hd = top_bit(heads & le);
-            const uint32_t n = heads & gt;                     // heads to the right: the run ends before them
-            const int c = top_bit(v & (n - 1u) & ~n);          // last contact at or left of the run's end
-            const bool has = c >= hd;
-            const int lc = __shfl_sync(0xFFFFFFFFu, lab, c);
-            if (((v >> lane) & 1u) && lab != lc) conf |= 1u << r;
-            if (!has && hd == lane) born |= 1u << r;
-            lab = has ? lc : row + hd;
-            par[row + lane] = lab;
+        int row = y0 * PW + 32 * sx, lab = 0;
+        uint32_t v = 0u;   // down bonds from the row above
+        // four rows at a time: everything that does not need the labels first,
+        // so that the chain from row to row is a shuffle and a select (rows past
+        // the tile's have no bonds)
+        for (int r = 0; r < 32; r += 4) {
+            int hd[4], c[4];
+            uint32_t dn[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint2 hv = *reinterpret_cast<const uint2 *>(&B[y0 + r + q][2 * sx]);
+                const uint32_t heads = run_heads(hv.x);
+                const uint32_t n = heads & gt;                // heads to the right: the run ends before them
+                hd[q] = top_bit(heads & le);
+                c[q] = top_bit(v & (n - 1u) & ~n);            // last contact at or left of the run's end
+                dn[q] = v;
+                v = hv.y;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q, row += PW) {
+                const bool has = c[q] >= hd[q];
+                const int lc = __shfl_sync(0xFFFFFFFFu, lab, c[q]);
+                if (((dn[q] >> lane) & 1u) && lab != lc) conf |= 1u << (r + q);
+                if (!has && hd[q] == lane) born |= 1u << (r + q);
+                lab = has ? lc : row + hd[q];
+                par[row + lane] = lab;
+            }
         }
+        if (rows < 32) born &= (1u << rows) - 1u;
         __syncwarp();
         const int col = y0 * PW + 32 * sx + lane;
         for (; conf; conf &= conf - 1) {

@@ -225,27 +225,35 @@ __device__ __forceinline__ uint32_t tile_label3(volatile int *par, const uint32_
         int labz[4] = {0, 0, 0, 0};
         uint32_t zw[4] = {0u, 0u, 0u, 0u};
         for (int zz = 0; zz < 8 && zb + zz < td; ++zz) {
-            int laby = 0;
-            uint32_t yw = 0u;
+            // first everything of the four rows that does not need the labels
+            // (rows past the tile's have no bonds)
+            int hd[4], py[4], pz[4];
+            uint32_t yw[4], zo[4];
 #pragma unroll
             for (int yy = 0; yy < 4; ++yy) {
-                if (yb + yy >= th) break;
-                const int r = yb + yy + G::TY * (zb + zz), row = r * G::PW;
+                const int r = yb + yy + G::TY * (zb + zz);
                 const uint32_t heads = run_heads(B[r][0]);
-                const int hd = top_bit(heads & le);
                 const uint32_t n = heads & gt, m = (n - 1u) & ~n;   // m: up to the run's end
-                const int py = top_bit(yw & m), pz = top_bit(zw[yy] & m);
-                const int ly = __shfl_sync(FULL, laby, py), lz = __shfl_sync(FULL, labz[yy], pz);
-                const bool hy = py >= hd, hz = pz >= hd;
-                const int lab = hy ? ly : hz ? lz : row + hd;
+                hd[yy] = top_bit(heads & le);
+                yw[yy] = yy > 0 ? B[r - 1][1] : 0u;
+                zo[yy] = zw[yy];
+                py[yy] = top_bit(yw[yy] & m);
+                pz[yy] = top_bit(zo[yy] & m);
+                zw[yy] = B[r][2];
+            }
+            int laby = 0;
+#pragma unroll
+            for (int yy = 0; yy < 4; ++yy) {
+                const int row = (yb + yy + G::TY * (zb + zz)) * G::PW;
+                const int ly = __shfl_sync(FULL, laby, py[yy]), lz = __shfl_sync(FULL, labz[yy], pz[yy]);
+                const bool hy = py[yy] >= hd[yy], hz = pz[yy] >= hd[yy];
+                const int lab = hy ? ly : hz ? lz : row + hd[yy];
                 const uint32_t bit = 1u << (4 * zz + yy);
-                if (((yw >> lane) & 1u) && laby != lab) cy |= bit;
-                if (((zw[yy] >> lane) & 1u) && labz[yy] != lab) cz |= bit;
-                if (!hy && !hz && hd == lane) born |= bit;
+                if (((yw[yy] >> lane) & 1u) && laby != lab) cy |= bit;
+                if (((zo[yy] >> lane) & 1u) && labz[yy] != lab) cz |= bit;
+                if (!hy && !hz && hd[yy] == lane && yb + yy < th) born |= bit;
                 par[row + lane] = lab;
                 laby = labz[yy] = lab;
-                yw = B[r][1];
-                zw[yy] = B[r][2];
             }
         }
     }
