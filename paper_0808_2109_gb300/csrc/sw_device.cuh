@@ -1798,19 +1798,55 @@ static __global__ void k_call_begin(const Replica R, Replica *rep, int32_t *jbas
     }
 }
 
-// A served lattice's initial device state in one launch: the hot start, zero
-// observables (n_obs 8-byte words) and the threshold word.
-static __global__ void k_job_init(uint8_t *spin, int64_t N, uint32_t key0, uint32_t key1,
-                                  unsigned long long *obs, int64_t n_obs, uint64_t *thr_dev, uint64_t thr)
+// Served lattices' initial device state, all of a lane's newly admitted jobs in
+// one launch (blockIdx.y = job): the hot start, zero observables, the threshold
+// word and zeroed PCC scratch.
+struct JobInit {
+    uint8_t *spin;
+    int64_t N;
+    uint32_t key0, key1;
+    unsigned long long *obs;
+    int64_t n_obs;         // 8-byte words
+    uint64_t *thr_dev;
+    uint64_t thr;
+    uint32_t *zero;        // PCC scratch, null without
+    int64_t n_zero;        // 4-byte words
+};
+__device__ __forceinline__ void job_init(const JobInit &q)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) {
-        const U4 r = philox4x32_10((uint32_t)(i >> 7), 0u, 0u, STREAM_INIT, key0, key1);
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, di = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < q.N; i += di) {
+        const U4 r = philox4x32_10((uint32_t)(i >> 7), 0u, 0u, STREAM_INIT, q.key0, q.key1);
         const int bit = (int)(i & 127);
-        spin[i] = (uint8_t)((u4_word(r, bit >> 5) >> (bit & 31)) & 1u);
+        q.spin[i] = (uint8_t)((u4_word(r, bit >> 5) >> (bit & 31)) & 1u);
     }
-    if (i < n_obs) obs[i] = 0ull;
-    if (i == 0) *thr_dev = thr;
+    for (int64_t i = i0; i < q.n_obs; i += di) q.obs[i] = 0ull;
+    for (int64_t i = i0; i < q.n_zero; i += di) q.zero[i] = 0u;
+    if (i0 == 0) *q.thr_dev = q.thr;
+}
+static __global__ void k_job_init(const JobInit q)   // one job
+{
+    job_init(q);
+}
+static __global__ void k_jobs_init(const JobInit *jobs)
+{
+    job_init(jobs[blockIdx.y]);
+}
+
+// Finished jobs' observables and thresholds side by side (blockIdx.y = job), for
+// one copy to the host.
+struct JobGather {
+    const unsigned long long *obs;
+    int64_t n_obs;                  // 8-byte words
+    const uint64_t *thr_dev;
+    unsigned long long *out;        // n_obs words, then the threshold
+};
+static __global__ void k_jobs_gather(const JobGather *jobs)
+{
+    const JobGather q = jobs[blockIdx.y];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < q.n_obs; i += (int64_t)gridDim.x * blockDim.x)
+        q.out[i] = q.obs[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0) q.out[q.n_obs] = *q.thr_dev;
 }
 
 // Integer ceiling of the bond step: nblocks BOND-stream Philox blocks

@@ -128,14 +128,27 @@ cudaError_t enqueue_hot_start(uint8_t *spin, int64_t N, uint64_t seed, cudaStrea
     return cudaGetLastError();
 }
 
-cudaError_t enqueue_job_init(uint8_t *spin, int64_t N, uint64_t seed, void *obs, int64_t obs_bytes, uint64_t *thr_dev,
-                             uint64_t thr, cudaStream_t st)
+// Blocks a job: enough for `most` items, about 16K over all jobs.
+static unsigned job_blocks(int64_t most, int n)
 {
-    const int64_t n_obs = obs_bytes / 8;
-    const int64_t n = std::max(N, n_obs);
-    k_job_init<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(spin, N, (uint32_t)seed, (uint32_t)(seed >> 32),
-                                                            static_cast<unsigned long long *>(obs), n_obs, thr_dev,
-                                                            thr);
+    return (unsigned)std::min<int64_t>(std::max<int64_t>((most + 255) / 256, 1), std::max(1, 16384 / n));
+}
+
+cudaError_t enqueue_job_init(const JobInit &job, int64_t most, cudaStream_t st)
+{
+    k_job_init<<<job_blocks(most, 1), 256, 0, st>>>(job);
+    return cudaGetLastError();
+}
+
+cudaError_t enqueue_jobs_init(const JobInit *jobs_dev, int n, int64_t most, cudaStream_t st)
+{
+    k_jobs_init<<<dim3(job_blocks(most, n), (unsigned)n), 256, 0, st>>>(jobs_dev);
+    return cudaGetLastError();
+}
+
+cudaError_t enqueue_jobs_gather(const JobGather *jobs_dev, int n, int64_t most, cudaStream_t st)
+{
+    k_jobs_gather<<<dim3(job_blocks(most, n), (unsigned)n), 256, 0, st>>>(jobs_dev);
     return cudaGetLastError();
 }
 

@@ -30,9 +30,12 @@ __attribute__((visibility("hidden"))) cudaError_t enqueue_groups(int TH, SweepAr
                                                                  bool last, cudaStream_t st);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_hot_start(uint8_t *spin, int64_t N, uint64_t seed,
                                                                     cudaStream_t st);
-__attribute__((visibility("hidden"))) cudaError_t enqueue_job_init(uint8_t *spin, int64_t N, uint64_t seed, void *obs,
-                                                                   int64_t obs_bytes, uint64_t *thr_dev, uint64_t thr,
-                                                                   cudaStream_t st);
+// One job, and n <= 65535 jobs of at most `most` items each (one launch).
+__attribute__((visibility("hidden"))) cudaError_t enqueue_job_init(const JobInit &job, int64_t most, cudaStream_t st);
+__attribute__((visibility("hidden"))) cudaError_t enqueue_jobs_init(const JobInit *jobs_dev, int n, int64_t most,
+                                                                    cudaStream_t st);
+__attribute__((visibility("hidden"))) cudaError_t enqueue_jobs_gather(const JobGather *jobs_dev, int n, int64_t most,
+                                                                      cudaStream_t st);
 
 // Launches kernel k; chained: as a dependent of the kernel before it in the
 // stream, which it may overlap (chain_next / chain_wait in sw_device.cuh).  The

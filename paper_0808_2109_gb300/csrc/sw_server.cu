@@ -50,6 +50,13 @@ int th_of_lane(int l) { return (l & 3) == 0 ? 32 : (l & 3) == 1 ? 64 : (l & 3) =
 
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
+// A block that several jobs share: jobs of one lane admitted together with the
+// same number of sweeps, which therefore finish together.
+struct Slab {
+    void *p = nullptr;
+    int refs = 0;
+};
+
 struct Job {
     uint64_t id = 0;
     sw_job spec{};
@@ -60,6 +67,7 @@ struct Job {
     Clock::time_point t_submit, t_admit;
     // device state: every buffer is carved from one block
     void *block = nullptr;
+    Slab *slab = nullptr;   // block lies in it
     uint8_t *spin = nullptr;
     int32_t *label = nullptr;
     uint16_t *code = nullptr;
@@ -68,6 +76,8 @@ struct Job {
     int32_t *cid = nullptr, *ncand = nullptr;
     uint64_t *thr_dev = nullptr;
     DevObs *obs = nullptr;
+    uint32_t *pcc_zero = nullptr;   // PCC scratch that starts zeroed
+    int64_t pcc_words = 0;
     int32_t *psize = nullptr, *csize = nullptr;   // SW_FLAG_CSIZE
     unsigned long long *nlink = nullptr;          // SW_FLAG_WIND
     // placement
@@ -133,6 +143,8 @@ struct Lane {
     Replica *reps_dev = nullptr;
     int32_t *tile_rep_dev = nullptr;
     int32_t *jbase_dev = nullptr;
+    unsigned char *ws = nullptr;   // workspace (tables and gathered records)
+    size_t ws_cap = 0;
     std::vector<Replica> reps_host;
     std::vector<int32_t> tile_rep_host;
     std::vector<Job *> slot_job;
@@ -172,23 +184,63 @@ namespace {
 
 void free_job_device(Job *j, cudaStream_t st)
 {
-    if (j->block) cudaFreeAsync(j->block, st);
+    if (j->slab) {
+        if (--j->slab->refs == 0) {
+            cudaFreeAsync(j->slab->p, st);
+            delete j->slab;
+        }
+        j->slab = nullptr;
+    } else if (j->block) {
+        cudaFreeAsync(j->block, st);
+    }
     j->block = nullptr;
 }
 
-// Device state of a newly admitted job: one stream-ordered block for all its
-// buffers, zeroed PCC scratch, and one kernel for the hot start, the
-// observables and the threshold.
+// One allocation for each group of jobs to admit that share a lane and a number
+// of sweeps (at most SLAB_MAX bytes each; 512 allocations of their own took 3 of
+// the 30 ms of a batch).  Jobs that get no share allocate their own block.
+constexpr size_t SLAB_MAX = (size_t)1 << 30;
+void share_blocks(sw_server *s, const std::vector<Job *> &admit)
+{
+    std::map<std::pair<int, int>, std::vector<Job *>> groups;
+    for (Job *j : admit) groups[{j->lane, j->spec.nsweeps}].push_back(j);
+    for (auto &g : groups) {
+        const std::vector<Job *> &v = g.second;
+        for (size_t at = 0; at < v.size();) {
+            size_t end = at, bytes = 0;
+            while (end < v.size() && (end == at || bytes + v[end]->bytes <= SLAB_MAX)) bytes += v[end++]->bytes;
+            void *p = nullptr;
+            if (end - at > 1 && cudaMallocAsync(&p, bytes, s->lanes[g.first.first].stream) == cudaSuccess) {
+                Slab *slab = new Slab{p, (int)(end - at)};
+                size_t off = 0;
+                for (size_t i = at; i < end; ++i) {
+                    v[i]->slab = slab;
+                    v[i]->block = static_cast<unsigned char *>(p) + off;
+                    off += v[i]->bytes;
+                }
+            } else {
+                cudaGetLastError();
+            }
+            at = end;
+        }
+    }
+}
+
+// Device memory of a newly admitted job: its share of a slab or one
+// stream-ordered block for all its buffers (their first contents come with those of the lane's other new jobs,
+// init_jobs).
 cudaError_t job_alloc(Job *j, cudaStream_t st)
 {
-    const size_t N = (size_t)j->spec.L * j->spec.L;
     const bool csz = (j->spec.flags & SW_FLAG_CSIZE) != 0;
     const bool wnd = (j->spec.flags & SW_FLAG_WIND) != 0;
     const JobLayout o = job_layout(j->spec.L, j->TH, j->spec.nsweeps, j->pcc, csz, wnd);
-    cudaError_t e = sw_inject_alloc_failure() ? cudaErrorMemoryAllocation : cudaMallocAsync(&j->block, o.total, st);
-    if (e != cudaSuccess) {
-        j->block = nullptr;
-        return e;
+    if (sw_inject_alloc_failure()) return cudaErrorMemoryAllocation;
+    if (!j->block) {
+        const cudaError_t e = cudaMallocAsync(&j->block, o.total, st);
+        if (e != cudaSuccess) {
+            j->block = nullptr;
+            return e;
+        }
     }
     unsigned char *b = static_cast<unsigned char *>(j->block);
     j->spin = b + o.spin;
@@ -210,10 +262,71 @@ cudaError_t job_alloc(Job *j, cudaStream_t st)
         j->cid = reinterpret_cast<int32_t *>(b + o.cid);
         j->ncand = reinterpret_cast<int32_t *>(b + o.ncand);
         j->cov = reinterpret_cast<uint32_t *>(b + o.cov);
-        if ((e = cudaMemsetAsync(b + o.pmask, 0, o.pcc_end - o.pmask, st)) != cudaSuccess) return e;
+        j->pcc_zero = reinterpret_cast<uint32_t *>(b + o.pmask);
+        j->pcc_words = (int64_t)((o.pcc_end - o.pmask) / 4);
     }
-    return enqueue_job_init(j->spin, (int64_t)N, j->spec.seed, j->obs, (int64_t)j->spec.nsweeps * sizeof(DevObs),
-                            j->thr_dev, j->thr, st);
+    return cudaSuccess;
+}
+
+constexpr int JOBS_PER_LAUNCH = 32768;   // jobs of one init or gather launch (grid y)
+
+// The lane's workspace with room for `bytes` (used in the order of its stream,
+// given back with the server); null beyond WORKSPACE_MAX or without memory.
+constexpr size_t WORKSPACE_MAX = (size_t)64 << 20;
+unsigned char *lane_workspace(Lane &ln, size_t bytes)
+{
+    if (bytes <= ln.ws_cap) return ln.ws;
+    if (bytes > WORKSPACE_MAX) return nullptr;
+    std::lock_guard<std::mutex> lk(sw_capture_mutex());
+    if (ln.ws) cudaFree(ln.ws);   // waits for the work that uses it
+    ln.ws = nullptr;
+    ln.ws_cap = 0;
+    size_t cap = 1 << 16;
+    while (cap < bytes) cap *= 2;
+    if (cudaMalloc(&ln.ws, cap) != cudaSuccess) {
+        cudaGetLastError();
+        ln.ws = nullptr;
+        return nullptr;
+    }
+    ln.ws_cap = cap;
+    return ln.ws;
+}
+
+// First contents of the new jobs of a lane, in one launch (job by job where there
+// is no memory for their table).
+cudaError_t init_jobs(const std::vector<Job *> &jobs, Lane &ln)
+{
+    const cudaStream_t st = ln.stream;
+    for (size_t at = 0; at < jobs.size(); at += JOBS_PER_LAUNCH) {
+        const size_t n = std::min<size_t>(jobs.size() - at, JOBS_PER_LAUNCH);
+        std::vector<JobInit> table(n);
+        int64_t most = 0;
+        for (size_t i = 0; i < n; ++i) {
+            const Job *j = jobs[at + i];
+            JobInit &q = table[i];
+            q.spin = j->spin;
+            q.N = (int64_t)j->spec.L * j->spec.L;
+            q.key0 = (uint32_t)j->spec.seed;
+            q.key1 = (uint32_t)(j->spec.seed >> 32);
+            q.obs = reinterpret_cast<unsigned long long *>(j->obs);
+            q.n_obs = (int64_t)j->spec.nsweeps * (int64_t)(sizeof(DevObs) / 8);
+            q.thr_dev = j->thr_dev;
+            q.thr = j->thr;
+            q.zero = j->pcc_zero;
+            q.n_zero = j->pcc_words;
+            most = std::max({most, q.N, q.n_obs, q.n_zero});
+        }
+        unsigned char *ws = n > 1 ? lane_workspace(ln, n * sizeof(JobInit)) : nullptr;
+        cudaError_t e = cudaSuccess;
+        if (ws) {
+            e = cudaMemcpyAsync(ws, table.data(), n * sizeof(JobInit), cudaMemcpyHostToDevice, st);
+            if (e == cudaSuccess) e = enqueue_jobs_init(reinterpret_cast<const JobInit *>(ws), (int)n, most, st);
+        } else {
+            for (size_t i = 0; i < n && e == cudaSuccess; ++i) e = enqueue_job_init(table[i], most, st);
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 Replica replica_of(const Job *j)
@@ -398,25 +511,62 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
         heap.resize(need);
         stage = heap.data();
     }
+    // every lane's finished jobs side by side in device memory, then one copy; job
+    // by job where there is no memory for that
     std::vector<size_t> at(done.size());
     std::vector<cudaError_t> err(done.size(), cudaSuccess);
     bool used[N_LANES] = {};
     size_t off = 0;
-    for (size_t i = 0; i < done.size(); ++i) {
-        Job *j = done[i];
-        const cudaStream_t st = s->lanes[j->lane].stream;
-        used[j->lane] = true;
-        at[i] = off;
-        const size_t nobs = (size_t)j->spec.nsweeps, N = (size_t)j->spec.L * j->spec.L;
-        cudaError_t e = cudaMemcpyAsync(stage + off, j->obs, nobs * sizeof(DevObs), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && j->pcc)
-            e = cudaMemcpyAsync(stage + off + nobs, j->thr_dev, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && j->spec.spins_out)
-            e = cudaMemcpyAsync(j->spec.spins_out, j->spin, N, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && j->spec.labels_out)
-            e = cudaMemcpyAsync(j->spec.labels_out, j->label, N * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-        err[i] = e;
-        off += nobs + 1;
+    for (int l = 0; l < N_LANES; ++l) {
+        const cudaStream_t st = s->lanes[l].stream;
+        std::vector<size_t> mine;
+        const size_t off0 = off;
+        for (size_t i = 0; i < done.size(); ++i)
+            if (done[i]->lane == l) {
+                mine.push_back(i);
+                at[i] = off;
+                off += (size_t)done[i]->spec.nsweeps + 1;
+            }
+        if (mine.empty()) continue;
+        used[l] = true;
+        // workspace: the jobs' table, then their records
+        const size_t table_bytes = round256(mine.size() * sizeof(JobGather)), side_bytes = (off - off0) * sizeof(DevObs);
+        unsigned char *ws = mine.size() > 1 && mine.size() <= (size_t)JOBS_PER_LAUNCH
+                                ? lane_workspace(s->lanes[l], table_bytes + side_bytes) : nullptr;
+        if (ws) {
+            std::vector<JobGather> table;
+            int64_t most = 0;
+            for (size_t i : mine) {
+                const Job *j = done[i];
+                const int64_t words = (int64_t)j->spec.nsweeps * (int64_t)(sizeof(DevObs) / 8);
+                table.push_back(JobGather{reinterpret_cast<const unsigned long long *>(j->obs), words, j->thr_dev,
+                                          reinterpret_cast<unsigned long long *>(ws + table_bytes +
+                                                                                 (at[i] - off0) * sizeof(DevObs))});
+                most = std::max(most, words);
+            }
+            cudaError_t e = cudaMemcpyAsync(ws, table.data(), table.size() * sizeof(JobGather), cudaMemcpyHostToDevice, st);
+            if (e == cudaSuccess)
+                e = enqueue_jobs_gather(reinterpret_cast<const JobGather *>(ws), (int)mine.size(), most, st);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(stage + off0, ws + table_bytes, side_bytes, cudaMemcpyDeviceToHost, st);
+            for (size_t i : mine) err[i] = e;
+        } else {
+            for (size_t i : mine) {
+                const Job *j = done[i];
+                const size_t nobs = (size_t)j->spec.nsweeps;
+                err[i] = cudaMemcpyAsync(stage + at[i], j->obs, nobs * sizeof(DevObs), cudaMemcpyDeviceToHost, st);
+                if (err[i] == cudaSuccess)
+                    err[i] = cudaMemcpyAsync(stage + at[i] + nobs, j->thr_dev, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
+            }
+        }
+        for (size_t i : mine) {
+            const Job *j = done[i];
+            const size_t N = (size_t)j->spec.L * j->spec.L;
+            if (err[i] == cudaSuccess && j->spec.spins_out)
+                err[i] = cudaMemcpyAsync(j->spec.spins_out, j->spin, N, cudaMemcpyDeviceToHost, st);
+            if (err[i] == cudaSuccess && j->spec.labels_out)
+                err[i] = cudaMemcpyAsync(j->spec.labels_out, j->label, N * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+        }
     }
     cudaError_t lane_err[N_LANES] = {};
     for (int l = 0; l < N_LANES; ++l)
@@ -488,8 +638,10 @@ void worker_main(sw_server *s)
             }
             s->stats.pending = (int64_t)s->pending.size();
         }
+        std::vector<Job *> fresh[N_LANES];   // admitted, first contents to come
+        for (Job *j : admit) j->lane = lane_of_th(j->TH) + ((j->pcc || j->spec.flags) ? 4 : 0);
+        share_blocks(s, admit);
         for (Job *j : admit) {
-            j->lane = lane_of_th(j->TH) + ((j->pcc || j->spec.flags) ? 4 : 0);
             Lane &ln = s->lanes[j->lane];
             j->t_admit = Clock::now();
             j->jstart = s->launch_index;
@@ -522,10 +674,17 @@ void worker_main(sw_server *s)
             ln.reps_host[j->slot] = replica_of(j);
             ln.active += 1;
             ln.dirty = true;
+            fresh[j->lane].push_back(j);
             s->running.push_back(j);
             std::lock_guard<std::mutex> lk(s->mu);
             s->stats.admitted += 1;
         }
+        for (int l = 0; l < N_LANES; ++l)
+            if (!fresh[l].empty() && init_jobs(fresh[l], s->lanes[l]) != cudaSuccess) {
+                cudaGetLastError();
+                std::lock_guard<std::mutex> lk(s->mu);
+                s->worker_error = SW_ERR_CUDA;
+            }
         // ---- one step of every busy lane
         nvtxRangePushA("server step");
         bool any = false;
@@ -649,6 +808,7 @@ int sw_server_destroy(sw_server *s)
         if (ln.reps_dev) cudaFree(ln.reps_dev);
         if (ln.tile_rep_dev) cudaFree(ln.tile_rep_dev);
         if (ln.jbase_dev) cudaFree(ln.jbase_dev);
+        if (ln.ws) cudaFree(ln.ws);
         if (ln.stream) cudaStreamDestroy(ln.stream);
     }
     if (s->stage) cudaFreeHost(s->stage);
