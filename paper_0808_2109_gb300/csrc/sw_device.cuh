@@ -636,6 +636,113 @@ __device__ __forceinline__ void warp_add64(unsigned long long *dst, unsigned lon
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
 }
 
+// ---------------------------------------------------------- a tile's draws
+// Link l = 2i + d draws word (l mod 4) of Philox(l/4, k, BOND), i.e. sites 2m
+// and 2m+1 share block m.  Warp w draws rows 8w .. 8w+7, two at a time (four
+// independent blocks in flight per lane): lane m the m-th and the (32+m)-th
+// block of a row, counted from the one that holds the row's first site (gbase:
+// the tile's; uL: sites from row to row).  Four ballots per 32 blocks are the
+// row's below-threshold bits with even and odd positions apart: x and z the
+// right links, y and w the down links, left in row y of `raw`.  The thread that
+// owns a word interleaves them (13 operations a word against a shuffle, a shift
+// and two ballots a word for every lane of the warp).  An odd first site is the
+// second one of its row's first block, so the row's 128 sites reach into a 65th
+// block: lane r draws it for row r and returns its first two words' bits.
+__device__ __forceinline__ uint32_t draw_rows(uint32_t (*raw_rows)[2 * TWW], const SweepPhilox &ph, uint32_t tm1,
+                                              uint32_t gbase, uint32_t uL, int th, int tw)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto ballots = [&](const U4 &r) {
+        return make_uint4(__ballot_sync(0xFFFFFFFFu, below(r.x, tm1)), __ballot_sync(0xFFFFFFFFu, below(r.y, tm1)),
+                          __ballot_sync(0xFFFFFFFFu, below(r.z, tm1)), __ballot_sync(0xFFFFFFFFu, below(r.w, tm1)));
+    };
+    const int rows = min(8, th - 8 * warp);
+    uint4 *raw = reinterpret_cast<uint4 *>(&raw_rows[8 * warp][0]);
+    uint32_t b = gbase + (uint32_t)(8 * warp) * uL;   // the row's first site
+    if (tw > 64) {
+        for (int i = 0; i < rows; i += 2, b += 2u * uL, raw += 4) {
+            const uint32_t b0 = (b >> 1) + lane, b2 = ((b + uL) >> 1) + lane;
+            const U4 r0 = sweep_block(ph, b0, STREAM_BOND), r1 = sweep_block(ph, b0 + 32, STREAM_BOND);
+            const U4 r2 = sweep_block(ph, b2, STREAM_BOND), r3 = sweep_block(ph, b2 + 32, STREAM_BOND);
+            const uint4 q0 = ballots(r0), q1 = ballots(r1), q2 = ballots(r2), q3 = ballots(r3);
+            if (lane == 0) {
+                raw[0] = q0;
+                raw[1] = q1;
+                raw[2] = q2;
+                raw[3] = q3;
+            }
+        }
+    } else {
+        // blocks 32 .. 63 of a row have no sites in the tile
+        for (int i = 0; i < rows; i += 2, b += 2u * uL, raw += 4) {
+            const U4 r0 = sweep_block(ph, (b >> 1) + lane, STREAM_BOND);
+            const U4 r2 = sweep_block(ph, ((b + uL) >> 1) + lane, STREAM_BOND);
+            const uint4 q0 = ballots(r0), q2 = ballots(r2);
+            if (lane == 0) {
+                raw[0] = q0;
+                raw[2] = q2;
+            }
+        }
+    }
+    if (!((uL | gbase) & 1u)) return 0u;
+    const uint32_t g0 = gbase + (uint32_t)(8 * warp + (lane & 7)) * uL;
+    const U4 r = sweep_block(ph, (g0 >> 1) + 64u, STREAM_BOND);
+    return (below(r.x, tm1) ? 1u : 0u) | (below(r.y, tm1) ? 2u : 0u);
+}
+
+// The links drawn below the threshold of the thread's word (row tid / 4, word
+// tid mod 4): right links rh, down links rv.  All lanes of the warp.
+__device__ __forceinline__ void draw_words(const uint32_t (*raw_rows)[2 * TWW], uint32_t extra, uint32_t gbase,
+                                           uint32_t uL, uint32_t &rh, uint32_t &rv)
+{
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 2, wc = threadIdx.x & 3;
+    const uint4 raw = *reinterpret_cast<const uint4 *>(&raw_rows[wy][4 * (wc >> 1)]);
+    rh = interleave16(raw.x, raw.z, wc & 1);
+    rv = interleave16(raw.y, raw.w, wc & 1);
+    if (!((uL | gbase) & 1u)) return;
+    // rows that start on an odd site are one site ahead of their blocks
+    const uint32_t ex = __shfl_sync(0xFFFFFFFFu, extra, lane >> 2);
+    uint32_t nh = __shfl_down_sync(0xFFFFFFFFu, rh, 1), nv = __shfl_down_sync(0xFFFFFFFFu, rv, 1);
+    if (wc == TWW - 1) {
+        nh = ex;
+        nv = ex >> 1;
+    }
+    if ((gbase + (uint32_t)wy * uL) & 1u) {
+        rh = __funnelshift_r(rh, nh, 1);
+        rv = __funnelshift_r(rv, nv, 1);
+    }
+}
+
+// The SPIN-stream bits of a row's 128 sites from global site g0 on: bit (g mod
+// 128) of Philox(g / 128, k, SPIN) for site g, so the row spans the two blocks
+// from the one holding its first site.
+__device__ __forceinline__ void spin_row(const SweepPhilox &ph, uint32_t g0, uint32_t *out)
+{
+    const uint32_t pos = g0 & 127u;
+    const U4 r0 = sweep_block(ph, g0 >> 7, STREAM_SPIN);
+    U4 r1 = r0;
+    if (pos) r1 = sweep_block(ph, (g0 >> 7) + 1, STREAM_SPIN);
+    // the 8 words from the first one the row needs: words pos/32 .. pos/32 + 4
+    uint32_t w[5];
+    switch (pos >> 5) {
+    case 0: w[0] = r0.x; w[1] = r0.y; w[2] = r0.z; w[3] = r0.w; w[4] = r1.x; break;
+    case 1: w[0] = r0.y; w[1] = r0.z; w[2] = r0.w; w[3] = r1.x; w[4] = r1.y; break;
+    case 2: w[0] = r0.z; w[1] = r0.w; w[2] = r1.x; w[3] = r1.y; w[4] = r1.z; break;
+    default: w[0] = r0.w; w[1] = r1.x; w[2] = r1.y; w[3] = r1.z; w[4] = r1.w; break;
+    }
+#pragma unroll
+    for (int c = 0; c < TWW; ++c) out[c] = __funnelshift_r(w[c], w[c + 1], pos & 31u);
+}
+
+// A byte of a warp's eight rows from bits 4 r of e (row r).
+__device__ __forceinline__ uint32_t rows_byte(uint32_t e)
+{
+    e &= 0x11111111u;
+    e = (e | (e >> 3)) & 0x03030303u;
+    e = (e | (e >> 6)) & 0x000F000Fu;
+    return (e | (e >> 12)) & 0xFFu;
+}
+
 // ------------------------------------------------------------ shared layout
 template <int TH>
 struct TileSmem {
@@ -750,62 +857,12 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     if (tid < 4) sm.acc[tid] = 0;
     if ((F & FEAT_CSIZE) && tid < 2) sm.acc_c2[tid] = 0ull;
 
-    // ---- Step 1 (Sec. I) of sweep k, its random part: link l = 2i + d draws
-    // word (l mod 4) of Philox(l/4, k, BOND), i.e. sites 2m and 2m+1 share
-    // block m.  Warp w draws rows 8w .. 8w+7, two at a time (four independent
-    // blocks in flight per lane): lane m the m-th and the (32+m)-th block of a
-    // row, counted from the one that holds the row's first site.  Four ballots
-    // per 32 blocks are the row's below-threshold bits with even and odd
-    // positions apart: x and z the right links, y and w the down links.  The
-    // thread that owns a word interleaves them (13 operations a word against
-    // a shuffle, a shift and two ballots a word for every lane of the warp).
+    // ---- Step 1 (Sec. I) of sweep k, its random part
     const uint64_t k = R.sweep0 + (uint64_t)j;
     const uint64_t thr = (F & FEAT_PCC) && (R.flags & RF_PCC) ? *R.thr_dev : R.thr;
     const SweepPhilox ph = sweep_philox((uint32_t)k, (uint32_t)(k >> 32), R.key0, R.key1);
     const bool any_bond = start && thr != 0;      // t = 0: P = 0, nothing bonds
-    // an odd first site is the second one of its row's first block, so the
-    // row's 128 sites reach into a 65th block: lane r draws it for row r
-    uint32_t extra = 0u;
-    if (any_bond) {
-        const uint32_t tm1 = (uint32_t)(thr - 1);     // t in [1, 2^32] -> t - 1 fits 32 bits
-        auto ballots = [&](const U4 &r) {
-            return make_uint4(__ballot_sync(0xFFFFFFFFu, below(r.x, tm1)), __ballot_sync(0xFFFFFFFFu, below(r.y, tm1)),
-                              __ballot_sync(0xFFFFFFFFu, below(r.z, tm1)), __ballot_sync(0xFFFFFFFFu, below(r.w, tm1)));
-        };
-        const int rows = min(8, t.th - 8 * warp);
-        uint4 *raw = reinterpret_cast<uint4 *>(&sm.b[8 * warp][0]);
-        uint32_t b = gbase + (uint32_t)(8 * warp) * uL;   // the row's first site
-        if (t.tw > 64) {
-            for (int i = 0; i < rows; i += 2, b += 2u * uL, raw += 4) {
-                const uint32_t b0 = (b >> 1) + lane, b2 = ((b + uL) >> 1) + lane;
-                const U4 r0 = sweep_block(ph, b0, STREAM_BOND), r1 = sweep_block(ph, b0 + 32, STREAM_BOND);
-                const U4 r2 = sweep_block(ph, b2, STREAM_BOND), r3 = sweep_block(ph, b2 + 32, STREAM_BOND);
-                const uint4 q0 = ballots(r0), q1 = ballots(r1), q2 = ballots(r2), q3 = ballots(r3);
-                if (lane == 0) {
-                    raw[0] = q0;
-                    raw[1] = q1;
-                    raw[2] = q2;
-                    raw[3] = q3;
-                }
-            }
-        } else {
-            // blocks 32 .. 63 of a row have no sites in the tile
-            for (int i = 0; i < rows; i += 2, b += 2u * uL, raw += 4) {
-                const U4 r0 = sweep_block(ph, (b >> 1) + lane, STREAM_BOND);
-                const U4 r2 = sweep_block(ph, ((b + uL) >> 1) + lane, STREAM_BOND);
-                const uint4 q0 = ballots(r0), q2 = ballots(r2);
-                if (lane == 0) {
-                    raw[0] = q0;
-                    raw[2] = q2;
-                }
-            }
-        }
-        if ((uL | gbase) & 1u) {
-            const uint32_t g0 = gbase + (uint32_t)(8 * warp + (lane & 7)) * uL;
-            const U4 r = sweep_block(ph, (g0 >> 1) + 64u, STREAM_BOND);
-            extra = (below(r.x, tm1) ? 1u : 0u) | (below(r.y, tm1) ? 2u : 0u);
-        }
-    }
+    const uint32_t extra = any_bond ? draw_rows(sm.b, ph, (uint32_t)(thr - 1), gbase, uL, t.th, t.tw) : 0u;
 
     if (early) finish_loads();
     if (fin) {
@@ -935,35 +992,14 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         }
         if (start) {
             uint32_t rh = 0u, rv = 0u;   // links drawn below the threshold
-            if (any_bond) {
-                const uint4 raw = *reinterpret_cast<const uint4 *>(&sm.b[wy][4 * (wc >> 1)]);
-                rh = interleave16(raw.x, raw.z, wc & 1);
-                rv = interleave16(raw.y, raw.w, wc & 1);
-                if ((uL | gbase) & 1u) {
-                    // rows that start on an odd site are one site ahead of their blocks
-                    const uint32_t ex = __shfl_sync(0xFFFFFFFFu, extra, lane >> 2);
-                    uint32_t nh = __shfl_down_sync(0xFFFFFFFFu, rh, 1), nv = __shfl_down_sync(0xFFFFFFFFu, rv, 1);
-                    if (wc == TWW - 1) {
-                        nh = ex;
-                        nv = ex >> 1;
-                    }
-                    if ((gbase + (uint32_t)wy * uL) & 1u) {
-                        rh = __funnelshift_r(rh, nh, 1);
-                        rv = __funnelshift_r(rv, nv, 1);
-                    }
-                }
-            }
+            if (any_bond) draw_words(sm.b, extra, gbase, uL, rh, rv);
             const uint32_t h = rh & eqr, v = rv & eqd;
             const int nb = __reduce_add_sync(0xFFFFFFFFu, __popc(h) + __popc(v));
             if (lane == 0) atomicAdd(&sm.acc[2], nb);
             // crossing bonds: right edge (the last column's bit of every row, a
             // warp's eight rows a byte), bottom edge (the last row's down links)
             {
-                uint32_t e = __ballot_sync(0xFFFFFFFFu, wc == last_c && ((h >> last_b) & 1u)) >> last_c;
-                e &= 0x11111111u;            // bit 4 r: row r
-                e = (e | (e >> 3)) & 0x03030303u;
-                e = (e | (e >> 6)) & 0x000F000Fu;
-                e = (e | (e >> 12)) & 0xFFu;
+                const uint32_t e = rows_byte(__ballot_sync(0xFFFFFFFFu, wc == last_c && ((h >> last_b) & 1u)) >> last_c);
                 uint32_t *cross = R.cross + (size_t)t.lt * CROSS_WORDS;
                 if (lane == 0) reinterpret_cast<uint8_t *>(cross)[warp] = (uint8_t)e;
                 if (wy == t.th - 1) cross[TWW + wc] = v;
@@ -981,28 +1017,8 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     }
     if (start) {
         // The SPIN-stream bit of every site of the tile, for the clusters that end
-        // inside it (Sec. I step 3: one new random spin per cluster): bit (g mod
-        // 128) of Philox(g / 128, k, SPIN) for a site of global index g.  A row's
-        // 128 sites span the two blocks from the one holding its first site; one
-        // thread per row draws them and keeps the row's 128 bits.
-        if (tid < t.th) {
-            const int y = tid;
-            const uint32_t g0 = gbase + (uint32_t)y * uL;
-            const uint32_t pos = g0 & 127u;
-            const U4 r0 = sweep_block(ph, g0 >> 7, STREAM_SPIN);
-            U4 r1 = r0;
-            if (pos) r1 = sweep_block(ph, (g0 >> 7) + 1, STREAM_SPIN);
-            // the 8 words from the first one the row needs: words pos/32 .. pos/32 + 4
-            uint32_t w[5];
-            switch (pos >> 5) {
-            case 0: w[0] = r0.x; w[1] = r0.y; w[2] = r0.z; w[3] = r0.w; w[4] = r1.x; break;
-            case 1: w[0] = r0.y; w[1] = r0.z; w[2] = r0.w; w[3] = r1.x; w[4] = r1.y; break;
-            case 2: w[0] = r0.z; w[1] = r0.w; w[2] = r1.x; w[3] = r1.y; w[4] = r1.z; break;
-            default: w[0] = r0.w; w[1] = r1.x; w[2] = r1.y; w[3] = r1.z; w[4] = r1.w; break;
-            }
-#pragma unroll
-            for (int c = 0; c < TWW; ++c) sm.u.spb[y][c] = __funnelshift_r(w[c], w[c + 1], pos & 31u);
-        }
+        // inside it (Sec. I step 3: one new random spin per cluster), one thread a row.
+        if (tid < t.th) spin_row(ph, gbase + (uint32_t)tid * uL, sm.u.spb[tid]);
         if (ext) {
             for (int q = tid; q < S * 8; q += NT) (&sm.pm[0][0])[q] = 0u;
             // the tiles together clear what the last sweep's candidates left (the
@@ -1287,6 +1303,179 @@ __device__ __forceinline__ void wunite(unsigned long long *lk, const int2 *node,
         }
         const unsigned long long root = (unsigned long long)(uint32_t)hi;   // self link, offset 0
         if (atomicCAS(lk + hi, root, wind_link(lo, off)) == root) return;
+    }
+}
+
+// ------------------------------------------------------------------ k_one
+// Sweeps of a lattice that is a single tile (L <= 128, plain, periodic or open),
+// all in one block: the tile is the whole lattice, so its wrapping links are
+// united in the same forest, every cluster ends inside, no node, code or merge
+// is needed and the spins stay in shared memory from sweep to sweep.  Bound by the
+// latency of a sweep's phases, which one block alone on its SM cannot hide: L=64
+// 12.8 us a sweep against 20.9 as tile and merge kernels, L=128 19.7 against
+// 26.6, one sweep of L=64 with its launch 20 us against 42.
+struct OneArgs {
+    int32_t L, nsweeps, open;
+    uint32_t key0, key1;
+    uint64_t sweep0, thr;
+    const uint8_t *spin_in;
+    uint8_t *spin_out;       // after the last sweep (may be spin_in)
+    int32_t *label;          // of the last sweep
+    uint32_t *bondbits;      // of the last sweep, null: not wanted
+    DevObs *obs;             // nsweeps entries, written whole
+};
+
+template <int TH>
+struct OneSmem {
+    int par[TH * PW];               // union-find forest over the sites (padded rows)
+    __align__(16) uint32_t b[TH][2 * TWW];   // raw draws, then the bonds without the wrapping links
+    uint32_t sp[TH][TWW];           // spins as bits
+    uint32_t spb[TH][TWW];          // SPIN-stream bit of each site
+    uint32_t wr[TH / 32], wd[TWW];  // wrapping bonds: bit y of the last column's right, bit x of the last row's down links
+    int part[TileCfg<TH>::NW][4];   // per warp: bond_sum, mag (sweep before), nbonds, nclusters
+};
+
+template <int TH>
+__global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
+{
+    constexpr int NT = TileCfg<TH>::NT, NW = TileCfg<TH>::NW;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    OneSmem<TH> &sm = *reinterpret_cast<OneSmem<TH> *>(smem_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
+    const int L = a.L, wy = tid >> 2, wc = tid & 3;
+    const uint32_t uL = (uint32_t)L;
+    const int last_c = (L - 1) >> 5, last_b = (L - 1) & 31;
+    const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW), x = 32 * sx + lane;
+    const uint32_t vm = wy < L ? valid_mask(wc, L) : 0u;
+    const uint32_t vr = a.open && wy < L ? valid_mask(wc, L - 1) : vm, vd = a.open && wy == L - 1 ? 0u : vm;
+    for (int w = warp; w < TH * TWW; w += NW) {
+        const int y = w >> 2, xx = 32 * (w & 3) + lane;
+        const int spin = y < L && xx < L ? a.spin_in[(uint32_t)y * uL + (uint32_t)xx] : 0;
+        const uint32_t word = __ballot_sync(0xFFFFFFFFu, spin);
+        if (lane == 0) sm.sp[y][w & 3] = word;
+    }
+    __syncthreads();
+    for (int j = 0;; ++j) {
+        const bool start = j < a.nsweeps, last = j == a.nsweeps - 1;
+        const uint64_t k = a.sweep0 + (uint64_t)j;
+        const SweepPhilox ph = sweep_philox((uint32_t)k, (uint32_t)(k >> 32), a.key0, a.key1);
+        const bool any_bond = start && a.thr != 0;
+        const uint32_t extra = any_bond ? draw_rows(sm.b, ph, (uint32_t)(a.thr - 1), 0u, uL, L, L) : 0u;
+        if (start && tid < L) spin_row(ph, (uint32_t)tid * uL, sm.spb[tid]);
+        __syncwarp();
+        // the thread's word: spin agreement, the sums of the sweep before, bonds
+        {
+            uint32_t eqr = 0u, eqd = 0u, cur = 0u;
+            if (wy < L) {
+                cur = sm.sp[wy][wc];
+                uint32_t right = __funnelshift_r(cur, wc + 1 < TWW ? sm.sp[wy][wc + 1] : 0u, 1);
+                if (wc == last_c) right |= (sm.sp[wy][0] & 1u) << last_b;
+                eqr = ~(cur ^ right) & vr;
+                eqd = ~(cur ^ sm.sp[wy + 1 < L ? wy + 1 : 0][wc]) & vd;
+            }
+            const int bs = 2 * (__popc(eqr) + __popc(eqd)) - __popc(vr) - __popc(vd);
+            const int ws = __reduce_add_sync(0xFFFFFFFFu, bs);
+            const int wm = __reduce_add_sync(0xFFFFFFFFu, 2 * __popc(cur) - __popc(vm));
+            uint32_t rh = 0u, rv = 0u;
+            if (any_bond) draw_words(sm.b, extra, 0u, uL, rh, rv);
+            const uint32_t h = rh & eqr, v = rv & eqd;
+            const int nb = __reduce_add_sync(0xFFFFFFFFu, __popc(h) + __popc(v));
+            const uint32_t e = rows_byte(__ballot_sync(0xFFFFFFFFu, wc == last_c && ((h >> last_b) & 1u)) >> last_c);
+            if (lane == 0) {
+                sm.part[warp][0] = ws;
+                sm.part[warp][1] = wm;
+                sm.part[warp][2] = nb;
+                reinterpret_cast<uint8_t *>(sm.wr)[warp] = (uint8_t)e;
+            }
+            if (wy == L - 1) sm.wd[wc] = v;
+            if (last && a.bondbits && wy < L) {
+                a.bondbits[wy * 2 * TWW + wc] = h;
+                a.bondbits[wy * 2 * TWW + TWW + wc] = v;
+            }
+            __syncwarp();   // the warp's rows: every draw is read before it is overwritten
+            *reinterpret_cast<uint2 *>(&sm.b[wy][2 * wc]) =
+                make_uint2(h & valid_mask(wc, L - 1), wy < L - 1 ? v : 0u);
+        }
+        __syncthreads();
+        if (j > 0 && tid < 2) {   // sweep j-1's sums of its new spins
+            long long v = 0;
+            for (int w = 0; w < NW; ++w) v += sm.part[w][tid];
+            (tid ? a.obs[j - 1].mag : a.obs[j - 1].bond_sum) = (unsigned long long)v;
+        }
+        if (!start) return;
+        const uint32_t born = tile_label_rows<TH>(sm.par, sm.b, L, L);
+        for (int q = tid; q < TH + TW; q += NT) {   // the wrapping links
+            const bool right = q < TH;
+            const int p = right ? q : q - TH;
+            if (!(((right ? sm.wr[p >> 5] : sm.wd[p >> 5]) >> (p & 31)) & 1u)) continue;
+            volatile int *par = sm.par;
+            if (right) shook<2>(par, par[p * PW + L - 1], par[p * PW]);
+            else shook<2>(par, par[(L - 1) * PW + p], par[p]);
+        }
+        __syncthreads();
+        // every root's record: 0x80000000 | its new spin << 30 | its site; the
+        // other labels' nodes take a copy where it is there already
+        {
+            const int col = y0 * PW + x;
+            uint32_t linked = 0u;
+            int ncl = 0;
+            for (uint32_t bits = born; bits; bits &= bits - 1) {
+                const int r = __ffs(bits) - 1, node = col + r * PW;
+                if (sm.par[node] == node) {
+                    const uint32_t spin = (sm.spb[y0 + r][sx] >> lane) & 1u;
+                    sm.par[node] = (int)(0x80000000u | (spin << 30) | (uint32_t)((y0 + r) * L + x));
+                    ++ncl;
+                } else {
+                    linked |= 1u << r;
+                }
+            }
+            ncl = __reduce_add_sync(0xFFFFFFFFu, ncl);
+            if (lane == 0) sm.part[warp][3] = ncl;
+            for (; linked; linked &= linked - 1) {
+                const int node = col + (__ffs(linked) - 1) * PW;
+                int p = sm.par[node], q = sm.par[p];
+                while (q >= 0 && q != p) {
+                    p = q;
+                    q = sm.par[p];
+                }
+                sm.par[node] = q;   // (a root that has no record yet is its own entry)
+            }
+        }
+        __syncthreads();
+        // every site's new spin; after the last sweep also to memory, with the labels
+        for (int r = 0; r < 32; r += 4) {
+            int v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                v[q] = x < L && y0 + r + q < L ? sm.par[(y0 + r + q) * PW + x] : (int)0x80000000;
+            while ((v[0] & v[1] & v[2] & v[3]) >= 0) {   // some entry is no record yet
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (v[q] >= 0) v[q] = sm.par[v[q]];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t word = __ballot_sync(0xFFFFFFFFu, ((uint32_t)v[q] >> 30) & 1u);
+                if (lane == 0) sm.sp[y0 + r + q][sx] = word;
+                if (last && x < L && y0 + r + q < L) {
+                    const uint32_t g = (uint32_t)(y0 + r + q) * uL + (uint32_t)x;
+                    a.spin_out[g] = (uint8_t)(((uint32_t)v[q] >> 30) & 1u);
+                    a.label[g] = v[q] & 0x3FFFFFFF;
+                }
+            }
+        }
+        if (tid < 2) {
+            long long v = 0;
+            for (int w = 0; w < NW; ++w) v += sm.part[w][2 + tid];
+            DevObs &o = a.obs[j];
+            (tid ? o.nclusters : o.nbonds) = (unsigned long long)v;
+            if (tid == 0) {
+                o.spans_x = o.spans_y = 0;
+                o.threshold = a.thr;
+                o.csize2 = 0ull;
+            }
+        }
+        __syncthreads();
     }
 }
 

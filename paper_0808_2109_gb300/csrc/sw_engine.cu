@@ -43,8 +43,39 @@ cudaError_t tile_prepare()
     const void *fn[2] = {(const void *)k_tile<TH, 0>, (const void *)k_tile<TH, FEAT_TILE>};
     for (int f = 0; f < 2 && err == cudaSuccess; ++f)
         err = cudaFuncSetAttribute(fn[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem<TH>(true));
+    if (err == cudaSuccess)
+        err = cudaFuncSetAttribute((const void *)k_one<TH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)sizeof(OneSmem<TH>));
     if (err == cudaSuccess) done[dev] = true;
     return err;
+}
+
+// Sweeps of a one-tile lattice, in launches of a bounded length.
+template <int TH>
+cudaError_t launch_one(OneArgs a, cudaStream_t st)
+{
+    constexpr int32_t MOST = 4096;   // about 50 ms
+    const int32_t n = a.nsweeps;
+    cudaError_t e = cudaSuccess;
+    for (int32_t at = 0; at < n && e == cudaSuccess; at += MOST) {
+        a.nsweeps = std::min(MOST, n - at);
+        k_one<TH><<<1, TileCfg<TH>::NT, sizeof(OneSmem<TH>), st>>>(a);
+        e = cudaGetLastError();
+        a.sweep0 += (uint64_t)a.nsweeps;
+        a.obs += a.nsweeps;
+        a.spin_in = a.spin_out;
+    }
+    return e;
+}
+
+cudaError_t enqueue_one(int TH, const OneArgs &a, cudaStream_t st)
+{
+    switch (TH) {
+    case 32: return launch_one<32>(a, st);
+    case 64: return launch_one<64>(a, st);
+    case 96: return launch_one<96>(a, st);
+    default: return launch_one<128>(a, st);
+    }
 }
 
 template <int TH>
@@ -554,6 +585,26 @@ int run_sweeps(sw_ctx *c, int32_t n)
         } else {
             SW_CUDA(potts_enqueue_sweeps(c->pd, n, c->sweep, obs, c->stream));
         }
+        c->obs_tail += n;
+        c->sweep += (uint64_t)n;
+        c->swept = true;
+        return SW_OK;
+    }
+    if (c->n_tiles == 1 && !c->pcc && !c->wind && !c->psize && !c->profiling) {
+        OneArgs a{};
+        a.L = c->L;
+        a.nsweeps = n;
+        a.open = c->open ? 1 : 0;
+        a.key0 = c->rep.key0;
+        a.key1 = c->rep.key1;
+        a.sweep0 = c->sweep;
+        a.thr = c->thr;
+        a.spin_in = c->spin;
+        a.spin_out = c->spin;
+        a.label = c->label;
+        a.bondbits = c->bondbits;
+        a.obs = c->obs + c->obs_tail;
+        SW_CUDA(enqueue_one(c->TH, a, c->stream));
         c->obs_tail += n;
         c->sweep += (uint64_t)n;
         c->swept = true;

@@ -87,7 +87,8 @@ int setup_device(int dev, unsigned char **out)
     if (!g_scratch_dev[dev]) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return SW_ERR_CUDA;
-        if (prepare_th(TH_STATIC) != cudaSuccess) return SW_ERR_CUDA;
+        for (int th : {32, 64, 96, TH_STATIC})
+            if (prepare_th(th) != cudaSuccess) return SW_ERR_CUDA;
         g_scratch_dev[dev] = static_cast<unsigned char *>(p);
     }
     *out = g_scratch_dev[dev];
@@ -117,6 +118,22 @@ extern "C" int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_
     if (rc != SW_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaGetLastError();
+
+    if (L <= TW) {
+        // one tile: one block does the whole sweep in its own shared memory
+        OneArgs o{};
+        o.L = L;
+        o.nsweeps = 1;
+        o.key0 = (uint32_t)seed;
+        o.key1 = (uint32_t)(seed >> 32);
+        o.sweep0 = sweep;
+        o.thr = threshold;
+        o.spin_in = spin_in;
+        o.spin_out = spin_out;
+        o.label = labels_out;
+        o.obs = reinterpret_cast<DevObs *>(obs_out);
+        return enqueue_one((L + 31) / 32 * 32, o, st) == cudaSuccess ? SW_OK : SW_ERR_CUDA;
+    }
 
     const int tiles_x = (L + TW - 1) / TW, tiles_y = (L + TH_STATIC - 1) / TH_STATIC;
     Replica R{};

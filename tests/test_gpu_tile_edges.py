@@ -53,3 +53,46 @@ def test_potts_word_and_block_edges(sw, orc, dim, L, q, csize):
                 np.testing.assert_array_equal(lat.spins(), ref.spin)
                 np.testing.assert_array_equal(lat.labels(), ref.label)
                 np.testing.assert_array_equal(lat.bonds(), ref.bond)
+
+
+# Lattices of a single tile run all sweeps of a call in one block.
+@pytest.mark.parametrize("opts", [{}, {"open": True}])
+@pytest.mark.parametrize("L,tile_h", [(2, 0), (3, 128), (31, 0), (32, 32), (33, 0), (63, 96), (64, 0), (65, 0),
+                                      (96, 96), (97, 0), (127, 0), (128, 0)])
+def test_one_tile_lattices(sw, orc, L, tile_h, opts):
+    for T in (1.5, 2.269185, 3.5):
+        ref = orc.sw_chain(L, 1.0, T, L, **opts)
+        with sw.Lattice(L, T=T, seed=L, tile_h=tile_h, **opts) as lat:
+            for n in (1, 4):
+                lat.sweep(n)
+                assert_obs_equal(lat.observables(), ref.run(n))
+                np.testing.assert_array_equal(lat.spins(), ref.spin)
+                np.testing.assert_array_equal(lat.labels(), ref.label)
+                np.testing.assert_array_equal(lat.bonds(), ref.bond)
+
+
+def test_one_tile_call_longer_than_a_launch(sw, orc):
+    ref = orc.sw_chain(12, 1.0, 2.269185, 5)
+    with sw.Lattice(12, T=2.269185, seed=5) as lat:
+        lat.sweep(4099)   # a launch runs at most 4096 sweeps
+        assert_obs_equal(lat.observables(), ref.run(4099))
+        np.testing.assert_array_equal(lat.spins(), ref.spin)
+        np.testing.assert_array_equal(lat.labels(), ref.label)
+
+
+@pytest.mark.parametrize("L", [2, 33, 96, 128])
+def test_static_sweep_of_one_tile(sw, L):
+    torch = pytest.importorskip("torch")
+    thr = sw.sw_threshold(1.0, 2.269185)
+    with sw.Lattice(L, p=thr / 2.0 ** 32, seed=7) as ref:
+        spins = torch.from_numpy(ref.spins()).cuda()
+        out, labels = torch.empty_like(spins), torch.empty(L * L, dtype=torch.int32, device="cuda")
+        obs = torch.full((sw.OBS_DTYPE.itemsize,), 0xAB, dtype=torch.uint8, device="cuda")
+        for k in range(2):
+            sw.sw_sweep_static((spins if k == 0 else out).data_ptr(), out.data_ptr(), labels.data_ptr(),
+                               obs.data_ptr(), L, thr, 7, k, torch.cuda.current_stream())
+            torch.cuda.synchronize()
+            ref.sweep(1)
+            assert obs.cpu().numpy().tobytes() == ref.observables().tobytes()
+            np.testing.assert_array_equal(out.cpu().numpy(), ref.spins())
+            np.testing.assert_array_equal(labels.cpu().numpy(), ref.labels())
