@@ -364,6 +364,21 @@ __device__ __forceinline__ void shook(volatile int *par, int a, int b)
     sunite(par, a, b);
 }
 
+// Two links at once, a1-b1 only where on1: their first atomics run together.  One
+// block alone on its SM waits for each round trip (k_one: L=64 12.8 -> 12.2 us a
+// sweep); where other CTAs fill the wait the second link's selects cost more (the
+// tile kernel at L=4096 is not faster with it).
+template <int STEPS>
+__device__ __forceinline__ void shook_pair(volatile int *par, int a0, int b0, bool on1, int a1, int b1)
+{
+    const int h0 = max(a0, b0), l0 = min(a0, b0), h1 = max(a1, b1), l1 = min(a1, b1);
+    int o0 = h0, o1 = h1;
+    if (a0 != b0) o0 = atomicCAS((int *)&par[h0], h0, l0);
+    if (on1 && a1 != b1) o1 = atomicCAS((int *)&par[h1], h1, l1);
+    if (o0 != h0) shook<STEPS - 1>(par, o0, l0);
+    if (o1 != h1) shook<STEPS - 1>(par, o1, l1);
+}
+
 // As sunite, reporting whether this call linked two sets (false: a and b
 // were already in one set).
 __device__ __forceinline__ bool sunite_linked(volatile int *par, int a, int b)
@@ -475,8 +490,8 @@ __device__ __forceinline__ uint32_t run_heads(uint32_t h)
 // per column, the single-swap unions and the label nodes' copies of their root's
 // record (two loads a code) to 1.19 ms.
 // Returns, to lane x, the rows of column x of the warp's sub-tile whose site
-// started a label (every root is one of them).
-template <int TH>
+// started a label (every root is one of them).  PAIRS: two conflicts at a time.
+template <int TH, bool PAIRS = false>
 __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
 {
     constexpr int NT = TileCfg<TH>::NT;
@@ -517,6 +532,15 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
         if (rows < 32) born &= (1u << rows) - 1u;
         __syncwarp();
         const int col = y0 * PW + 32 * sx + lane;
+        while (PAIRS && conf) {
+            const int i0 = col + (__ffs(conf) - 1) * PW;
+            conf &= conf - 1;
+            const bool two = conf != 0u;
+            const int i1 = two ? col + (__ffs(conf) - 1) * PW : i0;
+            conf &= conf - 1;
+            const int a0 = par[i0 - PW], b0 = par[i0], a1 = par[i1 - PW], b1 = par[i1];
+            shook_pair<4>(par, a0, b0, two, a1, b1);
+        }
         for (; conf; conf &= conf - 1) {
             const int i = col + (__ffs(conf) - 1) * PW;
             shook<4>(par, par[i - PW], par[i]);
@@ -647,7 +671,9 @@ __device__ __forceinline__ void warp_add64(unsigned long long *dst, unsigned lon
 // owns a word interleaves them (13 operations a word against a shuffle, a shift
 // and two ballots a word for every lane of the warp).  An odd first site is the
 // second one of its row's first block, so the row's 128 sites reach into a 65th
-// block: lane r draws it for row r and returns its first two words' bits.
+// block: lane r draws it for row r and returns its first two words' bits.  U row
+// pairs are unrolled: k_one, which has registers to spare, is 1-2% faster with 4.
+template <int U>
 __device__ __forceinline__ uint32_t draw_rows(uint32_t (*raw_rows)[2 * TWW], const SweepPhilox &ph, uint32_t tm1,
                                               uint32_t gbase, uint32_t uL, int th, int tw)
 {
@@ -660,6 +686,7 @@ __device__ __forceinline__ uint32_t draw_rows(uint32_t (*raw_rows)[2 * TWW], con
     uint4 *raw = reinterpret_cast<uint4 *>(&raw_rows[8 * warp][0]);
     uint32_t b = gbase + (uint32_t)(8 * warp) * uL;   // the row's first site
     if (tw > 64) {
+#pragma unroll U
         for (int i = 0; i < rows; i += 2, b += 2u * uL, raw += 4) {
             const uint32_t b0 = (b >> 1) + lane, b2 = ((b + uL) >> 1) + lane;
             const U4 r0 = sweep_block(ph, b0, STREAM_BOND), r1 = sweep_block(ph, b0 + 32, STREAM_BOND);
@@ -674,6 +701,7 @@ __device__ __forceinline__ uint32_t draw_rows(uint32_t (*raw_rows)[2 * TWW], con
         }
     } else {
         // blocks 32 .. 63 of a row have no sites in the tile
+#pragma unroll U
         for (int i = 0; i < rows; i += 2, b += 2u * uL, raw += 4) {
             const U4 r0 = sweep_block(ph, (b >> 1) + lane, STREAM_BOND);
             const U4 r2 = sweep_block(ph, ((b + uL) >> 1) + lane, STREAM_BOND);
@@ -862,7 +890,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     const uint64_t thr = (F & FEAT_PCC) && (R.flags & RF_PCC) ? *R.thr_dev : R.thr;
     const SweepPhilox ph = sweep_philox((uint32_t)k, (uint32_t)(k >> 32), R.key0, R.key1);
     const bool any_bond = start && thr != 0;      // t = 0: P = 0, nothing bonds
-    const uint32_t extra = any_bond ? draw_rows(sm.b, ph, (uint32_t)(thr - 1), gbase, uL, t.th, t.tw) : 0u;
+    const uint32_t extra = any_bond ? draw_rows<1>(sm.b, ph, (uint32_t)(thr - 1), gbase, uL, t.th, t.tw) : 0u;
 
     if (early) finish_loads();
     if (fin) {
@@ -1311,9 +1339,9 @@ __device__ __forceinline__ void wunite(unsigned long long *lk, const int2 *node,
 // all in one block: the tile is the whole lattice, so its wrapping links are
 // united in the same forest, every cluster ends inside, no node, code or merge
 // is needed and the spins stay in shared memory from sweep to sweep.  Bound by the
-// latency of a sweep's phases, which one block alone on its SM cannot hide: L=64
-// 12.8 us a sweep against 20.9 as tile and merge kernels, L=128 19.7 against
-// 26.6, one sweep of L=64 with its launch 20 us against 42.
+// latency of a sweep's phases, which one block alone on its SM cannot hide (hence
+// the conflicts and the records two at a time and the unrolled draws): L=64 12.2 us
+// a sweep against 20.9 as tile and merge kernels, L=128 19.0 against 26.6, one sweep of L=64 with its launch 20 us against 42.
 struct OneArgs {
     int32_t L, nsweeps, open;
     uint32_t key0, key1;
@@ -1360,7 +1388,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
         const uint64_t k = a.sweep0 + (uint64_t)j;
         const SweepPhilox ph = sweep_philox((uint32_t)k, (uint32_t)(k >> 32), a.key0, a.key1);
         const bool any_bond = start && a.thr != 0;
-        const uint32_t extra = any_bond ? draw_rows(sm.b, ph, (uint32_t)(a.thr - 1), 0u, uL, L, L) : 0u;
+        const uint32_t extra = any_bond ? draw_rows<4>(sm.b, ph, (uint32_t)(a.thr - 1), 0u, uL, L, L) : 0u;
         if (start && tid < L) spin_row(ph, (uint32_t)tid * uL, sm.spb[tid]);
         __syncwarp();
         // the thread's word: spin agreement, the sums of the sweep before, bonds
@@ -1403,7 +1431,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
             (tid ? a.obs[j - 1].mag : a.obs[j - 1].bond_sum) = (unsigned long long)v;
         }
         if (!start) return;
-        const uint32_t born = tile_label_rows<TH>(sm.par, sm.b, L, L);
+        const uint32_t born = tile_label_rows<TH, true>(sm.par, sm.b, L, L);
         for (int q = tid; q < TH + TW; q += NT) {   // the wrapping links
             const bool right = q < TH;
             const int p = right ? q : q - TH;
@@ -1419,15 +1447,23 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
             const int col = y0 * PW + x;
             uint32_t linked = 0u;
             int ncl = 0;
-            for (uint32_t bits = born; bits; bits &= bits - 1) {
-                const int r = __ffs(bits) - 1, node = col + r * PW;
-                if (sm.par[node] == node) {
-                    const uint32_t spin = (sm.spb[y0 + r][sx] >> lane) & 1u;
-                    sm.par[node] = (int)(0x80000000u | (spin << 30) | (uint32_t)((y0 + r) * L + x));
+            auto record = [&](int r, int node, int p, uint32_t word) {
+                if (p == node) {
+                    sm.par[node] = (int)(0x80000000u | (((word >> lane) & 1u) << 30) | (uint32_t)((y0 + r) * L + x));
                     ++ncl;
                 } else {
                     linked |= 1u << r;
                 }
+            };
+            for (uint32_t bits = born; bits;) {
+                const int r0 = __ffs(bits) - 1;
+                bits &= bits - 1;
+                const int r1 = bits ? __ffs(bits) - 1 : r0;
+                bits &= bits - 1;
+                const int p0 = sm.par[col + r0 * PW], p1 = sm.par[col + r1 * PW];
+                const uint32_t w0 = sm.spb[y0 + r0][sx], w1 = sm.spb[y0 + r1][sx];
+                record(r0, col + r0 * PW, p0, w0);
+                if (r1 != r0) record(r1, col + r1 * PW, p1, w1);
             }
             ncl = __reduce_add_sync(0xFFFFFFFFu, ncl);
             if (lane == 0) sm.part[warp][3] = ncl;
