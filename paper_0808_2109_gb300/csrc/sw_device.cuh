@@ -489,15 +489,23 @@ __device__ __forceinline__ uint32_t run_heads(uint32_t h)
 // at L=16384, T_c (111 -> 81M warp instructions a launch at L=4096), and masks
 // per column, the single-swap unions and the label nodes' copies of their root's
 // record (two loads a code) to 1.19 ms.
-// Returns, to lane x, the rows of column x of the warp's sub-tile whose site
+//
+// k_one, whose warps have nobody to hide behind, takes sub-tiles of fewer rows (RS)
+// and leaves out the words of a row that its lattice does not reach (WX in use).
+template <int WX, int RS>
+struct SubTile {
+    __device__ static int sx() { return (threadIdx.x >> 5) & (WX - 1); }
+    __device__ static int y0() { return RS * ((threadIdx.x >> 5) / WX); }
+};
+
+// 1.  Returns, to lane x, the rows of column x of the warp's sub-tile whose site
 // started a label (every root is one of them).  PAIRS: two conflicts at a time.
-template <int TH, bool PAIRS = false>
-__device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
+template <int WX, int RS, bool PAIRS>
+__device__ __forceinline__ uint32_t label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
 {
-    constexpr int NT = TileCfg<TH>::NT;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
-    const int rows = 32 * sx < tw ? min(32, th - y0) : 0;
+    const int lane = threadIdx.x & 31;
+    const int sx = SubTile<WX, RS>::sx(), y0 = SubTile<WX, RS>::y0();
+    const int rows = 32 * sx < tw ? min(RS, th - y0) : 0;
     uint32_t born = 0u, conf = 0u;
     if (rows > 0) {
         const uint32_t le = 0xFFFFFFFFu >> (31 - lane), gt = ~le;
@@ -506,7 +514,7 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
         // four rows at a time: everything that does not need the labels first,
         // so that the chain from row to row is a shuffle and a select (rows past
         // the tile's have no bonds)
-        for (int r = 0; r < 32; r += 4) {
+        for (int r = 0; r < RS; r += 4) {
             int hd[4], c[4];
             uint32_t dn[4];
 #pragma unroll
@@ -529,7 +537,7 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
                 par[row + lane] = lab;
             }
         }
-        if (rows < 32) born &= (1u << rows) - 1u;
+        if (rows < RS) born &= (1u << rows) - 1u;
         __syncwarp();
         const int col = y0 * PW + 32 * sx + lane;
         while (PAIRS && conf) {
@@ -547,33 +555,45 @@ __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uin
         }
         if (32 * sx + lane >= tw) born = 0u;
     }
-    __syncthreads();
+    return born;
+}
 
-    // ---- 2. links across sub-tile boundaries: vertical boundaries between
-    //         sub-tile columns, horizontal ones between sub-tile rows.  (Skipping a
-    //         link whose sites point at the same nodes as the one before it along
-    //         the boundary costs more than the unions it saves: 1433 us a sweep
-    //         against 1426 at L=16384, T_c.)
+// 2.  Links across sub-tile boundaries: vertical boundaries between sub-tile
+// columns, horizontal ones between sub-tile rows.  The q-th of EDGES: whether it is
+// a bond, and its sites' forest indices.  (Skipping a link whose sites point at the
+// same nodes as the one before it along the boundary costs more than the unions it
+// saves: 1433 us a sweep against 1426 at L=16384, T_c.)
+template <int TH, int WX, int RS>
+struct EdgeLinks {
+    static constexpr int NV = (WX - 1) * TH, EDGES = NV + (TH / RS - 1) * 32 * WX;
+    __device__ static bool link(int q, const uint32_t (*B)[2 * TWW], int th, int &ia, int &ib)
     {
-        constexpr int NV = (TWW - 1) * TH;
-        constexpr int NH = (TH / 32 - 1) * TW;
-        for (int q = threadIdx.x; q < NV + NH; q += NT) {
-            int ia, ib;
-            if (q < NV) {
-                const int bnd = q / TH + 1, y = q % TH;     // link (32 bnd - 1, y) - (32 bnd, y)
-                if (y >= th || !(B[y][2 * bnd - 2] >> 31)) continue;
-                ia = y * PW + 32 * bnd - 1;
-                ib = ia + 1;
-            } else {
-                const int r = q - NV;
-                const int bnd = r / TW + 1, x = r % TW;     // link (x, 32 bnd - 1) - (x, 32 bnd)
-                const int y = 32 * bnd - 1;
-                if (y + 1 >= th || !((B[y][2 * (x >> 5) + 1] >> (x & 31)) & 1u)) continue;
-                ia = y * PW + x;
-                ib = ia + PW;
-            }
-            shook<2>(par, par[ia], par[ib]);
+        if (q < NV) {
+            const int bnd = q / TH + 1, y = q % TH;             // link (32 bnd - 1, y) - (32 bnd, y)
+            if (y >= th || !(B[y][2 * bnd - 2] >> 31)) return false;
+            ia = y * PW + 32 * bnd - 1;
+            ib = ia + 1;
+        } else {
+            const int r = q - NV;
+            const int y = RS * (r / (32 * WX) + 1) - 1, x = r % (32 * WX);   // link (x, y) - (x, y + 1)
+            if (y + 1 >= th || !((B[y][2 * (x >> 5) + 1] >> (x & 31)) & 1u)) return false;
+            ia = y * PW + x;
+            ib = ia + PW;
         }
+        return true;
+    }
+};
+
+// Both, for all threads of a tile CTA; returns what label_rows does.
+template <int TH>
+__device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
+{
+    using E = EdgeLinks<TH, TWW, 32>;
+    const uint32_t born = label_rows<TWW, 32, false>(par, B, th, tw);
+    __syncthreads();
+    for (int q = threadIdx.x; q < E::EDGES; q += TileCfg<TH>::NT) {
+        int ia, ib;
+        if (E::link(q, B, th, ia, ib)) shook<2>(par, par[ia], par[ib]);
     }
     __syncthreads();
     return born;
@@ -1339,9 +1359,12 @@ __device__ __forceinline__ void wunite(unsigned long long *lk, const int2 *node,
 // all in one block: the tile is the whole lattice, so its wrapping links are
 // united in the same forest, every cluster ends inside, no node, code or merge
 // is needed and the spins stay in shared memory from sweep to sweep.  Bound by the
-// latency of a sweep's phases, which one block alone on its SM cannot hide (hence
-// the conflicts and the records two at a time and the unrolled draws): L=64 12.2 us
-// a sweep against 20.9 as tile and merge kernels, L=128 19.0 against 26.6, one sweep of L=64 with its launch 20 us against 42.
+// latency of a sweep's phases, which one block alone on its SM cannot hide: sub-tiles
+// of 8 or 16 rows instead of 32, so that twice the warps walk half the rows (OneCfg;
+// L=32 8.9 -> 5.6 us a sweep, L=64 12.2 -> 9.2, L=128 19.0 -> 17.3; 8 rows at L=64 9.5,
+// 32 rows at L=128 18.0), conflicts and records two at a time, eight look-ups of
+// spins in flight, unrolled draws.  As tile and merge kernels L=64 took 20.9 us a
+// sweep and L=128 26.6, and one sweep of L=64 with its launch 42 us against 17.
 struct OneArgs {
     int32_t L, nsweeps, open;
     uint32_t key0, key1;
@@ -1354,26 +1377,35 @@ struct OneArgs {
 };
 
 template <int TH>
+struct OneCfg {
+    static constexpr int WX = TH == 32 ? 1 : TH == 64 ? 2 : TWW;   // the words of a row that L <= TH sites reach
+    static constexpr int RS = TH == 32 ? 8 : 16;
+    static constexpr int NT = 32 * WX * (TH / RS);
+};
+
+template <int TH>
 struct OneSmem {
     int par[TH * PW];               // union-find forest over the sites (padded rows)
     __align__(16) uint32_t b[TH][2 * TWW];   // raw draws, then the bonds without the wrapping links
     uint32_t sp[TH][TWW];           // spins as bits
     uint32_t spb[TH][TWW];          // SPIN-stream bit of each site
     uint32_t wr[TH / 32], wd[TWW];  // wrapping bonds: bit y of the last column's right, bit x of the last row's down links
-    int part[TileCfg<TH>::NW][4];   // per warp: bond_sum, mag (sweep before), nbonds, nclusters
+    int part[OneCfg<TH>::NT / 32][4];   // per warp: bond_sum, mag (sweep before), nbonds, nclusters
 };
 
 template <int TH>
-__global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
+__global__ void __launch_bounds__(OneCfg<TH>::NT, 1) k_one(const OneArgs a)
 {
-    constexpr int NT = TileCfg<TH>::NT, NW = TileCfg<TH>::NW;
+    constexpr int WX = OneCfg<TH>::WX, RS = OneCfg<TH>::RS, NT = OneCfg<TH>::NT, NW = NT / 32;
+    constexpr int WT = TileCfg<TH>::NT;   // threads with a word of the tile; their warps draw
+    using E = EdgeLinks<TH, WX, RS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OneSmem<TH> &sm = *reinterpret_cast<OneSmem<TH> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
     const int L = a.L, wy = tid >> 2, wc = tid & 3;
     const uint32_t uL = (uint32_t)L;
     const int last_c = (L - 1) >> 5, last_b = (L - 1) & 31;
-    const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW), x = 32 * sx + lane;
+    const int sx = SubTile<WX, RS>::sx(), y0 = SubTile<WX, RS>::y0(), x = 32 * sx + lane;
     const uint32_t vm = wy < L ? valid_mask(wc, L) : 0u;
     const uint32_t vr = a.open && wy < L ? valid_mask(wc, L - 1) : vm, vd = a.open && wy == L - 1 ? 0u : vm;
     for (int w = warp; w < TH * TWW; w += NW) {
@@ -1388,11 +1420,11 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
         const uint64_t k = a.sweep0 + (uint64_t)j;
         const SweepPhilox ph = sweep_philox((uint32_t)k, (uint32_t)(k >> 32), a.key0, a.key1);
         const bool any_bond = start && a.thr != 0;
-        const uint32_t extra = any_bond ? draw_rows<4>(sm.b, ph, (uint32_t)(a.thr - 1), 0u, uL, L, L) : 0u;
-        if (start && tid < L) spin_row(ph, (uint32_t)tid * uL, sm.spb[tid]);
-        __syncwarp();
-        // the thread's word: spin agreement, the sums of the sweep before, bonds
-        {
+        if (WT == NT || tid < WT) {
+            const uint32_t extra = any_bond ? draw_rows<4>(sm.b, ph, (uint32_t)(a.thr - 1), 0u, uL, L, L) : 0u;
+            if (start && tid < L) spin_row(ph, (uint32_t)tid * uL, sm.spb[tid]);
+            __syncwarp();
+            // the thread's word: spin agreement, the sums of the sweep before, bonds
             uint32_t eqr = 0u, eqd = 0u, cur = 0u;
             if (wy < L) {
                 cur = sm.sp[wy][wc];
@@ -1427,18 +1459,26 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
         __syncthreads();
         if (j > 0 && tid < 2) {   // sweep j-1's sums of its new spins
             long long v = 0;
-            for (int w = 0; w < NW; ++w) v += sm.part[w][tid];
+            for (int w = 0; w < WT / 32; ++w) v += sm.part[w][tid];
             (tid ? a.obs[j - 1].mag : a.obs[j - 1].bond_sum) = (unsigned long long)v;
         }
         if (!start) return;
-        const uint32_t born = tile_label_rows<TH, true>(sm.par, sm.b, L, L);
-        for (int q = tid; q < TH + TW; q += NT) {   // the wrapping links
-            const bool right = q < TH;
-            const int p = right ? q : q - TH;
-            if (!(((right ? sm.wr[p >> 5] : sm.wd[p >> 5]) >> (p & 31)) & 1u)) continue;
+        const uint32_t born = label_rows<WX, RS, true>(sm.par, sm.b, L, L);
+        __syncthreads();
+        // links between sub-tiles and the wrapping ones
+        for (int q = tid; q < E::EDGES + TH + 32 * WX; q += NT) {
+            int ia, ib;
+            if (q < E::EDGES) {
+                if (!E::link(q, sm.b, L, ia, ib)) continue;
+            } else {
+                const bool right = q < E::EDGES + TH;
+                const int i = q - E::EDGES - (right ? 0 : TH);
+                if (!(((right ? sm.wr[i >> 5] : sm.wd[i >> 5]) >> (i & 31)) & 1u)) continue;
+                ia = right ? i * PW + L - 1 : (L - 1) * PW + i;
+                ib = right ? i * PW : i;
+            }
             volatile int *par = sm.par;
-            if (right) shook<2>(par, par[p * PW + L - 1], par[p * PW]);
-            else shook<2>(par, par[(L - 1) * PW + p], par[p]);
+            shook<2>(par, par[ia], par[ib]);
         }
         __syncthreads();
         // every root's record: 0x80000000 | its new spin << 30 | its site; the
@@ -1478,19 +1518,24 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
             }
         }
         __syncthreads();
-        // every site's new spin; after the last sweep also to memory, with the labels
-        for (int r = 0; r < 32; r += 4) {
-            int v[4];
+        // every site's new spin, eight rows' look-ups in flight; after the last
+        // sweep also to memory, with the labels
+        for (int r = 0; r < RS; r += 8) {
+            int v[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+            for (int q = 0; q < 8; ++q)
                 v[q] = x < L && y0 + r + q < L ? sm.par[(y0 + r + q) * PW + x] : (int)0x80000000;
-            while ((v[0] & v[1] & v[2] & v[3]) >= 0) {   // some entry is no record yet
+            for (bool more = true; more;) {   // some entry is no record yet
+                more = false;
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (v[q] >= 0) v[q] = sm.par[v[q]];
+                for (int q = 0; q < 8; ++q)
+                    if (v[q] >= 0) {
+                        v[q] = sm.par[v[q]];
+                        more = true;
+                    }
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < 8; ++q) {
                 const uint32_t word = __ballot_sync(0xFFFFFFFFu, ((uint32_t)v[q] >> 30) & 1u);
                 if (lane == 0) sm.sp[y0 + r + q][sx] = word;
                 if (last && x < L && y0 + r + q < L) {
@@ -1502,7 +1547,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, 1) k_one(const OneArgs a)
         }
         if (tid < 2) {
             long long v = 0;
-            for (int w = 0; w < NW; ++w) v += sm.part[w][2 + tid];
+            for (int w = 0; w < (tid ? NW : WT / 32); ++w) v += sm.part[w][2 + tid];
             DevObs &o = a.obs[j];
             (tid ? o.nclusters : o.nbonds) = (unsigned long long)v;
             if (tid == 0) {

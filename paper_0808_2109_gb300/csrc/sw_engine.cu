@@ -59,7 +59,7 @@ cudaError_t launch_one(OneArgs a, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     for (int32_t at = 0; at < n && e == cudaSuccess; at += MOST) {
         a.nsweeps = std::min(MOST, n - at);
-        k_one<TH><<<1, TileCfg<TH>::NT, sizeof(OneSmem<TH>), st>>>(a);
+        k_one<TH><<<1, OneCfg<TH>::NT, sizeof(OneSmem<TH>), st>>>(a);
         e = cudaGetLastError();
         a.sweep0 += (uint64_t)a.nsweeps;
         a.obs += a.nsweeps;
@@ -68,9 +68,13 @@ cudaError_t launch_one(OneArgs a, cudaStream_t st)
     return e;
 }
 
-cudaError_t enqueue_one(int TH, const OneArgs &a, cudaStream_t st)
+// The height of k_one for a side of at most 128: the fewest rows that hold it,
+// whatever height the lattice's tile kernel has.
+int one_height(int L) { return (L + 31) / 32 * 32; }
+
+cudaError_t enqueue_one(const OneArgs &a, cudaStream_t st)
 {
-    switch (TH) {
+    switch (one_height(a.L)) {
     case 32: return launch_one<32>(a, st);
     case 64: return launch_one<64>(a, st);
     case 96: return launch_one<96>(a, st);
@@ -382,6 +386,7 @@ int ctx_create(sw_ctx **out, int32_t L, uint64_t thr, uint64_t seed, bool pcc, u
     const size_t N = (size_t)L * L;
     const size_t nt = (size_t)c->n_tiles;
     if ((e = prepare_th(c->TH)) != cudaSuccess) return fail(e);
+    if (c->n_tiles == 1 && (e = prepare_th(one_height(L))) != cudaSuccess) return fail(e);
     if ((e = cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking)) != cudaSuccess) return fail(e);
     if ((e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking)) != cudaSuccess) return fail(e);
     c->stream = c->own_stream;
@@ -604,7 +609,7 @@ int run_sweeps(sw_ctx *c, int32_t n)
         a.label = c->label;
         a.bondbits = c->bondbits;
         a.obs = c->obs + c->obs_tail;
-        SW_CUDA(enqueue_one(c->TH, a, c->stream));
+        SW_CUDA(enqueue_one(a, c->stream));
         c->obs_tail += n;
         c->sweep += (uint64_t)n;
         c->swept = true;

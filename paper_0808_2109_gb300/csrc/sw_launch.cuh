@@ -24,8 +24,8 @@ __attribute__((visibility("hidden"))) cudaError_t enqueue_merge(int TH, const Sw
                                                                 cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat,
                                                                     cudaStream_t st, bool chained);
-// All sweeps of a lattice that is one tile of height TH (k_one).
-__attribute__((visibility("hidden"))) cudaError_t enqueue_one(int TH, const OneArgs &a, cudaStream_t st);
+// All sweeps of a one-tile lattice, L <= 128 (k_one).
+__attribute__((visibility("hidden"))) cudaError_t enqueue_one(const OneArgs &a, cudaStream_t st);
 // Launch groups j = 0 .. m-1 of one lattice; last: the final one is a call's
 // last and has no merge.
 __attribute__((visibility("hidden"))) cudaError_t enqueue_groups(int TH, SweepArgs a, bool pcc, int feat, int m,

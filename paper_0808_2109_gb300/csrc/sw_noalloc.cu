@@ -132,7 +132,7 @@ extern "C" int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_
         o.spin_out = spin_out;
         o.label = labels_out;
         o.obs = reinterpret_cast<DevObs *>(obs_out);
-        return enqueue_one((L + 31) / 32 * 32, o, st) == cudaSuccess ? SW_OK : SW_ERR_CUDA;
+        return enqueue_one(o, st) == cudaSuccess ? SW_OK : SW_ERR_CUDA;
     }
 
     const int tiles_x = (L + TW - 1) / TW, tiles_y = (L + TH_STATIC - 1) / TH_STATIC;
