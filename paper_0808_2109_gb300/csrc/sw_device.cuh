@@ -125,6 +125,10 @@ __device__ __forceinline__ int lattice_launch(const SweepArgs &a, const Replica 
     return a.j + *a.jbase - R.jstart;
 }
 
+// SMs of the GPU this is written for: the blocks of a grid that start at once
+// are about this many times a kernel's blocks per SM.
+constexpr int FIRST_WAVE_SMS = 152;
+
 // Programmatic dependent launch: the kernels of a call form one chain in which
 // each may start while the one before it drains.  Every kernel lets its
 // successor start at once, and every block waits (griddepcontrol.wait: all of
@@ -139,7 +143,11 @@ __device__ __forceinline__ int lattice_launch(const SweepArgs &a, const Replica 
 // 104 us).  Where a grid does not fill the GPU that has a price: blocks started
 // ahead go to the few SMs with room and run crowded there.  So
 //   - the merge kernels of the topological rule and of PCC let theirs start after
-//     their own wait (every option at L=1001: 92 us against 111);
+//     their own wait (every option at L=1001: 92 us against 111), and so do those of
+//     32-row tiles and of grids of at most one tile an SM, unless four such grids fit
+//     side by side (32 rows: L=1001 30.9 us against 34.3, L=2048 45.4 against 48.1;
+//     96 rows: L=1200 33.0 against 33.6, but L=2048 49.3 against 44.9; 3D Potts L=80
+//     43.9 against 49.1);
 //   - the cover kernel of PCC lets the tile kernel start only when it ends (the
 //     tiles of such a lattice have nothing to do before: 2D Potts L=1024 58 us
 //     against 76);
@@ -152,6 +160,10 @@ __device__ __forceinline__ void chain_next()
 __device__ __forceinline__ void chain_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ bool chain_crowds(int n_tiles, bool any_size = false)
+{
+    return 4 * n_tiles > FIRST_WAVE_SMS && (any_size || n_tiles <= FIRST_WAVE_SMS);
 }
 
 // ------------------------------------------------------------------ Philox
@@ -395,10 +407,6 @@ __device__ __forceinline__ bool sunite_linked(volatile int *par, int a, int b)
         if (atomicCAS((int *)&par[b], b, a) == b) return true;
     }
 }
-
-// SMs of the GPU this is written for: the blocks of a grid that start at once
-// are about this many times a kernel's blocks per SM.
-constexpr int FIRST_WAVE_SMS = 152;
 
 // Threads of a tile CTA: one warp per 32 x 32 sub-tile.
 template <int TH>
@@ -1632,11 +1640,11 @@ __device__ __forceinline__ const Replica *launch_lattice(const SweepArgs &a, int
 
 // The same at the start of a merge kernel (W: with the topological rule): the
 // successor may start, the predecessor's work is done.
-template <bool W>
+template <int TH, bool W>
 __device__ __forceinline__ const Replica *merge_lattice(const SweepArgs &a, int g, int &j)
 {
     const Replica *R = launch_lattice(a, g, j);
-    const bool late = W || (R && (R->flags & RF_PCC));
+    const bool late = W || (R && (R->flags & RF_PCC)) || chain_crowds(a.n_tiles, TH == 32);
     if (!late) chain_next();
     chain_wait();
     if (late) chain_next();
@@ -1657,7 +1665,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::UT, (W ? 40 : 64) / (MergeCfg<TH
     constexpr int S = SL::S, EPT = 2;
     __shared__ uint16_t links[32 * MC::LW];
     int j;
-    const Replica *Rp = merge_lattice<W>(a, blockIdx.x, j);
+    const Replica *Rp = merge_lattice<TH, W>(a, blockIdx.x, j);
     if (!Rp) return;
     const Replica &R = *Rp;
     const Tile t = tile_of(R, blockIdx.x, TH);
@@ -1816,7 +1824,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_jump(const SweepArgs 
 {
     using MC = MergeCfg<TH>;
     int j;
-    const Replica *Rp = merge_lattice<true>(a, blockIdx.x, j);
+    const Replica *Rp = merge_lattice<TH, true>(a, blockIdx.x, j);
     if (!Rp || !(Rp->flags & RF_WIND)) return;
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;   // the lattice's own nodes
@@ -1851,7 +1859,7 @@ __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_merge_resolve(const SweepA
     __shared__ int nwalks;
     if (threadIdx.x == 0) nwalks = 0;
     int j;
-    const Replica *Rp = merge_lattice<W>(a, blockIdx.x, j);
+    const Replica *Rp = merge_lattice<TH, W>(a, blockIdx.x, j);
     if (!Rp) return;
     const Replica &R = *Rp;
     const int base = (blockIdx.x - R.tile_base) * MC::S;

@@ -86,7 +86,8 @@ template <int TH>
 cudaError_t launch_tile(const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
     return launch_kernel(pcc || (feat & FEAT_TILE) ? k_tile<TH, FEAT_TILE> : k_tile<TH, 0>, dim3(a.n_tiles),
-                         TileCfg<TH>::NT, tile_smem<TH>(pcc), st, chained, a);
+                         TileCfg<TH>::NT, tile_smem<TH>(pcc), st, chained,
+                         chain_all_shared(a.n_tiles, pcc, (feat & FEAT_WIND) != 0), a);
 }
 
 // The merge of launch group j: unions across tile edges, every node's resolved
@@ -95,11 +96,11 @@ template <int TH>
 cudaError_t launch_merge(const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
     constexpr int MT = MergeCfg<TH>::MT;
-    const bool wind = (feat & FEAT_WIND) != 0;
+    const bool wind = (feat & FEAT_WIND) != 0, all_shared = chain_all_shared(a.n_tiles, pcc, wind);
     const dim3 tiles(a.n_tiles);
     cudaError_t e = cudaSuccess;
     auto go = [&](auto *k, dim3 grid, unsigned threads, auto... args) {
-        if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, args...);
+        if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, all_shared, args...);
     };
     go(wind ? k_merge_union<TH, true> : k_merge_union<TH, false>, tiles, MergeCfg<TH>::UT, a);
     if (wind) go(k_wind_jump<TH>, tiles, MT, a);
@@ -214,10 +215,20 @@ int sw_cuda_fail(cudaError_t e, int line = 0)
     return SW_ERR_CUDA;
 }
 
-// Tile height used for an L x L lattice: a SW_FLAG_TILE_* flag, else the
-// smallest height that covers short lattices, else 96 (three CTAs fit on an
-// SM, against two for 128).
-int pick_tile_height(int L, uint32_t flags)
+// Tile height used for an L x L lattice: a SW_FLAG_TILE_* flag, else the first of
+//   - one tile for a side of at most 128, where it has no features (k_one) or the
+//     topological rule (L=110 35.3 us a sweep against 40.5 in 32-row tiles), or at
+//     most 64;
+//   - 32 rows while they are at most six CTAs an SM (L <= 1920): the sweep is then
+//     bound by the latency of a tile, which is shortest where one warp walks 32 rows
+//     and a border has few nodes (L=300 26.7 us against 29.3 with 96 rows, L=1001
+//     31.0 against 32.2, L=1600 36.2 against 47.1; cluster sizes at L=1001 43.1
+//     against 57.9; at L=2048 45.3 against 44.9).  PCC and the topological rule pay
+//     more for the longer borders: PCC takes 32 rows up to half a CTA an SM (L <=
+//     512; 45.7 against 49.3 at L=512, 54.1 against 53.4 at 1001), the rule alone up
+//     to a third (L <= 384; 38.2 against 39.4 at L=200, 44.0 against 42.9 at 512);
+//   - 96 rows (four CTAs fit on an SM, three of 128).
+int pick_tile_height(int L, uint32_t flags, bool pcc)
 {
     if (flags & SW_FLAG_TILE_32) return 32;
     if (flags & SW_FLAG_TILE_64) return 64;
@@ -225,8 +236,10 @@ int pick_tile_height(int L, uint32_t flags)
     if (flags & SW_FLAG_TILE_128) return 128;
     if (L <= 32) return 32;
     if (L <= 64) return 64;
-    if (L <= 128) return 128;
-    return 96;
+    const bool wind = (flags & SW_FLAG_WIND) != 0;
+    if (L <= 128 && (wind || !(pcc || (flags & SW_FLAG_CSIZE)))) return 128;
+    const int64_t tiles = (int64_t)((L + TW - 1) / TW) * ((L + 31) / 32);
+    return tiles <= (pcc ? FIRST_WAVE_SMS / 2 : wind ? FIRST_WAVE_SMS / 3 : 6 * FIRST_WAVE_SMS) ? 32 : 96;
 }
 
 std::atomic<int> g_alloc_skip{0}, g_alloc_failures{0};   // sw_debug_fail_allocations
@@ -373,7 +386,7 @@ int ctx_create(sw_ctx **out, int32_t L, uint64_t thr, uint64_t seed, bool pcc, u
     if (e != cudaSuccess) return fail(e);
     c->L = L;
     c->nsites = (int64_t)L * L;
-    c->TH = pick_tile_height(L, flags);
+    c->TH = pick_tile_height(L, flags, pcc);
     c->S = slots_of(c->TH);
     c->tiles_x = (L + TW - 1) / TW;
     c->tiles_y = (L + c->TH - 1) / c->TH;

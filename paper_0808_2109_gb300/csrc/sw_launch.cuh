@@ -39,23 +39,44 @@ __attribute__((visibility("hidden"))) cudaError_t enqueue_jobs_init(const JobIni
 __attribute__((visibility("hidden"))) cudaError_t enqueue_jobs_gather(const JobGather *jobs_dev, int n, int64_t most,
                                                                       cudaStream_t st);
 
+// Whether a chain's kernels ask for the largest shared memory of an SM.  The split
+// between it and the L1 cache changes only on an idle SM: left to itself, an SM with
+// blocks of the merge kernels has room for no tile until they are gone, and the
+// tiles started ahead crowd on the other SMs (L=600 in 64-row tiles 43 us a sweep
+// against 32, 3D Potts L=128 84 against 71, every option at L=1920 81 against 68).
+// The PCC kernels read through L1 (L=1001 52.5 us, with the preference 54.0), and so
+// do the unions of the topological rule, which a grid of one wave does not crowd
+// (L=800 46.1 against 47.9); a grid that leaves half the GPU to its successors has
+// nothing to gain (2D Potts L=64 22.6 against 23.3).
+inline bool chain_all_shared(int64_t n_tiles, bool pcc, bool wind)
+{
+    return !pcc && (wind ? n_tiles > FIRST_WAVE_SMS : 8 * n_tiles > FIRST_WAVE_SMS);
+}
+
 // Launches kernel k; chained: as a dependent of the kernel before it in the
 // stream, which it may overlap (chain_next / chain_wait in sw_device.cuh).  The
 // first kernel after anything else in the stream is not chained.
 template <typename... P, typename... A>
 cudaError_t launch_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, bool chained,
-                          A... args)
+                          bool all_shared, A... args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = chained ? 1 : 0;
+    cudaLaunchAttribute at[2]{};
+    unsigned n = 0;
+    if (all_shared) {
+        at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    }
+    if (chained) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 

@@ -12,6 +12,7 @@
 // nodes) is fully rewritten by each sweep before it is read, so only the
 // lattice descriptor, the tile table and the caller's observables are set up
 // (zeroed where they accumulate) at the start of every call.
+// A lattice of one tile (L <= 128) is a single kernel that needs none of this.
 //
 // Costs and rules:
 //   - SW_STATIC_MAX_L x SW_STATIC_MAX_L is the largest lattice; the array
@@ -21,7 +22,7 @@
 //     different streams, or from different threads) race and corrupt each
 //     other.  Serialise them.
 //   - The first call on a device looks the array's device address up
-//     (cudaGetSymbolAddress) and raises the tile kernel's shared-memory limit
+//     (cudaGetSymbolAddress) and raises the tile kernels' shared-memory limits
 //     on that device; make that first call before any stream capture begins.
 //   - The kernels store spins 8 bytes, labels 16 bytes and observables 8
 //     bytes at a time: spin_out must be 8-byte, labels_out 16-byte and
@@ -135,7 +136,13 @@ extern "C" int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_
         return enqueue_one(o, st) == cudaSuccess ? SW_OK : SW_ERR_CUDA;
     }
 
-    const int tiles_x = (L + TW - 1) / TW, tiles_y = (L + TH_STATIC - 1) / TH_STATIC;
+    // 32 rows where the scratch holds as many tiles of them, L <= 512 (a call at
+    // L=300 with its copies 55 us against 65 in 128-row tiles; sw_engine.cu's
+    // pick_tile_height says why), with fewer nodes and codes than MAX_TILES_STATIC of
+    // the highest
+    const int tiles_x = (L + TW - 1) / TW;
+    const int th = tiles_x * ((L + 31) / 32) <= MAX_TILES_STATIC ? 32 : TH_STATIC;
+    const int tiles_y = (L + th - 1) / th;
     Replica R{};
     R.L = L;
     R.tiles_x = tiles_x;
@@ -173,8 +180,8 @@ extern "C" int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_
     a.n_tiles = tiles_x * tiles_y;
     a.jbase = reinterpret_cast<const int32_t *>(scratch + OFF_JBASE);
     a.j = 0;   // start the sweep (bonds, tile labels, border nodes) ...
-    if (enqueue_launch_th(TH_STATIC, a, false, 0, st, false) != cudaSuccess) return SW_ERR_CUDA;
+    if (enqueue_launch_th(th, a, false, 0, st, false) != cudaSuccess) return SW_ERR_CUDA;
     a.j = 1;   // ... and finish it (cluster flip, spins, labels, observables)
-    if (enqueue_tile(TH_STATIC, a, false, 0, st, true) != cudaSuccess) return SW_ERR_CUDA;
+    if (enqueue_tile(th, a, false, 0, st, true) != cudaSuccess) return SW_ERR_CUDA;
     return SW_OK;
 }

@@ -1137,7 +1137,7 @@ struct PMC {
 template <int DIM, bool W>
 __global__ void __launch_bounds__(PMC<DIM>::UT, W ? PMC<DIM>::WB : PMC<DIM>::UB) k_pmerge_union(const PottsDev p, int j, DevObs *obs)
 {
-    const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
+    const bool late = W || (p.flags & RF_PCC) || chain_crowds(p.ntiles);   // (sw_device.cuh)
     if (!late) chain_next();
     chain_wait();
     if (late) chain_next();
@@ -1271,7 +1271,7 @@ __global__ void __launch_bounds__(PMC<DIM>::UT, W ? PMC<DIM>::WB : PMC<DIM>::UB)
 template <int DIM, bool W>
 __global__ void __launch_bounds__(PMC<DIM>::MT) k_pmerge_resolve(const PottsDev p, int j, bool last, uint64_t sweep0, DevObs *obs)
 {
-    const bool late = W || (p.flags & RF_PCC);   // (sw_device.cuh)
+    const bool late = W || (p.flags & RF_PCC) || chain_crowds(p.ntiles);   // (sw_device.cuh)
     if (!late) chain_next();
     chain_wait();
     if (late) chain_next();
@@ -1498,13 +1498,19 @@ cudaError_t potts_prepare()
     return err;
 }
 
+bool all_shared(const PottsDev &p)
+{
+    return chain_all_shared(p.ntiles, (p.flags & RF_PCC) != 0, (p.flags & RF_WIND) != 0);
+}
+
 template <int DIM>
 cudaError_t launch_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
                         bool chained)
 {
     const bool feat = (p.flags & (RF_PCC | RF_OPEN | RF_CSIZE | RF_WIND)) != 0;
     return launch_kernel(feat ? k_ptile<DIM, FEAT_TILE> : k_ptile<DIM, 0>, dim3((unsigned)p.ntiles), PG<DIM>::NT,
-                         ptile_smem<DIM>((p.flags & RF_PCC) && !(p.flags & RF_WIND)), st, chained, p, j, nsweeps, sweep0, obs);
+                         ptile_smem<DIM>((p.flags & RF_PCC) && !(p.flags & RF_WIND)), st, chained, all_shared(p), p, j, nsweeps,
+                         sweep0, obs);
 }
 
 template <int DIM>
@@ -1516,7 +1522,7 @@ cudaError_t launch_merge(const PottsDev &p, int j, int nsweeps, uint64_t sweep0,
     const dim3 tiles((unsigned)p.ntiles);
     cudaError_t e = cudaSuccess;
     auto go = [&](auto *k, dim3 grid, unsigned threads, auto... args) {
-        if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, args...);
+        if (e == cudaSuccess) e = launch_kernel(k, grid, threads, 0, st, chained, all_shared(p), args...);
     };
     const bool last = j == nsweeps - 1;
     if (wind) {

@@ -96,3 +96,37 @@ def test_static_sweep_of_one_tile(sw, L):
             assert obs.cpu().numpy().tobytes() == ref.observables().tobytes()
             np.testing.assert_array_equal(out.cpu().numpy(), ref.spins())
             np.testing.assert_array_equal(labels.cpu().numpy(), ref.labels())
+
+
+# The height that a lattice gets without asking, at both sides of the rule's lines.
+@pytest.mark.parametrize("L,opts", [(64, {"csize": True}), (65, {"csize": True}), (65, {"pcc": True}),
+                                    (128, {"wind": True}), (129, {}), (384, {"wind": True}), (385, {"wind": True}),
+                                    (512, {"pcc": True}), (513, {"pcc": True}), (1920, {}), (1921, {})])
+def test_default_heights(sw, orc, L, opts):
+    kw = {"pcc": True} if "pcc" in opts else {"T": 2.269185}
+    rest = {k: v for k, v in opts.items() if k != "pcc"}
+    with sw.Lattice(L, seed=L, **kw, **rest) as lat, sw.Lattice(L, seed=L, tile_h=64, **kw, **rest) as ref:
+        for n in (1, 3):
+            lat.sweep(n)
+            ref.sweep(n)
+            assert lat.observables().tobytes() == ref.observables().tobytes()
+            np.testing.assert_array_equal(lat.spins(), ref.spins())
+            np.testing.assert_array_equal(lat.labels(), ref.labels())
+            np.testing.assert_array_equal(lat.bonds(), ref.bonds())
+
+
+@pytest.mark.parametrize("L", [129, 512, 513, 1024])   # 32-row tiles up to L = 512
+def test_static_sweep_of_tiles(sw, L):
+    torch = pytest.importorskip("torch")
+    thr = sw.sw_threshold(1.0, 2.269185)
+    with sw.Lattice(L, p=thr / 2.0 ** 32, seed=7, tile_h=96) as ref:
+        spins = torch.from_numpy(ref.spins()).cuda()
+        out, labels = torch.empty_like(spins), torch.empty(L * L, dtype=torch.int32, device="cuda")
+        obs = torch.empty(sw.OBS_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        sw.sw_sweep_static(spins.data_ptr(), out.data_ptr(), labels.data_ptr(), obs.data_ptr(), L, thr, 7, 0,
+                           torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        ref.sweep(1)
+        assert obs.cpu().numpy().tobytes() == ref.observables().tobytes()
+        np.testing.assert_array_equal(out.cpu().numpy(), ref.spins())
+        np.testing.assert_array_equal(labels.cpu().numpy(), ref.labels())
