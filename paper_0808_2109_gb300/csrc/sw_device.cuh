@@ -463,6 +463,10 @@ __device__ __forceinline__ uint32_t interleave16(uint32_t X, uint32_t Z, int hf)
 constexpr uint32_t INFO_BORDER = 0x80000000u;
 constexpr uint32_t INFO_INTERIOR = 0x40000000u;
 __device__ __forceinline__ int info_slot(int v) { return (v & 0xFFFF) >> 2; }
+// Cluster sizes (RF_CSIZE): bits 16 to 29 of a record, of its copies and of the
+// entry of a node that points at its root by index count sites.
+constexpr int SIZE_SHIFT = 16, SIZE_MASK = 0x3FFF << SIZE_SHIFT, FOREST_MASK = 0x7FFF;
+static_assert(128 * PW <= FOREST_MASK + 1, "a forest index fits below the count");
 
 // Run heads of a 32-site row word inside one sub-tile: bit x is set iff
 // x == 0 or the link (x-1, x) is not a bond (bit 31 of h, the link leaving
@@ -1038,11 +1042,12 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             // clusters that touch a tile border: their sizes were summed at their
             // root nodes by the merge; each root node is in exactly one tile
             if (csz) {
+                long long c[SPT];
+#pragma unroll
+                for (int q = 0; q < SPT; ++q) c[q] = tid + q * NT < S ? R.csize[(size_t)t.lt * S + tid + q * NT] : 0;
                 unsigned long long c2 = 0ull;
-                for (int s = tid; s < S; s += NT) {
-                    const long long c = R.csize[(size_t)t.lt * S + s];
-                    c2 += (unsigned long long)(c * c);
-                }
+#pragma unroll
+                for (int q = 0; q < SPT; ++q) c2 += (unsigned long long)(c[q] * c[q]);
                 warp_add64(&sm.acc_c2[0], c2);
             }
         }
@@ -1141,7 +1146,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (lane == 0 && ncl) atomicAdd(&sm.acc[3], ncl);
             // the other labels' nodes take a copy of their root's record where it
             // is there already, so that most sites find it two loads away (cluster
-            // sizes are added at the roots: their index instead)
+            // sizes: those of interior clusters its index instead)
             for (; linked; linked &= linked - 1) {
                 const int x = col + (__ffs(linked) - 1) * PW;
                 int p = sm.par[x], q = sm.par[p];
@@ -1149,7 +1154,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                     p = q;
                     q = sm.par[p];
                 }
-                sm.par[x] = q == p || csz ? p : q;
+                sm.par[x] = q == p || (csz && q >= 0) ? p : q;
             }
         }
 #pragma unroll
@@ -1191,76 +1196,88 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             const int x = 32 * sx + lane;
             uint16_t *cp = code + y0 * TW + x;
             const int *pp = sm.par + y0 * PW + x;
-            if (!((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext)) && rows == 32 && 32 * sx + 32 <= t.tw) {
+            // Cluster sizes: every label's node counts its sites, a run at a time, in
+            // the bits of its entry that a record, its copy or a root's index leave
+            // free (SIZE_SHIFT; a label has at most 2^10 sites).  Gathered down the
+            // columns per root, three loads a site and a branch, the loop took 14.3K
+            // clocks a tile at L=2048, T_c, against 8.9K (plain codes 2.0K); a match of
+            // the row's labels before the atomics is slower, 71 us a sweep against 64.
+            auto count = [&](int r, int v) {
+                const uint32_t heads = run_heads(sm.b[y0 + r][2 * sx]), n = heads >> lane;
+                if (n & 1u) {
+                    const uint32_t len = n >> 1 ? (uint32_t)__ffs(n >> 1) : 32u - lane;
+                    atomicAdd(&sm.par[(born >> r) & 1u ? (y0 + r) * PW + x : v], (int)(len << SIZE_SHIFT));
+                }
+            };
+            auto entry = [&](int v) { return sm.par[(F & FEAT_CSIZE) ? v & FOREST_MASK : v]; };
+            if ((F & FEAT_CSIZE) && csz)
+                for (int s = tid; s < S; s += NT) sm.u.finfo[s] = 0u;   // the sizes of border pieces (below)
+            if (!((F & FEAT_PCC) && ext) && rows == 32 && 32 * sx + 32 <= t.tw) {
 #pragma unroll 2
                 for (int r = 0; r < 32; r += 4) {
                     int v[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) v[q] = pp[(r + q) * PW];
+                    if ((F & FEAT_CSIZE) && csz) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) count(r + q, v[q]);
+                    }
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
-                        if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = sm.par[v[q]];   // records: negative or >= INFO_INTERIOR
+                        if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = entry(v[q]);   // records: negative or >= INFO_INTERIOR
                     while (min(min((uint32_t)v[0], (uint32_t)v[1]), min((uint32_t)v[2], (uint32_t)v[3])) < INFO_INTERIOR) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = sm.par[v[q]];
+                            if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = entry(v[q]);
                     }
 #pragma unroll
                     for (int q = 0; q < 4; ++q) cp[(r + q) * TW] = (uint16_t)v[q];
                 }
             } else {
                 const bool site = x < t.tw;
-                // Cluster sizes and piece masks, gathered down the lane's column and
-                // added when its cluster changes: a size goes to bits 16-30 of the
-                // root's record (a piece holds at most TW*TH = 2^14 sites, an interior
-                // cluster at most (TW-2)(TH-2) < 2^14, so neither field overflows into
-                // the record's flag bits; the codes read bits 0-15 only), the columns
-                // and rows of a border piece to its masks (only a piece touching the
-                // border can belong to a spanning cluster).
-                const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext);
-                int cur = -1, cur_v = 0;
+                // Piece masks, gathered down the lane's column and added when its
+                // cluster changes: the columns and rows of a border piece (only a
+                // piece touching the border can belong to a spanning cluster).
+                int cur = 0;
                 uint32_t cur_rows = 0u;
                 auto flush = [&]() {
-                    if (!cur_rows) return;
-                    if (csz) atomicAdd(&sm.par[cur], __popc(cur_rows) << 16);
-                    if (ext && cur_v < 0) {
-                        const int sl = info_slot(cur_v);
+                    if (cur_rows && cur < 0) {
+                        const int sl = info_slot(cur);
                         atomicOr(&sm.pm[sl][sx], 1u << lane);
                         atomicOr(&sm.pm[sl][4 + (y0 >> 5)], cur_rows);
                     }
                 };
                 for (int r = 0; r < rows; r += 4) {   // four rows' look-ups in flight
-                    int v[4], root[4];
+                    int v[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        root[q] = (y0 + r + q) * PW + x;
+                    for (int q = 0; q < 4; ++q)
                         v[q] = site && r + q < rows ? pp[(r + q) * PW] : (int)(INFO_INTERIOR | 4u * S);
+                    if ((F & FEAT_CSIZE) && csz) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (site && r + q < rows) count(r + q, v[q]);
                     }
                     while (min(min((uint32_t)v[0], (uint32_t)v[1]), min((uint32_t)v[2], (uint32_t)v[3])) < INFO_INTERIOR) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            if ((uint32_t)v[q] < INFO_INTERIOR) {
-                                root[q] = v[q];
-                                v[q] = sm.par[v[q]];
-                            }
+                            if ((uint32_t)v[q] < INFO_INTERIOR) v[q] = entry(v[q]);
                     }
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         if (r + q >= rows) break;
                         cp[(r + q) * TW] = (uint16_t)v[q];
-                        if (gather && site) {
-                            const int key = csz ? root[q] : v[q];
+                        if ((F & FEAT_PCC) && ext && site) {
+                            const int key = v[q] & ~SIZE_MASK;
                             if (key != cur) {
                                 flush();
                                 cur = key;
-                                cur_v = v[q];
                                 cur_rows = 0u;
                             }
                             cur_rows |= 1u << (r + q);
                         }
                     }
                 }
-                if (gather) flush();
+                if ((F & FEAT_PCC) && ext) flush();
             }
         }
         if ((F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext)) {
@@ -1268,19 +1285,29 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (ext)
                 for (int q = tid; q < S * 8; q += NT) R.pmask[(size_t)t.lt * S * 8 + q] = (&sm.pm[0][0])[q];
             if (csz) {
-                // every root: an interior cluster adds its |C|^2; a border piece
-                // hands its size to its representative node for the merge
+                // every label's count to its piece: a border piece's by its slot, an
+                // interior cluster's (at most (TW-2)(TH-2) < 2^14 sites) at its root
                 const int col = 32 * (warp / TWW) * PW + 32 * (warp & (TWW - 1)) + lane;
+                for (uint32_t bits = born; bits; bits &= bits - 1) {
+                    const int v = sm.par[col + (__ffs(bits) - 1) * PW];
+                    if (v < 0)
+                        atomicAdd(&sm.u.finfo[info_slot(v)], (uint32_t)(v & SIZE_MASK) >> SIZE_SHIFT);
+                    else if ((uint32_t)v < INFO_INTERIOR)
+                        atomicAdd(&sm.par[v & FOREST_MASK], v & SIZE_MASK);
+                }
+                __syncthreads();
+                // an interior cluster adds its |C|^2; a border piece hands its size
+                // to its representative node for the merge
                 unsigned long long c2 = 0ull;
                 for (uint32_t bits = born; bits; bits &= bits - 1) {
                     const int v = sm.par[col + (__ffs(bits) - 1) * PW];
-                    if (v < 0) {   // piece size: bits 16-30 (bit 31 is the border flag)
-                        R.psize[(size_t)t.lt * S + info_slot(v)] = (int32_t)(((uint32_t)v >> 16) & 0x7FFFu);
-                    } else if ((uint32_t)v >= INFO_INTERIOR) {   // bits 16-29 (bit 30 is the flag)
-                        const unsigned long long size = ((uint32_t)v >> 16) & 0x3FFFu;
+                    if (v >= (int)INFO_INTERIOR) {
+                        const unsigned long long size = (uint32_t)(v & SIZE_MASK) >> SIZE_SHIFT;
                         c2 += size * size;
                     }
                 }
+                for (int s = tid; s < S; s += NT)
+                    if (const uint32_t size = sm.u.finfo[s]) R.psize[(size_t)t.lt * S + s] = (int32_t)size;
                 warp_add64(&sm.acc_c2[1], c2);
                 __syncthreads();
             }
