@@ -408,18 +408,20 @@ __device__ __forceinline__ bool sunite_linked(volatile int *par, int a, int b)
     }
 }
 
-// Threads of a tile CTA: one warp per 32 x 32 sub-tile.
-template <int TH>
+// Threads of a tile CTA: one warp per sub-tile of 32 columns by RS rows.  Sub-tiles
+// of 32 rows have the fewest links between them; where the grid leaves an SM with few
+// warps, more warps that walk fewer rows are faster (tile_rows in sw_launch.cuh).
+template <int TH, int RS = 32>
 struct TileCfg {
-    static constexpr int NT = 4 * TH;           // threads per CTA
+    static constexpr int WT = 4 * TH;           // threads with a 32-site word of the tile
+    static constexpr int NT = WT * (32 / RS);   // threads per CTA
     static constexpr int NW = NT / 32;          // warps = sub-tiles
-    static constexpr int SUBY = TH / 32;        // sub-tile rows
-    // CTAs per SM the register allocation must leave room for: as many as
-    // the shared memory allows (32 rows: eleven CTAs; 64 rows: six; 96 rows:
-    // four; 128 rows: three), which caps a thread at 40 registers.  The
-    // kernel is latency-bound in its union-find, so resident warps pay: three
-    // 128-row CTAs per SM run 19% faster than two.
-    static constexpr int MINB = TH == 32 ? 11 : TH == 64 ? 6 : TH == 96 ? 4 : 3;
+    // CTAs per SM the register allocation must leave room for: as many as the
+    // shared memory allows (32 rows: eleven CTAs; 64 rows: six; 96 rows: four; 128
+    // rows: three), which caps a thread at 40 registers, and with shorter sub-tiles
+    // as many as their grids have.  Resident warps pay: three 128-row CTAs per SM
+    // ran 19% faster than two.
+    static constexpr int MINB = RS == 8 ? 3 : RS == 16 ? 6 : TH == 32 ? 11 : TH == 64 ? 6 : TH == 96 ? 4 : 3;
 };
 
 // Root of x without writing, while other threads replace roots by border
@@ -597,13 +599,13 @@ struct EdgeLinks {
 };
 
 // Both, for all threads of a tile CTA; returns what label_rows does.
-template <int TH>
+template <int TH, int RS = 32>
 __device__ __forceinline__ uint32_t tile_label_rows(volatile int *par, const uint32_t (*B)[2 * TWW], int th, int tw)
 {
-    using E = EdgeLinks<TH, TWW, 32>;
-    const uint32_t born = label_rows<TWW, 32, false>(par, B, th, tw);
+    using E = EdgeLinks<TH, TWW, RS>;
+    const uint32_t born = label_rows<TWW, RS, false>(par, B, th, tw);
     __syncthreads();
-    for (int q = threadIdx.x; q < E::EDGES; q += TileCfg<TH>::NT) {
+    for (int q = threadIdx.x; q < E::EDGES; q += TileCfg<TH, RS>::NT) {
         int ia, ib;
         if (E::link(q, B, th, ia, ib)) shook<2>(par, par[ia], par[ib]);
     }
@@ -843,17 +845,17 @@ constexpr int FEAT_WIND = 4;    // topological rule (RF_WIND)
 constexpr int FEAT_PCC = 8;     // PCC piece masks (RF_PCC)
 constexpr int FEAT_TILE = FEAT_CSIZE | FEAT_OPEN | FEAT_WIND | FEAT_PCC;
 
-template <int TH, int F>
-__global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(const SweepArgs a)
+template <int TH, int RS, int F>
+__global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_tile(const SweepArgs a)
 {
     using SL = Slots<TH>;
     constexpr int S = SL::S;
-    constexpr int NT = TileCfg<TH>::NT;
-    constexpr int NW = TileCfg<TH>::NW;
+    using TC = TileCfg<TH, RS>;
+    constexpr int NT = TC::NT, NW = TC::NW, WT = TC::WT;
     constexpr int SPT = (S + NT - 1) / NT;   // node slots per thread
     constexpr int NQ = TH * TW / 8 / NT;     // 8-site groups per thread
     static_assert(NQ * 8 * NT == TH * TW, "tile sites must split into 8-site groups");
-    static_assert(TH * TWW == NT && NW * 8 == TH, "one 32-site word of the tile per thread, eight rows per warp");
+    static_assert(TH * TWW == WT, "one 32-site word of the tile per thread of the first WT, eight rows per warp");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileSmem<TH> &sm = *reinterpret_cast<TileSmem<TH> *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
@@ -912,7 +914,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     // A block of the first wave may start before the merge is done: it draws
     // first and then waits and loads.  Later ones find the merge done.  (A PCC
     // lattice's threshold comes from the merge: no draws before it.)
-    const bool early = g < FIRST_WAVE_SMS * TileCfg<TH>::MINB && !pcc;
+    const bool early = g < FIRST_WAVE_SMS * TC::MINB && !pcc;
     if (!early) finish_loads();
     if (tid < 4) sm.acc[tid] = 0;
     if ((F & FEAT_CSIZE) && tid < 2) sm.acc_c2[tid] = 0ull;
@@ -1017,7 +1019,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
     //      sweep k-1 and the bonds of sweep k
     const uint32_t vm = wy < t.th ? valid_mask(wc, t.tw) : 0u;
     const int last_c = (t.tw - 1) >> 5, last_b = (t.tw - 1) & 31;   // the tile's last column
-    {
+    if (WT == NT || tid < WT) {
         uint32_t eqr = 0u, eqd = 0u, cur = 0u;   // links that exist and join equal spins
         uint32_t vr = vm, vd = vm;
         if (wy < t.th) {
@@ -1038,17 +1040,6 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (lane == 0) {
                 atomicAdd(&sm.acc[0], ws);
                 atomicAdd(&sm.acc[1], wm);
-            }
-            // clusters that touch a tile border: their sizes were summed at their
-            // root nodes by the merge; each root node is in exactly one tile
-            if (csz) {
-                long long c[SPT];
-#pragma unroll
-                for (int q = 0; q < SPT; ++q) c[q] = tid + q * NT < S ? R.csize[(size_t)t.lt * S + tid + q * NT] : 0;
-                unsigned long long c2 = 0ull;
-#pragma unroll
-                for (int q = 0; q < SPT; ++q) c2 += (unsigned long long)(c[q] * c[q]);
-                warp_add64(&sm.acc_c2[0], c2);
             }
         }
         if (start) {
@@ -1075,6 +1066,17 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             *reinterpret_cast<uint2 *>(&sm.b[wy][2 * wc]) =
                 make_uint2(h & valid_mask(wc, t.tw - 1), wy < t.th - 1 ? v : 0u);
         }
+    }
+    // clusters that touch a tile border: their sizes were summed at their root
+    // nodes by the merge; each root node is in exactly one tile
+    if ((F & FEAT_CSIZE) && csz && fin) {
+        long long c[SPT];
+#pragma unroll
+        for (int q = 0; q < SPT; ++q) c[q] = tid + q * NT < S ? R.csize[(size_t)t.lt * S + tid + q * NT] : 0;
+        unsigned long long c2 = 0ull;
+#pragma unroll
+        for (int q = 0; q < SPT; ++q) c2 += (unsigned long long)(c[q] * c[q]);
+        warp_add64(&sm.acc_c2[0], c2);
     }
     if (start) {
         // The SPIN-stream bit of every site of the tile, for the clusters that end
@@ -1103,7 +1105,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
 
     if (start) {
         // Step 2 inside the tile (Hoshen-Kopelman's role in Sec. II.A slave step 1)
-        const uint32_t born = tile_label_rows<TH>(sm.par, sm.b, t.th, t.tw);
+        const uint32_t born = tile_label_rows<TH, RS>(sm.par, sm.b, t.th, t.tw);
 
         // One node per border site: key = global index of the piece's local root,
         // parent = the piece's first border slot (the representative).
@@ -1124,7 +1126,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         // born in column x of its sub-tile.
         const bool last_start = j == R.nsweeps - 1;
         {
-            const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
+            const int sx = SubTile<TWW, RS>::sx(), y0 = SubTile<TWW, RS>::y0();
             const int col = y0 * PW + 32 * sx + lane;
             uint32_t linked = 0u;
             int ncl = 0;
@@ -1191,8 +1193,8 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
         // Every site's 2-byte code, the low half of its root's record.  Lane =
         // column: a site's entry, its label's node, seldom a third one.
         {
-            const int sx = warp & (TWW - 1), y0 = 32 * (warp / TWW);
-            const int rows = min(32, t.th - y0);
+            const int sx = SubTile<TWW, RS>::sx(), y0 = SubTile<TWW, RS>::y0();
+            const int rows = min(RS, t.th - y0);
             const int x = 32 * sx + lane;
             uint16_t *cp = code + y0 * TW + x;
             const int *pp = sm.par + y0 * PW + x;
@@ -1212,9 +1214,9 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             auto entry = [&](int v) { return sm.par[(F & FEAT_CSIZE) ? v & FOREST_MASK : v]; };
             if ((F & FEAT_CSIZE) && csz)
                 for (int s = tid; s < S; s += NT) sm.u.finfo[s] = 0u;   // the sizes of border pieces (below)
-            if (!((F & FEAT_PCC) && ext) && rows == 32 && 32 * sx + 32 <= t.tw) {
+            if (!((F & FEAT_PCC) && ext) && rows == RS && 32 * sx + 32 <= t.tw) {
 #pragma unroll 2
-                for (int r = 0; r < 32; r += 4) {
+                for (int r = 0; r < RS; r += 4) {
                     int v[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) v[q] = pp[(r + q) * PW];
@@ -1244,7 +1246,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
                     if (cur_rows && cur < 0) {
                         const int sl = info_slot(cur);
                         atomicOr(&sm.pm[sl][sx], 1u << lane);
-                        atomicOr(&sm.pm[sl][4 + (y0 >> 5)], cur_rows);
+                        atomicOr(&sm.pm[sl][4 + (y0 >> 5)], cur_rows << (y0 & 31));
                     }
                 };
                 for (int r = 0; r < rows; r += 4) {   // four rows' look-ups in flight
@@ -1287,7 +1289,7 @@ __global__ void __launch_bounds__(TileCfg<TH>::NT, TileCfg<TH>::MINB) k_tile(con
             if (csz) {
                 // every label's count to its piece: a border piece's by its slot, an
                 // interior cluster's (at most (TW-2)(TH-2) < 2^14 sites) at its root
-                const int col = 32 * (warp / TWW) * PW + 32 * (warp & (TWW - 1)) + lane;
+                const int col = SubTile<TWW, RS>::y0() * PW + 32 * SubTile<TWW, RS>::sx() + lane;
                 for (uint32_t bits = born; bits; bits &= bits - 1) {
                     const int v = sm.par[col + (__ffs(bits) - 1) * PW];
                     if (v < 0)
@@ -1432,7 +1434,7 @@ template <int TH>
 __global__ void __launch_bounds__(OneCfg<TH>::NT, 1) k_one(const OneArgs a)
 {
     constexpr int WX = OneCfg<TH>::WX, RS = OneCfg<TH>::RS, NT = OneCfg<TH>::NT, NW = NT / 32;
-    constexpr int WT = TileCfg<TH>::NT;   // threads with a word of the tile; their warps draw
+    constexpr int WT = TileCfg<TH>::WT;   // threads with a word of the tile; their warps draw
     using E = EdgeLinks<TH, WX, RS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OneSmem<TH> &sm = *reinterpret_cast<OneSmem<TH> *>(smem_raw);

@@ -40,8 +40,11 @@ cudaError_t tile_prepare()
     if (dev < 0 || dev >= PREP_MAX_DEVICES) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
     if (done[dev]) return cudaSuccess;
-    const void *fn[2] = {(const void *)k_tile<TH, 0>, (const void *)k_tile<TH, FEAT_TILE>};
-    for (int f = 0; f < 2 && err == cudaSuccess; ++f)
+    constexpr int R1 = TH == 32 ? 16 : 32, R2 = TH == 32 ? 8 : 32;   // (tile_rows)
+    const void *fn[6] = {(const void *)k_tile<TH, 32, 0>, (const void *)k_tile<TH, 32, FEAT_TILE>,
+                         (const void *)k_tile<TH, R1, 0>, (const void *)k_tile<TH, R1, FEAT_TILE>,
+                         (const void *)k_tile<TH, R2, 0>, (const void *)k_tile<TH, R2, FEAT_TILE>};
+    for (int f = 0; f < (TH == 32 ? 6 : 2) && err == cudaSuccess; ++f)
         err = cudaFuncSetAttribute(fn[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem<TH>(true));
     if (err == cudaSuccess)
         err = cudaFuncSetAttribute((const void *)k_one<TH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -82,12 +85,23 @@ cudaError_t enqueue_one(const OneArgs &a, cudaStream_t st)
     }
 }
 
+template <int TH, int RS>
+cudaError_t launch_tile_rows(const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
+{
+    return launch_kernel(pcc || (feat & FEAT_TILE) ? k_tile<TH, RS, FEAT_TILE> : k_tile<TH, RS, 0>, dim3(a.n_tiles),
+                         TileCfg<TH, RS>::NT, tile_smem<TH>(pcc), st, chained,
+                         chain_all_shared(a.n_tiles, pcc, (feat & FEAT_WIND) != 0), a);
+}
+
 template <int TH>
 cudaError_t launch_tile(const SweepArgs &a, bool pcc, int feat, cudaStream_t st, bool chained)
 {
-    return launch_kernel(pcc || (feat & FEAT_TILE) ? k_tile<TH, FEAT_TILE> : k_tile<TH, 0>, dim3(a.n_tiles),
-                         TileCfg<TH>::NT, tile_smem<TH>(pcc), st, chained,
-                         chain_all_shared(a.n_tiles, pcc, (feat & FEAT_WIND) != 0), a);
+    if constexpr (TH == 32) {
+        const int rs = tile_rows(a.n_tiles);
+        if (rs == 8) return launch_tile_rows<TH, 8>(a, pcc, feat, st, chained);
+        if (rs == 16) return launch_tile_rows<TH, 16>(a, pcc, feat, st, chained);
+    }
+    return launch_tile_rows<TH, 32>(a, pcc, feat, st, chained);
 }
 
 // The merge of launch group j: unions across tile edges, every node's resolved
@@ -215,18 +229,17 @@ int sw_cuda_fail(cudaError_t e, int line = 0)
     return SW_ERR_CUDA;
 }
 
-// Tile height used for an L x L lattice: a SW_FLAG_TILE_* flag, else the first of
-//   - one tile for a side of at most 128, where it has no features (k_one) or the
-//     topological rule (L=110 35.3 us a sweep against 40.5 in 32-row tiles), or at
-//     most 64;
+// Tile height used for an L x L lattice: a SW_FLAG_TILE_* flag, else
+//   - one tile for a side of at most 128 without features (k_one);
 //   - 32 rows while they are at most six CTAs an SM (L <= 1920): the sweep is then
-//     bound by the latency of a tile, which is shortest where one warp walks 32 rows
-//     and a border has few nodes (L=300 26.7 us against 29.3 with 96 rows, L=1001
-//     31.0 against 32.2, L=1600 36.2 against 47.1; cluster sizes at L=1001 43.1
-//     against 57.9; at L=2048 45.3 against 44.9).  PCC and the topological rule pay
-//     more for the longer borders: PCC takes 32 rows up to half a CTA an SM (L <=
-//     512; 45.7 against 49.3 at L=512, 54.1 against 53.4 at 1001), the rule alone up
-//     to a third (L <= 384; 38.2 against 39.4 at L=200, 44.0 against 42.9 at 512);
+//     bound by the latency of a tile, which is shortest where a warp walks few rows
+//     (tile_rows) and a border has few nodes (L=300 22.1 us a sweep against 29.3 with
+//     96 rows, L=1001 27.5 against 32.2, L=1600 36.6 against 47.1; L=2048 46.3 against
+//     44.9).  PCC and the topological rule pay more for the longer borders: PCC takes
+//     32 rows up to four CTAs an SM (L=1500 58.4 against 61.6, L=1600 64.3 against
+//     62.3), the rule up to one (L=700 43.1 against 46.1, L=1001 49.8 against 48.4) and
+//     together with PCC or cluster sizes up to two (every option at L=1001 52.6 against
+//     55.3, PCC by the rule 51.6 against 52.6 and at L=1200 56.5 against 53.5);
 //   - 96 rows (four CTAs fit on an SM, three of 128).
 int pick_tile_height(int L, uint32_t flags, bool pcc)
 {
@@ -234,12 +247,11 @@ int pick_tile_height(int L, uint32_t flags, bool pcc)
     if (flags & SW_FLAG_TILE_64) return 64;
     if (flags & SW_FLAG_TILE_96) return 96;
     if (flags & SW_FLAG_TILE_128) return 128;
-    if (L <= 32) return 32;
-    if (L <= 64) return 64;
-    const bool wind = (flags & SW_FLAG_WIND) != 0;
-    if (L <= 128 && (wind || !(pcc || (flags & SW_FLAG_CSIZE)))) return 128;
+    const bool wind = (flags & SW_FLAG_WIND) != 0, csize = (flags & SW_FLAG_CSIZE) != 0;
+    if (L <= 128 && !wind && !csize && !pcc) return L <= 32 ? 32 : L <= 64 ? 64 : 128;
+    const int per_sm = wind ? (pcc || csize ? 2 : 1) : pcc ? 4 : 6;
     const int64_t tiles = (int64_t)((L + TW - 1) / TW) * ((L + 31) / 32);
-    return tiles <= (pcc ? FIRST_WAVE_SMS / 2 : wind ? FIRST_WAVE_SMS / 3 : 6 * FIRST_WAVE_SMS) ? 32 : 96;
+    return tiles <= per_sm * FIRST_WAVE_SMS ? 32 : 96;
 }
 
 std::atomic<int> g_alloc_skip{0}, g_alloc_failures{0};   // sw_debug_fail_allocations

@@ -53,6 +53,16 @@ inline bool chain_all_shared(int64_t n_tiles, bool pcc, bool wind)
     return !pcc && (wind ? n_tiles > FIRST_WAVE_SMS : 8 * n_tiles > FIRST_WAVE_SMS);
 }
 
+// Rows of a sub-tile of the 32-row tiles: 8 (16 warps a CTA) while there is at most
+// one CTA an SM, 16 up to six, 32 beyond (8, 16 and 32 rows at T_c: L=300 22.2, 23.7
+// and 27.3 us a sweep, L=700 24.0, 25.7 and 29.5, L=1400 36.9, 31.3 and 33.6, L=1920
+// 45.4, 38.9 and 43.0, L=4096 153, 121 and 112; with cluster sizes L=300 27.6, 30.3 and
+// 36.2).
+inline int tile_rows(int n_tiles)
+{
+    return n_tiles <= FIRST_WAVE_SMS ? 8 : n_tiles <= 6 * FIRST_WAVE_SMS ? 16 : 32;
+}
+
 // Launches kernel k; chained: as a dependent of the kernel before it in the
 // stream, which it may overlap (chain_next / chain_wait in sw_device.cuh).  The
 // first kernel after anything else in the stream is not chained.

@@ -137,7 +137,7 @@ extern "C" int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_
     }
 
     // 32 rows where the scratch holds as many tiles of them, L <= 512 (a call at
-    // L=300 with its copies 55 us against 65 in 128-row tiles; sw_engine.cu's
+    // L=300 with its copies 42 us against 65 in 128-row tiles; sw_engine.cu's
     // pick_tile_height says why), with fewer nodes and codes than MAX_TILES_STATIC of
     // the highest
     const int tiles_x = (L + TW - 1) / TW;

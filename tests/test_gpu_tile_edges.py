@@ -101,7 +101,10 @@ def test_static_sweep_of_one_tile(sw, L):
 # The height that a lattice gets without asking, at both sides of the rule's lines.
 @pytest.mark.parametrize("L,opts", [(64, {"csize": True}), (65, {"csize": True}), (65, {"pcc": True}),
                                     (128, {"wind": True}), (129, {}), (384, {"wind": True}), (385, {"wind": True}),
-                                    (512, {"pcc": True}), (513, {"pcc": True}), (1920, {}), (1921, {})])
+                                    (512, {"pcc": True}), (513, {"pcc": True}), (1920, {}), (1921, {}),
+                                    (30, {"wind": True}), (768, {"wind": True}), (769, {"wind": True}),
+                                    (1056, {"wind": True, "csize": True}), (1057, {"wind": True, "csize": True}),
+                                    (1536, {"pcc": True}), (1537, {"pcc": True})])
 def test_default_heights(sw, orc, L, opts):
     kw = {"pcc": True} if "pcc" in opts else {"T": 2.269185}
     rest = {k: v for k, v in opts.items() if k != "pcc"}
@@ -130,3 +133,19 @@ def test_static_sweep_of_tiles(sw, L):
         assert obs.cpu().numpy().tobytes() == ref.observables().tobytes()
         np.testing.assert_array_equal(out.cpu().numpy(), ref.spins())
         np.testing.assert_array_equal(labels.cpu().numpy(), ref.labels())
+
+
+# 32-row tiles have sub-tiles of 8, 16 or 32 rows by the size of the grid.
+@pytest.mark.parametrize("opts", [{}, {"csize": True, "open": True}, {"pcc": True}, {"wind": True}])
+@pytest.mark.parametrize("L", [609, 801, 846, 1939, 1985])
+def test_rows_of_subtiles(sw, L, opts):
+    kw = {"pcc": True} if "pcc" in opts else {"T": 2.269185}
+    rest = {k: v for k, v in opts.items() if k != "pcc"}
+    with sw.Lattice(L, seed=L, tile_h=32, **kw, **rest) as lat, sw.Lattice(L, seed=L, tile_h=96, **kw, **rest) as ref:
+        for n in (1, 3):
+            lat.sweep(n)
+            ref.sweep(n)
+            assert lat.observables().tobytes() == ref.observables().tobytes()
+            np.testing.assert_array_equal(lat.spins(), ref.spins())
+            np.testing.assert_array_equal(lat.labels(), ref.labels())
+            np.testing.assert_array_equal(lat.bonds(), ref.bonds())
