@@ -68,7 +68,8 @@ __device__ __forceinline__ uint8_t cluster_state(uint32_t r, uint32_t klo, uint3
 
 // ------------------------------------------------------------ tile geometry
 // A tile is TX x TY (x TZ) sites; its rows (y, z) are row index r = y + TY z,
-// each of TWW 32-site words.  One thread per word: NT = 256 threads.
+// each of TWW 32-site words.  One thread per word: WT = 256 threads.  Where the grid
+// leaves an SM with few warps a CTA has M = 2 or 4 times as many (launch_tile).
 // Face nodes: for each axis a, a "-" face (local coordinate a = 0) and a "+"
 // face (the tile's last valid coordinate along a), each of Fa slots indexed
 // by the site's other coordinates (axis 0: y + TY z; axis 1: x + TX z; axis
@@ -80,8 +81,7 @@ struct PG {
     static constexpr int TZ = DIM == 2 ? 1 : 16;
     static constexpr int TWW = TX / 32;
     static constexpr int NR = TY * TZ;          // rows
-    static constexpr int NT = NR * TWW;         // threads
-    static constexpr int NW = NT / 32;          // warps
+    static constexpr int WT = NR * TWW;         // threads that own a word (and threads of a tile CTA, M = 1)
     static constexpr int NS = TX * TY * TZ;     // sites
     static constexpr int PW = TX + 1;           // forest row pitch (rows on distinct banks)
     static constexpr int RS = TX + 4;           // state row pitch in bytes (the halo column, padded)
@@ -91,9 +91,7 @@ struct PG {
     static constexpr int S = 2 * FT;            // node slots
     static constexpr int CW = FT / 32;          // crossing-bit words
     static constexpr int PMW = DIM == 2 ? 6 : 2;   // PCC coverage words of a piece
-    static constexpr int NQ = NS / 8 / NT;      // 8-site groups per thread
-    static constexpr int SPT = (S + NT - 1) / NT;  // node slots per thread
-    static_assert(NT == 256 && NQ == 4, "tile launch shape");
+    static_assert(WT == 256 && NS == 8 * 4 * WT, "tile launch shape");
     static_assert(F0 % 32 == 0 && F1 % 32 == 0 && F2 % 32 == 0, "faces of whole words");
     static_assert(S <= 0x7FFF, "slots fit the code");
 };
@@ -130,29 +128,32 @@ __device__ __forceinline__ bool slot_xyz(int s, const int (&e)[3], int &x, int &
     return x < e[0] && y < e[1] && z < e[2];
 }
 
-// The same for slot tid + NT q, the q-th of a tile kernel's thread (q is known
-// when the code is compiled, and with it the face).
-template <int DIM>
+// The same for slot tid + 256 M q, the q-th of a tile kernel's thread (q is known
+// when the code is compiled, and with it the face but for M = 4).
+template <int DIM, int M>
 __device__ __forceinline__ bool slot_of(int q, int tid, const int (&e)[3], int &x, int &y, int &z)
 {
     using G = PG<DIM>;
-    if constexpr (DIM == 2) {
-        static_assert(DIM != 2 || (G::NT == 256 && G::F0 == 64 && G::F1 == 128), "slots of a thread");
-        const bool side = tid < 128;   // q = 0: x-, x+, y-; q = 1: y+
+    if constexpr (M == 4) {
+        return slot_xyz<DIM>(tid + 1024 * q, e, x, y, z);
+    } else if constexpr (DIM == 2) {
+        static_assert(DIM != 2 || (G::F0 == 64 && G::F1 == 128), "slots of a thread");
+        const bool side = tid < 128;   // M = 1, q = 0: x-, x+, y-; q = 1: y+.  M = 2: all
         z = 0;
-        x = q == 0 ? (side ? (tid < 64 ? 0 : e[0] - 1) : tid - 128) : tid;
-        y = q == 0 ? (side ? tid & 63 : 0) : e[1] - 1;
+        x = q == 0 ? (side ? (tid < 64 ? 0 : e[0] - 1) : (tid - 128) & 127) : tid;
+        y = q == 0 ? (side ? tid & 63 : tid < 256 ? 0 : e[1] - 1) : e[1] - 1;
     } else {
-        static_assert(DIM != 3 || (G::NT == 256 && G::F0 == 256 && G::F1 == 512 && G::F2 == 512), "slots of a thread");
-        if (q < 2) {
-            x = q ? e[0] - 1 : 0;
+        static_assert(DIM != 3 || (G::F0 == 256 && G::F1 == 512 && G::F2 == 512), "slots of a thread");
+        const int f0 = M == 1 ? q : tid >> 8;   // q < 2 / M: x-, x+
+        if (q < 2 / M) {
+            x = f0 ? e[0] - 1 : 0;
             y = tid & 15;
-            z = tid >> 4;
+            z = (tid >> 4) & 15;
         } else {
-            const int f = tid + 256 * (q & 1);
+            const int f = M == 1 ? tid + 256 * (q & 1) : tid, face = M == 1 ? q >> 1 : q;   // 1, 2: y-, y+; 3, 4: z-, z+
             x = f & 31;
-            y = q < 6 ? (q < 4 ? 0 : e[1] - 1) : f >> 5;
-            z = q < 6 ? f >> 5 : (q < 8 ? 0 : e[2] - 1);
+            y = face == 1 ? 0 : face == 2 ? e[1] - 1 : f >> 5;
+            z = face < 3 ? f >> 5 : face == 3 ? 0 : e[2] - 1;
         }
     }
     return x < e[0] && y < e[1] && z < e[2];
@@ -198,7 +199,8 @@ struct alignas(16) WLink {
 // ------------------------------------------------- 3D tile union-find
 // Connected components of the bonds inside a 32 x 16 x 16 tile, B[r] = {+x,
 // +y, +z bonds} of row r = y + 16 z, all without the links that leave the
-// tile.  Warp w holds the rows y = 4 (w mod 4) .. + 3, z = 8 (w / 4) .. + 7,
+// tile.  Warp w holds the rows y = 4 (w mod 4) .. + 3, z = ZW (w / 4) .. + ZW - 1,
+// ZW = 8 / M,
 // lane = column, and goes through them with y innermost, the labels of the
 // row before along y and of the four rows before along z in registers:
 //   1. a run (maximal chain of x bonds in a row) takes the label of its last
@@ -214,17 +216,19 @@ struct alignas(16) WLink {
 // Links hang the larger root under the smaller, so roots are piece minima in
 // local row-major order, which is global order.  Returns, to lane x, the rows
 // (bit 4 zz + yy) of the warp whose site x started a label.
+template <int M>
 __device__ __forceinline__ uint32_t tile_label3(volatile int *par, const uint32_t (*B)[3], int tw, int th, int td)
 {
     using G = PG<3>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int yb = 4 * (warp & 3), zb = 8 * (warp >> 2);
+    constexpr int ZW = 8 / M;
+    const int yb = 4 * (warp & 3), zb = ZW * (warp >> 2);
     const uint32_t le = 0xFFFFFFFFu >> (31 - lane), gt = ~le;
     uint32_t born = 0u, cy = 0u, cz = 0u;
     {
         int labz[4] = {0, 0, 0, 0};
         uint32_t zw[4] = {0u, 0u, 0u, 0u};
-        for (int zz = 0; zz < 8 && zb + zz < td; ++zz) {
+        for (int zz = 0; zz < ZW && zb + zz < td; ++zz) {
             // first everything of the four rows that does not need the labels
             // (rows past the tile's have no bonds)
             int hd[4], py[4], pz[4];
@@ -269,14 +273,15 @@ __device__ __forceinline__ uint32_t tile_label3(volatile int *par, const uint32_
         shook<4>(par, par[i - G::TY * G::PW], par[i]);
     }
     __syncthreads();
-    // y bonds from rows y = 3, 7, 11 (every z), z bonds from layer z = 7 (every
-    // y): 64 rows, a quarter of a row's word a thread
+    // y bonds from rows y = 3, 7, 11 (every z), z bonds from the last layer of every
+    // warp but the top ones (every y): 64, 96 or 160 rows, a quarter of a row's word a
+    // thread
     {
         const int w = threadIdx.x >> 2, x0 = 8 * (threadIdx.x & 3);
         const bool yd = w < 48;
-        const int y = yd ? 4 * (w % 3) + 3 : w - 48, z = yd ? w / 3 : 7;
+        const int y = yd ? 4 * (w % 3) + 3 : w & 15, z = yd ? w / 3 : ZW * ((w >> 4) - 2) - 1;
         const int A = y + G::TY * z, step = (yd ? 1 : G::TY) * G::PW;
-        uint32_t bits = y < th && z < td ? (B[A][yd ? 1 : 2] >> x0) & 0xFFu : 0u;
+        uint32_t bits = w < 48 + 16 * (16 / ZW - 1) && y < th && z < td ? (B[A][yd ? 1 : 2] >> x0) & 0xFFu : 0u;
         int pa = -1, pb = -1;
         for (; bits; bits &= bits - 1) {
             const int i = A * G::PW + x0 + __ffs(bits) - 1;
@@ -354,12 +359,15 @@ __device__ __forceinline__ uint32_t interleave4x8(uint32_t v)
 // ----------------------------------------------------------------- k_ptile
 // Launch j finishes sweep j-1 (j >= 1) and starts sweep j (j < nsweeps).
 // F: FEAT_* bits compiled in (0: periodic plain lattices only).
-template <int DIM, int F>
-__global__ void __launch_bounds__(PG<DIM>::NT, 5)
+template <int DIM, int F, int M>
+__global__ void __launch_bounds__(M * PG<DIM>::WT, M == 1 ? 5 : M == 2 ? 2 : 1)
     k_ptile(const PottsDev p, int j, int nsweeps, uint64_t sweep0, DevObs *obs)
 {
     using G = PG<DIM>;
-    constexpr int NT = G::NT, NW = G::NW, S = G::S, TWW = G::TWW;
+    constexpr int WT = G::WT, NT = M * WT, NW = NT / 32, S = G::S, TWW = G::TWW;
+    constexpr int NQ = G::NS / 8 / NT;          // 8-site groups per thread
+    constexpr int SPT = (S + NT - 1) / NT;      // node slots per thread
+    constexpr int LR = 32 / M;                  // rows of a warp in the labelling
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PSmem<DIM> &sm = *reinterpret_cast<PSmem<DIM> *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -394,9 +402,10 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         z = r / G::TY;
         return y < th && z < td;
     };
-    // the thread's word of the tile: row wr = (wy, wz), sites 32 wc .. 32 wc + 31;
-    // warp w holds rows w NR / NW .. (w + 1) NR / NW - 1
-    constexpr int WROWS = G::NR / NW;
+    // the word of a thread of the first WT: row wr = (wy, wz), sites 32 wc .. 32 wc
+    // + 31; of their warps, w holds rows WROWS w .. WROWS (w + 1) - 1.  In 3D all warps
+    // draw, DROWS rows each
+    constexpr int WROWS = G::NR / (WT / 32), DROWS = DIM == 2 ? WROWS : G::NR / NW;
     const int wr = tid / TWW, wc = tid % TWW, wy = wr % G::TY, wz = wr / G::TY;
     const bool row_ok = wy < th && wz < td;
 
@@ -410,13 +419,13 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         const uint4 *code4 = reinterpret_cast<const uint4 *>(code);
         uint4 *scode4 = reinterpret_cast<uint4 *>(sm.f.s.code);
 #pragma unroll
-        for (int qq = 0; qq < G::NQ; ++qq) {
+        for (int qq = 0; qq < NQ; ++qq) {
             int x, y, z;
             const int idx = tid + qq * NT;
             if (group(idx, x, y, z)) cp_async16(scode4 + idx, code4 + idx);
         }
         for (int w = tid; w < S / 16; w += NT) cp_async16(sm.f.s.fst + 16 * w, p.nstate + nbase + 16 * w);
-        sm.f.s.fst[S + tid] = (uint8_t)tid;   // NT = 256
+        if (M == 1 || tid < 256) sm.f.s.fst[S + tid] = (uint8_t)tid;
     };
     // a block of the first wave draws first (sw_device.cuh's k_tile)
     const bool early = lt < FIRST_WAVE_SMS * 5 && !p.thr_dev;
@@ -497,9 +506,9 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             const bool bl = lane < 24;
             const uint32_t st_ = bl ? STREAM_BOND : STREAM_QSPIN;
             const uint32_t off = bl ? 3u * (lane & 7) + (lane >> 3) : (uint32_t)(lane - 24);
-            for (int i = 0; i < WROWS; i += 2) {
-                // two rows y, y + 1 of a layer (WROWS and TY are even)
-                const int r = WROWS * warp + i, y = r % G::TY, z = r / G::TY;
+            for (int i = 0; i < DROWS; i += 2) {
+                // two rows y, y + 1 of a layer (DROWS and TY are even)
+                const int r = DROWS * warp + i, y = r % G::TY, z = r / G::TY;
                 if (y >= th || z >= td) continue;
                 const uint32_t i0 = gidx(0, y, z) >> 2, i2 = i0 + (uL >> 2);
                 const U4 u0 = philox4x32_10((bl ? 3u * i0 : i0) + off, klo, khi, st_, k0, k1);
@@ -518,8 +527,8 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             // a row starts anywhere in a block: its 96 links lie in the 25 blocks
             // from the one that holds its first; lane x takes its three bits
             // from the ballots
-            for (int i = 0; i < WROWS; ++i) {
-                const int r = WROWS * warp + i, y = r % G::TY, z = r / G::TY;
+            for (int i = 0; i < DROWS; ++i) {
+                const int r = DROWS * warp + i, y = r % G::TY, z = r / G::TY;
                 if (y >= th || z >= td) continue;
                 const uint32_t l0 = 3u * gidx(0, y, z);
                 const U4 u = philox4x32_10((l0 >> 2) + lane, klo, khi, STREAM_BOND, k0, k1);
@@ -538,8 +547,9 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             // rows that start inside a QSPIN block: the blocks of all the warp's rows
             // dealt to its lanes
             const int nb = (tw + 3) / 4 + 1;   // blocks of a row
-            for (int i = lane; i < WROWS * nb; i += 32) {
-                const int r = WROWS * warp + i / nb, b = i % nb, y = r % G::TY, z = r / G::TY;
+            constexpr int QROWS = G::NR / NW;
+            for (int i = lane; i < QROWS * nb; i += 32) {
+                const int r = QROWS * warp + i / nb, b = i % nb, y = r % G::TY, z = r / G::TY;
                 if (y >= th || z >= td) continue;
                 const uint32_t i0 = gidx(0, y, z);
                 const uint32_t v = states4(philox4x32_10((i0 >> 2) + (uint32_t)b, klo, khi, STREAM_QSPIN, k0, k1));
@@ -588,7 +598,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         __syncthreads();
         const uint4 *scode4 = reinterpret_cast<const uint4 *>(sm.f.s.code);
 #pragma unroll
-        for (int qq = 0; qq < G::NQ; ++qq) {
+        for (int qq = 0; qq < NQ; ++qq) {
             int x, y, z;
             const int idx = tid + qq * NT;
             if (!group(idx, x, y, z)) continue;
@@ -644,7 +654,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
     // ---- the thread's word: state agreement along its links (four sites a
     //      comparison), the sums of sweep j-1 and the bonds of sweep j
     const bool last_start = j == nsweeps - 1;
-    {
+    if (M == 1 || tid < WT) {
         const uint32_t vm = row_ok ? valid_mask(wc, tw) : 0u;
         const uint32_t vx = open_x && row_ok ? valid_mask(wc, tw - 1) : vm;
         const uint32_t vy = open_y && wy == th - 1 ? 0u : vm;
@@ -676,16 +686,6 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             if (lane == 0) {
                 atomicAdd(&sm.acc[0], ws);
                 atomicAdd(&sm.acc[1], wm);
-            }
-            // clusters that touch a tile face: their sizes were summed at their
-            // root nodes by the merge; each root node is in exactly one tile
-            if (csz) {
-                unsigned long long c2 = 0ull;
-                for (int s = tid; s < S; s += NT) {
-                    const long long c = p.csize[nbase + s];
-                    c2 += (unsigned long long)(c * c);
-                }
-                warp_add64(&sm.acc_c2[0], c2);
             }
         }
         if (start) {
@@ -774,23 +774,34 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
             }
             put(bx & valid_mask(wc, tw - 1), wy < th - 1 ? by : 0u, wz < td - 1 ? bz : 0u);
         }
-        if (start && ext) {
-            for (int w = tid; w < S * G::PMW; w += NT) (&sm.pm[0][0])[w] = 0u;
-            // the tiles together clear what the last sweep's candidates left
-            // (the union kernel then resets their counts)
-            const int64_t W = (p.L + 31) / 32, FS = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
-            const int64_t i0 = (int64_t)lt * NT + tid, di = (int64_t)p.ntiles * NT;
-            for (int a = 0; a < DIM; ++a) {
-                const int64_t nc = p.ncand[a];
-                for (int64_t i = i0; i < nc * W; i += di) p.cov[a * FS * W + i] = 0u;
-                for (int64_t i = i0; i < nc; i += di) p.ccount[a * FS + i] = 0;
-            }
+    }
+    // clusters that touch a tile face: their sizes were summed at their root nodes
+    // by the merge; each root node is in exactly one tile
+    if (csz && fin) {
+        unsigned long long c2 = 0ull;
+#pragma unroll
+        for (int qq = 0; qq < SPT; ++qq) {
+            const long long c = tid + qq * NT < S ? p.csize[nbase + tid + qq * NT] : 0;
+            c2 += (unsigned long long)(c * c);
         }
-        if (start && lt == 0 && tid == 0) {
-            obs[j].threshold = thr;
-            obs[j].spans_x = 0;
-            obs[j].spans_y = 0;
+        warp_add64(&sm.acc_c2[0], c2);
+    }
+    if (start && ext) {
+        for (int w = tid; w < S * G::PMW; w += NT) (&sm.pm[0][0])[w] = 0u;
+        // the tiles together clear what the last sweep's candidates left (the union
+        // kernel then resets their counts)
+        const int64_t W = (p.L + 31) / 32, FS = DIM == 2 ? (int64_t)p.L : (int64_t)p.L * p.L;
+        const int64_t i0 = (int64_t)lt * NT + tid, di = (int64_t)p.ntiles * NT;
+        for (int a = 0; a < DIM; ++a) {
+            const int64_t nc = p.ncand[a];
+            for (int64_t i = i0; i < nc * W; i += di) p.cov[a * FS * W + i] = 0u;
+            for (int64_t i = i0; i < nc; i += di) p.ccount[a * FS + i] = 0;
         }
+    }
+    if (start && lt == 0 && tid == 0) {
+        obs[j].threshold = thr;
+        obs[j].spans_x = 0;
+        obs[j].spans_y = 0;
     }
     __syncthreads();
 
@@ -798,14 +809,14 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         // Step 2 inside the tile
         uint32_t born;
         if constexpr (DIM == 2)
-            born = tile_label_rows<64>(sm.f.par, sm.b, th, tw);
+            born = tile_label_rows<64, LR>(sm.f.par, sm.b, th, tw);
         else
-            born = tile_label3(sm.f.par, sm.b, tw, th, td);
+            born = tile_label3<M>(sm.f.par, sm.b, tw, th, td);
         // the warp's rows of the labelling: bit i of its masks is row lrow(i) and
         // its lanes are the sites lx
         const int lx = DIM == 2 ? 32 * (warp % TWW) + lane : lane;
         auto lrow = [&](int i) {
-            return DIM == 2 ? 32 * (warp / TWW) + i : 4 * (warp & 3) + (i & 3) + G::TY * (8 * (warp >> 2) + (i >> 2));
+            return DIM == 2 ? LR * (warp / TWW) + i : 4 * (warp & 3) + (i & 3) + G::TY * (LR / 4 * (warp >> 2) + (i >> 2));
         };
 
         // The labels' nodes that are no roots point at theirs, so that a site's
@@ -833,13 +844,13 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         // (A slot whose left neighbour has the same root leaves the mark to it: at
         // T_c a few big pieces hold most slots, and 32 lanes at one address wait
         // for each other.)
-        int rs[G::SPT];
+        int rs[SPT];
 #pragma unroll
-        for (int qq = 0; qq < G::SPT; ++qq) {
+        for (int qq = 0; qq < SPT; ++qq) {
             const int s = tid + qq * NT;
             int x, y, z;
             rs[qq] = -1;
-            if (s < S && slot_of<DIM>(qq, tid, t.e, x, y, z))
+            if (s < S && slot_of<DIM, M>(qq, tid, t.e, x, y, z))
                 rs[qq] = sroot_marked(sm.f.par, (y + G::TY * z) * G::PW + x);
             const int left = __shfl_up_sync(FULL, rs[qq], 1);
             if (rs[qq] >= 0 && (lane == 0 || left != rs[qq])) {
@@ -872,7 +883,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                 }
         }
 #pragma unroll
-        for (int qq = 0; qq < G::SPT; ++qq) {
+        for (int qq = 0; qq < SPT; ++qq) {
             const int s = tid + qq * NT;
             if (s >= S) break;
             const size_t node = nbase + s;
@@ -913,7 +924,7 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
         const bool gather = (F & (FEAT_CSIZE | FEAT_PCC)) && (csz || ext);
         if (!gather && !last_start && tw == G::TX && th == G::TY && td == G::TZ) {
 #pragma unroll 2
-            for (int i = 0; i < 32; i += 4) {
+            for (int i = 0; i < LR; i += 4) {
                 int v[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = sm.f.par[lrow(i + e) * G::PW + lx];
@@ -942,7 +953,8 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                     uint32_t *pm = sm.pm[cur_v & 0xFFFF];
                     if (DIM == 2) {
                         atomicOr(pm + (warp % TWW), 1u << lane);
-                        atomicOr(pm + 4 + warp / TWW, cur_rows);
+                        const int y0 = LR * (warp / TWW);
+                        atomicOr(pm + 4 + (y0 >> 5), cur_rows << (y0 & 31));
                     } else {
                         // bits y and 16 + z of the rows (bit 4 zz + yy of the mask)
                         uint32_t ys = cur_rows | (cur_rows >> 16);
@@ -954,11 +966,11 @@ __global__ void __launch_bounds__(PG<DIM>::NT, 5)
                         zs = (zs | (zs >> 6)) & 0x000F000Fu;
                         zs = (zs | (zs >> 12)) & 0xFFu;
                         atomicOr(pm, 1u << lane);
-                        atomicOr(pm + 1, ((ys & 0xFu) << (4 * (warp & 3))) | (zs << (16 + 8 * (warp >> 2))));
+                        atomicOr(pm + 1, ((ys & 0xFu) << (4 * (warp & 3))) | (zs << (16 + LR / 4 * (warp >> 2))));
                     }
                 }
             };
-            for (int i = 0; i < 32; i += 4) {   // four rows' look-ups in flight
+            for (int i = 0; i < LR; i += 4) {   // four rows' look-ups in flight
                 int v[4], root[4];
                 bool row[4];
 #pragma unroll
@@ -1488,12 +1500,15 @@ cudaError_t potts_prepare()
     if (dev < 0 || dev >= PREP_DEVICES) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
     if (done[dev]) return cudaSuccess;
-    const void *fn[4] = {(const void *)k_ptile<2, 0>, (const void *)k_ptile<2, FEAT_TILE>,
-                         (const void *)k_ptile<3, 0>, (const void *)k_ptile<3, FEAT_TILE>};
-    const int bytes[4] = {(int)ptile_smem<2>(true), (int)ptile_smem<2>(true), (int)ptile_smem<3>(true),
-                          (int)ptile_smem<3>(true)};
-    for (int f = 0; f < 4 && err == cudaSuccess; ++f)
-        err = cudaFuncSetAttribute(fn[f], cudaFuncAttributeMaxDynamicSharedMemorySize, bytes[f]);
+    auto set = [&](auto... k) {
+        ((err = err == cudaSuccess ? cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                          (int)std::max(ptile_smem<2>(true), ptile_smem<3>(true)))
+                                   : err),
+         ...);
+    };
+    set(k_ptile<2, 0, 1>, k_ptile<2, FEAT_TILE, 1>, k_ptile<2, 0, 2>, k_ptile<2, FEAT_TILE, 2>, k_ptile<2, 0, 4>,
+        k_ptile<2, FEAT_TILE, 4>, k_ptile<3, 0, 1>, k_ptile<3, FEAT_TILE, 1>, k_ptile<3, 0, 2>, k_ptile<3, FEAT_TILE, 2>,
+        k_ptile<3, 0, 4>, k_ptile<3, FEAT_TILE, 4>);
     if (err == cudaSuccess) done[dev] = true;
     return err;
 }
@@ -1503,14 +1518,32 @@ bool all_shared(const PottsDev &p)
     return chain_all_shared(p.ntiles, (p.flags & RF_PCC) != 0, (p.flags & RF_WIND) != 0);
 }
 
+template <int DIM, int M>
+cudaError_t launch_tile_cta(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
+                            bool chained)
+{
+    const bool feat = (p.flags & (RF_PCC | RF_OPEN | RF_CSIZE | RF_WIND)) != 0;
+    return launch_kernel(feat ? k_ptile<DIM, FEAT_TILE, M> : k_ptile<DIM, 0, M>, dim3((unsigned)p.ntiles), M * PG<DIM>::WT,
+                         ptile_smem<DIM>((p.flags & RF_PCC) && !(p.flags & RF_WIND)), st, chained, all_shared(p), p, j,
+                         nsweeps, sweep0, obs);
+}
+
+// M, the warps of a tile CTA by eights: a warp's rows in the labelling, its records and
+// its codes are a chain that an SM with one or two CTAs cannot hide, and more warps
+// have fewer rows each.  M = 4 up to two thirds of a CTA an SM (beyond, the blocks of
+// the next kernels have no room beside one), M = 2 up to two CTAs an SM in 2D and four
+// in 3D.  M = 1, 2 and 4, us a sweep at T_c: 2D, q=3, L=300 28.0, 24.3, 23.7; L=1024
+// 32.9, 29.6, 30.7; L=1500 45.6, 38.9; L=1700 45.6, 50.8; 3D, q=2, L=50 41.4, 32.9,
+// 30.6; L=96 50.8, 36.9, 38.1; L=128 71.3, 49.3; L=160 90.4, 83.9; L=200 136, 149; PCC
+// by the topological rule in 3D, L=50 64.2, 52.1, 49.4.
 template <int DIM>
 cudaError_t launch_tile(const PottsDev &p, int j, int nsweeps, uint64_t sweep0, DevObs *obs, cudaStream_t st,
                         bool chained)
 {
-    const bool feat = (p.flags & (RF_PCC | RF_OPEN | RF_CSIZE | RF_WIND)) != 0;
-    return launch_kernel(feat ? k_ptile<DIM, FEAT_TILE> : k_ptile<DIM, 0>, dim3((unsigned)p.ntiles), PG<DIM>::NT,
-                         ptile_smem<DIM>((p.flags & RF_PCC) && !(p.flags & RF_WIND)), st, chained, all_shared(p), p, j, nsweeps,
-                         sweep0, obs);
+    if (3 * p.ntiles <= 2 * FIRST_WAVE_SMS) return launch_tile_cta<DIM, 4>(p, j, nsweeps, sweep0, obs, st, chained);
+    if (p.ntiles <= (DIM == 2 ? 2 : 4) * FIRST_WAVE_SMS)
+        return launch_tile_cta<DIM, 2>(p, j, nsweeps, sweep0, obs, st, chained);
+    return launch_tile_cta<DIM, 1>(p, j, nsweeps, sweep0, obs, st, chained);
 }
 
 template <int DIM>

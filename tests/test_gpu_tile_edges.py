@@ -149,3 +149,27 @@ def test_rows_of_subtiles(sw, L, opts):
             np.testing.assert_array_equal(lat.spins(), ref.spins())
             np.testing.assert_array_equal(lat.labels(), ref.labels())
             np.testing.assert_array_equal(lat.bonds(), ref.bonds())
+
+
+# Potts tiles have 32, 16 or 8 warps by the size of the grid (the sizes above: 32).
+@pytest.mark.parametrize("opts", [{}, {"csize": True, "open": True}, {"wind": True}])
+@pytest.mark.parametrize("dim,L,q", [(2, 1290, 3), (2, 1681, 2), (3, 97, 3), (3, 161, 2)])
+def test_potts_warps_of_a_tile(sw, orc, dim, L, q, opts):
+    T = 1.0 / np.log(1 + np.sqrt(q)) if dim == 2 else (2.2557 if q == 2 else 1.8164)
+    ref = orc.PottsChain(dim, L, q, 1.0, T, L, **opts)
+    with sw.PottsLattice(dim, L, q, T=T, seed=L, **opts) as lat:
+        for n in (1, 2):
+            lat.sweep(n)
+            assert_obs_equal(lat.observables(), ref.run(n))
+            np.testing.assert_array_equal(lat.spins(), ref.spin)
+            np.testing.assert_array_equal(lat.labels(), ref.label)
+            np.testing.assert_array_equal(lat.bonds(), ref.bond)
+
+
+@pytest.mark.parametrize("dim,L", [(2, 200), (2, 1290), (3, 40), (3, 97)])
+def test_potts_pcc_warps_of_a_tile(sw, orc, dim, L):
+    ref = orc.PottsChain(dim, L, 2, 1.0, 1.0, 3, pcc=True)
+    with sw.PottsLattice(dim, L, 2, seed=3, pcc=True) as lat:
+        lat.sweep(4)
+        assert_obs_equal(lat.observables(), ref.run(4))
+        np.testing.assert_array_equal(lat.spins(), ref.spin)
