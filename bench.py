@@ -38,7 +38,7 @@ L2_BYTES = 129 << 20     # GB300 L2
 UNIT = "site-updates/ns"
 ALG_BYTES_PER_SITE = 10            # old spin in, label out, label in, new spin out
 PROFILE_FILE = os.path.join(ROOT, "profiles", "k_tile_L16384_Tc.md")
-LAUNCHES_PER_SWEEP = 4             # tile kernel, merge union, pointer jumping, resolve
+LAUNCHES_PER_SWEEP = 3             # tile kernel, merge union, resolve
 
 
 def parse_args():
@@ -430,7 +430,7 @@ def run_gb300(args):
                                           "seeds": f"{w.seed}..{w.seed + world - 1}"}),
             "tile_h": tile_h, "hbm_gbs_achieved": roofline["achieved"],
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "batched": batched, "served": served,
-            "gpu_launches": K * (LAUNCHES_PER_SWEEP * w.sweeps + 1),
+            "gpu_launches": K * (LAUNCHES_PER_SWEEP * w.sweeps + 2),   # a call: + its first kernel and the last finish
             "clocks": clk, "impl": "gb300",
         }
     if pool is not None:

@@ -225,7 +225,7 @@ int sw_sync(sw_ctx *ctx);
 typedef struct {
     int64_t tile_launches; /* launches of the tile kernel                   */
     double tile_ms;        /* their summed device time                      */
-    int64_t merge_groups;  /* launch groups (a group = the three merge kernels) */
+    int64_t merge_groups;  /* groups of merge kernels, one a launch of it    */
     double merge_ms;       /* summed device time of the merge groups         */
     int64_t tile_sites;    /* L*L (a Potts lattice: L^d)                     */
     int32_t tile_height;   /* rows per tile (tiles are 128 sites wide); 0 on a
@@ -392,7 +392,7 @@ int sw_server_get_stats(sw_server *srv, sw_server_stats *out);
  * one array is shared by every call: calls that overlap on the GPU (other
  * streams, other threads) race; run them one after another.  The first call
  * on a device sets the array up for that device (looks up its device address
- * and raises a kernel's shared-memory limit while the device is current):
+ * and raises its kernels' shared-memory limits while the device is current):
  * make it before any stream capture starts. */
 #define SW_STATIC_MAX_L 1024
 int sw_sweep_static(const uint8_t *spin_in, uint8_t *spin_out, int32_t *labels_out, sw_obs *obs_out,

@@ -17,6 +17,7 @@
 //            periodic wrap; the root of a global cluster is the minimum site
 //            index (the DPM rule "the smaller label wins", Sec. II.B step 5);
 //            then each node gets its cluster's root and new spin.
+//   k_one    all of it for a lattice of one tile, every sweep of a call in one block.
 //
 // Between launches only the 2-byte code per site and the node table cross
 // the SM boundary; spins stay in shared memory from one sweep to the next.
@@ -137,8 +138,9 @@ constexpr int FIRST_WAVE_SMS = 152;
 // tile table, launch offset, the threshold of a plain lattice) may be read
 // first, and so may draws be made.  No block returns without the wait, so a
 // kernel that has finished implies that all before it have.
-// A kernel lets its successor start first thing, so that short kernels are all
-// in place when their turn comes (L=64: 23.0 us a sweep against 24.9 when they
+// (Figures here compare the two sides of a rule on the kernels as they were when it
+// was set.)  A kernel lets its successor start first thing, so that short kernels are
+// all in place when their turn comes (L=64: 23.0 us a sweep against 24.9 when they
 // start after the wait and 27.0 without the chain; L=4096, T=3.0: 93.7, 97.9 and
 // 104 us).  Where a grid does not fill the GPU that has a price: blocks started
 // ahead go to the few SMs with room and run crowded there.  So
@@ -502,7 +504,8 @@ __device__ __forceinline__ uint32_t run_heads(uint32_t h)
 // and one code look-up a site took the 64-row tile kernel from 2.01 to 1.40 ms
 // at L=16384, T_c (111 -> 81M warp instructions a launch at L=4096), and masks
 // per column, the single-swap unions and the label nodes' copies of their root's
-// record (two loads a code) to 1.19 ms.
+// record (two loads a code) to 1.19 ms; four rows' words ahead of their labels made a
+// sweep 1 to 3% faster.
 //
 // k_one, whose warps have nobody to hide behind, takes sub-tiles of fewer rows (RS)
 // and leaves out the words of a row that its lattice does not reach (WX in use).

@@ -57,7 +57,7 @@ cudaError_t tile_prepare()
 template <int TH>
 cudaError_t launch_one(OneArgs a, cudaStream_t st)
 {
-    constexpr int32_t MOST = 4096;   // about 50 ms
+    constexpr int32_t MOST = 4096;   // about 70 ms at L=128
     const int32_t n = a.nsweeps;
     cudaError_t e = cudaSuccess;
     for (int32_t at = 0; at < n && e == cudaSuccess; at += MOST) {
@@ -562,7 +562,7 @@ cudaError_t next_event(sw_ctx *c, cudaEvent_t *ev)
 }
 
 // Profiling mode: the same launch groups, enqueued one by one, the tile
-// kernel and the three merge kernels of every group bracketed by events.
+// kernel and the merge kernels of every group bracketed by events.
 int enqueue_profiled(sw_ctx *c, int32_t n)
 {
     SweepArgs a = args_of(c);
