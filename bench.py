@@ -445,10 +445,9 @@ def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
     in this run: HBM (the algorithmic 10 B/site of a sweep against the
     measured copy bandwidth; the DRAM bytes ncu counted per launch beside it)
     and the integer pipe (the Philox blocks a launch draws against the
-    library's Philox probe).  Neither is what binds the kernel: it issues
-    instructions on about two thirds of its cycles and waits on dependent
-    shared-memory loads and barriers in the union-find (the ncu summaries in
-    profiles/)."""
+    library's Philox probe).  Neither is what binds the kernel: it issues on
+    72% of its cycles with the integer ALU pipe at 62% of its rate (the ncu
+    summaries in profiles/)."""
     N = w.L * w.L
     tile_s = st["tile_ms"] / st["tile_launches"] * 1e-3
     peak, peak_src = hbm_peak_gbs()
@@ -479,8 +478,8 @@ def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
                 "peak_source": "measured in this run: sw_bench_philox, 2^32 BOND blocks per launch"},
         "l2_gbs_peak": round(l2_peak, 1),
         "l2_peak_source": "measured in this run: sw_bench_l2, 32 MiB copy resident in L2",
-        "binding": "neither ceiling: instruction issue (about 2/3 of cycles) and dependent shared-memory "
-                   "latency in the union-find, with phase barriers (profiles/k_tile_L4096_full.md)",
+        "binding": "neither ceiling: the number of integer instructions (issue on 72% of cycles, the ALU pipe "
+                   "at 62% of its rate), then phase barriers (profiles/k_tile_L4096_full.md)",
     }
 
 
@@ -846,8 +845,8 @@ def run_potts(args):
                         "peak_blocks_per_s": round(philox_peak, 1),
                         "frac": round(blocks / tile_s / philox_peak, 4),
                         "peak_source": "measured in this run: sw_bench_philox, 2^32 BOND blocks per launch"},
-                "binding": "neither ceiling: instruction issue (70-76% of cycles) and the union-find's "
-                           "dependent shared-memory latency (profiles/k_potts_tiles_critical.md)"}
+                "binding": "neither ceiling: the number of integer instructions (issue on 71-75% of cycles, the ALU "
+                           "pipe at 55-62% of its rate; profiles/k_potts_tiles_critical.md)"}
     if traffic is not None:
         roofline["dram_gbs_measured"] = round(traffic / tile_s / 1e9, 1)
         roofline["frac_dram_measured"] = round(traffic / tile_s / 1e9 / hbm, 4)
