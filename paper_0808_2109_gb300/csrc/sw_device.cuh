@@ -446,6 +446,15 @@ __device__ __forceinline__ int top_bit(uint32_t v)
     return r;
 }
 
+// Takes the highest row out of a mask of rows (bfind and two operations, where the
+// lowest takes a bit reversal and an addition more).
+__device__ __forceinline__ int take_row(uint32_t &rows)
+{
+    const int r = top_bit(rows);
+    rows ^= 1u << r;
+    return r;
+}
+
 // The two 16-bit halves selected from X (even positions) and Z (odd
 // positions) interleaved into one word: bits of half hf (0 or 1) of each.
 __device__ __forceinline__ uint32_t interleave16(uint32_t X, uint32_t Z, int hf)
@@ -480,9 +489,16 @@ __device__ __forceinline__ uint32_t run_heads(uint32_t h)
     return ~((h & 0x7FFFFFFFu) << 1);
 }
 
+// The same as the tile kernels keep them for the labelling: bits 1 to 31 the run
+// heads, bit 0 (always a head) the link that leaves the sub-tile.
+__device__ __forceinline__ uint32_t heads_word(uint32_t h)
+{
+    return (run_heads(h) & ~1u) | (h >> 31);
+}
+
 // Connected components of the intra-tile bonds: B[y][2c] holds the right-link
-// bonds of word c of row y, B[y][2c + 1] its down-link bonds, both without the
-// links that leave the tile.  The tile is cut into 32 x 32 sub-tiles, one per
+// bonds of word c of row y as heads_word has them, B[y][2c + 1] its down-link bonds,
+// both without the links that leave the tile.  The tile is cut into 32 x 32 sub-tiles, one per
 // warp, lane = column:
 //   1. the warp goes down its 32 rows with every site's label in a register.
 //      A run (maximal chain of right bonds inside a sub-tile row) takes the
@@ -505,7 +521,9 @@ __device__ __forceinline__ uint32_t run_heads(uint32_t h)
 // at L=16384, T_c (111 -> 81M warp instructions a launch at L=4096), and masks
 // per column, the single-swap unions and the label nodes' copies of their root's
 // record (two loads a code) to 1.19 ms; four rows' words ahead of their labels made a
-// sweep 1 to 3% faster.
+// sweep 1 to 3% faster, and run heads kept by the thread of the word, births by label
+// and masks taken from the top another 1.5% (1350 -> 1330 us at L=16384, T_c; 2D Potts
+// L=8192, q=3, 449 -> 442).
 //
 // k_one, whose warps have nobody to hide behind, takes sub-tiles of fewer rows (RS)
 // and leaves out the words of a row that its lattice does not reach (WX in use).
@@ -537,9 +555,8 @@ __device__ __forceinline__ uint32_t label_rows(volatile int *par, const uint32_t
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const uint2 hv = *reinterpret_cast<const uint2 *>(&B[y0 + r + q][2 * sx]);
-                const uint32_t heads = run_heads(hv.x);
-                const uint32_t n = heads & gt;                // heads to the right: the run ends before them
-                hd[q] = top_bit(heads & le);
+                const uint32_t n = hv.x & gt;                 // heads to the right: the run ends before them
+                hd[q] = top_bit((hv.x & le) | 1u);
                 c[q] = top_bit(v & (n - 1u) & ~n);            // last contact at or left of the run's end
                 dn[q] = v;
                 v = hv.y;
@@ -549,8 +566,8 @@ __device__ __forceinline__ uint32_t label_rows(volatile int *par, const uint32_t
                 const bool has = c[q] >= hd[q];
                 const int lc = __shfl_sync(0xFFFFFFFFu, lab, c[q]);
                 if (((dn[q] >> lane) & 1u) && lab != lc) conf |= 1u << (r + q);
-                if (!has && hd[q] == lane) born |= 1u << (r + q);
                 lab = has ? lc : row + hd[q];
+                if (lab == row + lane) born |= 1u << (r + q);   // (a label is its first site's node)
                 par[row + lane] = lab;
             }
         }
@@ -566,8 +583,8 @@ __device__ __forceinline__ uint32_t label_rows(volatile int *par, const uint32_t
             const int a0 = par[i0 - PW], b0 = par[i0], a1 = par[i1 - PW], b1 = par[i1];
             shook_pair<4>(par, a0, b0, two, a1, b1);
         }
-        for (; conf; conf &= conf - 1) {
-            const int i = col + (__ffs(conf) - 1) * PW;
+        while (conf) {
+            const int i = col + take_row(conf) * PW;
             shook<4>(par, par[i - PW], par[i]);
         }
         if (32 * sx + lane >= tw) born = 0u;
@@ -587,7 +604,7 @@ struct EdgeLinks {
     {
         if (q < NV) {
             const int bnd = q / TH + 1, y = q % TH;             // link (32 bnd - 1, y) - (32 bnd, y)
-            if (y >= th || !(B[y][2 * bnd - 2] >> 31)) return false;
+            if (y >= th || !(B[y][2 * bnd - 2] & 1u)) return false;
             ia = y * PW + 32 * bnd - 1;
             ib = ia + 1;
         } else {
@@ -815,8 +832,8 @@ struct TileSmem {
                                     // finish half, the tile's site codes (TH * TW * 2 bytes)
     uint32_t sp[TH + 1][TWW];       // spins as bits, row TH = halo row
     uint32_t spx[TH / 32];          // halo column (the site right of the tile's last): bit y = row y
-    // row y: first the raw draws (below), then the intra-tile bonds, [2c] the
-    // right links and [2c + 1] the down links of word c
+    // row y: first the raw draws (below), then the intra-tile bonds, [2c] the right
+    // links (heads_word) and [2c + 1] the down links of word c
     __align__(16) uint32_t b[TH][2 * TWW];
     union {                         // never live at the same time:
         __align__(16) uint32_t finfo[Slots<TH>::S + 4];   // finish half: finals of the tile's own nodes,
@@ -1067,7 +1084,7 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
             }
             __syncwarp();   // the warp's rows: every draw is read before it is overwritten
             *reinterpret_cast<uint2 *>(&sm.b[wy][2 * wc]) =
-                make_uint2(h & valid_mask(wc, t.tw - 1), wy < t.th - 1 ? v : 0u);
+                make_uint2(heads_word(h & valid_mask(wc, t.tw - 1)), wy < t.th - 1 ? v : 0u);
         }
     }
     // clusters that touch a tile border: their sizes were summed at their root
@@ -1133,8 +1150,8 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
             const int col = y0 * PW + 32 * sx + lane;
             uint32_t linked = 0u;
             int ncl = 0;
-            for (uint32_t bits = born; bits; bits &= bits - 1) {
-                const int r = __ffs(bits) - 1;
+            for (uint32_t bits = born; bits;) {
+                const int r = take_row(bits);
                 const int x = col + r * PW;
                 const int p = sm.par[x];
                 if (p == x) {
@@ -1144,7 +1161,7 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
                     sm.par[x] = (int)(INFO_INTERIOR | c);
                     ++ncl;
                 } else if (p >= 0) {
-                    linked |= bits & -bits;
+                    linked |= 1u << r;
                 }
             }
             ncl = __reduce_add_sync(0xFFFFFFFFu, ncl);
@@ -1152,8 +1169,8 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
             // the other labels' nodes take a copy of their root's record where it
             // is there already, so that most sites find it two loads away (cluster
             // sizes: those of interior clusters its index instead)
-            for (; linked; linked &= linked - 1) {
-                const int x = col + (__ffs(linked) - 1) * PW;
+            while (linked) {
+                const int x = col + take_row(linked) * PW;
                 int p = sm.par[x], q = sm.par[p];
                 while ((uint32_t)q < INFO_INTERIOR && q != p) {
                     p = q;
@@ -1208,7 +1225,7 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
             // clocks a tile at L=2048, T_c, against 8.9K (plain codes 2.0K); a match of
             // the row's labels before the atomics is slower, 71 us a sweep against 64.
             auto count = [&](int r, int v) {
-                const uint32_t heads = run_heads(sm.b[y0 + r][2 * sx]), n = heads >> lane;
+                const uint32_t n = (sm.b[y0 + r][2 * sx] | 1u) >> lane;
                 if (n & 1u) {
                     const uint32_t len = n >> 1 ? (uint32_t)__ffs(n >> 1) : 32u - lane;
                     atomicAdd(&sm.par[(born >> r) & 1u ? (y0 + r) * PW + x : v], (int)(len << SIZE_SHIFT));
@@ -1494,7 +1511,7 @@ __global__ void __launch_bounds__(OneCfg<TH>::NT, 1) k_one(const OneArgs a)
             }
             __syncwarp();   // the warp's rows: every draw is read before it is overwritten
             *reinterpret_cast<uint2 *>(&sm.b[wy][2 * wc]) =
-                make_uint2(h & valid_mask(wc, L - 1), wy < L - 1 ? v : 0u);
+                make_uint2(heads_word(h & valid_mask(wc, L - 1)), wy < L - 1 ? v : 0u);
         }
         __syncthreads();
         if (j > 0 && tid < 2) {   // sweep j-1's sums of its new spins
