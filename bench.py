@@ -446,7 +446,7 @@ def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
     measured copy bandwidth; the DRAM bytes ncu counted per launch beside it)
     and the integer pipe (the Philox blocks a launch draws against the
     library's Philox probe).  Neither is what binds the kernel: it issues on
-    72% of its cycles with the integer ALU pipe at 62% of its rate (the ncu
+    72% of its cycles with the integer ALU pipe at 63% of its rate (the ncu
     summaries in profiles/)."""
     N = w.L * w.L
     tile_s = st["tile_ms"] / st["tile_launches"] * 1e-3
@@ -479,7 +479,7 @@ def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
         "l2_gbs_peak": round(l2_peak, 1),
         "l2_peak_source": "measured in this run: sw_bench_l2, 32 MiB copy resident in L2",
         "binding": "neither ceiling: the number of integer instructions (issue on 72% of cycles, the ALU pipe "
-                   "at 62% of its rate), then phase barriers (profiles/k_tile_L4096_full.md)",
+                   "at 63% of its rate), then phase barriers (profiles/k_tile_L4096_full.md)",
     }
 
 
@@ -846,7 +846,7 @@ def run_potts(args):
                         "frac": round(blocks / tile_s / philox_peak, 4),
                         "peak_source": "measured in this run: sw_bench_philox, 2^32 BOND blocks per launch"},
                 "binding": "neither ceiling: the number of integer instructions (issue on 71-75% of cycles, the ALU "
-                           "pipe at 55-62% of its rate; profiles/k_potts_tiles_critical.md)"}
+                           "pipe at 54-60% of its rate; profiles/k_potts_tiles_critical.md)"}
     if traffic is not None:
         roofline["dram_gbs_measured"] = round(traffic / tile_s / 1e9, 1)
         roofline["frac_dram_measured"] = round(traffic / tile_s / 1e9 / hbm, 4)
