@@ -289,6 +289,11 @@ int sw_bench_l2(const void *src_dev, void *dst_dev, int64_t bytes, int32_t reps,
  * n = 0 switches it off. */
 int sw_debug_fail_allocations(int32_t skip, int32_t n);
 
+/* The same for the servers' set-ups of newly admitted jobs (one for the jobs
+ * that join a tile height's lane together): the n after the first `skip` report
+ * an error and write nothing; their jobs end with SW_ERR_CUDA and never run. */
+int sw_debug_fail_setups(int32_t skip, int32_t n);
+
 /* ------------------------------------------------- batched and served runs
  * Many independent lattices on one GPU at once (the paper's decompositions
  * spread ONE lattice over processors, Sec. II; here independent lattices

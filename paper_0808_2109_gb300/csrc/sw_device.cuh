@@ -1110,7 +1110,7 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
             uint4 *cov4 = reinterpret_cast<uint4 *>(R.cov);
 #pragma unroll
             for (int ax = 0; ax < 2; ++ax) {
-                const int words = R.ncand[ax] * (ax == 0 ? R.tiles_x : R.tiles_y);
+                const int words = min(R.ncand[ax], L) * (ax == 0 ? R.tiles_x : R.tiles_y);   // (at most L candidates)
                 for (int i = i0; i < words; i += di) cov4[i] = make_uint4(0u, 0u, 0u, 0u);
                 cov4 += (size_t)L * R.tiles_x;
             }

@@ -254,7 +254,29 @@ int pick_tile_height(int L, uint32_t flags, bool pcc)
     return tiles <= per_sm * FIRST_WAVE_SMS ? 32 : 96;
 }
 
-std::atomic<int> g_alloc_skip{0}, g_alloc_failures{0};   // sw_debug_fail_allocations
+// Failures to inject (sw_debug_fail_*): of the next calls of hit, `skip` pass and
+// the `failures` after them are hits.
+struct Injection {
+    std::atomic<int> skip{0}, failures{0};
+    void set(int s, int n)
+    {
+        failures.store(0);
+        skip.store(s);
+        failures.store(n);
+    }
+    bool hit()
+    {
+        if (failures.load() <= 0) return false;
+        int s = skip.load();
+        while (s > 0)
+            if (skip.compare_exchange_weak(s, s - 1)) return false;   // this one still succeeds
+        int n = failures.load();
+        while (n > 0)
+            if (failures.compare_exchange_weak(n, n - 1)) return true;
+        return false;
+    }
+};
+Injection g_fail_alloc, g_fail_setup;
 
 template <typename T>
 cudaError_t dalloc(T **p, size_t count)
@@ -269,14 +291,12 @@ cudaError_t dalloc(T **p, size_t count)
 
 bool sw_inject_alloc_failure()
 {
-    if (g_alloc_failures.load() <= 0) return false;
-    int s = g_alloc_skip.load();
-    while (s > 0)
-        if (g_alloc_skip.compare_exchange_weak(s, s - 1)) return false;   // this one still succeeds
-    int n = g_alloc_failures.load();
-    while (n > 0)
-        if (g_alloc_failures.compare_exchange_weak(n, n - 1)) return true;
-    return false;
+    return g_fail_alloc.hit();
+}
+
+bool sw_inject_setup_failure()
+{
+    return g_fail_setup.hit();
 }
 
 std::mutex &sw_capture_mutex()
@@ -1184,9 +1204,14 @@ int sw_bench_l2(const void *src_dev, void *dst_dev, int64_t bytes, int32_t reps,
 int sw_debug_fail_allocations(int32_t skip, int32_t n)
 {
     if (skip < 0 || n < 0) return SW_ERR_ARG;
-    g_alloc_failures.store(0);
-    g_alloc_skip.store(skip);
-    g_alloc_failures.store(n);
+    g_fail_alloc.set(skip, n);
+    return SW_OK;
+}
+
+int sw_debug_fail_setups(int32_t skip, int32_t n)
+{
+    if (skip < 0 || n < 0) return SW_ERR_ARG;
+    g_fail_setup.set(skip, n);
     return SW_OK;
 }
 

@@ -25,4 +25,8 @@ __attribute__((visibility("hidden"))) std::mutex &sw_capture_mutex();
 // allocation failures remain, consuming one.  Every device allocation of the
 // library asks first and reports cudaErrorMemoryAllocation instead.
 __attribute__((visibility("hidden"))) bool sw_inject_alloc_failure();
+
+// The same for sw_debug_fail_setups: a server asks before it writes the first
+// contents of a lane's newly admitted jobs.
+__attribute__((visibility("hidden"))) bool sw_inject_setup_failure();
 #endif

@@ -296,6 +296,7 @@ unsigned char *lane_workspace(Lane &ln, size_t bytes)
 // is no memory for their table).
 cudaError_t init_jobs(const std::vector<Job *> &jobs, Lane &ln)
 {
+    if (sw_inject_setup_failure()) return cudaErrorUnknown;
     const cudaStream_t st = ln.stream;
     for (size_t at = 0; at < jobs.size(); at += JOBS_PER_LAUNCH) {
         const size_t n = std::min<size_t>(jobs.size() - at, JOBS_PER_LAUNCH);
@@ -612,6 +613,26 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
     s->cv_done.notify_all();
 }
 
+// Ends admitted jobs of a lane that never ran (and are in no table) with an error.
+void end_failed(sw_server *s, const std::vector<Job *> &jobs, Lane &ln, int rc)
+{
+    cudaGetLastError();
+    for (Job *j : jobs) free_job_device(j, ln.stream);
+    cudaStreamSynchronize(ln.stream);
+    std::lock_guard<std::mutex> lk(s->mu);
+    for (Job *j : jobs) {
+        sw_result res{};
+        res.status = rc;
+        res.L = j->spec.L;
+        res.nsweeps = j->spec.nsweeps;
+        s->used -= j->bytes;
+        s->finished[j->id] = res;
+        s->stats.finished += 1;
+        delete j;
+    }
+    s->cv_done.notify_all();
+}
+
 void worker_main(sw_server *s)
 {
     cudaSetDevice(s->dev);
@@ -654,19 +675,7 @@ void worker_main(sw_server *s)
                 if (j->slot < 0 || j->tile_base < 0) rc = SW_ERR_NOMEM;
             }
             if (rc != SW_OK) {
-                cudaGetLastError();
-                free_job_device(j, ln.stream);
-                cudaStreamSynchronize(ln.stream);
-                sw_result res{};
-                res.status = rc;
-                res.L = j->spec.L;
-                res.nsweeps = j->spec.nsweeps;
-                std::lock_guard<std::mutex> lk(s->mu);
-                s->used -= j->bytes;
-                s->finished[j->id] = res;
-                s->stats.finished += 1;
-                s->cv_done.notify_all();
-                delete j;
+                end_failed(s, {j}, ln, rc);
                 continue;
             }
             for (int i = 0; i < j->n_tiles; ++i) ln.tile_rep_host[j->tile_base + i] = j->slot;
@@ -679,11 +688,15 @@ void worker_main(sw_server *s)
             std::lock_guard<std::mutex> lk(s->mu);
             s->stats.admitted += 1;
         }
+        // jobs whose first contents cannot be written leave the lane again before its
+        // step: no kernel ever sees memory that nobody wrote
         for (int l = 0; l < N_LANES; ++l)
             if (!fresh[l].empty() && init_jobs(fresh[l], s->lanes[l]) != cudaSuccess) {
-                cudaGetLastError();
-                std::lock_guard<std::mutex> lk(s->mu);
-                s->worker_error = SW_ERR_CUDA;
+                for (Job *j : fresh[l]) {
+                    lane_release(s->lanes[l], j);
+                    s->running.erase(std::find(s->running.begin(), s->running.end(), j));
+                }
+                end_failed(s, fresh[l], s->lanes[l], SW_ERR_CUDA);
             }
         // ---- one step of every busy lane
         nvtxRangePushA("server step");

@@ -144,6 +144,7 @@ SIGNATURES = {
     "sw_save": ([_P, _P, _u64], ctypes.c_int),
     "sw_load": ([_P, _P, _u64], ctypes.c_int),
     "sw_debug_fail_allocations": ([_i32, _i32], ctypes.c_int),
+    "sw_debug_fail_setups": ([_i32, _i32], ctypes.c_int),
     "sw_destroy": ([_P], ctypes.c_int),
     "sw_set_stream": ([_P, _P], ctypes.c_int),
     "sw_sweep": ([_P, _i32], ctypes.c_int),
@@ -261,6 +262,10 @@ def sw_load(h, data: bytes) -> None:
 
 def sw_debug_fail_allocations(n: int, skip: int = 0) -> None:
     _check(lib().sw_debug_fail_allocations(skip, n), "sw_debug_fail_allocations")
+
+
+def sw_debug_fail_setups(n: int, skip: int = 0) -> None:
+    _check(lib().sw_debug_fail_setups(skip, n), "sw_debug_fail_setups")
 
 
 def sw_destroy(h) -> None:
