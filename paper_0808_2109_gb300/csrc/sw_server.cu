@@ -55,6 +55,7 @@ size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 struct Slab {
     void *p = nullptr;
     int refs = 0;
+    size_t bytes = 0;
 };
 
 struct Job {
@@ -182,10 +183,15 @@ struct sw_server {
 
 namespace {
 
-void free_job_device(Job *j, cudaStream_t st)
+// Gives a job's device memory back and returns the bytes that the budget gets with
+// it: none while other jobs hold the block that this one has a share of.
+size_t free_job_device(Job *j, cudaStream_t st)
 {
+    size_t freed = j->bytes;
     if (j->slab) {
+        freed = 0;
         if (--j->slab->refs == 0) {
+            freed = j->slab->bytes;
             cudaFreeAsync(j->slab->p, st);
             delete j->slab;
         }
@@ -194,6 +200,7 @@ void free_job_device(Job *j, cudaStream_t st)
         cudaFreeAsync(j->block, st);
     }
     j->block = nullptr;
+    return freed;
 }
 
 // One allocation for each group of jobs to admit that share a lane and a number
@@ -211,7 +218,7 @@ void share_blocks(sw_server *s, const std::vector<Job *> &admit)
             while (end < v.size() && (end == at || bytes + v[end]->bytes <= SLAB_MAX)) bytes += v[end++]->bytes;
             void *p = nullptr;
             if (end - at > 1 && cudaMallocAsync(&p, bytes, s->lanes[g.first.first].stream) == cudaSuccess) {
-                Slab *slab = new Slab{p, (int)(end - at)};
+                Slab *slab = new Slab{p, (int)(end - at), bytes};
                 size_t off = 0;
                 for (size_t i = at; i < end; ++i) {
                     v[i]->slab = slab;
@@ -226,9 +233,9 @@ void share_blocks(sw_server *s, const std::vector<Job *> &admit)
     }
 }
 
-// Device memory of a newly admitted job: its share of a slab or one
-// stream-ordered block for all its buffers (their first contents come with those of the lane's other new jobs,
-// init_jobs).
+// Device memory of a newly admitted job: its share of a slab or one stream-ordered
+// block for all its buffers (their first contents come with those of the lane's
+// other new jobs, init_jobs).
 cudaError_t job_alloc(Job *j, cudaStream_t st)
 {
     const bool csz = (j->spec.flags & SW_FLAG_CSIZE) != 0;
@@ -573,6 +580,7 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
     for (int l = 0; l < N_LANES; ++l)
         if (used[l]) lane_err[l] = cudaStreamSynchronize(s->lanes[l].stream);
     std::vector<sw_result> res(done.size());
+    size_t freed = 0;
     const auto now = Clock::now();
     for (size_t i = 0; i < done.size(); ++i) {
         Job *j = done[i];
@@ -596,15 +604,15 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
         r.queued_s = secs(j->t_submit, j->t_admit);
         r.run_s = secs(j->t_admit, now);
         lane_release(ln, j);
-        free_job_device(j, ln.stream);
+        freed += free_job_device(j, ln.stream);
     }
     // the frees complete before the budget counts the bytes as available
     for (int l = 0; l < N_LANES; ++l)
         if (used[l]) cudaStreamSynchronize(s->lanes[l].stream);
     std::lock_guard<std::mutex> lk(s->mu);
+    s->used -= freed;
     for (size_t i = 0; i < done.size(); ++i) {
         Job *j = done[i];
-        s->used -= j->bytes;
         s->finished[j->id] = res[i];
         s->stats.finished += 1;
         s->stats.site_updates += (int64_t)j->spec.L * j->spec.L * j->spec.nsweeps;
@@ -617,15 +625,16 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
 void end_failed(sw_server *s, const std::vector<Job *> &jobs, Lane &ln, int rc)
 {
     cudaGetLastError();
-    for (Job *j : jobs) free_job_device(j, ln.stream);
+    size_t freed = 0;
+    for (Job *j : jobs) freed += free_job_device(j, ln.stream);
     cudaStreamSynchronize(ln.stream);
     std::lock_guard<std::mutex> lk(s->mu);
+    s->used -= freed;
     for (Job *j : jobs) {
         sw_result res{};
         res.status = rc;
         res.L = j->spec.L;
         res.nsweeps = j->spec.nsweeps;
-        s->used -= j->bytes;
         s->finished[j->id] = res;
         s->stats.finished += 1;
         delete j;

@@ -82,3 +82,40 @@ def test_failed_setup_leaves_other_jobs_alone(sw, orc):
             assert_obs_equal(out["obs"], lat.observables())
             np.testing.assert_array_equal(out["spins"], lat.spins())
         _run_one(sw, srv, orc, 6)
+
+
+def _bytes_in_use(sw, srv, specs):
+    """The budget's bytes that these jobs take together, once all of them run."""
+    ids = srv.submit(specs)
+    deadline = time.time() + 60
+    while srv.stats()["active"] < len(specs) and time.time() < deadline:
+        time.sleep(0.001)
+    return ids, srv.stats()["bytes_in_use"]
+
+
+def test_shared_block_stays_charged_until_its_last_job(sw, orc):
+    """Jobs of one lane and length share a block.  One of them fails at its
+    admission: the block stays, and so do its bytes."""
+    spec = {"L": 300, "T": 2.3, "sweeps": 6000, "tile_h": 96}
+    with sw.Server() as srv:
+        _, two = _bytes_in_use(sw, srv, [dict(spec, seed=r) for r in range(2)])
+        srv.wait_all(60.0)
+        sw.sw_debug_fail_allocations(1)
+        try:
+            bad, good = srv.submit([dict(spec, seed=1), dict(spec, seed=2)], want_spins=True)
+            while (got := srv.poll(bad)) is None:
+                time.sleep(0.001)
+        finally:
+            sw.sw_debug_fail_allocations(0)
+        assert got[0].status == sw.SW_ERR_NOMEM
+        held = srv.stats()["bytes_in_use"]
+        assert srv.poll(good) is None   # still running
+        assert held == two
+        srv.wait_all(60.0)
+        res, out = srv.poll(good)
+        assert res.status == 0
+        with sw.Lattice(300, T=2.3, seed=2) as lat:
+            lat.sweep(6000)
+            assert_obs_equal(out["obs"], lat.observables())
+            np.testing.assert_array_equal(out["spins"], lat.spins())
+        assert srv.stats()["bytes_in_use"] == 0
