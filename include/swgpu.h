@@ -339,12 +339,13 @@ typedef struct {
 typedef struct {
     int64_t submitted, admitted, finished, pending, active;
     int64_t site_updates;   /* L*L*nsweeps summed over finished jobs              */
-    size_t bytes_in_use, bytes_budget;
+    size_t bytes_in_use, bytes_budget;   /* bytes_in_use: of admitted jobs        */
     int64_t launches;       /* launch groups run by the worker                    */
 } sw_server_stats;
 
 /* Create a server on the current device with a budget of device bytes for
- * lattice state (0 = 80% of the free memory).  Errors: SW_ERR_NOMEM,
+ * lattice state and the tables that set jobs up and gather their results (these
+ * take what the jobs leave; 0 = 80% of the free memory).  Errors: SW_ERR_NOMEM,
  * SW_ERR_CUDA. */
 int sw_server_create(sw_server **out, size_t device_bytes, uint32_t flags);
 

@@ -163,7 +163,8 @@ struct Lane {
 
 struct sw_server {
     int dev = 0;
-    size_t budget = 0, used = 0;
+    size_t budget = 0, used = 0;   // used: the admitted jobs' blocks
+    size_t workspaces = 0;         // the lanes' workspaces (the worker's; part of the budget beside them)
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     std::deque<Job *> pending;
@@ -277,31 +278,42 @@ cudaError_t job_alloc(Job *j, cudaStream_t st)
 
 constexpr int JOBS_PER_LAUNCH = 32768;   // jobs of one init or gather launch (grid y)
 
-// The lane's workspace with room for `bytes` (used in the order of its stream,
-// given back with the server); null beyond WORKSPACE_MAX or without memory.
+// The lane's workspace with room for `bytes` (used in the order of its stream, kept
+// for the next call and given back with the server or when a job needs its part of
+// the budget); null beyond WORKSPACE_MAX, what the budget has left or without memory.
 constexpr size_t WORKSPACE_MAX = (size_t)64 << 20;
-unsigned char *lane_workspace(Lane &ln, size_t bytes)
+void free_workspace(sw_server *s, Lane &ln)
+{
+    if (!ln.ws) return;
+    std::lock_guard<std::mutex> lk(sw_capture_mutex());
+    cudaFree(ln.ws);   // waits for the work that uses it
+    ln.ws = nullptr;
+    s->workspaces -= ln.ws_cap;
+    ln.ws_cap = 0;
+}
+
+unsigned char *lane_workspace(sw_server *s, Lane &ln, size_t bytes)
 {
     if (bytes <= ln.ws_cap) return ln.ws;
     if (bytes > WORKSPACE_MAX) return nullptr;
-    std::lock_guard<std::mutex> lk(sw_capture_mutex());
-    if (ln.ws) cudaFree(ln.ws);   // waits for the work that uses it
-    ln.ws = nullptr;
-    ln.ws_cap = 0;
     size_t cap = 1 << 16;
     while (cap < bytes) cap *= 2;
+    if (s->used + s->workspaces - ln.ws_cap + cap > s->budget) return nullptr;
+    free_workspace(s, ln);
+    std::lock_guard<std::mutex> lk(sw_capture_mutex());
     if (cudaMalloc(&ln.ws, cap) != cudaSuccess) {
         cudaGetLastError();
         ln.ws = nullptr;
         return nullptr;
     }
     ln.ws_cap = cap;
+    s->workspaces += cap;
     return ln.ws;
 }
 
 // First contents of the new jobs of a lane, in one launch (job by job where there
 // is no memory for their table).
-cudaError_t init_jobs(const std::vector<Job *> &jobs, Lane &ln)
+cudaError_t init_jobs(sw_server *s, const std::vector<Job *> &jobs, Lane &ln)
 {
     if (sw_inject_setup_failure()) return cudaErrorUnknown;
     const cudaStream_t st = ln.stream;
@@ -324,7 +336,7 @@ cudaError_t init_jobs(const std::vector<Job *> &jobs, Lane &ln)
             q.n_zero = j->pcc_words;
             most = std::max({most, q.N, q.n_obs, q.n_zero});
         }
-        unsigned char *ws = n > 1 ? lane_workspace(ln, n * sizeof(JobInit)) : nullptr;
+        unsigned char *ws = n > 1 ? lane_workspace(s, ln, n * sizeof(JobInit)) : nullptr;
         cudaError_t e = cudaSuccess;
         if (ws) {
             e = cudaMemcpyAsync(ws, table.data(), n * sizeof(JobInit), cudaMemcpyHostToDevice, st);
@@ -540,7 +552,7 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
         // workspace: the jobs' table, then their records
         const size_t table_bytes = round256(mine.size() * sizeof(JobGather)), side_bytes = (off - off0) * sizeof(DevObs);
         unsigned char *ws = mine.size() > 1 && mine.size() <= (size_t)JOBS_PER_LAUNCH
-                                ? lane_workspace(s->lanes[l], table_bytes + side_bytes) : nullptr;
+                                ? lane_workspace(s, s->lanes[l], table_bytes + side_bytes) : nullptr;
         if (ws) {
             std::vector<JobGather> table;
             int64_t most = 0;
@@ -657,13 +669,21 @@ void worker_main(sw_server *s)
                 s->cv_work.wait(lk, [s] { return s->stop || !s->pending.empty(); });
                 if (s->stop) break;
             }
-            for (auto it = s->pending.begin(); it != s->pending.end();) {
-                if (s->used + (*it)->bytes <= s->budget) {
-                    s->used += (*it)->bytes;
-                    admit.push_back(*it);
-                    it = s->pending.erase(it);
+            for (size_t at = 0; at < s->pending.size();) {
+                Job *const j = s->pending[at];
+                if (s->used + j->bytes <= s->budget && s->used + s->workspaces + j->bytes > s->budget) {
+                    // it fits but for the lanes' workspaces: they go (no lane runs between
+                    // steps, and a submission only adds to the end of the queue)
+                    lk.unlock();
+                    for (Lane &ln : s->lanes) free_workspace(s, ln);
+                    lk.lock();
+                }
+                if (s->used + s->workspaces + j->bytes <= s->budget) {
+                    s->used += j->bytes;
+                    admit.push_back(j);
+                    s->pending.erase(s->pending.begin() + (std::ptrdiff_t)at);
                 } else {
-                    ++it;
+                    ++at;
                 }
             }
             s->stats.pending = (int64_t)s->pending.size();
@@ -700,7 +720,7 @@ void worker_main(sw_server *s)
         // jobs whose first contents cannot be written leave the lane again before its
         // step: no kernel ever sees memory that nobody wrote
         for (int l = 0; l < N_LANES; ++l)
-            if (!fresh[l].empty() && init_jobs(fresh[l], s->lanes[l]) != cudaSuccess) {
+            if (!fresh[l].empty() && init_jobs(s, fresh[l], s->lanes[l]) != cudaSuccess) {
                 for (Job *j : fresh[l]) {
                     lane_release(s->lanes[l], j);
                     s->running.erase(std::find(s->running.begin(), s->running.end(), j));

@@ -119,3 +119,40 @@ def test_shared_block_stays_charged_until_its_last_job(sw, orc):
             assert_obs_equal(out["obs"], lat.observables())
             np.testing.assert_array_equal(out["spins"], lat.spins())
         assert srv.stats()["bytes_in_use"] == 0
+
+
+def test_workspaces_stay_inside_the_budget(sw, orc):
+    """Jobs that fill the budget leave nothing for the tables that gather their
+    results (64 MiB here): the server then holds no device memory beside them once
+    they are done.  With room left it keeps them, until a job needs that room."""
+    import torch
+    specs = [{"L": 3, "T": 2.3, "sweeps": 6000, "seed": r, "tile_h": 32} for r in range(128)]
+    with sw.Server() as srv:
+        _, total = _bytes_in_use(sw, srv, specs)
+        srv.wait_all(120.0)
+
+    def run(budget):
+        srv = sw.Server(device_bytes=budget)
+        ids = srv.submit(specs)
+        srv.wait_all(120.0)
+        for r in (0, 77, 127):
+            res, out = srv.poll(ids[r])
+            assert res.status == 0
+            assert_obs_equal(out["obs"], orc.sw_chain(3, 1.0, 2.3, r).run(6000))
+        return srv
+
+    def held(srv):
+        """Device bytes that the server itself gives back (the jobs' blocks stay in
+        the allocator's pool)."""
+        torch.cuda.synchronize()
+        free0, _ = torch.cuda.mem_get_info()
+        srv.close()
+        return torch.cuda.mem_get_info()[0] - free0
+
+    assert held(run(total)) < 48 << 20
+    srv = run(4 * total)   # the workspace is kept ...
+    (i,) = srv.submit([{"L": 3, "T": 2.3, "sweeps": int(3.9 * 128 * 6000), "seed": 1, "tile_h": 32}])
+    while srv.stats()["pending"]:
+        time.sleep(0.001)
+    assert srv.stats()["bytes_in_use"] + (64 << 20) > 4 * total
+    assert held(srv) < 48 << 20   # ... and given back for a job that needs all of the budget
