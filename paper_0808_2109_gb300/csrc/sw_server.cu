@@ -146,6 +146,10 @@ struct Lane {
     int32_t *jbase_dev = nullptr;
     unsigned char *ws = nullptr;   // workspace (tables and gathered records)
     size_t ws_cap = 0;
+    // host sides of copies in flight: a copy from pageable memory may outlast its call,
+    // so they live until the lane's step has been waited for
+    std::vector<JobInit> init_table;
+    int32_t jbase_host = 0;
     std::vector<Replica> reps_host;
     std::vector<int32_t> tile_rep_host;
     std::vector<Job *> slot_job;
@@ -317,9 +321,10 @@ cudaError_t init_jobs(sw_server *s, const std::vector<Job *> &jobs, Lane &ln)
 {
     if (sw_inject_setup_failure()) return cudaErrorUnknown;
     const cudaStream_t st = ln.stream;
+    ln.init_table.resize(jobs.size());
     for (size_t at = 0; at < jobs.size(); at += JOBS_PER_LAUNCH) {
         const size_t n = std::min<size_t>(jobs.size() - at, JOBS_PER_LAUNCH);
-        std::vector<JobInit> table(n);
+        JobInit *table = ln.init_table.data() + at;
         int64_t most = 0;
         for (size_t i = 0; i < n; ++i) {
             const Job *j = jobs[at + i];
@@ -339,7 +344,7 @@ cudaError_t init_jobs(sw_server *s, const std::vector<Job *> &jobs, Lane &ln)
         unsigned char *ws = n > 1 ? lane_workspace(s, ln, n * sizeof(JobInit)) : nullptr;
         cudaError_t e = cudaSuccess;
         if (ws) {
-            e = cudaMemcpyAsync(ws, table.data(), n * sizeof(JobInit), cudaMemcpyHostToDevice, st);
+            e = cudaMemcpyAsync(ws, table, n * sizeof(JobInit), cudaMemcpyHostToDevice, st);
             if (e == cudaSuccess) e = enqueue_jobs_init(reinterpret_cast<const JobInit *>(ws), (int)n, most, st);
         } else {
             for (size_t i = 0; i < n && e == cudaSuccess; ++i) e = enqueue_job_init(table[i], most, st);
@@ -535,6 +540,7 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
     // by job where there is no memory for that
     std::vector<size_t> at(done.size());
     std::vector<cudaError_t> err(done.size(), cudaSuccess);
+    std::vector<JobGather> tables[N_LANES];   // (alive until the lanes have been waited for)
     bool used[N_LANES] = {};
     size_t off = 0;
     for (int l = 0; l < N_LANES; ++l) {
@@ -554,7 +560,7 @@ void retire_all(sw_server *s, const std::vector<Job *> &done)
         unsigned char *ws = mine.size() > 1 && mine.size() <= (size_t)JOBS_PER_LAUNCH
                                 ? lane_workspace(s, s->lanes[l], table_bytes + side_bytes) : nullptr;
         if (ws) {
-            std::vector<JobGather> table;
+            std::vector<JobGather> &table = tables[l];
             int64_t most = 0;
             for (size_t i : mine) {
                 const Job *j = done[i];
@@ -755,8 +761,8 @@ void worker_main(sw_server *s)
                     s->worker_error = SW_ERR_CUDA;
                 }
             }
-            const int32_t jb = s->launch_index;
-            cudaMemcpyAsync(ln.jbase_dev, &jb, sizeof(int32_t), cudaMemcpyHostToDevice, ln.stream);
+            ln.jbase_host = s->launch_index;
+            cudaMemcpyAsync(ln.jbase_dev, &ln.jbase_host, sizeof(int32_t), cudaMemcpyHostToDevice, ln.stream);
             if (ln.graph) cudaGraphLaunch(ln.graph, ln.stream);
         }
         if (!any) {
