@@ -39,6 +39,16 @@ UNIT = "site-updates/ns"
 ALG_BYTES_PER_SITE = 10            # old spin in, label out, label in, new spin out
 PROFILE_FILE = os.path.join(ROOT, "profiles", "k_tile_L16384_Tc.md")
 LAUNCHES_PER_SWEEP = 3             # tile kernel, merge union, resolve
+ONE_TILE_L, ONE_TILE_SWEEPS = 128, 4096   # a lattice of one tile: sweeps of a call in one launch
+
+
+def launches_of_call(L: int, tile_h: int, sweeps: int) -> int:
+    """The library's kernels of one sw_sweep call on a plain lattice: one launch
+    per ONE_TILE_SWEEPS sweeps where one tile holds it, else the call's first
+    kernel, every sweep's and the last finish."""
+    if L <= min(ONE_TILE_L, tile_h):
+        return -(-sweeps // ONE_TILE_SWEEPS)
+    return LAUNCHES_PER_SWEEP * sweeps + 2
 
 
 def parse_args():
@@ -374,7 +384,9 @@ def run_gb300(args):
     st = lat.profile_read()
     lat.profile(False)
     lat.observables()
-    roofline = tile_roofline(torch, swgpu, stream, w, tile_h, st, ms / (K * w.sweeps))
+    # (a launch of the one-tile kernel runs many sweeps: its time is counted a sweep)
+    starts = st["tile_launches"] if st["merge_groups"] else prof_steps * w.sweeps
+    roofline = tile_roofline(torch, swgpu, stream, w, tile_h, st, starts, ms / (K * w.sweeps))
 
     # ---- end to end through the public API with pinned host buffers
     e2e_steps = max(1, min(K, 5))
@@ -430,7 +442,7 @@ def run_gb300(args):
                                           "seeds": f"{w.seed}..{w.seed + world - 1}"}),
             "tile_h": tile_h, "hbm_gbs_achieved": roofline["achieved"],
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "batched": batched, "served": served,
-            "gpu_launches": K * (LAUNCHES_PER_SWEEP * w.sweeps + 2),   # a call: + its first kernel and the last finish
+            "gpu_launches": K * launches_of_call(w.L, tile_h, w.sweeps),
             "clocks": clk, "impl": "gb300",
         }
     if pool is not None:
@@ -440,7 +452,7 @@ def run_gb300(args):
     return out
 
 
-def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
+def tile_roofline(torch, swgpu, stream, w, tile_h, st, starts, ms_per_sweep):
     """Both ceilings of the dominant kernel (the tile kernel), each measured
     in this run: HBM (the algorithmic 10 B/site of a sweep against the
     measured copy bandwidth; the DRAM bytes ncu counted per launch beside it)
@@ -449,10 +461,10 @@ def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
     72% of its cycles with the integer ALU pipe at 63% of its rate (the ncu
     summaries in profiles/)."""
     N = w.L * w.L
-    tile_s = st["tile_ms"] / st["tile_launches"] * 1e-3
+    tile_s = st["tile_ms"] / starts * 1e-3
     peak, peak_src = hbm_peak_gbs()
     achieved = ALG_BYTES_PER_SITE * N / tile_s / 1e9
-    traffic = profile_traffic(kernel_source_sha(), tile_h)
+    traffic = profile_traffic(kernel_source_sha(), tile_h) if st["merge_groups"] else None
     blocks = philox_calls_per_start(w.L)
     philox_peak = measure_philox_peak(torch, swgpu, stream)
     l2_peak = measure_l2_peak(torch, swgpu, stream)
@@ -463,7 +475,7 @@ def tile_roofline(torch, swgpu, stream, w, tile_h, st, ms_per_sweep):
         "frac": round(achieved / peak, 4),
         "traffic": traffic,
         "peak_source": peak_src,
-        "kernel": f"k_tile<{tile_h}> (fused finish/start of a sweep)",
+        "kernel": f"k_tile<{tile_h}> (fused finish/start of a sweep)" if st["merge_groups"] else "k_one (a whole sweep)",
         "bytes_per_site_algorithmic": ALG_BYTES_PER_SITE,
         "units_per_launch": N,
         "tile_kernel_avg_ms": round(tile_s * 1e3, 4),

@@ -223,9 +223,13 @@ int sw_sync(sw_ctx *ctx);
  * CUDA events recorded around them.  (Measurement support: the paper's
  * per-step timings, Sec. II.C, have no other counterpart here.) */
 typedef struct {
-    int64_t tile_launches; /* launches of the tile kernel                   */
+    int64_t tile_launches; /* launches of the tile kernel: a call's sweeps + 1; on a
+                              plain Ising lattice of one tile (L <= 128, no cluster
+                              sizes, topological rule or PCC), whose kernel runs up
+                              to 4096 sweeps of a call, launches of that one        */
     double tile_ms;        /* their summed device time                      */
-    int64_t merge_groups;  /* groups of merge kernels, one a launch of it    */
+    int64_t merge_groups;  /* groups of merge kernels, one a launch of the tile
+                              kernel (the last of a call is empty); 0 there  */
     double merge_ms;       /* summed device time of the merge groups         */
     int64_t tile_sites;    /* L*L (a Potts lattice: L^d)                     */
     int32_t tile_height;   /* rows per tile (tiles are 128 sites wide); 0 on a

@@ -57,11 +57,10 @@ cudaError_t tile_prepare()
 template <int TH>
 cudaError_t launch_one(OneArgs a, cudaStream_t st)
 {
-    constexpr int32_t MOST = 4096;   // about 70 ms at L=128
     const int32_t n = a.nsweeps;
     cudaError_t e = cudaSuccess;
-    for (int32_t at = 0; at < n && e == cudaSuccess; at += MOST) {
-        a.nsweeps = std::min(MOST, n - at);
+    for (int32_t at = 0; at < n && e == cudaSuccess; at += a.nsweeps) {
+        a.nsweeps = std::min(ONE_SWEEPS, n - at);
         k_one<TH><<<1, OneCfg<TH>::NT, sizeof(OneSmem<TH>), st>>>(a);
         e = cudaGetLastError();
         a.sweep0 += (uint64_t)a.nsweeps;
@@ -362,7 +361,7 @@ struct sw_ctx {
     std::vector<cudaEvent_t> ev_pool;      // events owned by the context
     std::vector<cudaEvent_t> ev_marks;     // per launch group: tile start, tile end, merge end
     size_t ev_used = 0;
-    int64_t prof_groups = 0;
+    int64_t prof_groups = 0, prof_merges = 0;
     double prof_tile_ms = 0.0, prof_merge_ms = 0.0;
 };
 
@@ -640,7 +639,7 @@ int run_sweeps(sw_ctx *c, int32_t n)
         c->swept = true;
         return SW_OK;
     }
-    if (c->n_tiles == 1 && !c->pcc && !c->wind && !c->psize && !c->profiling) {
+    if (c->n_tiles == 1 && !c->pcc && !c->wind && !c->psize) {
         OneArgs a{};
         a.L = c->L;
         a.nsweeps = n;
@@ -654,7 +653,22 @@ int run_sweeps(sw_ctx *c, int32_t n)
         a.label = c->label;
         a.bondbits = c->bondbits;
         a.obs = c->obs + c->obs_tail;
-        SW_CUDA(enqueue_one(a, c->stream));
+        if (c->profiling) {
+            for (int32_t at = 0; at < n; at += a.nsweeps) {
+                cudaEvent_t e0, e1;
+                SW_CUDA(next_event(c, &e0));
+                SW_CUDA(next_event(c, &e1));
+                a.nsweeps = std::min(ONE_SWEEPS, n - at);
+                SW_CUDA(cudaEventRecord(e0, c->stream));
+                SW_CUDA(enqueue_one(a, c->stream));
+                SW_CUDA(cudaEventRecord(e1, c->stream));
+                c->ev_marks.insert(c->ev_marks.end(), {e0, e1, e1});   // no merge
+                a.sweep0 += (uint64_t)a.nsweeps;
+                a.obs += a.nsweeps;
+            }
+        } else {
+            SW_CUDA(enqueue_one(a, c->stream));
+        }
         c->obs_tail += n;
         c->sweep += (uint64_t)n;
         c->swept = true;
@@ -1021,16 +1035,17 @@ int sw_profile_read(sw_ctx *ctx, sw_kernel_stats *out)
         ctx->prof_tile_ms += t;
         ctx->prof_merge_ms += m;
         ctx->prof_groups += 1;
+        ctx->prof_merges += ctx->ev_marks[i + 1] != ctx->ev_marks[i + 2] ? 1 : 0;
     }
     ctx->ev_marks.clear();
     ctx->ev_used = 0;
     out->tile_launches = ctx->prof_groups;
     out->tile_ms = ctx->prof_tile_ms;
-    out->merge_groups = ctx->prof_groups;
+    out->merge_groups = ctx->prof_merges;
     out->merge_ms = ctx->prof_merge_ms;
     out->tile_sites = ctx->is_potts ? ctx->nsites : (int64_t)ctx->L * ctx->L;
     out->tile_height = ctx->is_potts ? 0 : ctx->TH;
-    ctx->prof_groups = 0;
+    ctx->prof_groups = ctx->prof_merges = 0;
     ctx->prof_tile_ms = ctx->prof_merge_ms = 0.0;
     return SW_OK;
 }

@@ -24,7 +24,9 @@ __attribute__((visibility("hidden"))) cudaError_t enqueue_merge(int TH, const Sw
                                                                 cudaStream_t st, bool chained);
 __attribute__((visibility("hidden"))) cudaError_t enqueue_launch_th(int TH, const SweepArgs &a, bool pcc, int feat,
                                                                     cudaStream_t st, bool chained);
-// All sweeps of a one-tile lattice, L <= 128 (k_one).
+// All sweeps of a one-tile lattice, L <= 128 (k_one), ONE_SWEEPS of them a launch
+// (about 70 ms at L=128).
+constexpr int32_t ONE_SWEEPS = 4096;
 __attribute__((visibility("hidden"))) cudaError_t enqueue_one(const OneArgs &a, cudaStream_t st);
 // Launch groups j = 0 .. m-1 of one lattice; last: the final one is a call's
 // last and has no merge.
