@@ -138,23 +138,26 @@ constexpr int FIRST_WAVE_SMS = 152;
 // tile table, launch offset, the threshold of a plain lattice) may be read
 // first, and so may draws be made.  No block returns without the wait, so a
 // kernel that has finished implies that all before it have.
-// (Figures here compare the two sides of a rule on the kernels as they were when it
-// was set.)  A kernel lets its successor start first thing, so that short kernels are
-// all in place when their turn comes (L=64: 23.0 us a sweep against 24.9 when they
-// start after the wait and 27.0 without the chain; L=4096, T=3.0: 93.7, 97.9 and
-// 104 us).  Where a grid does not fill the GPU that has a price: blocks started
-// ahead go to the few SMs with room and run crowded there.  So
+// A kernel lets its successor start first thing, so that short kernels are
+// all in place when their turn comes (L=2048: 44.2 us a sweep against 48.5 when the
+// merge kernels let theirs start after their own wait and 49.9 without the chain;
+// L=4096, T=3.0: 85.8, 87.0 and 93.7; L=300 21.5 and, without the chain, 24.7; every
+// option at L=1920 65.4 and 72.7).  Where a grid does not fill the GPU that has a
+// price: blocks started ahead go to the few SMs with room and run crowded there.
+// (Figures with "then" compare the two sides on the kernels as they were when the rule
+// was set.)  So
 //   - the merge kernels of the topological rule and of PCC let theirs start after
-//     their own wait (every option at L=1001: 92 us against 111), and so do those of
-//     32-row tiles and of grids of at most one tile an SM, unless four such grids fit
-//     side by side (32 rows: L=1001 30.9 us against 34.3, L=2048 45.4 against 48.1;
-//     96 rows: L=1200 33.0 against 33.6, but L=2048 49.3 against 44.9; 3D Potts L=80
-//     43.9 against 49.1);
+//     their own wait (every option at L=1001, then 92 us against 111), and so do those
+//     of 32-row tiles and of grids of at most one tile an SM, unless four such grids fit
+//     side by side (32 rows: L=600 23.1 us against 25.1, L=1001 26.9 against 29.4,
+//     L=1200 28.4 against 31.7; 2D Potts L=64, two tiles, 16.5 first thing against 17.8;
+//     3D Potts L=80 then 43.9 against 49.1, but since its tiles have 32 warps 32.5
+//     against 31.7: the line for Potts grids is due for another look);
 //   - the cover kernel of PCC lets the tile kernel start only when it ends (the
-//     tiles of such a lattice have nothing to do before: 2D Potts L=1024 58 us
+//     tiles of such a lattice have nothing to do before: 2D Potts L=1024 then 58 us
 //     against 76);
 //   - the Potts tile kernel under the topological rule, whose unions are long,
-//     lets them start before its codes (3D L=128: 85 us against 109).
+//     lets them start before its codes (3D L=128, then 85 us against 109).
 __device__ __forceinline__ void chain_next()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -264,11 +267,6 @@ __device__ __forceinline__ uint32_t valid_mask(int c, int tw)
     const int n = tw - 32 * c;
     return n >= 32 ? 0xFFFFFFFFu : (n <= 0 ? 0u : ((1u << n) - 1u));
 }
-
-// Resolved final (root | spin << 30) of an edge slot: a representative holds
-// its cluster's, and so does every top or left slot (the ones a neighbour
-// reads for its halo).  Only nfinal is read: the tile kernel that reads a
-// neighbour's finals rewrites that neighbour's nodes concurrently.
 
 // ------------------------------------------------------------ tile geometry
 struct Tile {
@@ -927,7 +925,8 @@ __global__ void __launch_bounds__(TileCfg<TH, RS>::NT, TileCfg<TH, RS>::MINB) k_
         for (int s = tid; s < S / 4; s += NT) cp_async16(sm.u.finfo + 4 * s, nf + 4 * s);
         if (tid < 2) sm.u.finfo[S + tid] = tid ? FINAL_SPIN : 0u;
         // the halos' finals (new spins of the top row of the tile below and of
-        // the left column of the tile to the right)
+        // the left column of the tile to the right).  Every slot of a tile has its
+        // cluster's; the neighbours' nodes are not read: they rewrite them meanwhile.
         if (warp < TWW && tid < t.tw) fb = R.nfinal[(size_t)t.g_down * S + SL::TOP + tid];
         if (tid < t.th) fr = R.nfinal[(size_t)t.g_right * S + SL::LEFT + tid];
     };
@@ -1866,8 +1865,10 @@ __global__ void __launch_bounds__(MergeCfg<TH>::UT, (W ? 40 : 64) / (MergeCfg<TH
 
 // Topological rule: one round of pointer jumping over the representatives'
 // links (the wind unions hang roots under roots, so walks grow longer than on
-// the plain path, which has no such round: without it the merge takes 0.21 ms
-// instead of 0.23 at L=16384, T_c, 64-row tiles, 17 us instead of 20 at L=64).
+// the plain path, which has no such round).  It was kept for a gain of 5% (69.4 -> 66.2
+// us a sweep) on the kernels of its time; with the present ones it still gives 2% at
+// L=1001 (49.0 -> 48.0) and costs elsewhere: L=300 34.6 us a sweep without it and 35.1
+// with, L=2048 62.7 and 68.4, every option at L=1001 49.9 and 52.3, at L=4096 159 and 162.
 template <int TH>
 __global__ void __launch_bounds__(MergeCfg<TH>::MT) k_wind_jump(const SweepArgs a)
 {

@@ -236,9 +236,12 @@ int sw_cuda_fail(cudaError_t e, int line = 0)
 //     96 rows, L=1001 27.5 against 32.2, L=1600 36.6 against 47.1; L=2048 46.3 against
 //     44.9).  PCC and the topological rule pay more for the longer borders: PCC takes
 //     32 rows up to four CTAs an SM (L=1500 58.4 against 61.6, L=1600 64.3 against
-//     62.3), the rule up to one (L=700 43.1 against 46.1, L=1001 49.8 against 48.4) and
-//     together with PCC or cluster sizes up to two (every option at L=1001 52.6 against
-//     55.3, PCC by the rule 51.6 against 52.6 and at L=1200 56.5 against 53.5);
+//     62.3), the rule up to one (L=700 43.7 against 45.4, L=900 49.7 against 47.5,
+//     L=1001 51.4 against 48.9) and together with PCC or cluster sizes up to two (with
+//     cluster sizes L=800 52.2 against 55.1, L=1001 57.9 against 57.9, L=1056 56.2
+//     against 61.1 and, past the line, L=1057 58.3 against 61.8, L=1200 61.2 against 62.6;
+//     every option at L=1001 52.3 against 54.3; PCC by the rule L=1001 51.2 against 51.8,
+//     L=1200 56.5 against 53.2);
 //   - 96 rows (four CTAs fit on an SM, three of 128).
 int pick_tile_height(int L, uint32_t flags, bool pcc)
 {

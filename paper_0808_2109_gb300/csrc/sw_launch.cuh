@@ -44,12 +44,15 @@ __attribute__((visibility("hidden"))) cudaError_t enqueue_jobs_gather(const JobG
 // Whether a chain's kernels ask for the largest shared memory of an SM.  The split
 // between it and the L1 cache changes only on an idle SM: left to itself, an SM with
 // blocks of the merge kernels has room for no tile until they are gone, and the
-// tiles started ahead crowd on the other SMs (L=600 in 64-row tiles 43 us a sweep
-// against 32, 3D Potts L=128 84 against 71, every option at L=1920 81 against 68).
-// The PCC kernels read through L1 (L=1001 52.5 us, with the preference 54.0), and so
-// do the unions of the topological rule, which a grid of one wave does not crowd
-// (L=800 46.1 against 47.9); a grid that leaves half the GPU to its successors has
-// nothing to gain (2D Potts L=64 22.6 against 23.3).
+// tiles started ahead crowd on the other SMs (every option at L=1920 65.4 us a sweep
+// with the preference against 76.3).  The PCC kernels read through L1 (L=1001 46.9 us,
+// with the preference 47.7), and so do the unions of the topological rule, which a grid
+// of one wave does not crowd (L=800 46.4 either way); a grid that leaves half the GPU to
+// its successors has nothing to gain (2D Potts L=64 16.5 either way).  For plain
+// lattices the line was set on 64-row tiles (L=600 32 us against 43) and on Potts tiles
+// of 8 warps (3D L=128 71 against 84), which those sizes no longer have: now L=600 to
+// 2048 are within 1% either way, 2D Potts L=1024 takes 29.0 with the preference against
+// 28.5 and 3D L=128 48.2 against 45.8, so that this part is due for another look.
 inline bool chain_all_shared(int64_t n_tiles, bool pcc, bool wind)
 {
     return !pcc && (wind ? n_tiles > FIRST_WAVE_SMS : 8 * n_tiles > FIRST_WAVE_SMS);

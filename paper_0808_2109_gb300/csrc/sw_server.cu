@@ -210,7 +210,9 @@ size_t free_job_device(Job *j, cudaStream_t st)
 
 // One allocation for each group of jobs to admit that share a lane and a number
 // of sweeps (at most SLAB_MAX bytes each; 512 allocations of their own took 3 of
-// the 30 ms of a batch).  Jobs that get no share allocate their own block.
+// the 30 ms of a batch of equal lengths).  A job that no other new one of its lane
+// equals in length allocates its own block, as every job of a trace of mixed lengths
+// may have to.
 constexpr size_t SLAB_MAX = (size_t)1 << 30;
 void share_blocks(sw_server *s, const std::vector<Job *> &admit)
 {
@@ -465,6 +467,8 @@ void lane_release(Lane &ln, Job *j)
     ln.dirty = true;
 }
 
+// (The grid is the lane's capacity, idle entries included, and only grows: the launch
+// rules that go by the number of tiles go by that, also after a large load has gone.)
 SweepArgs lane_args(Lane &ln)
 {
     SweepArgs a{};
